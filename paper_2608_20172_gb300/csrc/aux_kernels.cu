@@ -128,19 +128,25 @@ __global__ void __launch_bounds__(kWarps * 32) pre_kernel(Problem p, BwdWorkspac
   }
 }
 
-// One block, fixed summation order (deterministic), fp64 accumulation.
-__global__ void __launch_bounds__(1024) dlambda_kernel(BwdWorkspace ws, int n_main, float* out) {
-  __shared__ double red[1024];
+// One block, fixed summation order (deterministic), fp64 accumulation: per thread, then per
+// warp by shuffles, then the warps in order (a tree of barriers over 1024 threads cost 3 us
+// more).
+__global__ void __launch_bounds__(1024) dlambda_kernel(const float* pre, int n_pre,
+                                                       const float* main, int n_main, float* out) {
+  __shared__ double red[32];
   double s = 0.0;
-  const int n = ws.n_pre_blocks + n_main;
-  for (int i = threadIdx.x; i < n; i += 1024) s += (double)ws.dlam_part[i];
-  red[threadIdx.x] = s;
+  for (int i = threadIdx.x; i < n_pre; i += 1024) s += (double)pre[i];
+  for (int i = threadIdx.x; i < n_main; i += 1024) s += (double)main[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = (float)s;
   }
-  if (threadIdx.x == 0) *out = (float)red[0];
 }
 
 cudaError_t launch_pre(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
@@ -152,8 +158,9 @@ cudaError_t launch_pre(const Problem& p, const BwdWorkspace& ws, cudaStream_t s)
   return cudaGetLastError();
 }
 
-cudaError_t launch_dlambda(const Problem& p, const BwdWorkspace& ws, int n_main, cudaStream_t s) {
-  dlambda_kernel<<<1, 1024, 0, s>>>(ws, n_main, p.dlambda);
+cudaError_t launch_dlambda(const Problem& p, const BwdWorkspace& ws, const float* main, int n_main,
+                           cudaStream_t s) {
+  dlambda_kernel<<<1, 1024, 0, s>>>(ws.dlam_part, ws.n_pre_blocks, main, n_main, p.dlambda);
   return cudaGetLastError();
 }
 

@@ -82,14 +82,16 @@ bool supports(relation_dtype dt, int d);
 cudaError_t launch_fwd(const Problem& p, cudaStream_t s);
 cudaError_t launch_bwd(const Problem& p, const BwdWorkspace& ws, cudaStream_t s);
 int main_ctas(const Problem& p);  // tile-kernel CTAs writing a dlambda partial
+float* main_partials(const BwdWorkspace& ws);  // where they write it
 }  // namespace simt
 
 namespace bwd_common {
 // Per-row Self part of the CUDA-core backward (D_i, F_ii, dS_ii and dlambda partials).
 cudaError_t launch_pre(const Problem& p, const BwdWorkspace& ws, cudaStream_t s);
-// Deterministic dlambda reduction of the pre-pass partials and the first n_main tile-kernel
-// partials.
-cudaError_t launch_dlambda(const Problem& p, const BwdWorkspace& ws, int n_main, cudaStream_t s);
+// Deterministic dlambda reduction of the pre-pass partials and the n_main tile-kernel
+// partials at `main`.
+cudaError_t launch_dlambda(const Problem& p, const BwdWorkspace& ws, const float* main, int n_main,
+                           cudaStream_t s);
 }  // namespace bwd_common
 
 namespace tc {

@@ -477,7 +477,8 @@ relation_status relation_bwd_stages(const void* q, const void* k, const void* v,
   cudaError_t e = cudaSuccess;
   if ((stages & 1) && (e = rel::bwd_common::launch_pre(p, ws, s)) != cudaSuccess) return from_cuda(e);
   if ((stages & 2) && (e = rel::simt::launch_bwd(p, ws, s)) != cudaSuccess) return from_cuda(e);
-  if (stages & 4) e = rel::bwd_common::launch_dlambda(p, ws, rel::simt::main_ctas(p), s);
+  if (stages & 4) e = rel::bwd_common::launch_dlambda(p, ws, rel::simt::main_partials(ws),
+                                                   rel::simt::main_ctas(p), s);
   return from_cuda(e);
 }
 
@@ -525,9 +526,9 @@ int relation_launch_count(relation_dtype dt, int d_h, relation_kernel kernel, in
   const int fam = pick_family(kernel, dt, d_h, backward != 0);
   if (fam == 0) return 0;
   if (!backward) return 1;
-  // SIMT: row pre-pass, dK/dV kernel, dQ kernel, dlambda reduction;
+  // SIMT: row pre-pass, tile kernel (dK/dV and dQ CTAs), dlambda reduction;
   // tcgen05: row pass, tile kernel, finalisation (dQ conversion + dlambda reduction)
-  return fam == 2 ? rel::tc::bwd_launches() : 4;
+  return fam == 2 ? rel::tc::bwd_launches() : 3;
 }
 
 relation_status relation_selftest_wait_timeout(int* dev_status, int timeout_us,

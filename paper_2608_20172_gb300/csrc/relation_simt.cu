@@ -5,18 +5,31 @@
 // approximate transcendental instructions) and every (dtype, d_h) the tensor-core
 // kernels do not cover.
 //
-// Forward (Sec. 5.1, App. A.3): one CTA owns 64 query rows of one head; 4 threads
-// share a row, each holding a quarter of q_i and of the Exchange accumulator z.  Key
-// and value tiles of 64 rows are staged in shared memory as fp32.  Per tile the row's
-// Exchange entries E_ij = SiLU(U_ij) (j < i) update the running (m, l, z) state; the
-// diagonal entry gives S_i = sigmoid(U_ii / tau_S) and is kept out of the scan.  The
-// epilogue applies the count correction and the Self-Exchange split:
+// Work split.  A CTA of W warps owns 8 W rows of one head (queries in the forward and dQ,
+// keys in dK / dV), eight per warp, and walks the other side in staged tiles of 64 rows.
+// Within a warp, lane = 16 ty + tx: the products over d (U, dP) give each lane a 4 x 4 tile
+// (rows 4 ty .., the tile's rows 16 i + tx), the products over the tile (z, dV, dK, dQ) a
+// tile of 4 rows x D / 16 columns, so that eight 16-byte shared-memory reads feed 64
+// multiply-adds (32 packed ones in the products over d).  The rows of a warp meet no other
+// warp's: the weights pass between the two kinds of product through a warp-private
+// [8][64] buffer.  Bound: shared-memory bandwidth and the FP32 pipe (backward: 78 % of the
+// wavefronts, 58 % of the pipe), 2 + 7 products of d_h over the causal pairs (forward +
+// backward); the forward's longest CTAs also end alone.  Measured, B 2, H 8, T 1000, d 64,
+// forward + backward: 1478 -> 331 us (forward 567 -> 107, backward tiles 920 -> 209) against a
+// thread per quarter row (one 16-byte shared read per four multiply-adds, two shuffles per
+// entry); B 1, H 2, T 128, d 32: 49 -> 11 and 77 -> 12 us.
+//
+// Forward (Sec. 5.1, App. A.3): per tile the row's Exchange entries E_ij = SiLU(U_ij) (j < i)
+// update the running (m, l, z) state; the diagonal entry gives S_i = sigmoid(U_ii / tau_S)
+// and is kept out of the scan.  The epilogue applies the count correction and the
+// Self-Exchange split:
 //   A_i = m + log l - lambda log i, g_i = sigmoid(A_i - S_i),
 //   Y_i = (1 - g_i) v_i + g_i z / l,  logZ_i = logaddexp(S_i, A_i)   (App. A.3.5).
 //
 // Backward (App. A.1.7): the Self part and D_i come from the shared row kernel
-// (bwd_common.cu); a key-stationary kernel accumulates dK, dV over query tiles and a
-// query-stationary kernel accumulates dQ over key tiles, both recomputing
+// (aux_kernels.cu); one launch holds key-stationary CTAs that accumulate dK, dV over query
+// tiles and query-stationary CTAs that accumulate dQ over key tiles (together, so that a
+// short sequence fills more of the GPU), both recomputing
 //   P_ij = exp(E_ij - lambda log i - logZ_i), dR_ij = P_ij (dO_i . v_j - D_i),
 //   dS_ij = dR_ij SiLU'(u_ij)  for j < i.
 // No atomics: every output element is written by exactly one thread.
@@ -28,9 +41,15 @@
 namespace rel {
 namespace simt {
 
-constexpr int kRows = 64;     // query (or key) rows per CTA
-constexpr int kTile = 64;     // rows per staged tile
-constexpr int kThreads = 256; // 4 threads per row
+constexpr int kTile = 64;       // rows per staged tile
+constexpr int kWarpRows = 8;    // rows per warp
+constexpr int PW = kTile + 4;   // row stride of the warp-private weight buffer
+// shared-memory row stride of a staged tile: 16 consecutive rows' 16-byte reads spread over
+// the banks (two wavefronts for 256 bytes)
+template <int D>
+struct Ld {
+  static constexpr int V = D + 4;
+};
 
 template <typename TI>
 struct IO;
@@ -39,8 +58,14 @@ struct IO<float> {
   static __device__ __forceinline__ float4 load4(const float* p) {
     return *reinterpret_cast<const float4*>(p);
   }
+  static __device__ __forceinline__ float2 load2(const float* p) {
+    return *reinterpret_cast<const float2*>(p);
+  }
   static __device__ __forceinline__ void store4(float* p, float4 v) {
     *reinterpret_cast<float4*>(p) = v;
+  }
+  static __device__ __forceinline__ void store2(float* p, float2 v) {
+    *reinterpret_cast<float2*>(p) = v;
   }
 };
 template <>
@@ -52,6 +77,9 @@ struct IO<__nv_bfloat16> {
     float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
     return make_float4(fa.x, fa.y, fb.x, fb.y);
   }
+  static __device__ __forceinline__ float2 load2(const __nv_bfloat16* p) {
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
+  }
   static __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
     __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y);
     __nv_bfloat162 b = __floats2bfloat162_rn(v.z, v.w);
@@ -60,173 +88,316 @@ struct IO<__nv_bfloat16> {
     raw.y = *reinterpret_cast<uint32_t*>(&b);
     *reinterpret_cast<uint2*>(p) = raw;
   }
+  static __device__ __forceinline__ void store2(__nv_bfloat16* p, float2 v) {
+    *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v.x, v.y);
+  }
 };
 
-__device__ __forceinline__ float sigmoidf_acc(float x) { return 1.0f / (1.0f + expf(-x)); }
+// The denominator is at least 1: __fdividef (2 ulp, 0 for a denominator above 2^126) takes no
+// branch, so that a lane's 16 entries overlap; the IEEE division's range check kept them apart.
+__device__ __forceinline__ float sigmoidf_acc(float x) { return __fdividef(1.0f, 1.0f + expf(-x)); }
 
-// Thread `part` of a row group owns the float4 chunks part, part + 4, part + 8, ...
+// A lane's columns of a row of D: D = 32: 2 tx .., D = 64: 4 tx .., D = 128: 4 tx .. and
+// 64 + 4 tx ..
 template <int D>
-struct Chunks {
-  static constexpr int N = D / 16;  // float4 chunks per thread
-  static __device__ __forceinline__ int col(int part, int c) { return (part + 4 * c) * 4; }
+struct Cols {
+  static constexpr int N = D / 16;
+  static constexpr int V = N < 4 ? N : 4;  // per access
+  static __device__ __forceinline__ int at(int tx, int c) { return (c / V) * 64 + tx * V; }
 };
-
 template <typename TI, int D>
-__device__ __forceinline__ void load_row_chunks(const TI* row, int part, float (&x)[D / 4]) {
+__device__ __forceinline__ void load_cols(const TI* row, int tx, float (&x)[D / 16]) {
+  using C = Cols<D>;
 #pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 t = IO<TI>::load4(row + Chunks<D>::col(part, c));
-    x[4 * c + 0] = t.x; x[4 * c + 1] = t.y; x[4 * c + 2] = t.z; x[4 * c + 3] = t.w;
+  for (int c = 0; c < C::N; c += C::V) {
+    if constexpr (C::V == 2) {
+      const float2 t = IO<TI>::load2(row + C::at(tx, c));
+      x[c] = t.x; x[c + 1] = t.y;
+    } else {
+      const float4 t = IO<TI>::load4(row + C::at(tx, c));
+      x[c] = t.x; x[c + 1] = t.y; x[c + 2] = t.z; x[c + 3] = t.w;
+    }
   }
 }
-
-template <int D>
-__device__ __forceinline__ float dot_part(const float (&x)[D / 4], const float* srow, int part) {
-  float acc = 0.f;
-#pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 t = *reinterpret_cast<const float4*>(srow + Chunks<D>::col(part, c));
-    acc = fmaf(x[4 * c + 0], t.x, acc);
-    acc = fmaf(x[4 * c + 1], t.y, acc);
-    acc = fmaf(x[4 * c + 2], t.z, acc);
-    acc = fmaf(x[4 * c + 3], t.w, acc);
-  }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  return acc;
-}
-
-template <int D>
-__device__ __forceinline__ void axpy_part(float (&y)[D / 4], float a, const float* srow, int part) {
-#pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 t = *reinterpret_cast<const float4*>(srow + Chunks<D>::col(part, c));
-    y[4 * c + 0] = fmaf(a, t.x, y[4 * c + 0]);
-    y[4 * c + 1] = fmaf(a, t.y, y[4 * c + 1]);
-    y[4 * c + 2] = fmaf(a, t.z, y[4 * c + 2]);
-    y[4 * c + 3] = fmaf(a, t.w, y[4 * c + 3]);
-  }
-}
-
-// Stage rows [r0, r0 + kTile) of one head of `src` into shared memory as fp32
-// (rows >= T are zero).
 template <typename TI, int D>
-__device__ __forceinline__ void stage_tile(float* dst, const TI* src, long long sT, int r0, int T) {
-  for (int idx = threadIdx.x; idx < kTile * (D / 4); idx += kThreads) {
-    int rr = idx / (D / 4), c4 = idx % (D / 4);
-    int r = r0 + rr;
-    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < T) t = IO<TI>::load4(src + (long long)r * sT + 4 * c4);
-    *reinterpret_cast<float4*>(dst + rr * D + 4 * c4) = t;
+__device__ __forceinline__ void store_cols(TI* row, int tx, const float (&x)[D / 16]) {
+  using C = Cols<D>;
+#pragma unroll
+  for (int c = 0; c < C::N; c += C::V) {
+    if constexpr (C::V == 2)
+      IO<TI>::store2(row + C::at(tx, c), make_float2(x[c], x[c + 1]));
+    else
+      IO<TI>::store4(row + C::at(tx, c), make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]));
   }
+}
+
+// Stage `rows` rows from r0 of one head into shared memory as fp32 (rows >= T are zero).
+// fp32 rows go by cp.async (16 bytes, zero-filled past T) and are complete after
+// stage_wait and a barrier; bf16 rows are converted on the way.
+template <typename TI, int D, int NT>
+__device__ __forceinline__ void stage(float* dst, const TI* src, long long sT, int r0, int rows,
+                                      int T) {
+  constexpr int LD = Ld<D>::V;
+  for (int idx = threadIdx.x; idx < rows * (D / 4); idx += NT) {
+    const int rr = idx / (D / 4), c4 = idx % (D / 4);
+    const int r = r0 + rr;
+    float* to = dst + rr * LD + 4 * c4;
+    if constexpr (sizeof(TI) == 4) {
+      const TI* from = src + (long long)min(r, T - 1) * sT + 4 * c4;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(to)), "l"(from),
+                   "r"(r < T ? 16 : 0)
+                   : "memory");
+    } else {
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < T) t = IO<TI>::load4(src + (long long)r * sT + 4 * c4);
+      *reinterpret_cast<float4*>(to) = t;
+    }
+  }
+}
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void stage_wait() {  // all but the last N groups have landed
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// s[r][i] = a_(4 ty + r) . b_(16 i + tx): rows of a (the warp's eight) and of a staged tile
+template <int D>
+__device__ __forceinline__ void dots(const float* a, const float* b, int ty, int tx,
+                                     float (&s)[4][4]) {
+  constexpr int LD = Ld<D>::V;
+  float2 acc[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[r][i] = make_float2(0.f, 0.f);
+  const float* ar = a + 4 * ty * LD;
+  const float* br = b + tx * LD;
+#pragma unroll 4
+  for (int d = 0; d < D; d += 4) {
+    float4 x[4], y[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(ar + r * LD + d);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[i] = *reinterpret_cast<const float4*>(br + 16 * i * LD + d);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[r][i] = __ffma2_rn(make_float2(x[r].x, x[r].y), make_float2(y[i].x, y[i].y), acc[r][i]);
+        acc[r][i] = __ffma2_rn(make_float2(x[r].z, x[r].w), make_float2(y[i].z, y[i].w), acc[r][i]);
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[r][i] = acc[r][i].x + acc[r][i].y;
+}
+
+// z[r] += sum_(k in [k0, k1)) w[4 ty + r][k] b_k over the lane's columns; k0, k1 multiples of
+// 4.  MASK: only the entries with use(r, k), so that a masked row of b (which may hold
+// anything) never enters, not even times zero.
+template <int D, bool MASK, typename F>
+__device__ __forceinline__ void axpys(const float* w, const float* b, int ty, int tx, int k0,
+                                      int k1, float (&z)[4][D / 16], F use) {
+  constexpr int LD = Ld<D>::V;
+  const float* wr = w + 4 * ty * PW;
+#pragma unroll 2
+  for (int k = k0; k < k1; k += 4) {
+    float4 p4[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) p4[r] = *reinterpret_cast<const float4*>(wr + r * PW + k);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      float v[D / 16];
+      load_cols<float, D>(b + (k + e) * LD, tx, v);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float pv = e == 0 ? p4[r].x : e == 1 ? p4[r].y : e == 2 ? p4[r].z : p4[r].w;
+        if (!MASK || use(r, k + e)) {
+#pragma unroll
+          for (int c = 0; c < D / 16; ++c) z[r][c] = fmaf(pv, v[c], z[r][c]);
+        }
+      }
+    }
+  }
+}
+
+// Sum / maximum over the 16 lanes that share a row
+__device__ __forceinline__ float row_sum(float x) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+__device__ __forceinline__ float row_max(float x) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
 }
 
 // ---------------------------------------------------------------------------
 // Forward
 // ---------------------------------------------------------------------------
-template <typename TI, int D>
-__global__ void __launch_bounds__(kThreads) fwd_kernel(Problem p) {
+template <int D, int W>
+constexpr size_t fwd_smem() {
+  return (size_t)(kWarpRows * W + 2 * kTile) * Ld<D>::V * 4 + (size_t)W * kWarpRows * PW * 4;
+}
+
+template <typename TI, int D, int W>
+__global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
+  constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
   extern __shared__ float4 smem_f4[];
-  float* Ks = reinterpret_cast<float*>(smem_f4);
-  float* Vs = Ks + kTile * D;
-  const int rl = threadIdx.x >> 2, part = threadIdx.x & 3;
-  const int bh = blockIdx.y, b = bh / p.H, h = bh % p.H;
-  const int q0 = blockIdx.x * kRows;
-  const int r = q0 + rl;
-  const bool row_ok = r < p.T;
+  float* Qs = reinterpret_cast<float*>(smem_f4);
+  float* Ks = Qs + ROWS * LD;
+  float* Vs = Ks + kTile * LD;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
+  float* Pw = Vs + kTile * LD + warp * kWarpRows * PW;
+  const float* Qw = Qs + warp * kWarpRows * LD;
+  const int BH = p.B * p.H;
+  const int qt = n_t - 1 - (int)(blockIdx.x / BH);  // most key tiles first
+  const int bh = (int)(blockIdx.x % BH), b = bh / p.H, h = bh % p.H;
+  const int q0 = qt * ROWS;
+  const int r0 = q0 + warp * kWarpRows + 4 * ty;  // the lane's rows r0 .. r0 + 3
   const long long base = (long long)b * p.sB + (long long)h * p.sH;
   const TI* Q = reinterpret_cast<const TI*>(p.q) + base;
   const TI* K = reinterpret_cast<const TI*>(p.k) + base;
   const TI* V = reinterpret_cast<const TI*>(p.v) + base;
 
-  float qv[D / 4], z[D / 4];
+  float z[4][D / 16], m[4], l[4], u_self[4];
 #pragma unroll
-  for (int c = 0; c < D / 4; ++c) { qv[c] = 0.f; z[c] = 0.f; }
-  if (row_ok) load_row_chunks<TI, D>(Q + (long long)r * p.sT, part, qv);
-
-  float m = -INFINITY, l = 0.f, s_self = 0.f;
-  const int kend = min(p.T, q0 + kRows);
+  for (int r = 0; r < 4; ++r) {
+    m[r] = -INFINITY;
+    l[r] = u_self[r] = 0.f;
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) z[r][c] = 0.f;
+  }
+  const int kend = min(p.T, q0 + ROWS);
+  stage<TI, D, NT>(Qs, Q, p.sT, q0, ROWS, p.T);
+  stage<TI, D, NT>(Ks, K, p.sT, 0, kTile, p.T);
+  stage_commit();
+  stage<TI, D, NT>(Vs, V, p.sT, 0, kTile, p.T);
+  stage_commit();
   for (int k0 = 0; k0 < kend; k0 += kTile) {
-    __syncthreads();
-    stage_tile<TI, D>(Ks, K, p.sT, k0, p.T);
-    stage_tile<TI, D>(Vs, V, p.sT, k0, p.T);
-    __syncthreads();
-    float e[kTile];
-    float mt = -INFINITY;
+    stage_wait<1>();
+    __syncthreads();  // Q and K are in
+    const int hist = q0 + warp * kWarpRows + kWarpRows - 1 - k0;  // the warp's last history key + 1
+    float sc[4];
+    {
+      float e[4][4];
+      dots<D>(Qw, Ks, ty, tx, e);
 #pragma unroll
-    for (int jj = 0; jj < kTile; ++jj) {
-      const float u = dot_part<D>(qv, Ks + jj * D, part) * p.inv_sqrt_d;
-      const int j = k0 + jj;
-      float ev = -INFINITY;
-      if (j < r) {
-        ev = u * sigmoidf_acc(u);                    // E_ij = SiLU(U_ij)
-      } else if (j == r) {
-        s_self = sigmoidf_acc(u / p.tau_s);          // S_i = sigmoid(U_ii / tau_S)
+      for (int r = 0; r < 4; ++r) {
+        float mt = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int j = k0 + 16 * i + tx;
+          const float u = e[r][i] * p.inv_sqrt_d;
+          const float ev = u * sigmoidf_acc(u);        // E_ij = SiLU(U_ij)
+          e[r][i] = j < r0 + r ? ev : -INFINITY;
+          u_self[r] = j == r0 + r ? u : u_self[r];
+          mt = fmaxf(mt, e[r][i]);
+        }
+        const float mn = fmaxf(m[r], row_max(mt));
+        // no history seen yet (mn = -inf): every weight is 0
+        sc[r] = mn == -INFINITY ? 1.f : expf(m[r] - mn);
+        float ls = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float w = mn == -INFINITY ? 0.f : expf(e[r][i] - mn);
+          ls += w;
+          Pw[(4 * ty + r) * PW + 16 * i + tx] = w;
+        }
+        l[r] = fmaf(l[r], sc[r], ls);  // this lane's share of the row sum
+        m[r] = mn;
       }
-      e[jj] = ev;
-      mt = fmaxf(mt, ev);
     }
-    const float mn = fmaxf(m, mt);
-    if (mn == -INFINITY) continue;                   // no history seen yet
-    const float sc = expf(m - mn);                   // e^{m - m'}; 0 for the empty state
-    l *= sc;
+    __syncthreads();  // K has been read
+    if (k0 + kTile < kend) stage<TI, D, NT>(Ks, K, p.sT, k0 + kTile, kTile, p.T);
+    stage_commit();
+    stage_wait<1>();
+    __syncthreads();  // V is in
 #pragma unroll
-    for (int c = 0; c < D / 4; ++c) z[c] *= sc;
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int jj = 0; jj < kTile; ++jj) {
-      const float w = expf(e[jj] - mn);             // exp(-inf) = 0 outside the history
-      l += w;
-      axpy_part<D>(z, w, Vs + jj * D, part);
-    }
-    m = mn;
+      for (int c = 0; c < D / 16; ++c) z[r][c] *= sc[r];
+    // keys every row of the warp has in its history, then the (at most 8) mixed ones
+    const int full = max(0, min(kTile, (hist - kWarpRows + 1) & ~3));
+    const int some = max(0, min(kTile, (hist + 3) & ~3));
+    axpys<D, false>(Pw, Vs, ty, tx, 0, full, z, [](int, int) { return true; });
+    axpys<D, true>(Pw, Vs, ty, tx, full, some, z, [&](int r, int k) { return k0 + k < r0 + r; });
+    __syncthreads();  // V has been read
+    if (k0 + kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + kTile, kTile, p.T);
+    stage_commit();
   }
-  if (!row_ok) return;
 
-  float g = 0.f, lz = s_self;
-  float inv_l = 0.f, fself = 1.0f;  // F_ii = 1 - g: the Self flow
-  if (r > 0 && l > 0.f) {
-    const float A = m + logf(l) - p.lambda * logf((float)(r + 1));
-    g = 1.0f / (1.0f + expf(s_self - A));
-    fself = 1.0f / (1.0f + expf(A - s_self));
-    const float hi = fmaxf(s_self, A), lo = fminf(s_self, A);
-    lz = hi + log1pf(expf(lo - hi));
-    inv_l = 1.0f / l;
-  }
-  float vi[D / 4];
-  load_row_chunks<TI, D>(V + (long long)r * p.sT, part, vi);
-  TI* Y = reinterpret_cast<TI*>(p.out) + base + (long long)r * p.sT;
 #pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 y;
-    y.x = (1.f - g) * vi[4 * c + 0] + g * (z[4 * c + 0] * inv_l);
-    y.y = (1.f - g) * vi[4 * c + 1] + g * (z[4 * c + 1] * inv_l);
-    y.z = (1.f - g) * vi[4 * c + 2] + g * (z[4 * c + 2] * inv_l);
-    y.w = (1.f - g) * vi[4 * c + 3] + g * (z[4 * c + 3] * inv_l);
-    IO<TI>::store4(Y + Chunks<D>::col(part, c), y);
+  for (int r = 0; r < 4; ++r) {
+    l[r] = row_sum(l[r]);
+    u_self[r] = row_sum(u_self[r]);  // held by the lane whose key it was, 0 elsewhere
   }
-  if (part == 0) {
-    p.logz[(long long)bh * p.T + r] = lz;
-    if (p.fself) p.fself[(long long)bh * p.T + r] = fself;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int row = r0 + r;
+    if (row >= p.T) continue;
+    const float lr = l[r], S = 1.0f / (1.0f + expf(-u_self[r] / p.tau_s));
+    float g = 0.f, lz = S;
+    float inv_l = 0.f, fself = 1.0f;  // F_ii = 1 - g: the Self flow
+    if (row > 0 && lr > 0.f) {
+      const float A = m[r] + logf(lr) - p.lambda * logf((float)(row + 1));
+      g = 1.0f / (1.0f + expf(S - A));
+      fself = 1.0f / (1.0f + expf(A - S));
+      const float hi = fmaxf(S, A), lo = fminf(S, A);
+      lz = hi + log1pf(expf(lo - hi));
+      inv_l = 1.0f / lr;
+    }
+    float y[D / 16];
+    load_cols<TI, D>(V + (long long)row * p.sT, tx, y);
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) y[c] = (1.f - g) * y[c] + g * (z[r][c] * inv_l);
+    store_cols<TI, D>(reinterpret_cast<TI*>(p.out) + base + (long long)row * p.sT, tx, y);
+    if (tx == 0) {
+      p.logz[(long long)bh * p.T + row] = lz;
+      if (p.fself) p.fself[(long long)bh * p.T + row] = fself;
+    }
   }
 }
 
 // ---------------------------------------------------------------------------
-// Backward: dK, dV (key-stationary)
+// Backward
 // ---------------------------------------------------------------------------
-template <typename TI, int D>
-__global__ void __launch_bounds__(kThreads) bwd_dkdv_kernel(Problem p, BwdWorkspace ws) {
-  extern __shared__ float4 smem_f4[];
-  float* Qs = reinterpret_cast<float*>(smem_f4);
-  float* Gs = Qs + kTile * D;        // dO tile
-  float* cs = Gs + kTile * D;        // -lambda log i - logZ_i
-  float* Ds = cs + kTile;            // D_i
-  float* ws_l = Ds + kTile;          // log i * F_ii (Exchange weight of dlambda)
-  __shared__ float red[kThreads / 32];
-  const int rl = threadIdx.x >> 2, part = threadIdx.x & 3;
-  const int bh = blockIdx.y, b = bh / p.H, h = bh % p.H;
-  const int k0 = blockIdx.x * kRows;
-  const int j = k0 + rl;
-  const bool key_ok = j < p.T;
+template <int D, int W>
+constexpr size_t bwd_smem() {
+  return (size_t)(2 * kWarpRows * W + 2 * kTile) * Ld<D>::V * 4 +
+         (size_t)W * kWarpRows * PW * 4 + 3 * kTile * 4 + W * 4;
+}
+
+// P_ij and dS_ij of one Exchange pair: ci = -lambda log i - logZ_i
+__device__ __forceinline__ void pair_grad(float u, float dP, float ci, float Di, float& P,
+                                          float& dR, float& dS) {
+  const float sg = sigmoidf_acc(u);
+  const float E = u * sg;
+  P = expf(E + ci);
+  dR = P * (dP - Di);
+  dS = dR * (sg + E * (1.f - sg));  // SiLU'(u) = sigma + E (1 - sigma)
+}
+
+// dK, dV (key-stationary): the CTA's ROWS keys over the query tiles from its first key on
+template <typename TI, int D, int W>
+__device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& ws, float* dlam_part,
+                                         float* smem, int kt, int bh) {
+  constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
+  float* Ks = smem;
+  float* Vs = Ks + ROWS * LD;
+  float* Qs = Vs + ROWS * LD;
+  float* Gs = Qs + kTile * LD;  // dO tile
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
+  float* Pw = Gs + kTile * LD + warp * kWarpRows * PW;
+  float* cs = Gs + kTile * LD + W * kWarpRows * PW;  // -lambda log i - logZ_i
+  float* Ds = cs + kTile;                            // D_i
+  float* wl = Ds + kTile;                            // log i * F_ii (Exchange weight of dlambda)
+  float* red = wl + kTile;
+  const int b = bh / p.H, h = bh % p.H;
+  const int k0 = kt * ROWS;
+  const int j0 = k0 + warp * kWarpRows + 4 * ty;  // the lane's keys j0 .. j0 + 3
   const long long base = (long long)b * p.sB + (long long)h * p.sH;
   const TI* Q = reinterpret_cast<const TI*>(p.q) + base;
   const TI* K = reinterpret_cast<const TI*>(p.k) + base;
@@ -234,144 +405,184 @@ __global__ void __launch_bounds__(kThreads) bwd_dkdv_kernel(Problem p, BwdWorksp
   const TI* G = reinterpret_cast<const TI*>(p.dout) + base;
   const float* logz = p.logz_in + (long long)bh * p.T;
   const float* Drow = ws.D + (long long)bh * p.T;
+  const float* Fs = ws.F_self + (long long)bh * p.T;
 
-  float kv[D / 4], vv[D / 4], dk[D / 4], dv[D / 4];
+  float dk[4][D / 16], dv[4][D / 16];
 #pragma unroll
-  for (int c = 0; c < D / 4; ++c) { kv[c] = vv[c] = dk[c] = dv[c] = 0.f; }
-  float dlam = 0.f;  // -sum_i log i F_ii dR_ij over this key's Exchange pairs
-  if (key_ok) {
-    load_row_chunks<TI, D>(K + (long long)j * p.sT, part, kv);
-    load_row_chunks<TI, D>(V + (long long)j * p.sT, part, vv);
-  }
-  for (int q0 = k0; q0 < p.T; q0 += kTile) {
-    __syncthreads();
-    stage_tile<TI, D>(Qs, Q, p.sT, q0, p.T);
-    stage_tile<TI, D>(Gs, G, p.sT, q0, p.T);
-    for (int ii = threadIdx.x; ii < kTile; ii += kThreads) {
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) dk[r][c] = dv[r][c] = 0.f;
+  float dlam = 0.f;  // -sum_i log i F_ii dR_ij over the lane's Exchange pairs
+  stage<TI, D, NT>(Ks, K, p.sT, k0, ROWS, p.T);
+  stage<TI, D, NT>(Vs, V, p.sT, k0, ROWS, p.T);
+  for (int q0 = k0 / kTile * kTile; q0 < p.T; q0 += kTile) {
+    __syncthreads();  // the previous tile has been read
+    stage<TI, D, NT>(Qs, Q, p.sT, q0, kTile, p.T);
+    stage<TI, D, NT>(Gs, G, p.sT, q0, kTile, p.T);
+    stage_commit();
+    for (int ii = threadIdx.x; ii < kTile; ii += NT) {
       const int i = q0 + ii;
       const float li = logf((float)(i + 1));
       cs[ii] = i < p.T ? -p.lambda * li - logz[i] : -INFINITY;
       Ds[ii] = i < p.T ? Drow[i] : 0.f;
-      ws_l[ii] = i < p.T ? li * ws.F_self[(long long)bh * p.T + i] : 0.f;
+      wl[ii] = i < p.T ? li * Fs[i] : 0.f;
     }
+    stage_wait<0>();
     __syncthreads();
-    for (int ii = 0; ii < kTile; ++ii) {
-      const int i = q0 + ii;
-      const float u = dot_part<D>(kv, Qs + ii * D, part) * p.inv_sqrt_d;
-      const float dP = dot_part<D>(vv, Gs + ii * D, part);
-      if (i > j && i < p.T) {
-        const float sg = sigmoidf_acc(u);
-        const float E = u * sg;
-        const float P = expf(E + cs[ii]);
-        const float dR = P * (dP - Ds[ii]);
-        const float dS = dR * (sg + E * (1.f - sg));   // SiLU'(u) = sigma + E (1 - sigma)
-        dlam = fmaf(-ws_l[ii], dR, dlam);
-        axpy_part<D>(dv, P, Gs + ii * D, part);
-        axpy_part<D>(dk, dS, Qs + ii * D, part);
+    float P[4][4], dS[4][4];
+    dots<D>(Ks + warp * kWarpRows * LD, Qs, ty, tx, P);
+    dots<D>(Vs + warp * kWarpRows * LD, Gs, ty, tx, dS);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int ii = 16 * i + tx, q = q0 + ii;
+      const float ci = cs[ii], Di = Ds[ii], wi = wl[ii];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float pv, dR, ds;
+        pair_grad(P[r][i] * p.inv_sqrt_d, dS[r][i], ci, Di, pv, dR, ds);
+        const bool in = q > j0 + r && q < p.T;
+        P[r][i] = in ? pv : 0.f;
+        dS[r][i] = in ? ds : 0.f;
+        dlam = in ? fmaf(-wi, dR, dlam) : dlam;
+        Pw[(4 * ty + r) * PW + ii] = P[r][i];
       }
     }
-  }
-  // per-CTA dlambda partial (the 4 threads of a key hold the same value: count part 0)
-  float c = part == 0 ? dlam : 0.f;
+    __syncwarp();
+    // queries after every key of the warp, and before them the (at most 8) mixed ones
+    const int first = k0 + warp * kWarpRows + 1 - q0;  // the first query any key takes
+    const int some = max(0, min(kTile, first & ~3));
+    const int full = max(0, min(kTile, (first + kWarpRows - 1 + 3) & ~3));
+    auto use = [&](int r, int k) { return q0 + k > j0 + r; };
+    axpys<D, true>(Pw, Gs, ty, tx, some, full, dv, use);
+    axpys<D, false>(Pw, Gs, ty, tx, full, kTile, dv, use);
+    __syncwarp();
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) Pw[(4 * ty + r) * PW + 16 * i + tx] = dS[r][i];
+    __syncwarp();
+    axpys<D, true>(Pw, Qs, ty, tx, some, full, dk, use);
+    axpys<D, false>(Pw, Qs, ty, tx, full, kTile, dk, use);
+  }
+  // the CTA's dlambda partial
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dlam += __shfl_xor_sync(0xffffffffu, dlam, o);
+  if (lane == 0) red[warp] = dlam;
   __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) t += red[w];
-    ws.dlam_part[ws.n_pre_blocks + blockIdx.y * gridDim.x + blockIdx.x] = t;
+    for (int w = 0; w < W; ++w) t += red[w];
+    dlam_part[kt * (p.B * p.H) + bh] = t;
   }
-  if (!key_ok) return;
   // Self terms of key j: dv_j += F_jj dO_j, dk_j += dS_jj q_j; then the 1/sqrt(d) of U.
-  const long long row = (long long)bh * p.T + j;
-  const float fs = ws.F_self[row], dss = ws.dS_self[row];
-  float qj[D / 4], gj[D / 4];
-  load_row_chunks<TI, D>(Q + (long long)j * p.sT, part, qj);
-  load_row_chunks<TI, D>(G + (long long)j * p.sT, part, gj);
-  TI* dK = reinterpret_cast<TI*>(p.dk) + base + (long long)j * p.sT;
-  TI* dV = reinterpret_cast<TI*>(p.dv) + base + (long long)j * p.sT;
 #pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 a, v4;
-    a.x = (dk[4 * c + 0] + dss * qj[4 * c + 0]) * p.inv_sqrt_d;
-    a.y = (dk[4 * c + 1] + dss * qj[4 * c + 1]) * p.inv_sqrt_d;
-    a.z = (dk[4 * c + 2] + dss * qj[4 * c + 2]) * p.inv_sqrt_d;
-    a.w = (dk[4 * c + 3] + dss * qj[4 * c + 3]) * p.inv_sqrt_d;
-    v4.x = dv[4 * c + 0] + fs * gj[4 * c + 0];
-    v4.y = dv[4 * c + 1] + fs * gj[4 * c + 1];
-    v4.z = dv[4 * c + 2] + fs * gj[4 * c + 2];
-    v4.w = dv[4 * c + 3] + fs * gj[4 * c + 3];
-    IO<TI>::store4(dK + Chunks<D>::col(part, c), a);
-    IO<TI>::store4(dV + Chunks<D>::col(part, c), v4);
+  for (int r = 0; r < 4; ++r) {
+    const int j = j0 + r;
+    if (j >= p.T) continue;
+    const float fs = Fs[j], dss = ws.dS_self[(long long)bh * p.T + j];
+    float qj[D / 16], gj[D / 16];
+    load_cols<TI, D>(Q + (long long)j * p.sT, tx, qj);
+    load_cols<TI, D>(G + (long long)j * p.sT, tx, gj);
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) {
+      qj[c] = (dk[r][c] + dss * qj[c]) * p.inv_sqrt_d;
+      gj[c] = dv[r][c] + fs * gj[c];
+    }
+    store_cols<TI, D>(reinterpret_cast<TI*>(p.dk) + base + (long long)j * p.sT, tx, qj);
+    store_cols<TI, D>(reinterpret_cast<TI*>(p.dv) + base + (long long)j * p.sT, tx, gj);
   }
 }
 
-// ---------------------------------------------------------------------------
-// Backward: dQ (query-stationary)
-// ---------------------------------------------------------------------------
-template <typename TI, int D>
-__global__ void __launch_bounds__(kThreads) bwd_dq_kernel(Problem p, BwdWorkspace ws) {
-  extern __shared__ float4 smem_f4[];
-  float* Ks = reinterpret_cast<float*>(smem_f4);
-  float* Vs = Ks + kTile * D;
-  const int rl = threadIdx.x >> 2, part = threadIdx.x & 3;
-  const int bh = blockIdx.y, b = bh / p.H, h = bh % p.H;
-  const int q0 = blockIdx.x * kRows;
-  const int i = q0 + rl;
-  const bool row_ok = i < p.T;
+// dQ (query-stationary): the CTA's ROWS queries over the key tiles up to its last query
+template <typename TI, int D, int W>
+__device__ __forceinline__ void bwd_dq(const Problem& p, const BwdWorkspace& ws, float* smem,
+                                       int qt, int bh) {
+  constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
+  float* Qs = smem;
+  float* Gs = Qs + ROWS * LD;
+  float* Ks = Gs + ROWS * LD;
+  float* Vs = Ks + kTile * LD;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
+  float* Pw = Vs + kTile * LD + warp * kWarpRows * PW;
+  const int b = bh / p.H, h = bh % p.H;
+  const int q0 = qt * ROWS;
+  const int r0 = q0 + warp * kWarpRows + 4 * ty;  // the lane's queries r0 .. r0 + 3
   const long long base = (long long)b * p.sB + (long long)h * p.sH;
   const TI* Q = reinterpret_cast<const TI*>(p.q) + base;
   const TI* K = reinterpret_cast<const TI*>(p.k) + base;
   const TI* V = reinterpret_cast<const TI*>(p.v) + base;
   const TI* G = reinterpret_cast<const TI*>(p.dout) + base;
-  const long long row = (long long)bh * p.T + i;
 
-  float qv[D / 4], gv[D / 4], dq[D / 4];
+  float dq[4][D / 16], ci[4], Di[4];
 #pragma unroll
-  for (int c = 0; c < D / 4; ++c) { qv[c] = gv[c] = dq[c] = 0.f; }
-  float ci = -INFINITY, Di = 0.f;
-  if (row_ok) {
-    load_row_chunks<TI, D>(Q + (long long)i * p.sT, part, qv);
-    load_row_chunks<TI, D>(G + (long long)i * p.sT, part, gv);
-    ci = -p.lambda * logf((float)(i + 1)) - p.logz_in[row];
-    Di = ws.D[row];
+  for (int r = 0; r < 4; ++r) {
+    const int i = r0 + r;
+    const long long row = (long long)bh * p.T + min(i, p.T - 1);
+    ci[r] = -p.lambda * logf((float)(i + 1)) - p.logz_in[row];
+    Di[r] = ws.D[row];
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) dq[r][c] = 0.f;
   }
-  const int kend = min(p.T, q0 + kRows);
+  const int kend = min(p.T, q0 + ROWS);
+  stage<TI, D, NT>(Qs, Q, p.sT, q0, ROWS, p.T);
+  stage<TI, D, NT>(Gs, G, p.sT, q0, ROWS, p.T);
+  stage<TI, D, NT>(Vs, V, p.sT, 0, kTile, p.T);
+  stage_commit();
   for (int k0 = 0; k0 < kend; k0 += kTile) {
-    __syncthreads();
-    stage_tile<TI, D>(Ks, K, p.sT, k0, p.T);
-    stage_tile<TI, D>(Vs, V, p.sT, k0, p.T);
-    __syncthreads();
-    for (int jj = 0; jj < kTile; ++jj) {
-      const int j = k0 + jj;
-      const float u = dot_part<D>(qv, Ks + jj * D, part) * p.inv_sqrt_d;
-      const float dP = dot_part<D>(gv, Vs + jj * D, part);
-      if (j < i && row_ok) {
-        const float sg = sigmoidf_acc(u);
-        const float E = u * sg;
-        const float P = expf(E + ci);
-        const float dR = P * (dP - Di);
-        const float dS = dR * (sg + E * (1.f - sg));
-        axpy_part<D>(dq, dS, Ks + jj * D, part);
-      }
-    }
-  }
-  if (!row_ok) return;
-  const float dss = ws.dS_self[row];
-  float ki[D / 4];
-  load_row_chunks<TI, D>(K + (long long)i * p.sT, part, ki);
-  TI* dQ = reinterpret_cast<TI*>(p.dq) + base + (long long)i * p.sT;
+    stage<TI, D, NT>(Ks, K, p.sT, k0, kTile, p.T);
+    stage_commit();
+    stage_wait<1>();
+    __syncthreads();  // V (and Q, dO) are in
+    float dS[4][4], u[4][4];
+    dots<D>(Gs + warp * kWarpRows * LD, Vs, ty, tx, dS);
+    stage_wait<0>();
+    __syncthreads();  // V has been read, K is in
+    if (k0 + kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + kTile, kTile, p.T);
+    stage_commit();
+    dots<D>(Qs + warp * kWarpRows * LD, Ks, ty, tx, u);
 #pragma unroll
-  for (int c = 0; c < Chunks<D>::N; ++c) {
-    float4 a;
-    a.x = (dq[4 * c + 0] + dss * ki[4 * c + 0]) * p.inv_sqrt_d;
-    a.y = (dq[4 * c + 1] + dss * ki[4 * c + 1]) * p.inv_sqrt_d;
-    a.z = (dq[4 * c + 2] + dss * ki[4 * c + 2]) * p.inv_sqrt_d;
-    a.w = (dq[4 * c + 3] + dss * ki[4 * c + 3]) * p.inv_sqrt_d;
-    IO<TI>::store4(dQ + Chunks<D>::col(part, c), a);
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float P, dR, ds;
+        pair_grad(u[r][i] * p.inv_sqrt_d, dS[r][i], ci[r], Di[r], P, dR, ds);
+        dS[r][i] = k0 + 16 * i + tx < r0 + r ? ds : 0.f;
+        Pw[(4 * ty + r) * PW + 16 * i + tx] = dS[r][i];
+      }
+    __syncwarp();
+    const int hist = q0 + warp * kWarpRows + kWarpRows - 1 - k0;
+    const int full = max(0, min(kTile, (hist - kWarpRows + 1) & ~3));
+    const int some = max(0, min(kTile, (hist + 3) & ~3));
+    axpys<D, false>(Pw, Ks, ty, tx, 0, full, dq, [](int, int) { return true; });
+    axpys<D, true>(Pw, Ks, ty, tx, full, some, dq, [&](int r, int k) { return k0 + k < r0 + r; });
+    __syncthreads();  // K has been read
   }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int i = r0 + r;
+    if (i >= p.T) continue;
+    const float dss = ws.dS_self[(long long)bh * p.T + i];
+    float ki[D / 16];
+    load_cols<TI, D>(K + (long long)i * p.sT, tx, ki);
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) ki[c] = (dq[r][c] + dss * ki[c]) * p.inv_sqrt_d;
+    store_cols<TI, D>(reinterpret_cast<TI*>(p.dq) + base + (long long)i * p.sT, tx, ki);
+  }
+}
+
+// Even CTAs dK / dV, odd ones dQ, the longest first in both.
+template <typename TI, int D, int W>
+__global__ void __launch_bounds__(32 * W) bwd_kernel(Problem p, BwdWorkspace ws, float* dlam_part,
+                                                     int n_t) {
+  extern __shared__ float4 smem_f4[];
+  float* smem = reinterpret_cast<float*>(smem_f4);
+  const int BH = p.B * p.H;
+  const int t = (int)((blockIdx.x >> 1) / BH), bh = (int)((blockIdx.x >> 1) % BH);
+  if (blockIdx.x & 1)
+    bwd_dq<TI, D, W>(p, ws, smem, n_t - 1 - t, bh);
+  else
+    bwd_dkdv<TI, D, W>(p, ws, dlam_part, smem, t, bh);
 }
 
 // ---------------------------------------------------------------------------
@@ -382,66 +593,74 @@ bool supports(relation_dtype dt, int d) {
   return d == 32 || d == 64 || d == 128;
 }
 
+// Warps per CTA (8 rows each).  Forward / backward tiles in us with 4 and with 2 warps: B 2,
+// H 8, T 1000, d 64: 107 / 209, 104 / 239; B 2, H 4, T 777, d 128: 95 / 175, 92 / 194; B 4, H 8,
+// T 1500, d 32: 189 / 520, 201 / 585; at T 128 alike.  Eight warps, both with IEEE division in
+// the sigmoid: 134 / 236 against 127 / 222, 150 / 215 against 130 / 195, 251 / 586 against
+// 228 / 566.
+constexpr int kWarps = 4;
+
+static int tiles(const Problem& p) {
+  return (p.T + kWarpRows * kWarps - 1) / (kWarpRows * kWarps);
+}
+
 template <typename TI, int D>
 static cudaError_t fwd_t(const Problem& p, cudaStream_t s) {
-  const size_t smem = 2u * kTile * D * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(fwd_kernel<TI, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  constexpr int W = kWarps;
+  constexpr size_t smem = fwd_smem<D, W>();
+  cudaError_t e = cudaFuncSetAttribute(fwd_kernel<TI, D, W>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((p.T + kRows - 1) / kRows, p.B * p.H);
-  fwd_kernel<TI, D><<<grid, kThreads, smem, s>>>(p);
+  const int n_t = tiles(p);
+  const long long grid = (long long)n_t * p.B * p.H;
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  fwd_kernel<TI, D, W><<<(unsigned)grid, 32 * W, smem, s>>>(p, n_t);
   return cudaGetLastError();
 }
 
 template <typename TI, int D>
 static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
-  const size_t smem_kv = 2u * kTile * D * sizeof(float) + 3u * kTile * sizeof(float);
-  const size_t smem_q = 2u * kTile * D * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(bwd_dkdv_kernel<TI, D>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kv);
+  constexpr int W = kWarps;
+  constexpr size_t smem = bwd_smem<D, W>();
+  static_assert(smem <= 232448, "shared memory");
+  cudaError_t e = cudaFuncSetAttribute(bwd_kernel<TI, D, W>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(bwd_dq_kernel<TI, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_q);
-  if (e != cudaSuccess) return e;
-  dim3 grid((p.T + kRows - 1) / kRows, p.B * p.H);
-  bwd_dkdv_kernel<TI, D><<<grid, kThreads, smem_kv, s>>>(p, ws);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  bwd_dq_kernel<TI, D><<<grid, kThreads, smem_q, s>>>(p, ws);
+  const int n_t = tiles(p);
+  const long long grid = 2LL * n_t * p.B * p.H;
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  bwd_kernel<TI, D, W><<<(unsigned)grid, 32 * W, smem, s>>>(p, ws, main_partials(ws), n_t);
   return cudaGetLastError();
 }
 
-int main_ctas(const Problem& p) { return ((p.T + kRows - 1) / kRows) * p.B * p.H; }
+// The tile kernel's dlambda partials, one per dK / dV CTA (at most one per 16 rows): in the
+// tensor-core path's per-query scalars (four floats per row), which this path does not use.
+float* main_partials(const BwdWorkspace& ws) { return ws.stats; }
+int main_ctas(const Problem& p) { return tiles(p) * p.B * p.H; }
+
+template <int D>
+static cudaError_t fwd_d(const Problem& p, cudaStream_t s) {
+  return p.dtype == RELATION_F32 ? fwd_t<float, D>(p, s) : fwd_t<__nv_bfloat16, D>(p, s);
+}
+template <int D>
+static cudaError_t bwd_d(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
+  return p.dtype == RELATION_F32 ? bwd_t<float, D>(p, ws, s) : bwd_t<__nv_bfloat16, D>(p, ws, s);
+}
 
 cudaError_t launch_fwd(const Problem& p, cudaStream_t s) {
-  if (p.dtype == RELATION_F32) {
-    switch (p.d) {
-      case 32: return fwd_t<float, 32>(p, s);
-      case 64: return fwd_t<float, 64>(p, s);
-      case 128: return fwd_t<float, 128>(p, s);
-    }
-  } else {
-    switch (p.d) {
-      case 32: return fwd_t<__nv_bfloat16, 32>(p, s);
-      case 64: return fwd_t<__nv_bfloat16, 64>(p, s);
-      case 128: return fwd_t<__nv_bfloat16, 128>(p, s);
-    }
+  switch (p.d) {
+    case 32: return fwd_d<32>(p, s);
+    case 64: return fwd_d<64>(p, s);
+    case 128: return fwd_d<128>(p, s);
   }
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_bwd(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
-  if (p.dtype == RELATION_F32) {
-    switch (p.d) {
-      case 32: return bwd_t<float, 32>(p, ws, s);
-      case 64: return bwd_t<float, 64>(p, ws, s);
-      case 128: return bwd_t<float, 128>(p, ws, s);
-    }
-  } else {
-    switch (p.d) {
-      case 32: return bwd_t<__nv_bfloat16, 32>(p, ws, s);
-      case 64: return bwd_t<__nv_bfloat16, 64>(p, ws, s);
-      case 128: return bwd_t<__nv_bfloat16, 128>(p, ws, s);
-    }
+  switch (p.d) {
+    case 32: return bwd_d<32>(p, ws, s);
+    case 64: return bwd_d<64>(p, ws, s);
+    case 128: return bwd_d<128>(p, ws, s);
   }
   return cudaErrorInvalidValue;
 }
