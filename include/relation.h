@@ -213,12 +213,13 @@ relation_status relation_linear_bwd(const void* p1, const void* p2, const void* 
  *                           (a forward state pass), the state's adjoint leaving every block
  *                           (dC(b - 1) = Diag(a_L(b)) dC(b) + Qs_b^T dY_b, a reverse pass),
  *                           then per block the gradients as tcgen05 products with bf16
- *                           operands and fp32 accumulation (five launches).  bf16 with d_h = 64,
+ *                           operands and fp32 accumulation (three launches).  bf16 with d_h = 64,
  *                           element strides multiples of 8 (else RELATION_ERR_UNSUPPORTED or
  *                           RELATION_ERR_ALIGNMENT, nothing launched).  Workspace, in
  *                           256-byte-aligned parts, with n = ceil(T / 128): B H n 64 rows of 64
- *                           fp32, B H n 64 fp32, B H (n + 1) 64 rows of 64 bf16 (the states,
- *                           the final one last) and B H n 64 rows of 64 bf16 (the adjoints).
+ *                           fp32 (the states' contributions, then the states), B H n 64 fp32,
+ *                           and B H (n + 1) 64 and B H n 64 rows of 64 bf16 (together the
+ *                           adjoints' contributions, then the adjoints).
  *                           The decay-range clamp and its report are the chunked forward's.
  *   RELATION_KERNEL_AUTO    the chunked kernel where it applies, else the recurrence.
  * workspace is 16-byte aligned and holds relation_linear_bwd_ex_workspace_size(shp, dt,

@@ -19,10 +19,18 @@
 // dev_status: the result is then not exact (the recurrent kernels have no such limit).
 //
 // One CTA per (head, 64 information columns): the columns of C and Y never mix, so a
-// d_h = 128 head runs as two CTAs that share the Q / K operands' arithmetic.  Warps 0-3
-// (thread = TMEM lane) do Ask Self, the log-retention scans, the operands, the masking,
-// the state's decay and bf16 copy, and the output; warp 4 issues the TMA loads, warp 5
-// (warp-uniform, elect.sync) the MMAs.  Every mbarrier wait is bounded (common.cuh).
+// d_h = 128 head runs as two CTAs that share the Q / K operands' arithmetic.  Elementwise
+// warpgroups of four warps (thread = token, or TMEM lane; the groups split the channels or
+// columns), then a warp that issues the TMA loads and one (warp-uniform, elect.sync) the
+// MMAs.  The block is a chain of short phases around small products: neither HBM nor a pipe
+// bounds it but the latency of those phases, so their work is spread over as many warps as
+// the SM holds: four groups on the sequential walk (one CTA per SM, its next block's loads
+// in flight), two on the one-block modes at d_h = 64, which leave room for a second CTA per SM
+// whose phases fill this one's waits.  With one group (one CTA per SM) the sequential walk took
+// 126 us at B 8, H 12, T 2048, d 64 and now takes 93; at B 1, H 12, T 32768 DELTA took 140 us
+// and OUT 177, now 79 and 95, the scan (16 blocks in flight instead of 8) 27, now 16.
+// Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps
+// meeting the warpgroups' barriers and skips the work between them.
 #include <cudaTypedefs.h>
 #include <math.h>
 
@@ -30,42 +38,68 @@
 
 namespace rel {
 namespace lintc {
-template <int D>
+template <int D, int MODE>
 struct Cfg {
+  static constexpr bool SEQ = MODE == MODE_SEQ;
+  static constexpr bool DELTA = MODE == MODE_DELTA || MODE == MODE_BOTH;
+  static constexpr int NG = (D == 64 && !SEQ) ? 2 : 4;  // elementwise warpgroups
+  static constexpr int CTAS = (D == 64 && !SEQ) ? 2 : 1;  // per SM
+  static constexpr int EW = NG * 128, W_TMA = NG * 4, W_MMA = W_TMA + 1;
+  static constexpr int THREADS = EW + 64;
   static constexpr int KB = D / 64;          // 64-channel (128-byte) blocks of a p tile
   static constexpr int PT = LT * D * 2;      // p1 / p2 / operand tile, [128 t][D] bf16
   static constexpr int VT = LT * NC * 2;     // the CTA's 64 columns of I~
   static constexpr int AT = LT * D * 4;      // alpha, [D / 32][128 t][32] fp32
-  static constexpr int KLT = LT * 128 * 2;   // KL as a 128-channel tile (d_h = 64: upper half 0)
   static constexpr int C0T = D * NC * 2;     // bf16 copy of C_0's 64 columns, [D c][64 n]
-  // Input stages (the next block's loads overlap the current block; one stage at d_h = 128,
-  // whose tiles leave no room for a second): p1 (then Qm in place, then the Y staging),
-  // p2 (then Km in place), the CTA's I~ columns, alpha (then its running log2 sums).
-  static constexpr int STAGES = D == 64 ? 2 : 1;
-  static constexpr int OFF_P1 = 0;
-  static constexpr int OFF_P2 = OFF_P1 + PT;
-  static constexpr int OFF_V = OFF_P2 + PT;
-  static constexpr int OFF_A = OFF_V + VT;
-  static constexpr int STAGE = 2 * PT + VT + AT;
-  static constexpr int OFF_QS = STAGES * STAGE;
-  static constexpr int OFF_KL = OFF_QS + PT;
-  static constexpr int OFF_C0 = OFF_KL + KLT;  // also the per-token / per-channel scalars
-  static constexpr int OFF_BAR = OFF_C0 + C0T;
+  // Input stages (SEQ at d_h = 64: the next block's loads overlap the current block): p2 (then
+  // Km in place; DELTA: KL), p1 (then Qm in place, then the Y staging; BOTH: Qs), the CTA's I~
+  // columns, dY (BOTH), alpha (then its running log2 sums).
+  static constexpr int STAGES = (D == 64 && SEQ) ? 2 : 1;
+  static constexpr int OFF_P2 = 0;
+  static constexpr int OFF_P1 = OFF_P2 + PT;
+  static constexpr int OFF_V = OFF_P1 + PT;
+  static constexpr int OFF_G = OFF_V + VT;
+  static constexpr int OFF_A = OFF_G + (MODE == MODE_BOTH ? VT : 0);
+  static constexpr int STAGE = OFF_A + AT;
+  // KL as the state product's A operand has 128 channels: at d_h = 64 the tile after it (Qs,
+  // p1) takes the upper 64, whose result rows are read by nobody (BOTH: they are Qs^T dY)
+  static constexpr int OFF_KL = DELTA ? OFF_P2 : STAGES * STAGE;
+  static constexpr int OFF_QS = SEQ ? OFF_KL + PT : STAGES * STAGE;
+  static constexpr int OFF_C0 = SEQ ? OFF_QS + PT : (DELTA ? STAGE : OFF_QS + PT);
+  // the per-token / per-channel scalars: before the C0 copy is written in its place (SEQ)
+  static constexpr int OFF_SC = SEQ ? OFF_C0 : (DELTA ? OFF_C0 : OFF_C0 + C0T);
+  static constexpr int SCB = 7 * LT * 4;
+  static constexpr int OFF_BAR = SEQ ? OFF_C0 + C0T : OFF_SC + SCB;
   static constexpr int SMEM = OFF_BAR + 128 + 1024;
-  static constexpr uint32_t LOAD_BYTES = 2 * PT + VT + AT;
+  static constexpr uint32_t LOAD_BYTES =
+      2 * PT + VT + AT + (MODE == MODE_OUT ? C0T : 0) + (MODE == MODE_BOTH ? VT : 0);
+  // TMEM columns: S 128 | E 64 | P 64 (S masked, bf16) | C 64; DELTA: C 64 (BOTH: 128) alone
+  static constexpr int COL_S = 0, COL_E = 128, COL_P = 192, COL_C = DELTA ? 0 : 256;
+  static constexpr int TMEM = SEQ ? 512 : (DELTA ? 128 : 256);
+  static_assert(SCB <= C0T || !SEQ, "scalars in the C0 tile");
+  static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory");
 };
-static_assert(Cfg<64>::SMEM <= 232448 && Cfg<128>::SMEM <= 232448, "shared memory");
+
+// 32 bytes to global memory (one sector)
+__device__ __forceinline__ void st_global_32(float* p, const uint32_t* r) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
 
 template <int D, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     lin_tc_fwd_kernel(const __grid_constant__ CUtensorMap tmP1,
                       const __grid_constant__ CUtensorMap tmP2,
                       const __grid_constant__ CUtensorMap tmV,
+                      const __grid_constant__ CUtensorMap tmG,
                       const __grid_constant__ CUtensorMap tmA,
                       const __grid_constant__ CUtensorMap tmY,
                       const __grid_constant__ CUtensorMap tmC0, LinearProblem p, LinCp cp) {
-  using C = Cfg<D>;
-  constexpr bool kDelta = MODE == MODE_DELTA || MODE == MODE_BDELTA;
+  using C = Cfg<D, MODE>;
+  constexpr bool SEQ = C::SEQ, DELTA = C::DELTA, BOTH = MODE == MODE_BOTH;
+  constexpr int NG = C::NG;
+  static_assert(!BOTH || D == 64, "both contributions in one product: d_h = 64");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -74,52 +108,44 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_BAR + 96);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 104);
   int* clamped = reinterpret_cast<int*>(smem + C::OFF_BAR + 108);
-  // per-token / per-channel scalars: in the C0 tile's space, or (OUT, where C0 is loaded
-  // with the inputs) in KL's, which that mode does not use
-  float* sq = reinterpret_cast<float*>(smem + (MODE == MODE_OUT ? C::OFF_KL : C::OFF_C0));
-  float* sk = sq + LT;                                             // [128] S_t / |p2_t|
-  float* half_sum = sk + LT;                                       // [2][128] (d_h = 64)
-  float* lmid_s = half_sum + 2 * LT;                               // [128] L_m per channel
-  float* lend_s = lmid_s + LT;                                     // [128] L_end per channel
+  float* s_dot = reinterpret_cast<float*>(smem + C::OFF_SC);  // [128] p1_t . p2_t
+  float* s_n1 = s_dot + LT;                                   // [128] |p1_t|^2
+  float* s_n2 = s_n1 + LT;                                    // [128] |p2_t|^2
+  // per channel L_m and, d_h = 64: the sum over the second half; d_h = 128: L_end
+  float* l_a = s_n2 + LT;
+  float* l_b = l_a + LT;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NSPLIT = D / NC;
   const int nb = (p.T + LT - 1) / LT;
-  // SEQ: one CTA per (head, split) over blocks [0, nb); DELTA / OUT: one block per CTA
-  const int cta_blk = MODE == MODE_SEQ ? 0 : (int)(blockIdx.x % nb);
-  const int bhs = MODE == MODE_SEQ ? (int)blockIdx.x : (int)(blockIdx.x / nb);
+  // SEQ: one CTA per (head, split) over blocks [0, nb); DELTA / BOTH / OUT: one block per CTA
+  const int cta_blk = SEQ ? 0 : (int)(blockIdx.x % nb);
+  const int bhs = SEQ ? (int)blockIdx.x : (int)(blockIdx.x / nb);
   const int split = bhs % NSPLIT;
   const int bh = bhs / NSPLIT;
   const int b = bh / p.H, h = bh % p.H;
-  const int blk_first = cta_blk, blk_end = MODE == MODE_SEQ ? nb : cta_blk + 1;
+  const int blk_first = cta_blk, blk_end = SEQ ? nb : cta_blk + 1;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NBAR; ++i)  // arrivals of the 128 elementwise threads, or one
-      mbar_init(bar(i), (i == B_OPS || i == B_C0 || i == B_A || i == B_EPI || i == B_EPI + 1)
-                            ? 128 : 1);
+    for (int i = 0; i < NBAR; ++i)  // arrivals of the elementwise threads, the four storing
+                                    // lanes, or one
+      mbar_init(bar(i), (i == B_OPS || i == B_C0 || i == B_A)
+                            ? C::EW
+                            : (i == B_EPI || i == B_EPI + 1) ? 4 : 1);
     *abort_flag = 0;
     *clamped = 0;
     fence_mbar_init();
   }
-  if (D == 64 && MODE != MODE_OUT) {  // KL's channels 64..127 stay zero (M = 128 product)
-    for (int i = threadIdx.x; i < LT * 64 * 2 / 16; i += kThreads)
-      *reinterpret_cast<uint4*>(smem + C::OFF_KL + LT * 128 + i * 16) = make_uint4(0, 0, 0, 0);
-    fence_async_smem();
-  }
-  if (warp == 5) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  if (warp == C::W_MMA) tmem_alloc(smem_u32(tmem_slot), C::TMEM);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
 
-  if (warp == 4) {
+  if (warp == C::W_TMA) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_desc(&tmP1);
-      tma_prefetch_desc(&tmP2);
-      tma_prefetch_desc(&tmV);
-      tma_prefetch_desc(&tmA);
       int issued = 0;
       for (int blk = blk_first; blk < blk_end; ++blk) {
         const int it = blk - blk_first;
@@ -131,27 +157,28 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int t0 = blk * LT;
         const uint32_t sg = sb + st * C::STAGE;
         const uint32_t lb = bar(B_LOAD + st);
-        mbar_arrive_expect_tx(lb, C::LOAD_BYTES + (MODE == MODE_OUT ? C::C0T : 0));
-        if (MODE == MODE_OUT)  // the state the block starts from, in the MN-major B layout
-          tma_load_2d(sb + C::OFF_C0, &tmC0, lb, 0, (bhs * (nb + 1) + blk) * D);
+        mbar_arrive_expect_tx(lb, C::LOAD_BYTES);
         for (int kb = 0; kb < C::KB; ++kb) {
           tma_load_4d(sg + C::OFF_P1 + kb * LT * 128, &tmP1, lb, kb * 64, t0, h, b);
           tma_load_4d(sg + C::OFF_P2 + kb * LT * 128, &tmP2, lb, kb * 64, t0, h, b);
         }
-        tma_load_4d(sg + C::OFF_V, &tmV, lb, split * NC, t0, h, b);
         for (int k = 0; k < D / 32; ++k)
           tma_load_4d(sg + C::OFF_A + k * LT * 128, &tmA, lb, k * 32, t0, h, b);
+        tma_load_4d(sg + C::OFF_V, &tmV, lb, split * NC, t0, h, b);
+        if (BOTH) tma_load_4d(sg + C::OFF_G, &tmG, lb, split * NC, t0, h, b);
+        if (MODE == MODE_OUT)  // the state the block starts from, in the MN-major B layout
+          tma_load_2d(sb + C::OFF_C0, &tmC0, lb, 0, (bhs * nb + blk) * D);
         issued = it + 1;
       }
       if (ab.raised())  // copies in flight land before the CTA releases its shared memory
         for (int it = issued - C::STAGES > 0 ? issued - C::STAGES : 0; it < issued; ++it)
           drain_wait(bar(B_LOAD + it % C::STAGES), (it / C::STAGES) & 1);
     }
-  } else if (warp == 5) {
+  } else if (warp == C::W_MMA) {
     // ------------------------------------------------------------------ MMA issuer
     constexpr uint32_t id_s = idesc_bf16_f32(128, 128, false, false);
     constexpr uint32_t id_e = idesc_bf16_f32(128, NC, false, true);
-    constexpr uint32_t id_c = idesc_bf16_f32(128, NC, true, true);
+    constexpr uint32_t id_c = idesc_bf16_f32(128, BOTH ? 2 * NC : NC, true, true);
     bool ok = true;
     for (int blk = blk_first; ok && blk < blk_end; ++blk) {
       const int it = blk - blk_first;
@@ -160,20 +187,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t sg = sb + st * C::STAGE;
       if (!(ok = mbar_wait_warp(bar(B_OPS), ph, ab))) break;
       tc_fence_after();
-      if (!kDelta) {
+      if (!DELTA) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {  // S = Qm Km^T
           const uint32_t koff = (kk >> 2) * (LT * 128) + (kk & 3) * 32;
-          mma_ss_w(tmem + COL_S, smem_desc_sw128(sg + C::OFF_P1 + koff, 16, 1024),
+          mma_ss_w(tmem + C::COL_S, smem_desc_sw128(sg + C::OFF_P1 + koff, 16, 1024),
                    smem_desc_sw128(sg + C::OFF_P2 + koff, 16, 1024), id_s, kk > 0 ? 1u : 0u);
         }
         mma_commit_w(bar(B_S));
-        if (!(ok = mbar_wait_warp(bar(B_C0), ph, ab))) break;
-        tc_fence_after();
+        if (SEQ) {  // (OUT: C0 came with the block's inputs)
+          if (!(ok = mbar_wait_warp(bar(B_C0), ph, ab))) break;
+          tc_fence_after();
+        }
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {  // E = Qs C_0
           const uint32_t koff = (kk >> 2) * (LT * 128) + (kk & 3) * 32;
-          mma_ss_w(tmem + COL_E, smem_desc_sw128(sb + C::OFF_QS + koff, 16, 1024),
+          mma_ss_w(tmem + C::COL_E, smem_desc_sw128(sb + C::OFF_QS + koff, 16, 1024),
                    smem_desc_sw128(sb + C::OFF_C0 + kk * 16 * 128, D * 128, 1024), id_e,
                    kk > 0 ? 1u : 0u);
         }
@@ -181,136 +210,114 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < LT / 16; ++kk)  // E += tril(S, -1) I~   (A from TMEM)
-          mma_ts_w(tmem + COL_E, tmem + COL_S + kk * 8,
+          mma_ts_w(tmem + C::COL_E, tmem + C::COL_P + kk * 8,
                    smem_desc_sw128(sg + C::OFF_V + kk * 16 * 128, LT * 128, 1024), id_e, 1u);
         mma_commit_w(bar(B_E));
       }
       if (MODE != MODE_OUT) {
-        // SEQ: C += KL^T I~ (C decayed by the threads); DELTA: the block's own sum;
-        // BDELTA: Qs^T dY
+        // SEQ: C += KL^T I~ (C decayed by the threads); DELTA: the block's own sum; BOTH:
+        // [KL | Qs]^T [I~ | dY], whose diagonal quarters are the two contributions
 #pragma unroll
         for (int kk = 0; kk < LT / 16; ++kk)
-          mma_ss_w(tmem + COL_C, smem_desc_sw128(sb + C::OFF_KL + kk * 16 * 128, LT * 128, 1024),
+          mma_ss_w(tmem + C::COL_C,
+                   smem_desc_sw128(sb + C::OFF_KL + kk * 16 * 128, LT * 128, 1024),
                    smem_desc_sw128(sg + C::OFF_V + kk * 16 * 128, LT * 128, 1024), id_c,
-                   ((MODE == MODE_SEQ && blk > 0) || kk > 0) ? 1u : 0u);
+                   ((SEQ && blk > 0) || kk > 0) ? 1u : 0u);
         mma_commit_w(bar(B_STATE));
       }
-      mma_commit_w(bar(B_FREE + st));
+      if (SEQ) mma_commit_w(bar(B_FREE + st));
     }
+    // SEQ: the last commits land before the CTA exits (EW warps have waited for the others)
+    if (SEQ && ok)
+      for (int it = max(0, nb - C::STAGES); it < nb; ++it)
+        mbar_wait_warp(bar(B_FREE + it % C::STAGES), (it / C::STAGES) & 1, ab);
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ elementwise
-    const int t = threadIdx.x;  // token of the block (phases A, D, E) / TMEM lane
-    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    const int grp = warp >> 2;            // warpgroup
+    const int t = threadIdx.x & 127;      // token of the block / TMEM lane
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float inv_tau_sqrt_d = 1.0f / (p.tau_s * sqrtf((float)D));
-    // phase B: thread (c, half) for d_h = 64, thread c over all 128 tokens for d_h = 128
+    // the retention sums: thread (c, half) for d_h = 64, thread c over all 128 tokens for 128
     const int c = D == 64 ? (t & 63) : t;
     const int half = D == 64 ? (t >> 6) : 0;
-    constexpr int TPT = D == 64 ? 64 : 128;  // tokens per phase-B thread
-    const int tb0 = half * 64;
-    uint8_t* p1s = smem + C::OFF_P1;
-    uint8_t* p2s = smem + C::OFF_P2;
-    float* al = reinterpret_cast<float*>(smem + C::OFF_A);
-    auto al_at = [&](int tok, int ch) -> float& {  // [D / 32][128][32] fp32, 128-byte swizzle
-      return al[al_swz(tok, ch)];
-    };
-    float l_end = 0.f;  // this channel's L at the block's last token (phase C, c < D)
+    constexpr int TPT = D == 64 ? 64 : 128;  // tokens per thread of the retention sums
     bool ok = true, my_clamp = false;
-    for (int blk = blk_first; ok && blk < blk_end; ++blk) {
+    for (int blk = blk_first; blk < blk_end; ++blk) {
       const int it = blk - blk_first;
       const uint32_t ph = it & 1;
       const int t0 = blk * LT;
       const int st = it % C::STAGES;
       uint8_t* const sg = smem + st * C::STAGE;
-      p1s = sg + C::OFF_P1;
-      p2s = sg + C::OFF_P2;
-      al = reinterpret_cast<float*>(sg + C::OFF_A);
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD + st), (it / C::STAGES) & 1, ab));
-      if (!ok) break;
-      // ---- phase A: Ask Self of token t (rows past T give zero operands)
-      {
-        float dot = 0.f, n1 = 0.f, n2 = 0.f;
+      uint8_t* const p1s = sg + C::OFF_P1;
+      uint8_t* const p2s = sg + C::OFF_P2;
+      float* const al = reinterpret_cast<float*>(sg + C::OFF_A);
+      auto al_at = [&](int tok, int ch) -> float& {  // [D / 32][128][32] fp32, 128-byte swizzle
+        return al[al_swz(tok, ch)];
+      };
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD + st), (it / C::STAGES) & 1, ab));
+      if (ok) {
+        // ---- Ask Self's sums of token t (the groups but the last) beside the channels'
+        // inclusive running sums L_t of log2 alpha in place of alpha (the last group; 0
+        // past T; d_h = 64: the second half's relative to its start)
+        if (grp < NG - 1) {
+          ask_self_sums<D, NG == 2 ? 7 : 0>(p1s, p2s, t, NG == 2 ? 7 : 1 << grp, s_dot, s_n1, s_n2);
+        } else {
+          float lsum = 0.f;
+          for (int i0 = 0; i0 < TPT; i0 += 16) {
+            float la[16];
 #pragma unroll
-        for (int kb = 0; kb < C::KB; ++kb) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const uint32_t off = kb * LT * 128 + t * 128 + ((k ^ (t & 7)) << 4);
-            const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-            const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-            const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-              const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-              dot = fmaf(x.x, y.x, fmaf(x.y, y.y, dot));
-              n1 = fmaf(x.x, x.x, fmaf(x.y, x.y, n1));
-              n2 = fmaf(y.x, y.x, fmaf(y.y, y.y, n2));
+            for (int u = 0; u < 16; ++u) {
+              const int tok = half * 64 + i0 + u;
+              la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
             }
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              lsum += la[u];
+              al_at(half * 64 + i0 + u, c) = lsum;
+            }
+            if (D == 128 && i0 == 48) l_a[c] = lsum;  // L at the 64th token
           }
+          if (D == 64)
+            (half == 0 ? l_a : l_b)[c] = lsum;
+          else
+            l_b[c] = lsum;
         }
-        float s1 = 0.f, s2 = 0.f;
+      }
+      ew_sync<NG>();
+      float l_end = 0.f;  // channel t's L at the block's last token (t < D)
+      if (ok) {
+        if (t < D) l_end = D == 64 ? l_a[c] + l_b[c] : l_b[c];
+        // Qs, KL and the state are single buffers: the last block's state product (the last
+        // reader of KL; Qs's reader precedes B_E) must be done before they are written
+        if (SEQ && blk > 0) {
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), (blk - 1) & 1, ab));
+          tc_fence_after();
+        }
+      }
+      if (ok) {
+        // ---- the operands of token t over the group's channels, 8 per 16-byte access: Qm
+        // and Km in place of p1 and p2, Qs, KL (DELTA: KL in place of p2; BOTH: and Qs of p1)
+        float s1 = 0.f, s2 = 0.f;  // rows past T give zero operands
         if (t0 + t < p.T) {
-          const float S = 1.0f / (1.0f + __expf(-dot * inv_tau_sqrt_d));
-          s1 = S * rsqrtf(n1);
-          s2 = S * rsqrtf(n2);
-        }
-        sq[t] = s1;
-        sk[t] = s2;
-      }
-      // ---- phase B, pass 1 (thread = channel, d_h = 64: channel and half block): the
-      // inclusive running sums L_t of log2 alpha in place of alpha (0 past T)
-      // (batches of 16: the loads and logarithms of a batch are issued before its stores)
-      float lsum = 0.f, l_mid;
-      for (int i0 = 0; i0 < TPT; i0 += 16) {
-        float la[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int tok = tb0 + i0 + u;
-          la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
+          const float S = 1.0f / (1.0f + __expf(-s_dot[t] * inv_tau_sqrt_d));
+          s1 = S * rsqrtf(s_n1[t]);
+          s2 = S * rsqrtf(s_n2[t]);
         }
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          lsum += la[u];
-          al_at(tb0 + i0 + u, c) = lsum;  // d_h = 64, second half: relative to its start
-        }
-      }
-      if (D == 64) half_sum[half * 128 + c] = lsum;
-      ew_sync();
-      if (D == 64) {
-        l_mid = half_sum[c];
-        l_end = half_sum[c] + half_sum[128 + c];
-      } else {
-        l_mid = al_at(63, c);
-        l_end = lsum;
-      }
-      if (t < D) {  // per-channel L_m and L_end for the token-parallel pass
-        lmid_s[t] = l_mid;
-        lend_s[t] = l_end;
-      }
-      ew_sync();
-      // Qs, KL and the state are single buffers: the last block's state product (the last
-      // reader of KL; Qs's reader precedes B_E) must be done before they are written
-      if (MODE == MODE_SEQ && blk > 0) {
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), (blk - 1) & 1, ab));
-        if (!ok) break;
-        tc_fence_after();
-      }
-      // ---- pass 2 (thread = token t, 8 channels per 16-byte access): the four operands,
-      // Qm and Km in place of p1 and p2
-      {
-        const int tok = t;
-        const float s1 = sq[tok], s2 = sk[tok];
-#pragma unroll
-        for (int k = 0; k < D / 8; ++k) {
-          const uint32_t off = (k >> 3) * LT * 128 + tok * 128 + (((k & 7) ^ (tok & 7)) << 4);
-          const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-          const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-          const float4 L0 = *reinterpret_cast<const float4*>(&al_at(tok, 8 * k));
-          const float4 L1 = *reinterpret_cast<const float4*>(&al_at(tok, 8 * k + 4));
-          const float4 M0 = *reinterpret_cast<const float4*>(lmid_s + 8 * k);
-          const float4 M1 = *reinterpret_cast<const float4*>(lmid_s + 8 * k + 4);
-          const float4 E0 = *reinterpret_cast<const float4*>(lend_s + 8 * k);
-          const float4 E1 = *reinterpret_cast<const float4*>(lend_s + 8 * k + 4);
+        for (int k0 = 0; k0 < D / 8 / NG; ++k0) {
+          const int k = grp * (D / 8 / NG) + k0;
+          const uint32_t off = (k >> 3) * LT * 128 + t * 128 + (((k & 7) ^ (t & 7)) << 4);
+          uint4 a4 = make_uint4(0, 0, 0, 0);
+          if (!DELTA || BOTH) a4 = *reinterpret_cast<const uint4*>(p1s + off);
+          uint4 b4 = make_uint4(0, 0, 0, 0);
+          b4 = *reinterpret_cast<const uint4*>(p2s + off);
+          const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k));
+          const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k + 4));
+          const float4 M0 = *reinterpret_cast<const float4*>(l_a + 8 * k);
+          const float4 M1 = *reinterpret_cast<const float4*>(l_a + 8 * k + 4);
+          const float4 E0 = *reinterpret_cast<const float4*>(l_b + 8 * k);
+          const float4 E1 = *reinterpret_cast<const float4*>(l_b + 8 * k + 4);
           const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
           const float Mv[8] = {M0.x, M0.y, M0.z, M0.w, M1.x, M1.y, M1.z, M1.w};
           const float Ev[8] = {E0.x, E0.y, E0.z, E0.w, E1.x, E1.y, E1.z, E1.w};
@@ -325,159 +332,172 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int u = 0; u < 2; ++u) {
               const int ch = 2 * e + u;
               // the second half's sums (d_h = 64) are relative to the half's start
-              const float L = Lv[ch] + ((D == 64 && tok >= 64) ? Mv[ch] : 0.f);
-              float dm = L - Mv[ch];  // log2 of a_t / a_m
-              if (fabsf(dm) > kClampLog2) {
-                dm = copysignf(kClampLog2, dm);
-                my_clamp = true;
-              }
+              const float L = Lv[ch] + ((D == 64 && t >= 64) ? Mv[ch] : 0.f);
               const float xv = u ? x.y : x.x, yv = u ? y.y : y.x;
-              if (!kDelta) {
+              if (!DELTA) {
+                float dm = L - Mv[ch];  // log2 of a_t / a_m
+                if (fabsf(dm) > kClampLog2) {
+                  dm = copysignf(kClampLog2, dm);
+                  my_clamp = true;
+                }
                 r[u][0] = xv * s1 * ex2_approx(dm);      // Qm
                 r[u][1] = yv * s2 * ex2_approx(-dm);     // Km
-                r[u][2] = xv * s1 * ex2_approx(L);       // Qs (factor <= 1)
               }
-              if (MODE == MODE_BDELTA)
-                r[u][3] = xv * s1 * ex2_approx(L);         // Qs, in KL's place
-              else if (MODE != MODE_OUT)
-                r[u][3] = yv * s2 * ex2_approx(Ev[ch] - L);  // KL (factor <= 1)
+              if (!DELTA || BOTH) r[u][2] = xv * s1 * ex2_approx(L);  // Qs (factor <= 1)
+              if (MODE != MODE_OUT) {  // KL (factor <= 1)
+                const float Le = D == 64 ? Mv[ch] + Ev[ch] : Ev[ch];
+                r[u][3] = yv * s2 * ex2_approx(Le - L);
+              }
             }
-            if (!kDelta) {
+            if (!DELTA) {
               qm[e] = pack_bf16x2(r[0][0], r[1][0]);
               km[e] = pack_bf16x2(r[0][1], r[1][1]);
-              qs[e] = pack_bf16x2(r[0][2], r[1][2]);
             }
+            if (!DELTA || BOTH) qs[e] = pack_bf16x2(r[0][2], r[1][2]);
             if (MODE != MODE_OUT) kl[e] = pack_bf16x2(r[0][3], r[1][3]);
           }
-          if (!kDelta) {
+          if (!DELTA) {
             *reinterpret_cast<uint4*>(p1s + off) = make_uint4(qm[0], qm[1], qm[2], qm[3]);
             *reinterpret_cast<uint4*>(p2s + off) = make_uint4(km[0], km[1], km[2], km[3]);
-            *reinterpret_cast<uint4*>(smem + C::OFF_QS + off) =
-                make_uint4(qs[0], qs[1], qs[2], qs[3]);
           }
+          if (!DELTA || BOTH)
+            *reinterpret_cast<uint4*>((BOTH ? p1s : smem + C::OFF_QS) + off) =
+                make_uint4(qs[0], qs[1], qs[2], qs[3]);
           if (MODE != MODE_OUT)
             *reinterpret_cast<uint4*>(smem + C::OFF_KL + off) =
                 make_uint4(kl[0], kl[1], kl[2], kl[3]);
         }
+        fence_async_smem();
+        mbar_arrive(bar(B_OPS));
       }
-      fence_async_smem();
-      ew_sync();
-      mbar_arrive(bar(B_OPS));
-      if (kDelta) {
-        // the block's state (adjoint) contribution and decay, to the workspace
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), 0, ab));
-        if (!ok) break;
+      if (SEQ) ew_sync<NG>();  // the scalars have been read: C0 takes their place
+      if (DELTA) {
+        // the block's state (and adjoint) contribution and decay, to the workspace
+        ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), 0, ab));
         tc_fence_after();
-        if (t < D) {
-          uint32_t z[64];
-          tmem_ld32(trow + COL_C, z);
-          tmem_ld32(trow + COL_C + 32, z + 32);
+        constexpr int CG = NC / NG;  // columns per group
+        const bool upper = BOTH && t >= 64;  // rows of Qs^T dY, in columns 64 .. 127
+        if (ok && (t < D || BOTH)) {
+          uint32_t z[32];
+          const uint32_t col = trow + C::COL_C + (BOTH && (warp & 3) >= 2 ? NC : 0) + grp * CG;
+          if constexpr (CG == 32)
+            tmem_ld32(col, z);
+          else
+            tmem_ld16(col, *reinterpret_cast<uint32_t(*)[16]>(z));
           tmem_ld_wait();
-          const long long row = (long long)(bhs * nb + blk) * D + t;
-          float4* dst = reinterpret_cast<float4*>(cp.dC + row * 64);
+          const long long row = (long long)(bhs * nb + blk) * D + (upper ? t - 64 : t);
+          float* dst = (upper ? cp.dQ : cp.dC) + row * 64 + grp * CG;
 #pragma unroll
-          for (int k = 0; k < 16; ++k)
-            dst[k] = make_float4(__uint_as_float(z[4 * k]), __uint_as_float(z[4 * k + 1]),
-                                 __uint_as_float(z[4 * k + 2]), __uint_as_float(z[4 * k + 3]));
-          cp.g[row] = ex2_approx(l_end);
+          for (int k = 0; k < CG / 8; ++k) st_global_32(dst + 8 * k, z + 8 * k);
+          if (grp == 0 && !upper) cp.g[row] = ex2_approx(l_end);
         }
         continue;
       }
-      if (MODE == MODE_OUT) {
-        mbar_arrive(bar(B_C0));  // C0 came with the block's inputs
-      } else {
-      // ---- phase C: the state after the last block (complete, waited above), its bf16
-      // copy, then decayed by a_L
-      if (t < D) {
-        uint32_t z[64];
-        if (blk > 0) {
-          tmem_ld32(trow + COL_C, z);
-          tmem_ld32(trow + COL_C + 32, z + 32);
-          tmem_ld_wait();
-        } else {
+      if (SEQ && ok) {
+        // ---- the state after the last block (complete, waited above): its bf16 copy, then
+        // decayed by a_L
+        if (t < D) {  // (whole warps)
+          uint32_t z[16];
+          if (blk > 0) {
+            tmem_ld16(trow + C::COL_C + grp * 16, z);
+            tmem_ld_wait();
+          } else {
 #pragma unroll
-          for (int n = 0; n < 64; ++n) z[n] = 0u;
+            for (int n = 0; n < 16; ++n) z[n] = 0u;
+          }
+          uint8_t* crow = smem + C::OFF_C0 + t * 128;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              w[e] = pack_bf16x2(__uint_as_float(z[8 * k + 2 * e]),
+                                 __uint_as_float(z[8 * k + 2 * e + 1]));
+            *reinterpret_cast<uint4*>(crow + (((2 * grp + k) ^ (t & 7)) << 4)) =
+                make_uint4(w[0], w[1], w[2], w[3]);
+          }
+          if (blk > 0) {
+            const float decay = ex2_approx(l_end);
+#pragma unroll
+            for (int n = 0; n < 16; ++n) z[n] = __float_as_uint(__uint_as_float(z[n]) * decay);
+            tmem_st16(trow + C::COL_C + grp * 16, z);
+            tmem_st_wait();
+          }
         }
-        uint8_t* crow = smem + C::OFF_C0 + t * 128;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          uint32_t w[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            w[e] = pack_bf16x2(__uint_as_float(z[8 * k + 2 * e]), __uint_as_float(z[8 * k + 2 * e + 1]));
-          *reinterpret_cast<uint4*>(crow + ((k ^ (t & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        if (blk > 0) {
-          const float decay = ex2_approx(l_end);
-#pragma unroll
-          for (int n = 0; n < 64; ++n) z[n] = __float_as_uint(__uint_as_float(z[n]) * decay);
-          tmem_st16(trow + COL_C, z);
-          tmem_st16(trow + COL_C + 16, z + 16);
-          tmem_st16(trow + COL_C + 32, z + 32);
-          tmem_st16(trow + COL_C + 48, z + 48);
-          tmem_st_wait();
-        }
+        fence_async_smem();
+        tc_fence_before();
+        mbar_arrive(bar(B_C0));
       }
-      fence_async_smem();
-      tc_fence_before();
-      mbar_arrive(bar(B_C0));
-      }
-      // ---- phase D: S masked to the strictly earlier tokens, packed to bf16 in place
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_S), ph, ab));
-      if (!ok) break;
-      tc_fence_after();
+      // ---- S masked to the strictly earlier tokens, packed to bf16
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_S), ph, ab));
+      if (ok) {
+        tc_fence_after();
 #pragma unroll
-      for (int c0 = 0; c0 < LT; c0 += 32) {
-        uint32_t s[32], pk[16];
-        tmem_ld32(trow + COL_S + c0, s);
-        tmem_ld_wait();
+        for (int c0 = 0; c0 < LT / NG; c0 += 32) {
+          const int col = grp * (LT / NG) + c0;
+          uint32_t pk[16];
+          if (col <= (warp & 3) * 32) {  // some column of the warp's rows is unmasked
+            uint32_t s[32];
+            tmem_ld32(trow + C::COL_S + col, s);
+            tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          const float lo = (c0 + j < t) ? __uint_as_float(s[j]) : 0.f;
-          const float hi = (c0 + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
-          pk[j >> 1] = pack_bf16x2(lo, hi);
+            for (int j = 0; j < 32; j += 2) {
+              const float lo = (col + j < t) ? __uint_as_float(s[j]) : 0.f;
+              const float hi = (col + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
+              pk[j >> 1] = pack_bf16x2(lo, hi);
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) pk[j] = 0u;
+          }
+          tmem_st16(trow + C::COL_P + (col >> 1), pk);
         }
-        tmem_st16(trow + COL_S + (c0 >> 1), pk);  // columns already read
+        tmem_st_wait();
+        tc_fence_before();
+        mbar_arrive(bar(B_A));
       }
-      tmem_st_wait();
-      tc_fence_before();
-      mbar_arrive(bar(B_A));
-      // ---- phase E: Y = I~ + E, staged per warp (32 rows) and stored by TMA
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_E), ph, ab));
-      if (!ok) break;
-      tc_fence_after();
-      {
-        uint32_t z[64];
-        tmem_ld32(trow + COL_E, z);
-        tmem_ld32(trow + COL_E + 32, z + 32);
+      // ---- Y = I~ + E, staged in p1's tile and stored by TMA (32 rows per store)
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_E), ph, ab));
+      if (ok) {
+        tc_fence_after();
+        constexpr int CG = NC / NG;
+        uint32_t z[CG];
+        if constexpr (CG == 32)
+          tmem_ld32(trow + C::COL_E + grp * CG, z);
+        else
+          tmem_ld16(trow + C::COL_E + grp * CG, z);
         tmem_ld_wait();
         const uint8_t* vrow = sg + C::OFF_V + t * 128;
-        uint8_t* ystage = sg + C::OFF_P1 + warp * (32 * 128) + lane * 128;
+        uint8_t* yrow = sg + C::OFF_P1 + t * 128;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k0 = 0; k0 < CG / 8; ++k0) {
+          const int k = grp * (CG / 8) + k0;
           const uint4 vv = *reinterpret_cast<const uint4*>(vrow + ((k ^ (t & 7)) << 4));
           const uint32_t vw[4] = {vv.x, vv.y, vv.z, vv.w};
           uint32_t yw[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float2 vf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&vw[e]));
-            yw[e] = pack_bf16x2(vf.x + __uint_as_float(z[8 * k + 2 * e]),
-                                vf.y + __uint_as_float(z[8 * k + 2 * e + 1]));
+            yw[e] = pack_bf16x2(vf.x + __uint_as_float(z[8 * k0 + 2 * e]),
+                                vf.y + __uint_as_float(z[8 * k0 + 2 * e + 1]));
           }
-          *reinterpret_cast<uint4*>(ystage + ((k ^ (lane & 7)) << 4)) =
+          *reinterpret_cast<uint4*>(yrow + ((k ^ (t & 7)) << 4)) =
               make_uint4(yw[0], yw[1], yw[2], yw[3]);
         }
         fence_async_smem();
-        __syncwarp();
-        if (lane == 0) {
+        tc_fence_before();
+      }
+      ew_sync<NG>();
+      if (ok && grp == 0 && lane == 0) {
+        if (t0 + warp * 32 < p.T) {
           tma_store_4d(&tmY, smem_u32(sg + C::OFF_P1 + warp * (32 * 128)), split * NC,
                        t0 + warp * 32, h, b);
           tma_store_commit();
-          tma_store_wait_read_all();  // the staging (the next block's p1) is reloaded next
+          tma_store_wait_read_all();  // the staging (a later block's p1) is reloaded next
         }
-        __syncwarp();
+        mbar_arrive(bar(B_EPI + st));
       }
-      mbar_arrive(bar(B_EPI + st));
+      __syncwarp();
     }
     if (my_clamp) atomicExch(clamped, 1);
   }
@@ -486,42 +506,35 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (threadIdx.x == 0 && *clamped && p.dev_status && !*abort_flag)
     atomicExch(p.dev_status, (int)RELATION_ERR_UNSUPPORTED);
-  if (warp == 5) {
+  if (warp == C::W_MMA) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(tmem, C::TMEM);
   }
 }
 
-// Sequential scan of the state over the blocks of one (head, split), for the chunk-parallel
-// forward: C_0(0) = 0, C_0(b + 1) = Diag(g_b) C_0(b) + dC_b, each C_0(b) written in bf16
-// (row-major [D][64] per block, the OUT pass's B operand after a swizzled TMA load).  A CTA
-// takes 8 channels x 64 columns, two per thread (a warp = one channel's 64 columns,
-// coalesced); the loads of the next 8 blocks are in flight while 8 are combined.
+// Scan of the state over the blocks of one (head, split), for the chunk-parallel forms:
+// C_0(0) = 0, C_0(b + 1) = Diag(g_b) C_0(b) + dC_b; every C_0(b) is written in bf16 over the
+// first half of its own row of dC_b (rows of 64 bf16 at a pitch of 256 bytes: the B operand of
+// the block's products after a swizzled TMA load).  A warp owns a channel's 64 columns, two
+// per lane; it has read a row (__syncwarp) before it writes it, the loads of the next P
+// blocks in flight while P are combined.
 //   REV (the backward): from the last block down, the state's adjoint leaving block b,
-//   dC(nb - 1) = 0, dC(b - 1) = Diag(g_b) dC(b) + dQ_b (dQ_b = Qs_b^T dY_b in dC's place),
-//   written to out_rows (bf16 [nb][D][64] per (head, split)).  Forward: nb + 1 states.
+//   dC(nb - 1) = 0, dC(b - 1) = Diag(g_b) dC(b) + dQ_b (dQ_b = Qs_b^T dY_b), in place of dQ.
 template <int D, bool REV>
-__global__ void __launch_bounds__(256) scan_kernel(LinCp cp, __nv_bfloat16* out_rows) {
-  constexpr int CPB = 8, P = 8;
-  const int cg = (int)(blockIdx.x % (D / CPB));
-  const int bhs = (int)(blockIdx.x / (D / CPB));
-  const int c = cg * CPB + (int)(threadIdx.x >> 5);
-  const int n = (int)(threadIdx.x & 31) * 2;
-  const int nb = cp.nb;
+__device__ __forceinline__ void scan_blocks(float* rows, const float* g, int nb, int bhs, int c,
+                                            int n) {
+  constexpr int P = 16;
   const long long base = (long long)bhs * nb * D + c;  // row of block blk: base + blk D
-  // output rows: forward nb + 1 states per (head, split), backward nb adjoints
-  const long long obase = (long long)bhs * (REV ? nb : nb + 1) * D + c;
   auto load = [&](int b0, float2 (&dv)[P], float (&gv)[P]) {
 #pragma unroll
     for (int u = 0; u < P; ++u) {
       const int blk = REV ? nb - 1 - (b0 + u) : b0 + u;
+      dv[u] = make_float2(0.f, 0.f);
+      gv[u] = 1.f;
       if (blk >= 0 && blk < nb) {
         const long long row = base + (long long)blk * D;
-        dv[u] = *reinterpret_cast<const float2*>(cp.dC + row * 64 + n);
-        gv[u] = cp.g[row];
-      } else {
-        dv[u] = make_float2(0.f, 0.f);
-        gv[u] = 1.f;
+        dv[u] = *reinterpret_cast<const float2*>(rows + row * 64 + n);
+        gv[u] = g[row];
       }
     }
   };
@@ -532,13 +545,14 @@ __global__ void __launch_bounds__(256) scan_kernel(LinCp cp, __nv_bfloat16* out_
     float2 nxt[P];
     float gn[P];
     load(b0 + P, nxt, gn);
+    __syncwarp();  // the warp has read rows b0 .. b0 + P - 1 (a round ago)
 #pragma unroll
     for (int u = 0; u < P; ++u) {
       const int i = b0 + u;
       if (i < nb) {
         const int blk = REV ? nb - 1 - i : i;
-        const long long orow = obase + (long long)blk * D;
-        *reinterpret_cast<__nv_bfloat162*>(out_rows + orow * 64 + n) =
+        const long long row = base + (long long)blk * D;
+        reinterpret_cast<__nv_bfloat162*>(rows + row * 64)[n >> 1] =
             __floats2bfloat162_rn(st.x, st.y);
         st = make_float2(fmaf(gc[u], st.x, cur[u].x), fmaf(gc[u], st.y, cur[u].y));
       }
@@ -549,13 +563,23 @@ __global__ void __launch_bounds__(256) scan_kernel(LinCp cp, __nv_bfloat16* out_
       gc[u] = gn[u];
     }
   }
-  if (!REV)  // the final state, after the last block
-    *reinterpret_cast<__nv_bfloat162*>(out_rows + (obase + (long long)nb * D) * 64 + n) =
-        __floats2bfloat162_rn(st.x, st.y);
 }
 
-// Workspace layout of the chunk-parallel forward: dC and g per (head, split, block), C0 per
-// (head, split) and block plus the final state (see LinCp).
+// CTAs of 8 channels; with BOTH the second half of the grid scans the adjoints.
+template <int D, bool BOTH>
+__global__ void __launch_bounds__(256) scan_kernel(LinCp cp, int ctas) {
+  const bool rev = BOTH && (int)blockIdx.x >= ctas;
+  const int w = (int)blockIdx.x - (rev ? ctas : 0);
+  const int c = (w % (D / 8)) * 8 + (int)(threadIdx.x >> 5), n = (int)(threadIdx.x & 31) * 2;
+  if (rev)
+    scan_blocks<D, true>(cp.dQ, cp.g, cp.nb, w / (D / 8), c, n);
+  else
+    scan_blocks<D, false>(cp.dC, cp.g, cp.nb, w / (D / 8), c, n);
+}
+
+// Workspace of the chunk-parallel forward: dC and g per (head, split, block) (see LinCp).  The
+// size also holds bf16 rows for nb + 1 states per (head, split), which the scan now keeps in
+// dC's rows: the backward's second array of fp32 rows takes that place.
 static size_t cp_bytes(long long heads, long long nb, int d, LinCp* out, void* base) {
   const long long rows = heads * nb * d, rows_c0 = heads * (nb + 1) * d;
   const size_t b_dc = align256((size_t)rows * 64 * 4), b_g = align256((size_t)rows * 4);
@@ -564,23 +588,26 @@ static size_t cp_bytes(long long heads, long long nb, int d, LinCp* out, void* b
     uint8_t* q = static_cast<uint8_t*>(base);
     out->dC = reinterpret_cast<float*>(q);
     out->g = reinterpret_cast<float*>(q + b_dc);
-    out->c0 = reinterpret_cast<__nv_bfloat16*>(q + b_dc + b_g);
+    out->dQ = nullptr;
   }
   return b_dc + b_g + b_c0;
 }
 
+template <int D, int MODE>
+static cudaError_t set_smem() {
+  return cudaFuncSetAttribute(lin_tc_fwd_kernel<D, MODE>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D, MODE>::SMEM);
+}
+
 template <int D>
 static cudaError_t fwd_t(const LinearProblem& lp, void* workspace, cudaStream_t s) {
-  const int smem = Cfg<D>::SMEM;
   const bool cp_path = workspace != nullptr;
   cudaError_t e;
-  for (auto fn : {lin_tc_fwd_kernel<D, MODE_SEQ>, lin_tc_fwd_kernel<D, MODE_DELTA>,
-                  lin_tc_fwd_kernel<D, MODE_OUT>})
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-        cudaSuccess) {
-      note_failure("linear chunked forward: shared memory attribute");
-      return e;
-    }
+  if ((e = cp_path ? set_smem<D, MODE_DELTA>() : set_smem<D, MODE_SEQ>()) != cudaSuccess ||
+      (cp_path && (e = set_smem<D, MODE_OUT>()) != cudaSuccess)) {
+    note_failure("linear chunked forward: shared memory attribute");
+    return e;
+  }
   Problem p{};  // the bf16 tensor-map helper's view of the shapes
   p.B = lp.B; p.T = lp.T; p.H = lp.H; p.d = lp.d;
   p.sB = lp.sB; p.sT = lp.sT; p.sH = lp.sH;
@@ -598,60 +625,63 @@ static cudaError_t fwd_t(const LinearProblem& lp, void* workspace, cudaStream_t 
   mc = m1;  // unused by the sequential mode
   if (cp_path) {
     cp_bytes(heads, nb, D, &cp, workspace);
-    if (!make_tmap_c0(&mc, cp.c0, heads * (nb + 1) * D, D)) {
+    if (!make_tmap_c0(&mc, cp.dC, heads * nb * D, D)) {
       note_failure("linear chunked forward: TMA descriptor of the workspace");
       return cudaErrorInvalidValue;
     }
   }
   if (!cp_path) {
     if (heads > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    lin_tc_fwd_kernel<D, MODE_SEQ><<<(unsigned)heads, kThreads, smem, s>>>(m1, m2, mv, ma, my, mc,
-                                                                          lp, cp);
+    using C = Cfg<D, MODE_SEQ>;
+    lin_tc_fwd_kernel<D, MODE_SEQ>
+        <<<(unsigned)heads, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
   } else {
-    const long long grid = heads * nb;
-    if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    lin_tc_fwd_kernel<D, MODE_DELTA><<<(unsigned)grid, kThreads, smem, s>>>(m1, m2, mv, ma, my, mc,
-                                                                           lp, cp);
+    const long long grid = heads * nb, ctas = heads * (D / 8);
+    if (grid > 0x7fffffffLL || ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    using CD = Cfg<D, MODE_DELTA>;
+    using CO = Cfg<D, MODE_OUT>;
+    lin_tc_fwd_kernel<D, MODE_DELTA>
+        <<<(unsigned)grid, CD::THREADS, CD::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
     if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
-    scan_kernel<D, false><<<(unsigned)(heads * (D / 8)), 256, 0, s>>>(cp, cp.c0);
+    scan_kernel<D, false><<<(unsigned)ctas, 256, 0, s>>>(cp, (int)ctas);
     if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
-    lin_tc_fwd_kernel<D, MODE_OUT><<<(unsigned)grid, kThreads, smem, s>>>(m1, m2, mv, ma, my, mc,
-                                                                         lp, cp);
+    lin_tc_fwd_kernel<D, MODE_OUT>
+        <<<(unsigned)grid, CO::THREADS, CO::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked forward: launch");
   return e;
 }
 
-// The state passes the chunked backward needs (relation_linear_tc_bwd.cu), in the
-// workspace laid out by bwd_bytes: the forward's states entering every block and the final
-// one (cp.c0), then the state's adjoint leaving every block (dcb, bf16 [heads][nb][D][64]).
-// Four launches: forward DELTA, forward scan, BDELTA (Qs^T dY per block), reverse scan.
-size_t bwd_bytes(long long heads, long long nb, int d, LinCp* cp, __nv_bfloat16** dcb,
-                 void* base) {
+// The state passes the chunked backward needs (relation_linear_tc_bwd.cu), in the workspace
+// laid out by bwd_bytes: the forward's states entering every block (bf16, in dC's rows) and the
+// state's adjoint leaving every block (bf16, in dQ's rows).  Two launches: the blocks'
+// contributions to both, and both scans.
+size_t bwd_bytes(long long heads, long long nb, int d, LinCp* cp, void* base) {
   const size_t f = cp_bytes(heads, nb, d, cp, base);
-  if (dcb) *dcb = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(base) + f);
+  // dQ's fp32 rows fill what the forward's nb + 1 and the adjoints' nb bf16 rows would take
+  if (cp)
+    cp->dQ = reinterpret_cast<float*>(static_cast<uint8_t*>(base) +
+                                      align256((size_t)(heads * nb * d) * 64 * 4) +
+                                      align256((size_t)(heads * nb * d) * 4));
   return f + align256((size_t)(heads * nb * d) * 64 * 2);
 }
 
-template <int D>
-cudaError_t states_t(const LinearProblem& lp, const void* dy, void* workspace, cudaStream_t s) {
-  const int smem = Cfg<D>::SMEM;
+cudaError_t launch_states(const LinearProblem& lp, const void* dy, void* workspace,
+                          cudaStream_t s) {
+  constexpr int D = 64;
   cudaError_t e;
-  for (auto fn : {lin_tc_fwd_kernel<D, MODE_DELTA>, lin_tc_fwd_kernel<D, MODE_BDELTA>})
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-        cudaSuccess) {
-      note_failure("linear chunked backward: shared memory attribute");
-      return e;
-    }
+  if ((e = set_smem<D, MODE_BOTH>()) != cudaSuccess) {
+    note_failure("linear chunked backward: shared memory attribute");
+    return e;
+  }
   Problem p{};
   p.B = lp.B; p.T = lp.T; p.H = lp.H; p.d = lp.d;
   p.sB = lp.sB; p.sT = lp.sT; p.sH = lp.sH;
   const int nb = (lp.T + LT - 1) / LT;
-  const long long heads = (long long)lp.B * lp.H * (D / NC);
+  const long long heads = (long long)lp.B * lp.H;
   LinCp cp{};
   cp.nb = nb;
-  __nv_bfloat16* dcb = nullptr;
-  bwd_bytes(heads, nb, D, &cp, &dcb, workspace);
+  bwd_bytes(heads, nb, D, &cp, workspace);
   CUtensorMap m1, m2, mv, mg, ma;
   if (!tc::make_tmap_bf16(&m1, lp.p1, p, LT) || !tc::make_tmap_bf16(&m2, lp.p2, p, LT) ||
       !tc::make_tmap_bf16(&mv, lp.v, p, LT) || !tc::make_tmap_bf16(&mg, dy, p, LT) ||
@@ -659,22 +689,17 @@ cudaError_t states_t(const LinearProblem& lp, const void* dy, void* workspace, c
     note_failure("linear chunked backward: TMA descriptors");
     return cudaErrorInvalidValue;
   }
-  const long long grid = heads * nb;
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  // (the Y map is unused in these modes; m1 stands in)
-  lin_tc_fwd_kernel<D, MODE_DELTA><<<(unsigned)grid, kThreads, smem, s>>>(m1, m2, mv, ma, m1, m1,
-                                                                         lp, cp);
+  const long long grid = heads * nb, ctas = heads * (D / 8);
+  if (grid > 0x7fffffffLL || 2 * ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  // (the Y and state maps are unused in this mode; m1 stands in)
+  using C = Cfg<D, MODE_BOTH>;
+  lin_tc_fwd_kernel<D, MODE_BOTH>
+      <<<(unsigned)grid, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mg, ma, m1, m1, lp, cp);
   if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked backward: launch"); return e; }
-  scan_kernel<D, false><<<(unsigned)(heads * (D / 8)), 256, 0, s>>>(cp, cp.c0);
-  if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked backward: launch"); return e; }
-  lin_tc_fwd_kernel<D, MODE_BDELTA><<<(unsigned)grid, kThreads, smem, s>>>(m1, m2, mg, ma, m1, m1,
-                                                                          lp, cp);
-  if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked backward: launch"); return e; }
-  scan_kernel<D, true><<<(unsigned)(heads * (D / 8)), 256, 0, s>>>(cp, dcb);
+  scan_kernel<D, true><<<(unsigned)(2 * ctas), 256, 0, s>>>(cp, (int)ctas);
   if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked backward: launch");
   return e;
 }
-template cudaError_t states_t<64>(const LinearProblem&, const void*, void*, cudaStream_t);
 
 }  // namespace lintc
 

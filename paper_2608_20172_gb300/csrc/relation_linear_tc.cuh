@@ -18,26 +18,23 @@ namespace lintc {
 
 constexpr int LT = 128;          // tokens per block
 constexpr int NC = 64;           // information columns per CTA
-constexpr int kThreads = 192;    // warps 0-3 elementwise, 4 TMA, 5 MMA
-constexpr int kTmemCols = 256;   // S 128 | E 64 | C 64
-constexpr int COL_S = 0, COL_E = 128, COL_C = 192;
 constexpr float kClampLog2 = 120.0f;
 
 // Modes of the kernel: SEQ walks all blocks of a (head, split) in order with the state in
 // TMEM; the chunk-parallel pair takes one block per CTA: DELTA writes the block's state
 // contribution sum_j KL_j I~_j^T and decay a_L (fp32) to the workspace, OUT reads the
 // state the block starts from (bf16, produced by scan_kernel) and writes the block's Y.
-// BDELTA is DELTA for the backward: the block's contribution to the state's adjoint,
-// Qs^T dY (Qs in KL's place, dY in I~'s).
-enum : int { MODE_SEQ = 0, MODE_DELTA = 1, MODE_OUT = 2, MODE_BDELTA = 3 };
+// BOTH (the backward, d_h = 64) is DELTA together with the block's contribution to the
+// state's adjoint, Qs^T dY.
+enum : int { MODE_SEQ = 0, MODE_DELTA = 1, MODE_OUT = 2, MODE_BOTH = 3 };
 
-// Workspace of the chunk-parallel forward, per (head, split, block): dC [D][64] fp32, the
-// decay g [D] fp32, and per (head, split) nb + 1 states C0 [D][64] bf16 (the state entering
-// every block, then the final one).
+// Workspace of the chunk-parallel forms, per (head, split, block): dC [D][64] fp32 (after the
+// scan every row's first 128 bytes hold the row of the state entering the block, bf16), the
+// decay g [D] fp32 and, for the backward, dQ [D][64] likewise (the adjoint leaving the block).
 struct LinCp {
   float* dC;
+  float* dQ;
   float* g;
-  __nv_bfloat16* c0;
   int nb;
 };
 
@@ -59,8 +56,9 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* m, 
       "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
-__device__ __forceinline__ void ew_sync() {  // the 128 elementwise threads
-  asm volatile("bar.sync 1, 128;" ::: "memory");
+template <int NG>
+__device__ __forceinline__ void ew_sync() {  // the elementwise warpgroups
+  asm volatile("bar.sync 1, %0;" ::"n"(NG * 128) : "memory");
 }
 // byte offset of element (row r, column c) in a tile of 128-byte-swizzled rows of 64
 // bf16 columns, blocks of `rows` rows per 64 columns
@@ -68,16 +66,51 @@ __device__ __forceinline__ uint32_t swz(int r, int c, int rows) {
   return (uint32_t)((c >> 6) * rows * 128 + r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4) +
                     (c & 7) * 2);
 }
+// Ask Self's sums of token t over its D channels (p1, p2: 128-byte-swizzled bf16 tiles),
+// those of `which`: 1 p1 . p2, 2 |p1|^2, 4 |p2|^2.  Each is one chain of multiply-adds in
+// channel order whichever thread takes it.  ALL = 7 where `which` is 7 at compile time.
+template <int D, int ALL>
+__device__ __forceinline__ void ask_self_sums(const uint8_t* p1s, const uint8_t* p2s, int t,
+                                              int which, float* dot, float* n1, float* n2) {
+  auto pass = [&](auto f, bool r1, bool r2) {
+#pragma unroll
+    for (int k = 0; k < D / 8; ++k) {
+      const uint32_t off = (k >> 3) * LT * 128 + t * 128 + (((k & 7) ^ (t & 7)) << 4);
+      uint4 a4 = make_uint4(0, 0, 0, 0), b4 = a4;
+      if (r1) a4 = *reinterpret_cast<const uint4*>(p1s + off);
+      if (r2) b4 = *reinterpret_cast<const uint4*>(p2s + off);
+      const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        f(__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e])),
+          __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e])));
+    }
+  };
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+  if (ALL == 7) {
+    pass([&](float2 x, float2 y) {
+      s0 = fmaf(x.x, y.x, fmaf(x.y, y.y, s0));
+      s1 = fmaf(x.x, x.x, fmaf(x.y, x.y, s1));
+      s2 = fmaf(y.x, y.x, fmaf(y.y, y.y, s2));
+    }, true, true);
+    dot[t] = s0;
+    n1[t] = s1;
+    n2[t] = s2;
+  } else if (which == 1) {
+    pass([&](float2 x, float2 y) { s0 = fmaf(x.x, y.x, fmaf(x.y, y.y, s0)); }, true, true);
+    dot[t] = s0;
+  } else if (which == 2) {
+    pass([&](float2 x, float2) { s1 = fmaf(x.x, x.x, fmaf(x.y, x.y, s1)); }, true, false);
+    n1[t] = s1;
+  } else {
+    pass([&](float2, float2 y) { s2 = fmaf(y.x, y.x, fmaf(y.y, y.y, s2)); }, false, true);
+    n2[t] = s2;
+  }
+}
 // element (token, channel) of [d / 32][128][32] fp32 tiles written by the swizzled
 // retention map: the 16-byte groups of a token's 128-byte row permuted by (token & 7)
 __device__ __forceinline__ int al_swz(int tok, int ch) {
   return (ch >> 5) * (LT * 32) + tok * 32 + ((((ch & 31) >> 2) ^ (tok & 7)) << 2) + (ch & 3);
-}
-__device__ __forceinline__ float ld_bf(const uint8_t* base, uint32_t off) {
-  return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(base + off));
-}
-__device__ __forceinline__ void st_bf(uint8_t* base, uint32_t off, float x) {
-  *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(x);
 }
 
 
@@ -105,8 +138,8 @@ inline bool make_tmap_alpha(CUtensorMap* m, const LinearProblem& p, bool swz = f
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2-D map over the bf16 C0 rows of the workspace: [rows][64], boxes of D rows, 128-byte
-// swizzle (the MN-major B layout of the E = Qs C_0 product).
+// 2-D map over the bf16 state rows of the workspace: [rows][64] at a pitch of 256 bytes, boxes
+// of D rows, 128-byte swizzle (the MN-major B layout of the E = Qs C_0 product).
 inline bool make_tmap_c0(CUtensorMap* m, void* base, long long rows, int d) {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -119,7 +152,7 @@ inline bool make_tmap_c0(CUtensorMap* m, void* base, long long rows, int d) {
     fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
   }
   cuuint64_t dims[2] = {64, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {128};
+  cuuint64_t strides[1] = {256};
   cuuint32_t box[2] = {64, (cuuint32_t)d};
   cuuint32_t estr[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
@@ -129,10 +162,8 @@ inline bool make_tmap_c0(CUtensorMap* m, void* base, long long rows, int d) {
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t bwd_bytes(long long heads, long long nb, int d, LinCp* cp, __nv_bfloat16** dcb,
-                 void* base);
-template <int D>
-cudaError_t states_t(const LinearProblem& lp, const void* dy, void* workspace, cudaStream_t s);
+size_t bwd_bytes(long long heads, long long nb, int d, LinCp* cp, void* base);
+cudaError_t launch_states(const LinearProblem& lp, const void* dy, void* workspace, cudaStream_t s);
 
 }  // namespace lintc
 }  // namespace rel

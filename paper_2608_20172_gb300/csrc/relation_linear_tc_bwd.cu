@@ -2,10 +2,10 @@
 // App. A.4; the paper writes out the forward only), bf16, d_h = 64.
 //
 // Reverse mode through the 128-token blocks of relation_linear_tc.cu, every block in
-// parallel.  The state passes come first (relation_linear_tc.cu, states_t): the state C_0
-// entering every block and the final one (forward DELTA + scan), and the state's adjoint
-// dC leaving every block, dC(b - 1) = Diag(a_L(b)) dC(b) + Qs_b^T dY_b (BDELTA + reverse
-// scan).  Then one CTA per block, with G = dY, A = tril(Qm Km^T, -1), dA = tril(G I~^T, -1):
+// parallel.  The state passes come first (relation_linear_tc.cu, launch_states): the blocks'
+// contributions to the state and to its adjoint in one launch, then the scans of the state
+// C_0 entering every block and of the adjoint dC leaving it,
+// dC(b - 1) = Diag(a_L(b)) dC(b) + Qs_b^T dY_b.  Then one CTA per block, with G = dY, A = tril(Qm Km^T, -1), dA = tril(G I~^T, -1):
 //   X  = dA Km + G (2^{L_m} C_0)^T        dq'_t = 2^{L_t - L_m} X_t
 //   Y  = dA^T Qm + Ys,  Ys = I~ (2^{L_end - L_m} dC)^T   dk'_j = 2^{L_m - L_j} Y_j
 //   dI~ = G + A^T G + KL dC
@@ -23,9 +23,15 @@
 // then cancel up to fp32 rounding, where rounding Qm and Km independently of q' and k'
 // would leave errors of the bf16 unit, divided by alpha_u.  The products are tcgen05
 // MMAs with fp32 accumulation in TMEM; the masked A and dA go through shared memory so that
-// the transposed products read them as MN-major operands.  Warps 0-3 (thread = token or
-// channel) do the elementwise work, warp 4 the TMA loads and stores, warp 5 (warp-uniform,
-// elect.sync) the MMAs.  Every mbarrier wait is bounded (common.cuh).
+// the transposed products read them as MN-major operands.  Four warpgroups do the
+// elementwise work (thread = token; the groups split the channels or columns; the sums whose
+// rounding the cancellation above rests on stay one chain each, in the order of the block's
+// tokens or channels, on different groups), then a warp the TMA loads and one (warp-uniform,
+// elect.sync) the MMAs.  One CTA per SM (212 KB), so latency bounds it: a block's phases and
+// barriers around small products, nothing else resident.  B 8, H 12, T 2048: 361 us with one
+// elementwise warpgroup, 197 with four; the state passes 161 us as four launches, 66 as two.
+// Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps meeting the
+// warpgroups' barriers and skips the work between them.
 #include "relation_linear_tc.cuh"
 
 namespace rel {
@@ -33,6 +39,8 @@ namespace lintc {
 namespace bwd {
 
 constexpr int D = 64;
+constexpr int NG = 4;                      // elementwise warpgroups
+constexpr int EW = NG * 128, W_TMA = NG * 4, W_MMA = W_TMA + 1, kThreads = EW + 64;
 constexpr int kTmemCols = 512;  // scratch S / dA 128 | X 64 | Y 64 | dI~ 64 | Ys 64
 constexpr int COL_SC = 0, COL_X = 128, COL_Y = 192, COL_DI = 256, COL_YS = 320;
 // shared memory (bytes): 128-token tiles of 64 bf16 columns are 16 KB
@@ -49,8 +57,8 @@ constexpr int C64 = 64 * 64 * 2;          // a [64 c][64 n] bf16 tile
 constexpr int OFF_C0 = OFF_DAS + 2 * T16; // C_0, then 2^{L_m} C_0 in place
 constexpr int OFF_DC = OFF_C0 + C64;      // dC (the state's adjoint leaving the block)
 constexpr int OFF_DCP = OFF_DC + C64;     // 2^{L_end - L_m} dC
-constexpr int OFF_SC = OFF_DCP + C64;     // scalars, 9 x 128 fp32
-constexpr int OFF_BAR = OFF_SC + 9 * LT * 4;
+constexpr int OFF_SC = OFF_DCP + C64;     // scalars, 15 x 128 fp32
+constexpr int OFF_BAR = OFF_SC + 15 * LT * 4;
 constexpr int SMEM = OFF_BAR + 128 + 1024;
 static_assert(SMEM <= 232448, "shared memory");
 constexpr uint32_t LOAD_BYTES = 4 * T16 + LT * 64 * 4 + 2 * C64;
@@ -81,16 +89,13 @@ __device__ __forceinline__ void qm_km(float x, float y, float s1, float s2, floa
 constexpr float kSmallAlpha = 1.0f / 1024.0f;
 
 // The small-retention fix-up's tiles (dY, p1, p2 loaded again), over the epilogue's dL and
-// Km Ys arrays once phase F has read them
+// Km Ys arrays once the suffix sums are out, and after them the list of its (token, channel)s
 constexpr int OFF_FIX_G = OFF_KL, OFF_FIX_P1 = OFF_KL + T16, OFF_FIX_P2 = OFF_KL + 2 * T16;
-static_assert(OFF_FIX_P2 + T16 <= OFF_C0 && OFF_KL % 1024 == 0, "fix-up tiles");
+constexpr int OFF_FIX_LIST = OFF_FIX_P2 + T16;  // up to 128 x 64 16-bit entries
+static_assert(OFF_FIX_LIST + LT * 64 * 2 <= OFF_C0 && OFF_FIX_LIST >= OFF_TS &&
+              OFF_KL % 1024 == 0, "fix-up tiles");
 
 enum : int { B_LOAD = 0, B_OPS, B_S, B_A, B_DA, B_DAS, B_MM, B_RELOAD, B_FIX, NBAR };
-
-// Some lane of the warp has a token flagged in its 64-bit mask.
-__device__ __forceinline__ bool small_any_warp(unsigned long long m) {
-  return __any_sync(0xffffffffu, m != 0ull);
-}
 
 __global__ void __launch_bounds__(kThreads, 1)
     lin_tc_bwd_kernel(const __grid_constant__ CUtensorMap tmP1,
@@ -98,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                       const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmG,
                       const __grid_constant__ CUtensorMap tmA,
-                      const __grid_constant__ CUtensorMap tmC0,  // states: [heads][nb + 1][64][64]
+                      const __grid_constant__ CUtensorMap tmC0,  // states: [heads][nb][64][64]
                       const __grid_constant__ CUtensorMap tmDC,  // adjoints: [heads][nb][64][64]
                       const __grid_constant__ CUtensorMap tmDP1,
                       const __grid_constant__ CUtensorMap tmDP2,
@@ -111,17 +116,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_BAR + 96);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_BAR + 104);
   int* clamped = reinterpret_cast<int*>(smem + OFF_BAR + 108);
-  volatile int* fix_any = reinterpret_cast<volatile int*>(smem + OFF_BAR + 112);
+  int* fix_count = reinterpret_cast<int*>(smem + OFF_BAR + 112);
   float* sc = reinterpret_cast<float*>(smem + OFF_SC);
-  float* sq = sc;                 // S_t / |p1_t|
-  float* sk = sc + LT;            // S_t / |p2_t|
-  float* s_self = sc + 2 * LT;    // S_t
-  float* r1 = sc + 3 * LT;        // 1 / |p1_t|
-  float* r2 = sc + 4 * LT;        // 1 / |p2_t|
-  float* half_sum = sc + 5 * LT;  // [2][128]: per-channel sums of the two halves (log2 alpha,
-                                  // then dL and Km Ys)
-  float* lmid_s = sc + 7 * LT;    // [128] L_m per channel
-  float* lend_s = sc + 8 * LT;    // [128] L_end per channel
+  float* s_dot = sc;             // p1_t . p2_t
+  float* s_n1 = sc + LT;         // |p1_t|^2
+  float* s_n2 = sc + 2 * LT;     // |p2_t|^2
+  float* sum_l = sc + 3 * LT;    // [2][64] per-channel sums over the half blocks: log2 alpha
+  float* sum_g = sc + 4 * LT;    // dL
+  float* sum_t = sc + 5 * LT;    // Km Ys
+  float* a1_s = sc + 6 * LT;     // [4][128] the groups' shares of p1_t . dq'_t
+  float* a2_s = sc + 10 * LT;    // [4][128] and of p2_t . dk'_t
+  float* e0_s = sc + 14 * LT;    // [64] the end term's state part
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blk = (int)(blockIdx.x % nb);
@@ -131,20 +136,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NBAR; ++i)
-      mbar_init(bar(i), (i == B_OPS || i == B_A || i == B_DAS) ? 128 : 1);
+      mbar_init(bar(i), (i == B_OPS || i == B_A || i == B_DAS) ? EW : 1);
     *abort_flag = 0;
     *clamped = 0;
-    *fix_any = 0;
+    *fix_count = 0;
     fence_mbar_init();
   }
-  if (warp == 5) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  if (warp == W_MMA) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
 
-  if (warp == 4) {
+  if (warp == W_TMA) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const uint32_t lb = bar(B_LOAD);
@@ -155,7 +160,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tma_load_4d(sb + OFF_G, &tmG, lb, 0, t0, h, b);
       for (int k = 0; k < 2; ++k)
         tma_load_4d(sb + OFF_AL + k * LT * 128, &tmA, lb, k * 32, t0, h, b);
-      tma_load_2d(sb + OFF_C0, &tmC0, lb, 0, (bh * (nb + 1) + blk) * D);
+      tma_load_2d(sb + OFF_C0, &tmC0, lb, 0, (bh * nb + blk) * D);
       tma_load_2d(sb + OFF_DC, &tmDC, lb, 0, (bh * nb + blk) * D);
       // p1 and p2 again (Qm and Km overwrote them) once the MMAs reading those are done
       bool ok = mbar_wait(bar(B_MM), 0, ab);
@@ -167,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       drain_wait(lb, 0);
       if (ok && ab.raised()) drain_wait(bar(B_RELOAD), 0);
     }
-  } else if (warp == 5) {
+  } else if (warp == W_MMA) {
     // ------------------------------------------------------------------ MMA issuer
     constexpr uint32_t id_s = idesc_bf16_f32(128, 128, false, false);  // S, dA
     constexpr uint32_t id_kk = idesc_bf16_f32(128, 64, false, false);  // A, B K-major
@@ -227,8 +232,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ elementwise
-    const int t = threadIdx.x;  // token of the block / TMEM lane; channel c = t & 63, half
-    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    const int grp = warp >> 2;        // warpgroup
+    const int t = threadIdx.x & 127;  // token of the block / TMEM lane; channel c = t & 63, half
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float inv_tau_sqrt_d = 1.0f / (p.tau_s * sqrtf((float)D));
     const int c = t & 63, half = t >> 6;
     uint8_t* const p1s = smem + OFF_P1;
@@ -239,284 +245,257 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     float* const gl = reinterpret_cast<float*>(smem + OFF_GL);  // dL [t][GS]
     float* const ts = reinterpret_cast<float*>(smem + OFF_TS);  // Km Ys [t][GS]
-    bool ok = true, my_clamp = false;
-    do {
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD), 0, ab));
-      if (!ok) break;
-      // ---- phase A (thread = token): S_t, 1 / |p1_t|, 1 / |p2_t| (zero past T)
-      {
-        float dot = 0.f, n1 = 0.f, n2 = 0.f;
+    auto bf2 = [](uint32_t w) { return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w)); };
+    bool my_clamp = false;
+    bool ok = __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD), 0, ab));
+    // ---- the sums of S_t, |p1_t|, |p2_t| (groups 0, 1, 2) beside the running sums of log2
+    // alpha in place of alpha (group 3: channel and half block, the second half's relative to
+    // its start; 16 tokens ahead)
+    if (ok) {
+      if (grp < 3) {
+        ask_self_sums<D, 0>(p1s, p2s, t, 1 << grp, s_dot, s_n1, s_n2);
+      } else {
+        float lsum = 0.f;
+        for (int i0 = 0; i0 < 64; i0 += 16) {
+          float la[16];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint32_t off = t * 128 + ((k ^ (t & 7)) << 4);
-          const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-          const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-          const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+          for (int u = 0; u < 16; ++u) {
+            const int tok = half * 64 + i0 + u;
+            la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
+          }
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-            const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-            dot = fmaf(x.x, y.x, fmaf(x.y, y.y, dot));
-            n1 = fmaf(x.x, x.x, fmaf(x.y, x.y, n1));
-            n2 = fmaf(y.x, y.x, fmaf(y.y, y.y, n2));
+          for (int u = 0; u < 16; ++u) {
+            lsum += la[u];
+            al_at(half * 64 + i0 + u, c) = lsum;
           }
         }
-        float S = 0.f, i1 = 0.f, i2 = 0.f;
-        if (t0 + t < p.T) {
-          S = 1.0f / (1.0f + __expf(-dot * inv_tau_sqrt_d));
-          i1 = rsqrtf(n1);
-          i2 = rsqrtf(n2);
-        }
-        sq[t] = S * i1;
-        sk[t] = S * i2;
-        s_self[t] = S;
-        r1[t] = i1;
-        r2[t] = i2;
+        sum_l[t] = lsum;
       }
-      // ---- phase B, pass 1 (thread = channel and half block): running sums of log2 alpha
-      // in place of alpha (the second half's relative to its start), 16 tokens ahead
-      float lsum = 0.f;
-      for (int i0 = 0; i0 < 64; i0 += 16) {
-        float la[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int tok = half * 64 + i0 + u;
-          la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          lsum += la[u];
-          al_at(half * 64 + i0 + u, c) = lsum;
-        }
+    }
+    ew_sync<NG>();
+    float S = 0.f, i1 = 0.f, i2 = 0.f, s1 = 0.f, s2 = 0.f;  // token t (zero past T)
+    if (ok) {
+      if (t0 + t < p.T) {
+        S = 1.0f / (1.0f + __expf(-s_dot[t] * inv_tau_sqrt_d));
+        i1 = rsqrtf(s_n1[t]);
+        i2 = rsqrtf(s_n2[t]);
+        s1 = S * i1;
+        s2 = S * i2;
       }
-      half_sum[half * 128 + c] = lsum;
-      ew_sync();
-      const float l_mid = half_sum[c], l_end = half_sum[c] + half_sum[128 + c];
-      if (half == 0) {
-        lmid_s[c] = l_mid;
-        lend_s[c] = l_end;
-        // C_0 scaled by 2^{L_m} in place, dC scaled by 2^{L_end - L_m} into its own tile
-        // (row c; both factors <= 1)
+      {
+        // C_0 scaled by 2^{L_m} in place, dC scaled by 2^{L_end - L_m} into its own tile (both
+        // factors <= 1): one 16-byte group of one row per thread
+        const int r = threadIdx.x >> 3, k = threadIdx.x & 7;
+        const float l_mid = sum_l[r], l_end = sum_l[r] + sum_l[64 + r];
         const float f0 = ex2_approx(l_mid), f1 = ex2_approx(l_end - l_mid);
-        uint8_t* r0 = smem + OFF_C0 + c * 128;
-        const uint8_t* rd = smem + OFF_DC + c * 128;
-        uint8_t* rp = smem + OFF_DCP + c * 128;
+        uint4* r0 = reinterpret_cast<uint4*>(smem + OFF_C0 + r * 128 + 16 * k);
+        const uint4 a4 = *r0;
+        const uint4 d4 = *reinterpret_cast<const uint4*>(smem + OFF_DC + r * 128 + 16 * k);
+        const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
+        uint32_t oa[4], od[4];
 #pragma unroll
-        for (int k0 = 0; k0 < 8; ++k0) {
-          const int k = (k0 + c) & 7;  // rows 128 bytes apart: rotate the 16-byte groups
-          const uint4 a4 = *reinterpret_cast<const uint4*>(r0 + 16 * k);
-          const uint4 d4 = *reinterpret_cast<const uint4*>(rd + 16 * k);
-          const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
-          uint32_t oa[4], od[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-            const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&dw[e]));
-            oa[e] = pack_bf16x2(x.x * f0, x.y * f0);
-            od[e] = pack_bf16x2(y.x * f1, y.y * f1);
-          }
-          *reinterpret_cast<uint4*>(r0 + 16 * k) = make_uint4(oa[0], oa[1], oa[2], oa[3]);
-          *reinterpret_cast<uint4*>(rp + 16 * k) = make_uint4(od[0], od[1], od[2], od[3]);
+        for (int e = 0; e < 4; ++e) {
+          const float2 x = bf2(aw[e]), y = bf2(dw[e]);
+          oa[e] = pack_bf16x2(x.x * f0, x.y * f0);
+          od[e] = pack_bf16x2(y.x * f1, y.y * f1);
         }
+        *r0 = make_uint4(oa[0], oa[1], oa[2], oa[3]);
+        *reinterpret_cast<uint4*>(smem + OFF_DCP + r * 128 + 16 * k) =
+            make_uint4(od[0], od[1], od[2], od[3]);
       }
-      ew_sync();
-      // ---- phase B, pass 2 (thread = token): Qm, Km in place of p1, p2, and KL
-      {
-        const float s1 = sq[t], s2 = sk[t];
+      // ---- Qm, Km in place of p1, p2, and KL: token t, the group's 16 channels
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint32_t off = t * 128 + ((k ^ (t & 7)) << 4);
-          const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-          const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-          const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k));
-          const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k + 4));
-          const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
-          const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
-          uint32_t qm[4], km[4], kl[4];
+      for (int k = 2 * grp, k1 = 0; k1 < 2; ++k, ++k1) {
+        const uint32_t off = t * 128 + ((k ^ (t & 7)) << 4);
+        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
+        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
+        const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k));
+        const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k + 4));
+        const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
+        const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+        uint32_t qm[4], km[4], kl[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-            const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-            float r[2][3];
+        for (int e = 0; e < 4; ++e) {
+          const float2 x = bf2(aw[e]), y = bf2(bw[e]);
+          float r[2][3];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const int ch = 8 * k + 2 * e + u;
-              const float Lm = lmid_s[ch];
-              const float L = Lv[2 * e + u] + (t >= 64 ? Lm : 0.f);
-              const float dm = dm_of(Lv[2 * e + u], Lm, t >= 64, my_clamp);
-              const float xv = u ? x.y : x.x, yv = u ? y.y : y.x;
-              qm_km(xv, yv, s1, s2, dm, r[u][0], r[u][1]);
-              r[u][2] = yv * s2 * ex2_approx(lend_s[ch] - L);       // KL (factor <= 1)
-            }
-            qm[e] = pack_bf16x2(r[0][0], r[1][0]);
-            km[e] = pack_bf16x2(r[0][1], r[1][1]);
-            kl[e] = pack_bf16x2(r[0][2], r[1][2]);
+          for (int u = 0; u < 2; ++u) {
+            const int ch = 8 * k + 2 * e + u;
+            const float Lm = sum_l[ch];
+            const float L = Lv[2 * e + u] + (t >= 64 ? Lm : 0.f);
+            const float dm = dm_of(Lv[2 * e + u], Lm, t >= 64, my_clamp);
+            const float xv = u ? x.y : x.x, yv = u ? y.y : y.x;
+            qm_km(xv, yv, s1, s2, dm, r[u][0], r[u][1]);
+            r[u][2] = yv * s2 * ex2_approx((Lm + sum_l[64 + ch]) - L);  // KL (factor <= 1)
           }
-          *reinterpret_cast<uint4*>(p1s + off) = make_uint4(qm[0], qm[1], qm[2], qm[3]);
-          *reinterpret_cast<uint4*>(p2s + off) = make_uint4(km[0], km[1], km[2], km[3]);
-          *reinterpret_cast<uint4*>(smem + OFF_KL + off) = make_uint4(kl[0], kl[1], kl[2], kl[3]);
+          qm[e] = pack_bf16x2(r[0][0], r[1][0]);
+          km[e] = pack_bf16x2(r[0][1], r[1][1]);
+          kl[e] = pack_bf16x2(r[0][2], r[1][2]);
         }
+        *reinterpret_cast<uint4*>(p1s + off) = make_uint4(qm[0], qm[1], qm[2], qm[3]);
+        *reinterpret_cast<uint4*>(p2s + off) = make_uint4(km[0], km[1], km[2], km[3]);
+        *reinterpret_cast<uint4*>(smem + OFF_KL + off) = make_uint4(kl[0], kl[1], kl[2], kl[3]);
       }
       fence_async_smem();
-      ew_sync();
       mbar_arrive(bar(B_OPS));
-      // ---- phase D: A = tril(S, -1), then dA = tril(G I~^T, -1), as bf16 rows [t][j] in
-      // shared memory (the products read them K-major and, transposed, MN-major)
-      for (int pass = 0; pass < 2; ++pass) {
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(pass == 0 ? B_S : B_DA), 0, ab));
-        if (!ok) break;
-        tc_fence_after();
-        uint8_t* dst = smem + (pass == 0 ? OFF_AS : OFF_DAS);
-#pragma unroll
-        for (int c0 = 0; c0 < LT; c0 += 32) {
-          uint32_t s[32], pk[16];
-          tmem_ld32(trow + COL_SC + c0, s);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const float lo = (c0 + j < t) ? __uint_as_float(s[j]) : 0.f;
-            const float hi = (c0 + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
-            pk[j >> 1] = pack_bf16x2(lo, hi);
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(dst + swz(t, c0 + 8 * q, LT)) =
-                make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-        }
-        fence_async_smem();
-        tc_fence_before();
-        mbar_arrive(bar(pass == 0 ? B_A : B_DAS));
-      }
-      if (!ok) break;
-      // ---- phase E (thread = token): every product done, p1 and p2 back in shared memory
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_MM), 0, ab) && mbar_wait(bar(B_RELOAD), 0, ab));
+    }
+    // ---- A = tril(S, -1), then dA = tril(G I~^T, -1), as bf16 rows [t][j] in shared memory
+    // (the products read them K-major and, transposed, MN-major): 32 columns per group
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(pass == 0 ? B_S : B_DA), 0, ab));
       if (!ok) break;
       tc_fence_after();
-      {
-        const float s1 = sq[t], s2 = sk[t], i1 = r1[t], i2 = r2[t], S = s_self[t];
-        uint8_t* const gs = smem + OFF_G;
-        bool unused_clamp = false;
-        // channels [c0, c0 + 32): X, Y = dA^T Qm + Ys, Ys (and dI~) from TMEM
-        auto load_xy = [&](int c0, uint32_t (&x)[32], uint32_t (&y)[32], uint32_t (&ys)[32],
-                           uint32_t* di) {
-          tmem_ld32(trow + COL_X + c0, x);
-          tmem_ld32(trow + COL_Y + c0, y);
-          tmem_ld32(trow + COL_YS + c0, ys);
-          if (di) tmem_ld32(trow + COL_DI + c0, di);
-          tmem_ld_wait();
-        };
-        // pass 1 (8 channels at a time): dq' = 2^{L_t - L_m} X, dk' = 2^{L_m - L_t} Y, the
-        // dots p1 . dq' and p2 . dk', dL = Qm X - Km Y and Km Ys (Qm, Km as the products
-        // read them), dv = dI~ + dY (in dY's place)
-        float A1 = 0.f, A2 = 0.f;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          uint32_t x[32], y[32], ys[32], di[32];
-          load_xy(c0, x, y, ys, di);
+      uint8_t* dst = smem + (pass == 0 ? OFF_AS : OFF_DAS);
+      const int c0 = 32 * grp;
+      uint32_t pk[16];
+      if (grp <= (warp & 3)) {  // some column of the warp's rows is unmasked
+        uint32_t s[32];
+        tmem_ld32(trow + COL_SC + c0, s);
+        tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int kc = (c0 >> 3) + k;
-            const uint32_t off = t * 128 + ((kc ^ (t & 7)) << 4);
-            const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-            const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-            const uint4 g4 = *reinterpret_cast<const uint4*>(gs + off);
-            const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc));
-            const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc + 4));
-            const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
-            const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w},
-                           gw[4] = {g4.x, g4.y, g4.z, g4.w};
-            float dl[8], tv[8];
-            uint32_t dvw[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 xa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-              const float2 yb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-              const float2 g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw[e]));
-              float dvv[2];
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int j = 8 * k + 2 * e + u;  // index within the 32 loaded columns
-                const int ch = 8 * kc + 2 * e + u;
-                const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
-                const float dm = dm_of(Lv[2 * e + u], lmid_s[ch], t >= 64, unused_clamp);
-                float qm, km;
-                qm_km(pv, kv, s1, s2, dm, qm, km);
-                const float X = __uint_as_float(x[j]), Ysv = __uint_as_float(ys[j]);
-                const float Y = __uint_as_float(y[j]) + Ysv;
-                A1 = fmaf(pv, ex2_approx(dm) * X, A1);
-                A2 = fmaf(kv, ex2_approx(-dm) * Y, A2);
-                dl[2 * e + u] = qm * X - km * Y;
-                tv[2 * e + u] = km * Ysv;
-                dvv[u] = __uint_as_float(di[j]) + (u ? g.y : g.x);
-              }
-              dvw[e] = pack_bf16x2(dvv[0], dvv[1]);
-            }
-            *reinterpret_cast<uint4*>(gs + off) = make_uint4(dvw[0], dvw[1], dvw[2], dvw[3]);
-            float* gr = gl + t * GS + 8 * kc;
-            *reinterpret_cast<float4*>(gr) = make_float4(dl[0], dl[1], dl[2], dl[3]);
-            *reinterpret_cast<float4*>(gr + 4) = make_float4(dl[4], dl[5], dl[6], dl[7]);
-            float* tr = ts + t * GS + 8 * kc;
-            *reinterpret_cast<float4*>(tr) = make_float4(tv[0], tv[1], tv[2], tv[3]);
-            *reinterpret_cast<float4*>(tr + 4) = make_float4(tv[4], tv[5], tv[6], tv[7]);
-          }
+        for (int j = 0; j < 32; j += 2) {
+          const float lo = (c0 + j < t) ? __uint_as_float(s[j]) : 0.f;
+          const float hi = (c0 + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
+          pk[j >> 1] = pack_bf16x2(lo, hi);
         }
-        // pass 2: through S_t and the normalisation of p1, p2 (written in their place)
-        //   dp1 = S/|p1| dq' - S/|p1|^3 (p1 . dq') p1 + du p2, and symmetrically dp2,
-        //   du = (p1 . dq' / |p1| + p2 . dk' / |p2|) S (1 - S) / (tau_S sqrt(d_h))
-        const float du = (i1 * A1 + i2 * A2) * S * (1.0f - S) * inv_tau_sqrt_d;
-        const float c1 = s1 * i1 * i1 * A1, c2 = s2 * i2 * i2 * A2;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          uint32_t x[32], y[32], ys[32];
-          load_xy(c0, x, y, ys, nullptr);
+      } else {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int kc = (c0 >> 3) + k;
-            const uint32_t off = t * 128 + ((kc ^ (t & 7)) << 4);
-            const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-            const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-            const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc));
-            const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc + 4));
-            const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
-            const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
-            uint32_t o1[4], o2[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 xa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-              const float2 yb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[e]));
-              float r1v[2], r2v[2];
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                const int j = 8 * k + 2 * e + u;
-                const int ch = 8 * kc + 2 * e + u;
-                const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
-                const float dm = dm_of(Lv[2 * e + u], lmid_s[ch], t >= 64, unused_clamp);
-                const float dq = ex2_approx(dm) * __uint_as_float(x[j]);
-                const float dk = ex2_approx(-dm) * (__uint_as_float(y[j]) + __uint_as_float(ys[j]));
-                r1v[u] = fmaf(s1, dq, fmaf(-c1, pv, du * kv));
-                r2v[u] = fmaf(s2, dk, fmaf(-c2, kv, du * pv));
-              }
-              o1[e] = pack_bf16x2(r1v[0], r1v[1]);
-              o2[e] = pack_bf16x2(r2v[0], r2v[1]);
-            }
-            *reinterpret_cast<uint4*>(p1s + off) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
-            *reinterpret_cast<uint4*>(p2s + off) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
-          }
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0 && t0 + warp * 32 < p.T) {  // this warp's 32 rows of dp1, dp2, dv
-          const uint32_t so = (uint32_t)warp * (32 * 128);
-          tma_store_4d(&tmDP1, sb + OFF_P1 + so, 0, t0 + warp * 32, h, b);
-          tma_store_4d(&tmDP2, sb + OFF_P2 + so, 0, t0 + warp * 32, h, b);
-          tma_store_4d(&tmDV, sb + OFF_G + so, 0, t0 + warp * 32, h, b);
-          tma_store_commit();
-        }
+        for (int j = 0; j < 16; ++j) pk[j] = 0u;
       }
-      // ---- phase F (thread = channel and half block): dalpha_u = (end + sum_{t >= u} dL_t)
-      // / alpha_u, end = sum_n (2^{L_m} C_0)[c][n] (2^{L_end - L_m} dC)[c][n] + sum_j Km_j Ys_j
-      ew_sync();
-      {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4*>(dst + swz(t, c0 + 8 * q, LT)) =
+            make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      fence_async_smem();
+      tc_fence_before();
+      mbar_arrive(bar(pass == 0 ? B_A : B_DAS));
+    }
+    // ---- every product done, p1 and p2 back in shared memory: token t, the group's channels
+    ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_MM), 0, ab) && mbar_wait(bar(B_RELOAD), 0, ab));
+    uint8_t* const gs = smem + OFF_G;
+    float dq[16], dk[16];
+    if (ok) {
+      tc_fence_after();
+      bool unused_clamp = false;
+      // dq' = 2^{L_t - L_m} X, dk' = 2^{L_m - L_t} Y (Y = dA^T Qm + Ys), the group's shares of
+      // p1 . dq' and p2 . dk', dL = Qm X - Km Y and Km Ys (Qm, Km as the products read them),
+      // dv = dI~ + dY (in dY's place)
+      uint32_t x[16], y[16], ys[16], di[16];
+      tmem_ld16(trow + COL_X + 16 * grp, x);
+      tmem_ld16(trow + COL_Y + 16 * grp, y);
+      tmem_ld16(trow + COL_YS + 16 * grp, ys);
+      tmem_ld16(trow + COL_DI + 16 * grp, di);
+      tmem_ld_wait();
+      float A1 = 0.f, A2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int kc = 2 * grp + k;
+        const uint32_t off = t * 128 + ((kc ^ (t & 7)) << 4);
+        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
+        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
+        const uint4 g4 = *reinterpret_cast<const uint4*>(gs + off);
+        const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc));
+        const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc + 4));
+        const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
+        const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w},
+                       gw[4] = {g4.x, g4.y, g4.z, g4.w};
+        float dl[8], tv[8];
+        uint32_t dvw[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 xa = bf2(aw[e]), yb = bf2(bw[e]), g = bf2(gw[e]);
+          float dvv[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int j = 8 * k + 2 * e + u;  // index within the group's 16 columns
+            const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
+            const float dm = dm_of(Lv[2 * e + u], sum_l[16 * grp + j], t >= 64, unused_clamp);
+            float qm, km;
+            qm_km(pv, kv, s1, s2, dm, qm, km);
+            const float X = __uint_as_float(x[j]), Ysv = __uint_as_float(ys[j]);
+            const float Y = __uint_as_float(y[j]) + Ysv;
+            dq[j] = ex2_approx(dm) * X;
+            dk[j] = ex2_approx(-dm) * Y;
+            A1 = fmaf(pv, dq[j], A1);
+            A2 = fmaf(kv, dk[j], A2);
+            dl[2 * e + u] = qm * X - km * Y;
+            tv[2 * e + u] = km * Ysv;
+            dvv[u] = __uint_as_float(di[j]) + (u ? g.y : g.x);
+          }
+          dvw[e] = pack_bf16x2(dvv[0], dvv[1]);
+        }
+        *reinterpret_cast<uint4*>(gs + off) = make_uint4(dvw[0], dvw[1], dvw[2], dvw[3]);
+        float* gr = gl + t * GS + 8 * kc;
+        *reinterpret_cast<float4*>(gr) = make_float4(dl[0], dl[1], dl[2], dl[3]);
+        *reinterpret_cast<float4*>(gr + 4) = make_float4(dl[4], dl[5], dl[6], dl[7]);
+        float* tr = ts + t * GS + 8 * kc;
+        *reinterpret_cast<float4*>(tr) = make_float4(tv[0], tv[1], tv[2], tv[3]);
+        *reinterpret_cast<float4*>(tr + 4) = make_float4(tv[4], tv[5], tv[6], tv[7]);
+      }
+      a1_s[grp * 128 + t] = A1;
+      a2_s[grp * 128 + t] = A2;
+    }
+    // dalpha's division reads alpha again, rows of 16 threads (in flight during the sums)
+    const long long abase = (long long)b * p.sB + (long long)h * p.sH + 4 * (threadIdx.x & 15);
+    const int arow = threadIdx.x >> 4;  // rows arow + 32 i
+    float4 av[4];
+    ew_sync<NG>();
+    if (ok) {
+      // through S_t and the normalisation of p1, p2 (written in their place)
+      //   dp1 = S/|p1| dq' - S/|p1|^3 (p1 . dq') p1 + du p2, and symmetrically dp2,
+      //   du = (p1 . dq' / |p1| + p2 . dk' / |p2|) S (1 - S) / (tau_S sqrt(d_h))
+      const float A1 = ((a1_s[t] + a1_s[128 + t]) + a1_s[256 + t]) + a1_s[384 + t];
+      const float A2 = ((a2_s[t] + a2_s[128 + t]) + a2_s[256 + t]) + a2_s[384 + t];
+      const float du = (i1 * A1 + i2 * A2) * S * (1.0f - S) * inv_tau_sqrt_d;
+      const float c1 = s1 * i1 * i1 * A1, c2 = s2 * i2 * i2 * A2;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t off = t * 128 + (((2 * grp + k) ^ (t & 7)) << 4);
+        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
+        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
+        const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+        uint32_t o1[4], o2[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 xa = bf2(aw[e]), yb = bf2(bw[e]);
+          float r1v[2], r2v[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int j = 8 * k + 2 * e + u;
+            const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
+            r1v[u] = fmaf(s1, dq[j], fmaf(-c1, pv, du * kv));
+            r2v[u] = fmaf(s2, dk[j], fmaf(-c2, kv, du * pv));
+          }
+          o1[e] = pack_bf16x2(r1v[0], r1v[1]);
+          o2[e] = pack_bf16x2(r2v[0], r2v[1]);
+        }
+        *reinterpret_cast<uint4*>(p1s + off) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+        *reinterpret_cast<uint4*>(p2s + off) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int tok = t0 + arow + 32 * i;
+        av[i] = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (tok < p.T)
+          av[i] = __ldg(reinterpret_cast<const float4*>(p.alpha + abase + (long long)tok * p.sT));
+      }
+      fence_async_smem();
+      // ---- per channel and half block: the sums of dL (group 0) and of Km Ys (group 1); per
+      // channel (group 2) end's state part, sum_n (2^{L_m} C_0)[c][n] (2^{L_end - L_m} dC)[c][n]
+      if (grp < 2) {
+        const float* src = (grp == 0 ? gl : ts) + half * 64 * GS + c;
+        float sum = 0.f;
+#pragma unroll
+        for (int i0 = 0; i0 < 64; i0 += 16) {  // 16 independent loads in flight
+          float v16[16];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) v16[u] = src[(i0 + u) * GS];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) sum += v16[u];
+        }
+        (grp == 0 ? sum_g : sum_t)[t] = sum;
+      } else if (grp == 2 && half == 0) {
         float e0 = 0.f;
         const uint8_t* rc0 = smem + OFF_C0 + c * 128;
         const uint8_t* rdp = smem + OFF_DCP + c * 128;
@@ -528,173 +507,189 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
-            const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&dw[e]));
+            const float2 x = bf2(aw[e]), y = bf2(dw[e]);
             e0 = fmaf(x.x, y.x, fmaf(x.y, y.y, e0));
           }
         }
-        float glh = 0.f, tsh = 0.f;
+        e0_s[c] = e0;
+      }
+    }
+    ew_sync<NG>();
+    if (ok && grp == 0) {
+      // the suffix sums end + sum_{t >= u} dL_t in dL's place; what the block's end and (for the
+      // first half) the later half carry comes first
+      float run = e0_s[c] + sum_t[c] + sum_t[64 + c] + (half == 0 ? sum_g[64 + c] : 0.f);
+      float* col = gl + half * 64 * GS + c;
 #pragma unroll
-        for (int i0 = 0; i0 < 64; i0 += 16) {  // 16 independent loads in flight
-          float g16[16], t16[16];
+      for (int i0 = 48; i0 >= 0; i0 -= 16) {
+        float g16[16];
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            g16[u] = gl[(half * 64 + i0 + u) * GS + c];
-            t16[u] = ts[(half * 64 + i0 + u) * GS + c];
-          }
+        for (int u = 0; u < 16; ++u) g16[u] = col[(i0 + u) * GS];
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            glh += g16[u];
-            tsh += t16[u];
-          }
-        }
-        half_sum[half * 128 + c] = glh;
-        half_sum[half * 128 + 64 + c] = tsh;
-        ew_sync();
-        // what the block's end and (for the first half) the later half carry
-        float run = e0 + half_sum[64 + c] + half_sum[128 + 64 + c] +
-                    (half == 0 ? half_sum[128 + c] : 0.f);
-        const float* arow = p.alpha + (long long)b * p.sB + (long long)h * p.sH + c;
-        float* drow = p.dalpha + (long long)b * p.sB + (long long)h * p.sH + c;
-        unsigned long long small = 0ull;  // tokens of the half with alpha < kSmallAlpha
-        for (int i0 = 48; i0 >= 0; i0 -= 16) {  // 16 tokens: loads first, then the suffix
-          float a16[16], g16[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            const int tok = half * 64 + i0 + u;
-            a16[u] = t0 + tok < p.T ? __ldg(arow + (long long)(t0 + tok) * p.sT) : 1.f;
-            g16[u] = gl[tok * GS + c];
-          }
-#pragma unroll
-          for (int u = 15; u >= 0; --u) {
-            const int tok = half * 64 + i0 + u;
-            run += g16[u];
-            if (t0 + tok < p.T) drow[(long long)(t0 + tok) * p.sT] = run / a16[u];
-            if (a16[u] < kSmallAlpha) small |= 1ull << (i0 + u);
-          }
-        }
-        // A small alpha_u (below 2^-10) leaves the suffix sum above a small remainder of
-        // terms that cancel, whose fp32 rounding the division magnifies.  There dalpha comes
-        // from the state entering u and the adjoint of Diag(alpha_u) C_{u-1}, channel c (row
-        // c), at the midpoint scale:
-        //   P_u = 2^{L_m} C_0 + sum_{j < u} Km_j I~_j,   Q_u = 2^{L_end - L_m} dC + sum_{t >= u} Qm_t dY_t,
-        //   dalpha_u = <P_u, Q_u> / alpha_u,
-        // where every term of P_u (u in the first half) or of Q_u (the second) carries the
-        // factor alpha_u, so nothing large cancels.  A block with such tokens loads dY, p1
-        // and p2 again (their tiles now hold the outputs) over the dL arrays, which every
-        // elementwise warp has read by then; one warp per (u, c), Km and Qm in fp32.
-        const bool warp_small = small_any_warp(small);  // every lane takes part in the vote
-        if (lane == 0 && warp_small) *fix_any = 1;
-        ew_sync();
-        if (*fix_any) {
-          if (threadIdx.x == 0) {
-            fence_async_smem();  // the dL arrays' generic accesses precede the copies
-            mbar_arrive_expect_tx(bar(B_FIX), 3 * T16);
-            tma_load_4d(sb + OFF_FIX_G, &tmG, bar(B_FIX), 0, t0, h, b);
-            tma_load_4d(sb + OFF_FIX_P1, &tmP1, bar(B_FIX), 0, t0, h, b);
-            tma_load_4d(sb + OFF_FIX_P2, &tmP2, bar(B_FIX), 0, t0, h, b);
-          }
-          if (!(ok = __all_sync(0xffffffffu, mbar_wait(bar(B_FIX), 0, ab)))) break;
-          const uint8_t* vt = smem + OFF_V;
-          const uint8_t* gt = smem + OFF_FIX_G;
-          const uint8_t* p1t = smem + OFF_FIX_P1;
-          const uint8_t* p2t = smem + OFF_FIX_P2;
-          const uint8_t* c0t = smem + OFF_C0;
-          const uint8_t* dct = smem + OFF_DCP;
-          const int t_live = min(LT, p.T - t0);
-          bool unused_clamp = false;
-          // lanes: token group g4 (tokens = g4 mod 4) and the 8 columns from nc (16-byte
-          // group lane & 7 of a 128-byte swizzled row)
-          const int g4 = lane >> 3;
-          auto row16 = [&](const uint8_t* tile, int r) {
-            return *reinterpret_cast<const uint4*>(
-                tile + r * 128 + ((((uint32_t)lane & 7) ^ ((uint32_t)r & 7)) << 4));
-          };
-          auto elem = [&](const uint8_t* tile, int r, int col) {
-            return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
-                tile + r * 128 + ((((uint32_t)col >> 3) ^ ((uint32_t)r & 7)) << 4) + (col & 7) * 2));
-          };
-          for (int i = 0; i < 64 && warp_small; ++i) {
-            unsigned fl = __ballot_sync(0xffffffffu, ((small >> i) & 1ull) != 0ull);
-            while (fl) {
-              const int src = __ffs(fl) - 1;
-              fl &= fl - 1;
-              const int cc = (warp & 1) * 32 + src;  // that lane's channel
-              const int u = half * 64 + i;
-              const float lmc = lmid_s[cc];
-              // Km of the tokens before u and Qm of those from u on, channel cc: lane l
-              // holds tokens l + 32 k
-              float kmr[4], qmr[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const int tok = lane + 32 * k;
-                const float dm = dm_of(al_at(tok, cc), lmc, tok >= 64, unused_clamp);
-                const float x2 = tok < u ? elem(p2t, tok, cc) : 0.f;
-                const float x1 = (tok >= u && tok < t_live) ? elem(p1t, tok, cc) : 0.f;
-                kmr[k] = x2 * sk[tok] * ex2_approx(-dm);
-                qmr[k] = x1 * sq[tok] * ex2_approx(dm);
-              }
-              float P[8], Q[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) P[e] = Q[e] = 0.f;
-#pragma unroll 4
-              for (int j0 = 0; j0 < LT; j0 += 4) {  // tokens j0 + g4
-                const int j = j0 + g4, kq = j0 >> 5;
-                const float ksel = kq == 0 ? kmr[0] : kq == 1 ? kmr[1] : kq == 2 ? kmr[2] : kmr[3];
-                const float qsel = kq == 0 ? qmr[0] : kq == 1 ? qmr[1] : kq == 2 ? qmr[2] : qmr[3];
-                const float km = __shfl_sync(0xffffffffu, ksel, (j0 & 31) + g4);
-                const float qm = __shfl_sync(0xffffffffu, qsel, (j0 & 31) + g4);
-                const uint4 v4 = row16(vt, j), d4 = row16(gt, j);
-                const uint32_t vw[4] = {v4.x, v4.y, v4.z, v4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const float2 fv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&vw[e]));
-                  const float2 fd = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&dw[e]));
-                  P[2 * e] = fmaf(km, fv.x, P[2 * e]);
-                  P[2 * e + 1] = fmaf(km, fv.y, P[2 * e + 1]);
-                  Q[2 * e] = fmaf(qm, fd.x, Q[2 * e]);
-                  Q[2 * e + 1] = fmaf(qm, fd.y, Q[2 * e + 1]);
-                }
-              }
-              // the four token groups' sums, the block-boundary rows, and <P_u, Q_u>
-              const uint4 c4 = row16(c0t, cc), e4 = row16(dct, cc);
-              const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w}, ew[4] = {e4.x, e4.y, e4.z, e4.w};
-              float pq = 0.f;
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float2 cf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&cw[e]));
-                const float2 ef = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ew[e]));
-#pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2) {
-                  float pe = P[2 * e + h2], qe = Q[2 * e + h2];
-                  pe += __shfl_xor_sync(0xffffffffu, pe, 8);
-                  pe += __shfl_xor_sync(0xffffffffu, pe, 16);
-                  qe += __shfl_xor_sync(0xffffffffu, qe, 8);
-                  qe += __shfl_xor_sync(0xffffffffu, qe, 16);
-                  pq = fmaf(pe + (h2 ? cf.y : cf.x), qe + (h2 ? ef.y : ef.x), pq);
-                }
-              }
-              pq += __shfl_xor_sync(0xffffffffu, pq, 1);
-              pq += __shfl_xor_sync(0xffffffffu, pq, 2);
-              pq += __shfl_xor_sync(0xffffffffu, pq, 4);
-              if (lane == src)
-                drow[(long long)(t0 + u) * p.sT] = pq / __ldg(arow + (long long)(t0 + u) * p.sT);
-            }
-          }
+        for (int u = 15; u >= 0; --u) {
+          run += g16[u];
+          col[(i0 + u) * GS] = run;
         }
       }
-    } while (false);
+    } else if (ok && grp == 1 && lane == 0) {  // 32 rows of dp1, dp2, dv per warp
+      const int r0 = (warp & 3) * 32;
+      if (t0 + r0 < p.T) {
+        const uint32_t so = (uint32_t)r0 * 128;
+        tma_store_4d(&tmDP1, sb + OFF_P1 + so, 0, t0 + r0, h, b);
+        tma_store_4d(&tmDP2, sb + OFF_P2 + so, 0, t0 + r0, h, b);
+        tma_store_4d(&tmDV, sb + OFF_G + so, 0, t0 + r0, h, b);
+        tma_store_commit();
+      }
+    }
+    ew_sync<NG>();
+    // ---- dalpha_u = (end + sum_{t >= u} dL_t) / alpha_u, rows of 16 threads; the (token,
+    // channel)s with a small alpha are listed for the fix-up
+    uint16_t* const fix_list = reinterpret_cast<uint16_t*>(smem + OFF_FIX_LIST);
+    if (ok) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int tok = arow + 32 * i;
+        const float4 r4 = *reinterpret_cast<const float4*>(gl + tok * GS + 4 * (threadIdx.x & 15));
+        const float a[4] = {av[i].x, av[i].y, av[i].z, av[i].w};
+        if (t0 + tok < p.T) {
+          *reinterpret_cast<float4*>(p.dalpha + abase + (long long)(t0 + tok) * p.sT) =
+              make_float4(r4.x / a[0], r4.y / a[1], r4.z / a[2], r4.w / a[3]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (a[e] < kSmallAlpha)
+              fix_list[atomicAdd(fix_count, 1)] =
+                  (uint16_t)(tok * 64 + 4 * (threadIdx.x & 15) + e);
+        }
+      }
+    }
+    ew_sync<NG>();
+    // A small alpha_u (below 2^-10) leaves the suffix sum above a small remainder of
+    // terms that cancel, whose fp32 rounding the division magnifies.  There dalpha comes
+    // from the state entering u and the adjoint of Diag(alpha_u) C_{u-1}, channel c (row
+    // c), at the midpoint scale:
+    //   P_u = 2^{L_m} C_0 + sum_{j < u} Km_j I~_j,   Q_u = 2^{L_end - L_m} dC + sum_{t >= u} Qm_t dY_t,
+    //   dalpha_u = <P_u, Q_u> / alpha_u,
+    // where every term of P_u (u in the first half) or of Q_u (the second) carries the
+    // factor alpha_u, so nothing large cancels.  A block with such tokens loads dY, p1
+    // and p2 again (their tiles now hold the outputs) over the dL arrays, which every
+    // elementwise warp has read by then; one warp per (u, c), Km and Qm in fp32.
+    const int n_fix = *reinterpret_cast<volatile int*>(fix_count);
+    if (ok && n_fix > 0) {
+      if (threadIdx.x == 0) {
+        fence_async_smem();  // the dL arrays' generic accesses precede the copies
+        mbar_arrive_expect_tx(bar(B_FIX), 3 * T16);
+        tma_load_4d(sb + OFF_FIX_G, &tmG, bar(B_FIX), 0, t0, h, b);
+        tma_load_4d(sb + OFF_FIX_P1, &tmP1, bar(B_FIX), 0, t0, h, b);
+        tma_load_4d(sb + OFF_FIX_P2, &tmP2, bar(B_FIX), 0, t0, h, b);
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_FIX), 0, ab));
+    }
+    if (ok && n_fix > 0) {
+      const uint8_t* vt = smem + OFF_V;
+      const uint8_t* gt = smem + OFF_FIX_G;
+      const uint8_t* p1t = smem + OFF_FIX_P1;
+      const uint8_t* p2t = smem + OFF_FIX_P2;
+      const uint8_t* c0t = smem + OFF_C0;
+      const uint8_t* dct = smem + OFF_DCP;
+      const int t_live = min(LT, p.T - t0);
+      bool unused_clamp = false;
+      // lanes: token group g4 (tokens = g4 mod 4) and the 8 columns of 16-byte group lane & 7
+      // of a 128-byte swizzled row
+      const int g4 = lane >> 3;
+      auto row16 = [&](const uint8_t* tile, int r) {
+        return *reinterpret_cast<const uint4*>(
+            tile + r * 128 + ((((uint32_t)lane & 7) ^ ((uint32_t)r & 7)) << 4));
+      };
+      auto elem = [&](const uint8_t* tile, int r, int col) {
+        return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
+            tile + r * 128 + ((((uint32_t)col >> 3) ^ ((uint32_t)r & 7)) << 4) + (col & 7) * 2));
+      };
+      // S_t / |p_t| of tokens lane + 32 k
+      float sq[4], sk[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int tok = lane + 32 * k;
+        sq[k] = sk[k] = 0.f;
+        if (t0 + tok < p.T) {
+          const float St = 1.0f / (1.0f + __expf(-s_dot[tok] * inv_tau_sqrt_d));
+          sq[k] = St * rsqrtf(s_n1[tok]);
+          sk[k] = St * rsqrtf(s_n2[tok]);
+        }
+      }
+      for (int i = warp; i < n_fix; i += NG * 4) {
+        const int u = fix_list[i] >> 6, cc = fix_list[i] & 63;
+        const float lmc = sum_l[cc];
+        // Km of the tokens before u and Qm of those from u on, channel cc: lane l
+        // holds tokens l + 32 k
+        float kmr[4], qmr[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int tok = lane + 32 * k;
+          const float dm = dm_of(al_at(tok, cc), lmc, tok >= 64, unused_clamp);
+          const float x2 = tok < u ? elem(p2t, tok, cc) : 0.f;
+          const float x1 = (tok >= u && tok < t_live) ? elem(p1t, tok, cc) : 0.f;
+          kmr[k] = x2 * sk[k] * ex2_approx(-dm);
+          qmr[k] = x1 * sq[k] * ex2_approx(dm);
+        }
+        float P[8], Q[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) P[e] = Q[e] = 0.f;
+#pragma unroll 4
+        for (int j0 = 0; j0 < LT; j0 += 4) {  // tokens j0 + g4
+          const int j = j0 + g4, kq = j0 >> 5;
+          const float ksel = kq == 0 ? kmr[0] : kq == 1 ? kmr[1] : kq == 2 ? kmr[2] : kmr[3];
+          const float qsel = kq == 0 ? qmr[0] : kq == 1 ? qmr[1] : kq == 2 ? qmr[2] : qmr[3];
+          const float km = __shfl_sync(0xffffffffu, ksel, (j0 & 31) + g4);
+          const float qm = __shfl_sync(0xffffffffu, qsel, (j0 & 31) + g4);
+          const uint4 v4 = row16(vt, j), d4 = row16(gt, j);
+          const uint32_t vw[4] = {v4.x, v4.y, v4.z, v4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 fv = bf2(vw[e]), fd = bf2(dw[e]);
+            P[2 * e] = fmaf(km, fv.x, P[2 * e]);
+            P[2 * e + 1] = fmaf(km, fv.y, P[2 * e + 1]);
+            Q[2 * e] = fmaf(qm, fd.x, Q[2 * e]);
+            Q[2 * e + 1] = fmaf(qm, fd.y, Q[2 * e + 1]);
+          }
+        }
+        // the four token groups' sums, the block-boundary rows, and <P_u, Q_u>
+        const uint4 c4 = row16(c0t, cc), e4 = row16(dct, cc);
+        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w}, ew[4] = {e4.x, e4.y, e4.z, e4.w};
+        float pq = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 cf = bf2(cw[e]), ef = bf2(ew[e]);
+#pragma unroll
+          for (int h2 = 0; h2 < 2; ++h2) {
+            float pe = P[2 * e + h2], qe = Q[2 * e + h2];
+            pe += __shfl_xor_sync(0xffffffffu, pe, 8);
+            pe += __shfl_xor_sync(0xffffffffu, pe, 16);
+            qe += __shfl_xor_sync(0xffffffffu, qe, 8);
+            qe += __shfl_xor_sync(0xffffffffu, qe, 16);
+            pq = fmaf(pe + (h2 ? cf.y : cf.x), qe + (h2 ? ef.y : ef.x), pq);
+          }
+        }
+        pq += __shfl_xor_sync(0xffffffffu, pq, 1);
+        pq += __shfl_xor_sync(0xffffffffu, pq, 2);
+        pq += __shfl_xor_sync(0xffffffffu, pq, 4);
+        if (lane == 0) {
+          const long long at = (long long)b * p.sB + (long long)h * p.sH +
+                               (long long)(t0 + u) * p.sT + cc;
+          p.dalpha[at] = pq / __ldg(p.alpha + at);
+        }
+      }
+    }
     if (lane == 0) tma_store_wait_read_all();
     if (my_clamp) atomicExch(clamped, 1);
   }
 
-  if (warp == 5) drain_wait(bar(B_MM), 0);  // no product in flight past the teardown
-  if (threadIdx.x == 0 && *fix_any) drain_wait(bar(B_FIX), 0);  // nor the fix-up's copies
+  if (warp == W_MMA) drain_wait(bar(B_MM), 0);  // no product in flight past the teardown
+  if (threadIdx.x == 0 && *fix_count > 0) drain_wait(bar(B_FIX), 0);  // nor the fix-up's copies
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *clamped && p.dev_status && !*abort_flag)
     atomicExch(p.dev_status, (int)RELATION_ERR_UNSUPPORTED);
-  if (warp == 5) {
+  if (warp == W_MMA) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
@@ -711,10 +706,10 @@ bool linear_tc_bwd_supports(const LinearProblem& p) {
 size_t linear_tc_bwd_workspace_bytes(const LinearProblem& p) {
   if (!linear_tc_bwd_supports(p)) return 0;
   const long long heads = (long long)p.B * p.H, nb = (p.T + lintc::LT - 1) / lintc::LT;
-  return lintc::bwd_bytes(heads, nb, 64, nullptr, nullptr, nullptr);
+  return lintc::bwd_bytes(heads, nb, 64, nullptr, nullptr);
 }
 
-// Five launches: the four state passes (states_t), then one CTA per (head, block).
+// Three launches: the two state passes (launch_states), then one CTA per (head, block).
 cudaError_t launch_linear_tc_bwd(const LinearProblem& p, cudaStream_t s) {
   using namespace lintc;
   if (!linear_tc_bwd_supports(p) || !p.workspace) return cudaErrorInvalidValue;
@@ -728,23 +723,22 @@ cudaError_t launch_linear_tc_bwd(const LinearProblem& p, cudaStream_t s) {
     note_failure("linear chunked backward: shared memory attribute");
     return e;
   }
-  if ((e = states_t<64>(p, p.dy, p.workspace, s)) != cudaSuccess) return e;
+  if ((e = launch_states(p, p.dy, p.workspace, s)) != cudaSuccess) return e;
   LinCp cp{};
-  __nv_bfloat16* dcb = nullptr;
-  bwd_bytes(heads, nb, 64, &cp, &dcb, p.workspace);
+  bwd_bytes(heads, nb, 64, &cp, p.workspace);
   Problem q{};  // the bf16 tensor-map helper's view of the shapes
   q.B = p.B; q.T = p.T; q.H = p.H; q.d = p.d;
   q.sB = p.sB; q.sT = p.sT; q.sH = p.sH;
   CUtensorMap m1, m2, mv, mg, ma, mc0, mdc, o1, o2, ov;
   if (!tc::make_tmap_bf16(&m1, p.p1, q, LT) || !tc::make_tmap_bf16(&m2, p.p2, q, LT) ||
       !tc::make_tmap_bf16(&mv, p.v, q, LT) || !tc::make_tmap_bf16(&mg, p.dy, q, LT) ||
-      !make_tmap_alpha(&ma, p, true) || !make_tmap_c0(&mc0, cp.c0, heads * (nb + 1) * 64, 64) ||
-      !make_tmap_c0(&mdc, dcb, heads * nb * 64, 64) || !tc::make_tmap_bf16(&o1, p.dp1, q, 32) ||
+      !make_tmap_alpha(&ma, p, true) || !make_tmap_c0(&mc0, cp.dC, heads * nb * 64, 64) ||
+      !make_tmap_c0(&mdc, cp.dQ, heads * nb * 64, 64) || !tc::make_tmap_bf16(&o1, p.dp1, q, 32) ||
       !tc::make_tmap_bf16(&o2, p.dp2, q, 32) || !tc::make_tmap_bf16(&ov, p.dv, q, 32)) {
     note_failure("linear chunked backward: TMA descriptors");
     return cudaErrorInvalidValue;
   }
-  bwd::lin_tc_bwd_kernel<<<(unsigned)grid, kThreads, bwd::SMEM, s>>>(m1, m2, mv, mg, ma, mc0, mdc,
+  bwd::lin_tc_bwd_kernel<<<(unsigned)grid, bwd::kThreads, bwd::SMEM, s>>>(m1, m2, mv, mg, ma, mc0, mdc,
                                                                     o1, o2, ov, p, nb);
   if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked backward: launch");
   return e;
