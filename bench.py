@@ -608,7 +608,7 @@ def linear_measure(binding, dev, peaks, steps=20, warmup=3):
                                  "unit": "TFLOP/s", "frac": tc_ach / peaks["bf16_tflops"],
                                  "algorithmic_flops_per_launch": tc_fl},
             "roofline_chunked_bwd": {"bound": "tensor",
-                                     "kernel": "chunked backward (five launches)",
+                                     "kernel": "chunked backward (three launches)",
                                      "achieved": tcb_ach, "peak": peaks["bf16_tflops"],
                                      "unit": "TFLOP/s", "frac": tcb_ach / peaks["bf16_tflops"],
                                      "flops_per_call": tcb_fl},

@@ -27,8 +27,9 @@
 // the SM holds: four groups on the sequential walk (one CTA per SM, its next block's loads
 // in flight), two on the one-block modes at d_h = 64, which leave room for a second CTA per SM
 // whose phases fill this one's waits.  With one group (one CTA per SM) the sequential walk took
-// 126 us at B 8, H 12, T 2048, d 64 and now takes 93; at B 1, H 12, T 32768 DELTA took 140 us
-// and OUT 177, now 79 and 95, the scan (16 blocks in flight instead of 8) 27, now 16.
+// 126 us at B 8, H 12, T 2048, d 64; four groups 93; with the logarithms on every warp, the next
+// block's sums taken while the output product runs and the stores on the TMA warp 82.  At B 1,
+// H 12, T 32768 DELTA, the scan and OUT took 140, 27 and 177 us, now 78, 16 and 95.
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps
 // meeting the warpgroups' barriers and skips the work between them.
 #include <cudaTypedefs.h>
@@ -66,17 +67,20 @@ struct Cfg {
   static constexpr int OFF_KL = DELTA ? OFF_P2 : STAGES * STAGE;
   static constexpr int OFF_QS = SEQ ? OFF_KL + PT : STAGES * STAGE;
   static constexpr int OFF_C0 = SEQ ? OFF_QS + PT : (DELTA ? STAGE : OFF_QS + PT);
-  // the per-token / per-channel scalars: before the C0 copy is written in its place (SEQ)
-  static constexpr int OFF_SC = SEQ ? OFF_C0 : (DELTA ? OFF_C0 : OFF_C0 + C0T);
-  static constexpr int SCB = 7 * LT * 4;
-  static constexpr int OFF_BAR = SEQ ? OFF_C0 + C0T : OFF_SC + SCB;
+  // the per-token / per-channel scalars; AHEAD: two sets, the next block's sums are taken while
+  // the current block's output product runs.  d_h = 128 SEQ has no room: they stand in the C0
+  // tile before the copy is written there
+  static constexpr bool AHEAD = STAGES == 2, IN_C0 = SEQ && D == 128;
+  static constexpr int OFF_SC = IN_C0 || DELTA ? OFF_C0 : OFF_C0 + C0T;
+  static constexpr int SCB = 5 * LT * 4;
+  static constexpr int OFF_BAR = IN_C0 ? OFF_C0 + C0T : OFF_SC + (AHEAD ? 2 : 1) * SCB;
   static constexpr int SMEM = OFF_BAR + 128 + 1024;
   static constexpr uint32_t LOAD_BYTES =
       2 * PT + VT + AT + (MODE == MODE_OUT ? C0T : 0) + (MODE == MODE_BOTH ? VT : 0);
   // TMEM columns: S 128 | E 64 | P 64 (S masked, bf16) | C 64; DELTA: C 64 (BOTH: 128) alone
   static constexpr int COL_S = 0, COL_E = 128, COL_P = 192, COL_C = DELTA ? 0 : 256;
   static constexpr int TMEM = SEQ ? 512 : (DELTA ? 128 : 256);
-  static_assert(SCB <= C0T || !SEQ, "scalars in the C0 tile");
+  static_assert(SCB <= C0T, "scalars in the C0 tile");
   static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory");
 };
 
@@ -108,12 +112,6 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_BAR + 96);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 104);
   int* clamped = reinterpret_cast<int*>(smem + C::OFF_BAR + 108);
-  float* s_dot = reinterpret_cast<float*>(smem + C::OFF_SC);  // [128] p1_t . p2_t
-  float* s_n1 = s_dot + LT;                                   // [128] |p1_t|^2
-  float* s_n2 = s_n1 + LT;                                    // [128] |p2_t|^2
-  // per channel L_m and, d_h = 64: the sum over the second half; d_h = 128: L_end
-  float* l_a = s_n2 + LT;
-  float* l_b = l_a + LT;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NSPLIT = D / NC;
@@ -127,11 +125,9 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   const int blk_first = cta_blk, blk_end = SEQ ? nb : cta_blk + 1;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NBAR; ++i)  // arrivals of the elementwise threads, the four storing
-                                    // lanes, or one
-      mbar_init(bar(i), (i == B_OPS || i == B_C0 || i == B_A)
-                            ? C::EW
-                            : (i == B_EPI || i == B_EPI + 1) ? 4 : 1);
+    for (int i = 0; i < NBAR; ++i)  // arrivals of the elementwise threads, or one
+      mbar_init(bar(i), (i == B_OPS || i == B_C0 || i == B_A || i == B_EPI || i == B_EPI + 1)
+                            ? C::EW : 1);
     *abort_flag = 0;
     *clamped = 0;
     fence_mbar_init();
@@ -146,13 +142,27 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   if (warp == C::W_TMA) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
+      // Y of block it (staged in its p1 tile) by TMA, once every elementwise thread has
+      // written its part and read the stage's I~
+      auto store_y = [&](int it) -> bool {
+        const int st = it % C::STAGES;
+        if (!mbar_wait(bar(B_EPI + st), (it / C::STAGES) & 1, ab)) return false;
+        for (int q = 0; q < LT && (blk_first + it) * LT + q < p.T; q += 32)
+          tma_store_4d(&tmY, sb + st * C::STAGE + C::OFF_P1 + q * 128, split * NC,
+                       (blk_first + it) * LT + q, h, b);
+        tma_store_commit();
+        tma_store_wait_read_all();  // before the stage is loaded again (or the CTA exits)
+        return true;
+      };
+      const int n_it = blk_end - blk_first;
       int issued = 0;
+      bool ok = true;
       for (int blk = blk_first; blk < blk_end; ++blk) {
         const int it = blk - blk_first;
         const int st = it % C::STAGES, use = it / C::STAGES;
-        // the stage's previous block: its MMAs and its output staging are done
-        if (use > 0 && (!mbar_wait(bar(B_FREE + st), (use - 1) & 1, ab) ||
-                        !mbar_wait(bar(B_EPI + st), (use - 1) & 1, ab)))
+        // the stage's previous block: its MMAs are done and its output is stored
+        if (use > 0 && (!(ok = store_y(it - C::STAGES)) ||
+                        !(ok = mbar_wait(bar(B_FREE + st), (use - 1) & 1, ab))))
           break;
         const int t0 = blk * LT;
         const uint32_t sg = sb + st * C::STAGE;
@@ -170,6 +180,8 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
           tma_load_2d(sb + C::OFF_C0, &tmC0, lb, 0, (bhs * nb + blk) * D);
         issued = it + 1;
       }
+      if (!DELTA)
+        for (int it = max(0, n_it - C::STAGES); ok && it < n_it; ++it) ok = store_y(it);
       if (ab.raised())  // copies in flight land before the CTA releases its shared memory
         for (int it = issued - C::STAGES > 0 ? issued - C::STAGES : 0; it < issued; ++it)
           drain_wait(bar(B_LOAD + it % C::STAGES), (it / C::STAGES) & 1);
@@ -243,6 +255,63 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     const int half = D == 64 ? (t >> 6) : 0;
     constexpr int TPT = D == 64 ? 64 : 128;  // tokens per thread of the retention sums
     bool ok = true, my_clamp = false;
+    // A block's scalars: p1_t . p2_t, |p1_t|^2, |p2_t|^2 per token, and per channel L_m and
+    // (d_h = 64) the sum over the second half or (128) L_end
+    auto scalars = [&](int it) {
+      return reinterpret_cast<float*>(smem + C::OFF_SC + (C::AHEAD ? (it & 1) * C::SCB : 0));
+    };
+    // The sums of block it, once it is loaded: log2 alpha in place of alpha (0 past T; every
+    // group), then Ask Self's sums (the groups but the last) beside the channels' inclusive
+    // running sums L_t in place of log2 alpha (the last group; d_h = 64: the second half's
+    // relative to its start).  The running sums are one chain per channel: with the logarithms
+    // on the same four warps they took 3900 cycles of a block's 10600.  Visible after the
+    // warpgroups' next barrier.
+    auto sums = [&](int it) {
+      const int t0 = (blk_first + it) * LT, st = it % C::STAGES;
+      uint8_t* const sg = smem + st * C::STAGE;
+      float* const al = reinterpret_cast<float*>(sg + C::OFF_A);
+      float* const s_dot = scalars(it);
+      float* const l_a = s_dot + 3 * LT;
+      float* const l_b = l_a + LT;
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD + st), (it / C::STAGES) & 1, ab));
+      if (ok) {
+#pragma unroll
+        for (int i0 = 0; i0 < LT * D / 4; i0 += C::EW) {
+          const int i = i0 + threadIdx.x;  // 16-byte group of the tile, of token (i / 8) % 128
+          const bool live = t0 + ((i >> 3) & 127) < p.T;
+          float4 v = reinterpret_cast<float4*>(al)[i];
+          v.x = live ? __log2f(v.x) : 0.f;
+          v.y = live ? __log2f(v.y) : 0.f;
+          v.z = live ? __log2f(v.z) : 0.f;
+          v.w = live ? __log2f(v.w) : 0.f;
+          reinterpret_cast<float4*>(al)[i] = v;
+        }
+      }
+      ew_sync<NG>();
+      if (!ok) return;
+      if (grp < NG - 1) {
+        ask_self_sums<D, NG == 2 ? 7 : 0>(sg + C::OFF_P1, sg + C::OFF_P2, t,
+                                          NG == 2 ? 7 : 1 << grp, s_dot, s_dot + LT, s_dot + 2 * LT);
+      } else {
+        float lsum = 0.f;
+        for (int i0 = 0; i0 < TPT; i0 += 16) {
+          float la[16];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) la[u] = al[al_swz(half * 64 + i0 + u, c)];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            lsum += la[u];
+            al[al_swz(half * 64 + i0 + u, c)] = lsum;
+          }
+          if (D == 128 && i0 == 48) l_a[c] = lsum;  // L at the 64th token
+        }
+        if (D == 64)
+          (half == 0 ? l_a : l_b)[c] = lsum;
+        else
+          l_b[c] = lsum;
+      }
+    };
+    if (C::AHEAD) sums(0);
     for (int blk = blk_first; blk < blk_end; ++blk) {
       const int it = blk - blk_first;
       const uint32_t ph = it & 1;
@@ -252,38 +321,15 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
       uint8_t* const p1s = sg + C::OFF_P1;
       uint8_t* const p2s = sg + C::OFF_P2;
       float* const al = reinterpret_cast<float*>(sg + C::OFF_A);
+      const float* const s_dot = scalars(it);
+      const float* const s_n1 = s_dot + LT;
+      const float* const s_n2 = s_n1 + LT;
+      const float* const l_a = s_n2 + LT;
+      const float* const l_b = l_a + LT;
       auto al_at = [&](int tok, int ch) -> float& {  // [D / 32][128][32] fp32, 128-byte swizzle
         return al[al_swz(tok, ch)];
       };
-      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD + st), (it / C::STAGES) & 1, ab));
-      if (ok) {
-        // ---- Ask Self's sums of token t (the groups but the last) beside the channels'
-        // inclusive running sums L_t of log2 alpha in place of alpha (the last group; 0
-        // past T; d_h = 64: the second half's relative to its start)
-        if (grp < NG - 1) {
-          ask_self_sums<D, NG == 2 ? 7 : 0>(p1s, p2s, t, NG == 2 ? 7 : 1 << grp, s_dot, s_n1, s_n2);
-        } else {
-          float lsum = 0.f;
-          for (int i0 = 0; i0 < TPT; i0 += 16) {
-            float la[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-              const int tok = half * 64 + i0 + u;
-              la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-              lsum += la[u];
-              al_at(half * 64 + i0 + u, c) = lsum;
-            }
-            if (D == 128 && i0 == 48) l_a[c] = lsum;  // L at the 64th token
-          }
-          if (D == 64)
-            (half == 0 ? l_a : l_b)[c] = lsum;
-          else
-            l_b[c] = lsum;
-        }
-      }
+      if (!C::AHEAD) sums(it);
       ew_sync<NG>();
       float l_end = 0.f;  // channel t's L at the block's last token (t < D)
       if (ok) {
@@ -370,7 +416,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         fence_async_smem();
         mbar_arrive(bar(B_OPS));
       }
-      if (SEQ) ew_sync<NG>();  // the scalars have been read: C0 takes their place
+      if (C::IN_C0) ew_sync<NG>();  // the scalars have been read: C0 takes their place
       if (DELTA) {
         // the block's state (and adjoint) contribution and decay, to the workspace
         ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), 0, ab));
@@ -456,7 +502,8 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         tc_fence_before();
         mbar_arrive(bar(B_A));
       }
-      // ---- Y = I~ + E, staged in p1's tile and stored by TMA (32 rows per store)
+      if (C::AHEAD && blk + 1 < blk_end) sums(it + 1);
+      // ---- Y = I~ + E, staged in p1's tile (stored by the TMA warp)
       ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_E), ph, ab));
       if (ok) {
         tc_fence_after();
@@ -486,18 +533,8 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         }
         fence_async_smem();
         tc_fence_before();
-      }
-      ew_sync<NG>();
-      if (ok && grp == 0 && lane == 0) {
-        if (t0 + warp * 32 < p.T) {
-          tma_store_4d(&tmY, smem_u32(sg + C::OFF_P1 + warp * (32 * 128)), split * NC,
-                       t0 + warp * 32, h, b);
-          tma_store_commit();
-          tma_store_wait_read_all();  // the staging (a later block's p1) is reloaded next
-        }
         mbar_arrive(bar(B_EPI + st));
       }
-      __syncwarp();
     }
     if (my_clamp) atomicExch(clamped, 1);
   }

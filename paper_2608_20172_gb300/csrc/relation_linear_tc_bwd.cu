@@ -27,9 +27,11 @@
 // elementwise work (thread = token; the groups split the channels or columns; the sums whose
 // rounding the cancellation above rests on stay one chain each, in the order of the block's
 // tokens or channels, on different groups), then a warp the TMA loads and one (warp-uniform,
-// elect.sync) the MMAs.  One CTA per SM (212 KB), so latency bounds it: a block's phases and
-// barriers around small products, nothing else resident.  B 8, H 12, T 2048: 361 us with one
-// elementwise warpgroup, 197 with four; the state passes 161 us as four launches, 66 as two.
+// elect.sync) the MMAs.  One CTA per SM (220 KB), so latency bounds it: a block's phases and
+// barriers around small products, nothing else resident.  B 8, H 12, T 2048, the whole backward:
+// 535 us with one elementwise warpgroup and four state launches, 270 with four groups and two,
+// 254 with p1 and p2 kept in registers past Qm and Km (they were loaded again) and the small
+// retentions' fix-up beside the products.
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps meeting the
 // warpgroups' barriers and skips the work between them.
 #include "relation_linear_tc.cuh"
@@ -45,8 +47,8 @@ constexpr int kTmemCols = 512;  // scratch S / dA 128 | X 64 | Y 64 | dI~ 64 | Y
 constexpr int COL_SC = 0, COL_X = 128, COL_Y = 192, COL_DI = 256, COL_YS = 320;
 // shared memory (bytes): 128-token tiles of 64 bf16 columns are 16 KB
 constexpr int T16 = LT * 64 * 2;
-constexpr int OFF_P1 = 0;                 // p1, then Qm in place, then p1 again, then dp1
-constexpr int OFF_P2 = OFF_P1 + T16;      // p2, then Km in place, then p2 again, then dp2
+constexpr int OFF_P1 = 0;                 // p1, then Qm in place, then dp1
+constexpr int OFF_P2 = OFF_P1 + T16;      // p2, then Km in place, then dp2
 constexpr int OFF_V = OFF_P2 + T16;       // I~
 constexpr int OFF_G = OFF_V + T16;        // dY, then dI~ (the dv output)
 constexpr int OFF_AL = OFF_G + T16;       // alpha, then its running log2 sums [2][128][32] fp32
@@ -58,7 +60,9 @@ constexpr int OFF_C0 = OFF_DAS + 2 * T16; // C_0, then 2^{L_m} C_0 in place
 constexpr int OFF_DC = OFF_C0 + C64;      // dC (the state's adjoint leaving the block)
 constexpr int OFF_DCP = OFF_DC + C64;     // 2^{L_end - L_m} dC
 constexpr int OFF_SC = OFF_DCP + C64;     // scalars, 15 x 128 fp32
-constexpr int OFF_BAR = OFF_SC + 15 * LT * 4;
+constexpr int kFix = 16;
+constexpr int OFF_COEF = OFF_SC + 15 * LT * 4;  // [kFix][128] fp32: Km / Qm of the fix-ups
+constexpr int OFF_BAR = OFF_COEF + kFix * LT * 4;
 constexpr int SMEM = OFF_BAR + 128 + 1024;
 static_assert(SMEM <= 232448, "shared memory");
 constexpr uint32_t LOAD_BYTES = 4 * T16 + LT * 64 * 4 + 2 * C64;
@@ -66,9 +70,6 @@ constexpr int GS = 68;  // row stride (floats) of the epilogue's [t][64] arrays:
 constexpr int OFF_GL = OFF_KL, OFF_TS = OFF_GL + LT * GS * 4;
 static_assert(OFF_TS + LT * GS * 4 <= OFF_C0, "epilogue arrays overlap the state tiles");
 
-// Qm and Km of one channel as the products read them (bf16), from p1, p2 (bf16 values),
-// S / |p|, and the channel's log2 ratio to the midpoint; the epilogue recomputes them
-// through this same function, bit for bit.
 __device__ __forceinline__ float dm_of(float lv, float lm, bool later, bool& clamped) {
   // log2 of a_t / a_m for one channel from its stored running sum (relative to the block's
   // start, or in the later half to the midpoint) and L_m, clamped to +-kClampLog2
@@ -79,23 +80,79 @@ __device__ __forceinline__ float dm_of(float lv, float lm, bool later, bool& cla
   }
   return dm;
 }
-__device__ __forceinline__ void qm_km(float x, float y, float s1, float s2, float dm, float& qm,
-                                      float& km) {
-  qm = __bfloat162float(__float2bfloat16_rn(x * s1 * ex2_approx(dm)));
-  km = __bfloat162float(__float2bfloat16_rn(y * s2 * ex2_approx(-dm)));
-}
-
-// Retention below this takes dalpha from the state and its adjoint at the token (phase F).
+// Retention below this takes dalpha from the state and its adjoint at the token (fix_up).
 constexpr float kSmallAlpha = 1.0f / 1024.0f;
 
-// The small-retention fix-up's tiles (dY, p1, p2 loaded again), over the epilogue's dL and
-// Km Ys arrays once the suffix sums are out, and after them the list of its (token, channel)s
+// A block with more than kFix (token, channel)s of small retention fixes them up at the end,
+// from dY, p1 and p2 loaded again over the epilogue's dL and Km Ys arrays once the suffix sums
+// are out, and after them the list of the (token, channel)s.
 constexpr int OFF_FIX_G = OFF_KL, OFF_FIX_P1 = OFF_KL + T16, OFF_FIX_P2 = OFF_KL + 2 * T16;
 constexpr int OFF_FIX_LIST = OFF_FIX_P2 + T16;  // up to 128 x 64 16-bit entries
 static_assert(OFF_FIX_LIST + LT * 64 * 2 <= OFF_C0 && OFF_FIX_LIST >= OFF_TS &&
               OFF_KL % 1024 == 0, "fix-up tiles");
 
-enum : int { B_LOAD = 0, B_OPS, B_S, B_A, B_DA, B_DAS, B_MM, B_RELOAD, B_FIX, NBAR };
+enum : int { B_LOAD = 0, B_OPS, B_S, B_A, B_DA, B_DAS, B_MM, B_FIX, NBAR };
+
+__device__ __forceinline__ float2 bf2(uint32_t w) {
+  return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w));
+}
+
+// dalpha of one (token u, channel c) with small retention, by one warp (the value is in lane 0).
+// A small alpha_u (below 2^-10) leaves the suffix sum above a small remainder of terms that
+// cancel, whose fp32 rounding the division magnifies.  There dalpha comes from the state
+// entering u and the adjoint of Diag(alpha_u) C_{u-1}, channel c (row c), at the midpoint scale:
+//   P_u = 2^{L_m} C_0 + sum_{j < u} Km_j I~_j,   Q_u = 2^{L_end - L_m} dC + sum_{t >= u} Qm_t dY_t,
+//   dalpha_u = <P_u, Q_u> / alpha_u,
+// where every term of P_u (u in the first half) or of Q_u (the second) carries the factor
+// alpha_u, so nothing large cancels.  coef: Km of the tokens before u and Qm of those from u
+// on, channel c, in fp32 (0 past T).  Tiles: 128-byte-swizzled rows of 64 bf16.
+__device__ __forceinline__ float fix_up(const float* coef, const uint8_t* v, const uint8_t* dy,
+                                        const uint8_t* c0, const uint8_t* dcp, int u, int c,
+                                        int lane) {
+  const int g4 = lane >> 3;  // tokens = g4 mod 4; the columns of 16-byte group lane & 7
+  auto row16 = [&](const uint8_t* tile, int r) {
+    return *reinterpret_cast<const uint4*>(
+        tile + r * 128 + ((((uint32_t)lane & 7) ^ ((uint32_t)r & 7)) << 4));
+  };
+  auto add = [&](float (&acc)[8], float f, const uint4 x) {
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 y = bf2(w[e]);
+      acc[2 * e] = fmaf(f, y.x, acc[2 * e]);
+      acc[2 * e + 1] = fmaf(f, y.y, acc[2 * e + 1]);
+    }
+  };
+  float P[8], Q[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) P[e] = Q[e] = 0.f;
+#pragma unroll 4
+  for (int j = g4; j < u; j += 4) add(P, coef[j], row16(v, j));
+#pragma unroll 4
+  for (int j = (u & ~3) + g4; j < LT; j += 4) add(Q, j >= u ? coef[j] : 0.f, row16(dy, j));
+  // the four token groups' sums, the block-boundary rows, and <P_u, Q_u>
+  __syncwarp();
+  const uint4 c4 = row16(c0, c), e4 = row16(dcp, c);
+  const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w}, ew[4] = {e4.x, e4.y, e4.z, e4.w};
+  float pq = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float2 cf = bf2(cw[e]), ef = bf2(ew[e]);
+#pragma unroll
+    for (int h2 = 0; h2 < 2; ++h2) {
+      float pe = P[2 * e + h2], qe = Q[2 * e + h2];
+      pe += __shfl_xor_sync(0xffffffffu, pe, 8);
+      pe += __shfl_xor_sync(0xffffffffu, pe, 16);
+      qe += __shfl_xor_sync(0xffffffffu, qe, 8);
+      qe += __shfl_xor_sync(0xffffffffu, qe, 16);
+      pq = fmaf(pe + (h2 ? cf.y : cf.x), qe + (h2 ? ef.y : ef.x), pq);
+    }
+  }
+  pq += __shfl_xor_sync(0xffffffffu, pq, 1);
+  pq += __shfl_xor_sync(0xffffffffu, pq, 2);
+  pq += __shfl_xor_sync(0xffffffffu, pq, 4);
+  return pq;
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
     lin_tc_bwd_kernel(const __grid_constant__ CUtensorMap tmP1,
@@ -116,7 +173,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_BAR + 96);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_BAR + 104);
   int* clamped = reinterpret_cast<int*>(smem + OFF_BAR + 108);
-  int* fix_count = reinterpret_cast<int*>(smem + OFF_BAR + 112);
+  int* fix_count = reinterpret_cast<int*>(smem + OFF_BAR + 112);  // small retentions found;
+  int* fix_late = reinterpret_cast<int*>(smem + OFF_BAR + 116);   // entries of the late list
   float* sc = reinterpret_cast<float*>(smem + OFF_SC);
   float* s_dot = sc;             // p1_t . p2_t
   float* s_n1 = sc + LT;         // |p1_t|^2
@@ -127,6 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* a1_s = sc + 6 * LT;     // [4][128] the groups' shares of p1_t . dq'_t
   float* a2_s = sc + 10 * LT;    // [4][128] and of p2_t . dk'_t
   float* e0_s = sc + 14 * LT;    // [64] the end term's state part
+  uint16_t* fix_early = reinterpret_cast<uint16_t*>(e0_s + 64);  // [kFix] (token, channel)s
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blk = (int)(blockIdx.x % nb);
@@ -139,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(bar(i), (i == B_OPS || i == B_A || i == B_DAS) ? EW : 1);
     *abort_flag = 0;
     *clamped = 0;
-    *fix_count = 0;
+    *fix_count = *fix_late = 0;
     fence_mbar_init();
   }
   if (warp == W_MMA) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
@@ -162,15 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tma_load_4d(sb + OFF_AL + k * LT * 128, &tmA, lb, k * 32, t0, h, b);
       tma_load_2d(sb + OFF_C0, &tmC0, lb, 0, (bh * nb + blk) * D);
       tma_load_2d(sb + OFF_DC, &tmDC, lb, 0, (bh * nb + blk) * D);
-      // p1 and p2 again (Qm and Km overwrote them) once the MMAs reading those are done
-      bool ok = mbar_wait(bar(B_MM), 0, ab);
-      if (ok) {
-        mbar_arrive_expect_tx(bar(B_RELOAD), 2 * T16);
-        tma_load_4d(sb + OFF_P1, &tmP1, bar(B_RELOAD), 0, t0, h, b);
-        tma_load_4d(sb + OFF_P2, &tmP2, bar(B_RELOAD), 0, t0, h, b);
-      }
       drain_wait(lb, 0);
-      if (ok && ab.raised()) drain_wait(bar(B_RELOAD), 0);
     }
   } else if (warp == W_MMA) {
     // ------------------------------------------------------------------ MMA issuer
@@ -245,12 +296,34 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     float* const gl = reinterpret_cast<float*>(smem + OFF_GL);  // dL [t][GS]
     float* const ts = reinterpret_cast<float*>(smem + OFF_TS);  // Km Ys [t][GS]
-    auto bf2 = [](uint32_t w) { return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w)); };
     bool my_clamp = false;
     bool ok = __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD), 0, ab));
-    // ---- the sums of S_t, |p1_t|, |p2_t| (groups 0, 1, 2) beside the running sums of log2
-    // alpha in place of alpha (group 3: channel and half block, the second half's relative to
-    // its start; 16 tokens ahead)
+    // ---- log2 alpha in place of alpha (0 past T), and the (token, channel)s with a small alpha
+    if (ok) {
+#pragma unroll
+      for (int i0 = 0; i0 < LT * D / 4; i0 += EW) {
+        const int i = i0 + threadIdx.x;  // 16-byte group of the tile
+        const int tok = (i >> 3) & 127;
+        const bool live = t0 + tok < p.T;
+        const float4 v = reinterpret_cast<const float4*>(al)[i];
+        float a[4] = {v.x, v.y, v.z, v.w};
+        if (live && fminf(fminf(a[0], a[1]), fminf(a[2], a[3])) < kSmallAlpha) {
+          const int ch = (i >> 10) * 32 + (((i & 7) ^ (tok & 7)) << 2);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (a[e] < kSmallAlpha) {
+              const int n = atomicAdd(fix_count, 1);
+              if (n < kFix) fix_early[n] = (uint16_t)(tok * 64 + ch + e);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e] = live ? __log2f(a[e]) : 0.f;
+        reinterpret_cast<float4*>(al)[i] = make_float4(a[0], a[1], a[2], a[3]);
+      }
+    }
+    ew_sync<NG>();
+    // ---- the sums of S_t, |p1_t|, |p2_t| (groups 0, 1, 2) beside the running sums L_t in place
+    // of log2 alpha (group 3: channel and half block, the second half's relative to its start)
     if (ok) {
       if (grp < 3) {
         ask_self_sums<D, 0>(p1s, p2s, t, 1 << grp, s_dot, s_n1, s_n2);
@@ -259,10 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i0 = 0; i0 < 64; i0 += 16) {
           float la[16];
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            const int tok = half * 64 + i0 + u;
-            la[u] = (t0 + tok < p.T) ? __log2f(al_at(tok, c)) : 0.f;
-          }
+          for (int u = 0; u < 16; ++u) la[u] = al_at(half * 64 + i0 + u, c);
 #pragma unroll
           for (int u = 0; u < 16; ++u) {
             lsum += la[u];
@@ -273,7 +343,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     ew_sync<NG>();
+    const int n_small = *reinterpret_cast<volatile int*>(fix_count);
+    const int n_early = n_small <= kFix ? n_small : 0;
+    float* const coef = reinterpret_cast<float*>(smem + OFF_COEF);
     float S = 0.f, i1 = 0.f, i2 = 0.f, s1 = 0.f, s2 = 0.f;  // token t (zero past T)
+    uint4 ra[2], rb[2];  // p1, p2 of token t, the group's 16 channels: Qm, Km take their place
     if (ok) {
       if (t0 + t < p.T) {
         S = 1.0f / (1.0f + __expf(-s_dot[t] * inv_tau_sqrt_d));
@@ -303,34 +377,52 @@ __global__ void __launch_bounds__(kThreads, 1)
         *reinterpret_cast<uint4*>(smem + OFF_DCP + r * 128 + 16 * k) =
             make_uint4(od[0], od[1], od[2], od[3]);
       }
+      // the early fix-ups' coefficients: Km before the token, Qm from it on (each thread reads
+      // the channels that it alone overwrites below)
+      for (int f = 0; f < n_early; ++f) {
+        const int u = fix_early[f] >> 6, ch = fix_early[f] & 63;
+        if ((ch >> 4) != grp) continue;
+        const float dm = dm_of(al_at(t, ch), sum_l[ch], t >= 64, my_clamp);
+        const uint8_t* tile = t < u ? p2s : p1s;
+        const float x = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
+            tile + t * 128 + (((ch >> 3) ^ (t & 7)) << 4) + (ch & 7) * 2));
+        coef[f * LT + t] = t < u ? x * s2 * ex2_approx(-dm) : x * s1 * ex2_approx(dm);
+      }
       // ---- Qm, Km in place of p1, p2, and KL: token t, the group's 16 channels
 #pragma unroll
-      for (int k = 2 * grp, k1 = 0; k1 < 2; ++k, ++k1) {
+      for (int k1 = 0; k1 < 2; ++k1) {
+        const int k = 2 * grp + k1;
         const uint32_t off = t * 128 + ((k ^ (t & 7)) << 4);
-        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
-        const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k));
-        const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k + 4));
-        const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
-        const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
+        ra[k1] = *reinterpret_cast<const uint4*>(p1s + off);
+        rb[k1] = *reinterpret_cast<const uint4*>(p2s + off);
+        const uint32_t aw[4] = {ra[k1].x, ra[k1].y, ra[k1].z, ra[k1].w};
+        const uint32_t bw[4] = {rb[k1].x, rb[k1].y, rb[k1].z, rb[k1].w};
         uint32_t qm[4], km[4], kl[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 x = bf2(aw[e]), y = bf2(bw[e]);
-          float r[2][3];
+        for (int q = 0; q < 2; ++q) {  // four channels
+          const float4 L4 = *reinterpret_cast<const float4*>(&al_at(t, 8 * k + 4 * q));
+          const float4 M4 = *reinterpret_cast<const float4*>(sum_l + 8 * k + 4 * q);
+          const float4 E4 = *reinterpret_cast<const float4*>(sum_l + 64 + 8 * k + 4 * q);
+          const float Lv[4] = {L4.x, L4.y, L4.z, L4.w}, Mv[4] = {M4.x, M4.y, M4.z, M4.w};
+          const float Ev[4] = {E4.x, E4.y, E4.z, E4.w};
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int ch = 8 * k + 2 * e + u;
-            const float Lm = sum_l[ch];
-            const float L = Lv[2 * e + u] + (t >= 64 ? Lm : 0.f);
-            const float dm = dm_of(Lv[2 * e + u], Lm, t >= 64, my_clamp);
-            const float xv = u ? x.y : x.x, yv = u ? y.y : y.x;
-            qm_km(xv, yv, s1, s2, dm, r[u][0], r[u][1]);
-            r[u][2] = yv * s2 * ex2_approx((Lm + sum_l[64 + ch]) - L);  // KL (factor <= 1)
+          for (int e = 0; e < 2; ++e) {
+            const float2 x = bf2(aw[2 * q + e]), y = bf2(bw[2 * q + e]);
+            float r[2][3];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int j = 2 * e + u;
+              const float L = Lv[j] + (t >= 64 ? Mv[j] : 0.f);
+              const float dm = dm_of(Lv[j], Mv[j], t >= 64, my_clamp);
+              const float xs = (u ? x.y : x.x) * s1, ys = (u ? y.y : y.x) * s2;
+              r[u][0] = xs * ex2_approx(dm);
+              r[u][1] = ys * ex2_approx(-dm);
+              r[u][2] = ys * ex2_approx((Mv[j] + Ev[j]) - L);  // KL (factor <= 1)
+            }
+            qm[2 * q + e] = pack_bf16x2(r[0][0], r[1][0]);
+            km[2 * q + e] = pack_bf16x2(r[0][1], r[1][1]);
+            kl[2 * q + e] = pack_bf16x2(r[0][2], r[1][2]);
           }
-          qm[e] = pack_bf16x2(r[0][0], r[1][0]);
-          km[e] = pack_bf16x2(r[0][1], r[1][1]);
-          kl[e] = pack_bf16x2(r[0][2], r[1][2]);
         }
         *reinterpret_cast<uint4*>(p1s + off) = make_uint4(qm[0], qm[1], qm[2], qm[3]);
         *reinterpret_cast<uint4*>(p2s + off) = make_uint4(km[0], km[1], km[2], km[3]);
@@ -371,8 +463,23 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       mbar_arrive(bar(pass == 0 ? B_A : B_DAS));
     }
-    // ---- every product done, p1 and p2 back in shared memory: token t, the group's channels
-    ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_MM), 0, ab) && mbar_wait(bar(B_RELOAD), 0, ab));
+    // ---- the few small retentions' dalpha while the products run (dY, I~ and the state tiles
+    // still stand), a warp each
+    if (n_early > 0) {
+      ew_sync<NG>();  // the coefficients and the scaled state tiles are written
+      if (ok && warp < n_early) {
+        const int u = fix_early[warp] >> 6, ch = fix_early[warp] & 63;
+        const long long at =
+            (long long)b * p.sB + (long long)h * p.sH + (long long)(t0 + u) * p.sT + ch;
+        const float a = __ldg(p.alpha + at);
+        const float pq = fix_up(coef + warp * LT, smem + OFF_V, smem + OFF_G, smem + OFF_C0,
+                                smem + OFF_DCP, u, ch, lane);
+        if (lane == 0) p.dalpha[at] = pq / a;
+      }
+      ew_sync<NG>();  // dY has been read: dv takes its place
+    }
+    // ---- every product done: token t, the group's channels
+    ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_MM), 0, ab));
     uint8_t* const gs = smem + OFF_G;
     float dq[16], dk[16];
     if (ok) {
@@ -381,20 +488,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       // dq' = 2^{L_t - L_m} X, dk' = 2^{L_m - L_t} Y (Y = dA^T Qm + Ys), the group's shares of
       // p1 . dq' and p2 . dk', dL = Qm X - Km Y and Km Ys (Qm, Km as the products read them),
       // dv = dI~ + dY (in dY's place)
-      uint32_t x[16], y[16], ys[16], di[16];
-      tmem_ld16(trow + COL_X + 16 * grp, x);
-      tmem_ld16(trow + COL_Y + 16 * grp, y);
-      tmem_ld16(trow + COL_YS + 16 * grp, ys);
-      tmem_ld16(trow + COL_DI + 16 * grp, di);
-      tmem_ld_wait();
       float A1 = 0.f, A2 = 0.f;
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const int kc = 2 * grp + k;
+        uint32_t x[8], y[8], ys[8], di[8];
+        tmem_ld8(trow + COL_X + 8 * kc, x);
+        tmem_ld8(trow + COL_Y + 8 * kc, y);
+        tmem_ld8(trow + COL_YS + 8 * kc, ys);
+        tmem_ld8(trow + COL_DI + 8 * kc, di);
+        tmem_ld_wait();
         const uint32_t off = t * 128 + ((kc ^ (t & 7)) << 4);
-        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
+        const uint4 a4 = ra[k], b4 = rb[k];
+        const uint4 m4 = *reinterpret_cast<const uint4*>(p1s + off);  // Qm, Km as the products
+        const uint4 n4 = *reinterpret_cast<const uint4*>(p2s + off);  // read them
         const uint4 g4 = *reinterpret_cast<const uint4*>(gs + off);
+        const float4 M0 = *reinterpret_cast<const float4*>(sum_l + 8 * kc);
+        const float4 M1 = *reinterpret_cast<const float4*>(sum_l + 8 * kc + 4);
+        const float Mv[8] = {M0.x, M0.y, M0.z, M0.w, M1.x, M1.y, M1.z, M1.w};
+        const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w}, nw[4] = {n4.x, n4.y, n4.z, n4.w};
         const float4 L0 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc));
         const float4 L1 = *reinterpret_cast<const float4*>(&al_at(t, 8 * kc + 4));
         const float Lv[8] = {L0.x, L0.y, L0.z, L0.w, L1.x, L1.y, L1.z, L1.w};
@@ -405,23 +517,23 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float2 xa = bf2(aw[e]), yb = bf2(bw[e]), g = bf2(gw[e]);
+          const float2 qm2 = bf2(mw[e]), km2 = bf2(nw[e]);
           float dvv[2];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const int j = 8 * k + 2 * e + u;  // index within the group's 16 columns
+            const int i = 2 * e + u, j = 8 * k + i;
             const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
-            const float dm = dm_of(Lv[2 * e + u], sum_l[16 * grp + j], t >= 64, unused_clamp);
-            float qm, km;
-            qm_km(pv, kv, s1, s2, dm, qm, km);
-            const float X = __uint_as_float(x[j]), Ysv = __uint_as_float(ys[j]);
-            const float Y = __uint_as_float(y[j]) + Ysv;
+            const float dm = dm_of(Lv[2 * e + u], Mv[2 * e + u], t >= 64, unused_clamp);
+            const float qm = u ? qm2.y : qm2.x, km = u ? km2.y : km2.x;
+            const float X = __uint_as_float(x[i]), Ysv = __uint_as_float(ys[i]);
+            const float Y = __uint_as_float(y[i]) + Ysv;
             dq[j] = ex2_approx(dm) * X;
             dk[j] = ex2_approx(-dm) * Y;
             A1 = fmaf(pv, dq[j], A1);
             A2 = fmaf(kv, dk[j], A2);
             dl[2 * e + u] = qm * X - km * Y;
             tv[2 * e + u] = km * Ysv;
-            dvv[u] = __uint_as_float(di[j]) + (u ? g.y : g.x);
+            dvv[u] = __uint_as_float(di[i]) + (u ? g.y : g.x);
           }
           dvw[e] = pack_bf16x2(dvv[0], dvv[1]);
         }
@@ -452,8 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const uint32_t off = t * 128 + (((2 * grp + k) ^ (t & 7)) << 4);
-        const uint4 a4 = *reinterpret_cast<const uint4*>(p1s + off);
-        const uint4 b4 = *reinterpret_cast<const uint4*>(p2s + off);
+        const uint4 a4 = ra[k], b4 = rb[k];
         const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
         uint32_t o1[4], o2[4];
 #pragma unroll
@@ -542,141 +653,67 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     ew_sync<NG>();
-    // ---- dalpha_u = (end + sum_{t >= u} dL_t) / alpha_u, rows of 16 threads; the (token,
-    // channel)s with a small alpha are listed for the fix-up
-    uint16_t* const fix_list = reinterpret_cast<uint16_t*>(smem + OFF_FIX_LIST);
+    // ---- dalpha_u = (end + sum_{t >= u} dL_t) / alpha_u, rows of 16 threads, but for small
+    // alphas: those were written above or are listed for the late fix-up
+    uint16_t* const late_list = reinterpret_cast<uint16_t*>(smem + OFF_FIX_LIST);
     if (ok) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int tok = arow + 32 * i;
         const float4 r4 = *reinterpret_cast<const float4*>(gl + tok * GS + 4 * (threadIdx.x & 15));
         const float a[4] = {av[i].x, av[i].y, av[i].z, av[i].w};
-        if (t0 + tok < p.T) {
-          *reinterpret_cast<float4*>(p.dalpha + abase + (long long)(t0 + tok) * p.sT) =
-              make_float4(r4.x / a[0], r4.y / a[1], r4.z / a[2], r4.w / a[3]);
+        const float d[4] = {r4.x / a[0], r4.y / a[1], r4.z / a[2], r4.w / a[3]};
+        float* const to = p.dalpha + abase + (long long)(t0 + tok) * p.sT;
+        if (t0 + tok >= p.T) continue;
+        if (!(fminf(fminf(a[0], a[1]), fminf(a[2], a[3])) < kSmallAlpha)) {
+          *reinterpret_cast<float4*>(to) = make_float4(d[0], d[1], d[2], d[3]);
+          continue;
+        }
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (a[e] < kSmallAlpha)
-              fix_list[atomicAdd(fix_count, 1)] =
-                  (uint16_t)(tok * 64 + 4 * (threadIdx.x & 15) + e);
+        for (int e = 0; e < 4; ++e) {
+          if (!(a[e] < kSmallAlpha))
+            to[e] = d[e];
+          else if (n_early == 0)
+            late_list[atomicAdd(fix_late, 1)] =
+                (uint16_t)(tok * 64 + 4 * (threadIdx.x & 15) + e);
         }
       }
     }
-    ew_sync<NG>();
-    // A small alpha_u (below 2^-10) leaves the suffix sum above a small remainder of
-    // terms that cancel, whose fp32 rounding the division magnifies.  There dalpha comes
-    // from the state entering u and the adjoint of Diag(alpha_u) C_{u-1}, channel c (row
-    // c), at the midpoint scale:
-    //   P_u = 2^{L_m} C_0 + sum_{j < u} Km_j I~_j,   Q_u = 2^{L_end - L_m} dC + sum_{t >= u} Qm_t dY_t,
-    //   dalpha_u = <P_u, Q_u> / alpha_u,
-    // where every term of P_u (u in the first half) or of Q_u (the second) carries the
-    // factor alpha_u, so nothing large cancels.  A block with such tokens loads dY, p1
-    // and p2 again (their tiles now hold the outputs) over the dL arrays, which every
-    // elementwise warp has read by then; one warp per (u, c), Km and Qm in fp32.
-    const int n_fix = *reinterpret_cast<volatile int*>(fix_count);
-    if (ok && n_fix > 0) {
-      if (threadIdx.x == 0) {
+    if (n_small > n_early) {  // more than kFix: their tiles again, a warp per (token, channel)
+      ew_sync<NG>();
+      const int n_late = *reinterpret_cast<volatile int*>(fix_late);
+      if (ok && threadIdx.x == 0) {
         fence_async_smem();  // the dL arrays' generic accesses precede the copies
         mbar_arrive_expect_tx(bar(B_FIX), 3 * T16);
         tma_load_4d(sb + OFF_FIX_G, &tmG, bar(B_FIX), 0, t0, h, b);
         tma_load_4d(sb + OFF_FIX_P1, &tmP1, bar(B_FIX), 0, t0, h, b);
         tma_load_4d(sb + OFF_FIX_P2, &tmP2, bar(B_FIX), 0, t0, h, b);
       }
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_FIX), 0, ab));
-    }
-    if (ok && n_fix > 0) {
-      const uint8_t* vt = smem + OFF_V;
-      const uint8_t* gt = smem + OFF_FIX_G;
-      const uint8_t* p1t = smem + OFF_FIX_P1;
-      const uint8_t* p2t = smem + OFF_FIX_P2;
-      const uint8_t* c0t = smem + OFF_C0;
-      const uint8_t* dct = smem + OFF_DCP;
-      const int t_live = min(LT, p.T - t0);
-      bool unused_clamp = false;
-      // lanes: token group g4 (tokens = g4 mod 4) and the 8 columns of 16-byte group lane & 7
-      // of a 128-byte swizzled row
-      const int g4 = lane >> 3;
-      auto row16 = [&](const uint8_t* tile, int r) {
-        return *reinterpret_cast<const uint4*>(
-            tile + r * 128 + ((((uint32_t)lane & 7) ^ ((uint32_t)r & 7)) << 4));
-      };
-      auto elem = [&](const uint8_t* tile, int r, int col) {
-        return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
-            tile + r * 128 + ((((uint32_t)col >> 3) ^ ((uint32_t)r & 7)) << 4) + (col & 7) * 2));
-      };
-      // S_t / |p_t| of tokens lane + 32 k
-      float sq[4], sk[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int tok = lane + 32 * k;
-        sq[k] = sk[k] = 0.f;
-        if (t0 + tok < p.T) {
-          const float St = 1.0f / (1.0f + __expf(-s_dot[tok] * inv_tau_sqrt_d));
-          sq[k] = St * rsqrtf(s_n1[tok]);
-          sk[k] = St * rsqrtf(s_n2[tok]);
-        }
-      }
-      for (int i = warp; i < n_fix; i += NG * 4) {
-        const int u = fix_list[i] >> 6, cc = fix_list[i] & 63;
-        const float lmc = sum_l[cc];
-        // Km of the tokens before u and Qm of those from u on, channel cc: lane l
-        // holds tokens l + 32 k
-        float kmr[4], qmr[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int tok = lane + 32 * k;
-          const float dm = dm_of(al_at(tok, cc), lmc, tok >= 64, unused_clamp);
-          const float x2 = tok < u ? elem(p2t, tok, cc) : 0.f;
-          const float x1 = (tok >= u && tok < t_live) ? elem(p1t, tok, cc) : 0.f;
-          kmr[k] = x2 * sk[k] * ex2_approx(-dm);
-          qmr[k] = x1 * sq[k] * ex2_approx(dm);
-        }
-        float P[8], Q[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) P[e] = Q[e] = 0.f;
-#pragma unroll 4
-        for (int j0 = 0; j0 < LT; j0 += 4) {  // tokens j0 + g4
-          const int j = j0 + g4, kq = j0 >> 5;
-          const float ksel = kq == 0 ? kmr[0] : kq == 1 ? kmr[1] : kq == 2 ? kmr[2] : kmr[3];
-          const float qsel = kq == 0 ? qmr[0] : kq == 1 ? qmr[1] : kq == 2 ? qmr[2] : qmr[3];
-          const float km = __shfl_sync(0xffffffffu, ksel, (j0 & 31) + g4);
-          const float qm = __shfl_sync(0xffffffffu, qsel, (j0 & 31) + g4);
-          const uint4 v4 = row16(vt, j), d4 = row16(gt, j);
-          const uint32_t vw[4] = {v4.x, v4.y, v4.z, v4.w}, dw[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 fv = bf2(vw[e]), fd = bf2(dw[e]);
-            P[2 * e] = fmaf(km, fv.x, P[2 * e]);
-            P[2 * e + 1] = fmaf(km, fv.y, P[2 * e + 1]);
-            Q[2 * e] = fmaf(qm, fd.x, Q[2 * e]);
-            Q[2 * e + 1] = fmaf(qm, fd.y, Q[2 * e + 1]);
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_FIX), 0, ab));
+      for (int f = warp; ok && f < n_late; f += NG * 4) {
+        const int u = late_list[f] >> 6, ch = late_list[f] & 63;
+        bool unused_clamp = false;
+        float* const cf = coef + warp * LT;
+        for (int tok = lane; tok < LT; tok += 32) {
+          float x = 0.f;
+          if (t0 + tok < p.T) {
+            const float St = 1.0f / (1.0f + __expf(-s_dot[tok] * inv_tau_sqrt_d));
+            const float dm = dm_of(al_at(tok, ch), sum_l[ch], tok >= 64, unused_clamp);
+            x = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
+                smem + (tok < u ? OFF_FIX_P2 : OFF_FIX_P1) + tok * 128 +
+                (((ch >> 3) ^ (tok & 7)) << 4) + (ch & 7) * 2));
+            x = tok < u ? x * (St * rsqrtf(s_n2[tok])) * ex2_approx(-dm)
+                        : x * (St * rsqrtf(s_n1[tok])) * ex2_approx(dm);
           }
+          cf[tok] = x;
         }
-        // the four token groups' sums, the block-boundary rows, and <P_u, Q_u>
-        const uint4 c4 = row16(c0t, cc), e4 = row16(dct, cc);
-        const uint32_t cw[4] = {c4.x, c4.y, c4.z, c4.w}, ew[4] = {e4.x, e4.y, e4.z, e4.w};
-        float pq = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 cf = bf2(cw[e]), ef = bf2(ew[e]);
-#pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2) {
-            float pe = P[2 * e + h2], qe = Q[2 * e + h2];
-            pe += __shfl_xor_sync(0xffffffffu, pe, 8);
-            pe += __shfl_xor_sync(0xffffffffu, pe, 16);
-            qe += __shfl_xor_sync(0xffffffffu, qe, 8);
-            qe += __shfl_xor_sync(0xffffffffu, qe, 16);
-            pq = fmaf(pe + (h2 ? cf.y : cf.x), qe + (h2 ? ef.y : ef.x), pq);
-          }
-        }
-        pq += __shfl_xor_sync(0xffffffffu, pq, 1);
-        pq += __shfl_xor_sync(0xffffffffu, pq, 2);
-        pq += __shfl_xor_sync(0xffffffffu, pq, 4);
-        if (lane == 0) {
-          const long long at = (long long)b * p.sB + (long long)h * p.sH +
-                               (long long)(t0 + u) * p.sT + cc;
-          p.dalpha[at] = pq / __ldg(p.alpha + at);
-        }
+        __syncwarp();
+        const float pq = fix_up(cf, smem + OFF_V, smem + OFF_FIX_G, smem + OFF_C0,
+                                smem + OFF_DCP, u, ch, lane);
+        const long long at =
+            (long long)b * p.sB + (long long)h * p.sH + (long long)(t0 + u) * p.sT + ch;
+        if (lane == 0) p.dalpha[at] = pq / __ldg(p.alpha + at);
+        __syncwarp();
       }
     }
     if (lane == 0) tma_store_wait_read_all();
@@ -684,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   if (warp == W_MMA) drain_wait(bar(B_MM), 0);  // no product in flight past the teardown
-  if (threadIdx.x == 0 && *fix_count > 0) drain_wait(bar(B_FIX), 0);  // nor the fix-up's copies
+  if (threadIdx.x == 0 && *fix_late > 0) drain_wait(bar(B_FIX), 0);  // nor the fix-up's copies
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *clamped && p.dev_status && !*abort_flag)

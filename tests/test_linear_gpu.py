@@ -313,3 +313,23 @@ def test_linear_chunked_at_the_longest_sweep_point():
         pu.check_recorded("linear 32768", "Y chunk-parallel", y_ws[b, :, h], ref, "bf16", "out")
         pu.check_recorded("linear 32768", "Y sequential", y_seq[b, :, h], ref, "bf16", "out")
     _check_grads("linear 32768 bwd", g, p1, p2, v, alpha, dy, heads)
+
+
+@pytest.mark.parametrize("n_small", [1, 16, 17, 300])
+@pytest.mark.parametrize("T", [128, 200])
+def test_linear_chunked_backward_small_retentions(n_small, T):
+    """The retention gradient at planted small retentions: up to 16 in a block go beside the
+    products, more through the tiles loaded again; both against the recurrence."""
+    w = workloads.custom(1, 2, T, 64, "bf16")
+    p1, p2, v, alpha, dy = workloads.make_linear_inputs(w, seed=5)
+    alpha = alpha.clamp_min(2.0 ** -9)  # none small but the planted ones
+    g = torch.Generator().manual_seed(n_small)
+    for h in range(w.H):
+        for i in torch.randperm(min(T, 128) * 64, generator=g)[:n_small].tolist():
+            alpha[0, i // 64, h, i % 64] = 2.0 ** -13
+    dev = torch.device("cuda:0")
+    args = [t.to(dev) for t in (p1, p2, v, alpha, dy)]
+    got = binding.linear_bwd(*args, kernel="tcgen05")[3].float().cpu().numpy()
+    ref = binding.linear_bwd(*args, kernel="simt")[3].float().cpu().numpy()
+    for h in range(w.H):
+        pu.check(f"dalpha head {h}", got[0, :, h], ref[0, :, h], "bf16", "grad")
