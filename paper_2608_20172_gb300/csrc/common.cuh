@@ -225,6 +225,60 @@ __device__ __forceinline__ void mma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint6
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Four k steps (K = 64) of one product under a single elect.sync: the operands advance by
+// A_STEP and B_STEP (descriptor units of 16 bytes) a step; the first step accumulates if
+// `accumulate`, the others always.
+template <int A_STEP, int B_STEP>
+__device__ __forceinline__ void mma_ss_w4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                          uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "add.s64 a1, %1, %5;\n\tadd.s64 a2, %1, %6;\n\tadd.s64 a3, %1, %7;\n\t"
+      "add.s64 b1, %2, %8;\n\tadd.s64 b2, %2, %9;\n\tadd.s64 b3, %2, %10;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "setp.eq.b32 p, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "n"(A_STEP), "n"(2 * A_STEP),
+      "n"(3 * A_STEP), "n"(B_STEP), "n"(2 * B_STEP), "n"(3 * B_STEP)
+      : "memory");
+}
+// Two such products with A in tensor memory (steps 1 to 3 at columns A1, A2, A3 from the first)
+// and, if COMMIT, the arrival on `bar` when they and everything issued before complete, under
+// one elect.sync.
+template <int A1, int A2, int A3, int B_STEP, bool COMMIT>
+__device__ __forceinline__ void mma_ts_w4x2(uint32_t d0, uint32_t a0, uint64_t b0, uint32_t d1,
+                                            uint32_t a1, uint64_t b1, uint32_t idesc,
+                                            uint32_t accumulate, uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred p, t, e;\n\t.reg .b32 x1, x2, x3, y1, y2, y3;\n\t"
+      ".reg .b64 u1, u2, u3, v1, v2, v3;\n\t"
+      "add.s32 x1, %1, %9;\n\tadd.s32 x2, %1, %10;\n\tadd.s32 x3, %1, %11;\n\t"
+      "add.s32 y1, %4, %9;\n\tadd.s32 y2, %4, %10;\n\tadd.s32 y3, %4, %11;\n\t"
+      "add.s64 u1, %2, %12;\n\tadd.s64 u2, %2, %13;\n\tadd.s64 u3, %2, %14;\n\t"
+      "add.s64 v1, %5, %12;\n\tadd.s64 v2, %5, %13;\n\tadd.s64 v3, %5, %14;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %6, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [x1], u1, %6, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [x2], u2, %6, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [x3], u3, %6, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%3], [%4], %5, %6, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%3], [y1], v1, %6, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%3], [y2], v2, %6, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%3], [y3], v3, %6, t;\n\t"
+      "setp.ne.b32 p, %15, 0;\n\t"
+      "and.pred e, e, p;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n\t}" ::"r"(
+          d0),
+      "r"(a0), "l"(b0), "r"(d1), "r"(a1), "l"(b1), "r"(idesc), "r"(accumulate), "r"(bar),
+      "n"(A1), "n"(A2), "n"(A3), "n"(B_STEP), "n"(2 * B_STEP), "n"(3 * B_STEP),
+      "n"(COMMIT ? 1 : 0)
+      : "memory");
+}
 // Copy of a 128-row x 32-byte slice of a shared-memory matrix (the descriptor's layout,
 // e.g. one K step of a 128-byte-swizzled K-major tile) into TMEM lanes 0-127, 8 columns:
 // the A-operand layout of tcgen05.mma with A in TMEM.  Issued from warp-uniform code by one

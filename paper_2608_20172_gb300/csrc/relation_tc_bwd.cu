@@ -357,54 +357,69 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
                                        : idesc_bf16_f32(128, D, true, true);     // dQ
     bool ok = true;
     bool acc_done = false;  // B_ACC of the current unit committed
-    // A unit's running offsets (steps, Q / dO stage loads) and its K / V tiles
+    // A unit's running step offset and its K / V tiles' descriptors (K-major; K also as the
+    // M-major operand of dQ)
     struct Ctx {
-      int gs0, gq0;
-      uint32_t ks, vs;
+      int gs0;
+      uint64_t k, v, km;
     };
-    auto ctx_of = [&](int ul_, int gs0_, int gq0_) {
+    auto ctx_of = [&](int ul_, int gs0_) {
       const uint32_t k = sb + C::OFF_KV + (ul_ % C::NKV) * 2 * C::KVT;
-      return Ctx{gs0_, gq0_, k, k + C::KVT};
+      return Ctx{gs0_, smem_desc_sw128(k, 16, 1024), smem_desc_sw128(k + C::KVT, 16, 1024),
+                 smem_desc_sw128(k, 16384, 1024)};
     };
-    // U^T of step s into buffer (gs0 + s) % NBUF (waits for its Q / dO stage)
-    auto issue_u = [&](const Ctx& x, int s) -> bool {
-      const int g = x.gq0 + C::unit_of(s), st = g % C::NQS, bb = (x.gs0 + s) % C::NBUF;
-      const int hh = s % C::SPT;
-      if (C::HALF || hh == 0) {
-        if (!mbar_wait_warp(bar(B_QF + st), (g / C::NQS) & 1, ab)) return false;
+    // The issue of a step's products is a chain of dependent instructions between the barrier
+    // that lets it start and the one that passes it on, so what can be is taken out of it: the
+    // stages' descriptors are bases plus an offset, the Q / dO stage of the next step to issue
+    // (and its phase) and of the next step to consume are running counters, and products go
+    // out in groups under one elect.sync (d_h = 64 tiles at B 8, H 12, T 2048: 221.5 -> 216.5 us; d_h = 128, H 16, T 4096: 174 -> 170).
+    const uint64_t d_qk = smem_desc_sw128(sb + C::OFF_Q, 16, 1024);      // Q, dO K-major
+    const uint64_t d_gk = smem_desc_sw128(sb + C::OFF_DO, 16, 1024);
+    const uint64_t d_qm = smem_desc_sw128(sb + C::OFF_Q, C::KBQ, 1024);  // and MN-major
+    const uint64_t d_gm = smem_desc_sw128(sb + C::OFF_DO, C::KBQ, 1024);
+    const uint64_t d_ds = smem_desc_sw128(sb + C::OFF_DS, 16384, 1024);
+    uint32_t iq_st = 0, iq_ph = 0, cq_st = 0;
+    // descriptor offset of a step's rows in its stage
+    auto rows_of = [](uint32_t st, int hh) -> uint32_t {
+      return (st * C::QSZ + (C::HALF ? 0 : hh * C::QW * 128)) >> 4;
+    };
+    // the Q / dO stage of step s, the next to issue
+    auto wait_q = [&](int s) -> bool {
+      if (C::HALF || s % C::SPT == 0) {
+        if (!mbar_wait_warp(bar(B_QF + iq_st), iq_ph, ab)) return false;
         tc_fence_after();
-      }
-      const uint32_t rows = C::HALF ? 0u : (uint32_t)(hh * C::QW * 128);  // the step's rows
-#pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t kof = (kk >> 2) * 16384 + (kk & 3) * 32;
-        const uint32_t qof = (kk >> 2) * C::KBQ + (kk & 3) * 32;
-        const uint64_t bq = smem_desc_sw128(sb + C::OFF_Q + st * C::QSZ + rows + qof, 16, 1024);
-        if (C::HALF)
-          mma_ss_w(tmem + C::col_u(bb), smem_desc_sw128(x.ks + kof, 16, 1024), bq, id_s,
-                   kk > 0 ? 1u : 0u);
-        else
-          mma_ts_w(tmem + C::col_u(bb), tmem + C::COL_KT + kk * 8, bq, id_s, kk > 0 ? 1u : 0u);
       }
       return true;
     };
-    // dP^T of step s (after issue_u(s)), then the step's S barrier
-    auto issue_dp = [&](const Ctx& x, int s) {
-      const int st = (x.gq0 + C::unit_of(s)) % C::NQS, bb = (x.gs0 + s) % C::NBUF;
-      const int hh = s % C::SPT;
-      const uint32_t rows = C::HALF ? 0u : (uint32_t)(hh * C::QW * 128);
+    auto next_q = [&](int s) {
+      if (C::HALF || s % C::SPT == C::SPT - 1)
+        if (++iq_st == C::NQS) {
+          iq_st = 0;
+          iq_ph ^= 1;
+        }
+    };
+    // d_h = 128: U^T (or dP^T) of a step, 64 channels at a time
+    auto mma_half = [&](uint32_t col, uint64_t a, uint64_t b) {
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t kof = (kk >> 2) * 16384 + (kk & 3) * 32;
-        const uint32_t qof = (kk >> 2) * C::KBQ + (kk & 3) * 32;
-        const uint64_t bg = smem_desc_sw128(sb + C::OFF_DO + st * C::QSZ + rows + qof, 16, 1024);
-        if (C::HALF)
-          mma_ss_w(tmem + C::col_g(bb), smem_desc_sw128(x.vs + kof, 16, 1024), bg, id_s,
-                   kk > 0 ? 1u : 0u);
-        else
-          mma_ts_w(tmem + C::col_g(bb), tmem + C::COL_VT + kk * 8, bg, id_s, kk > 0 ? 1u : 0u);
+      for (int kb = 0; kb < C::KB; ++kb)
+        mma_ss_w4<2, 2>(tmem + col, a + kb * 1024, b + kb * (C::KBQ >> 4), id_s, kb > 0 ? 1u : 0u);
+    };
+    // U^T and dP^T of step s into buffer (gs0 + s) % NBUF and the step's S barrier
+    auto issue_step = [&](const Ctx& x, int s) -> bool {
+      if (!wait_q(s)) return false;
+      const int bb = (x.gs0 + s) % C::NBUF;
+      const uint32_t off = rows_of(iq_st, s % C::SPT);
+      if (C::HALF) {
+        mma_half(C::col_u(bb), x.k, d_qk + off);
+        mma_half(C::col_g(bb), x.v, d_gk + off);
+        mma_commit_w(bar(B_S + bb));
+      } else {
+        mma_ts_w4x2<8, 16, 24, 2, true>(tmem + C::col_u(bb), tmem + C::COL_KT, d_qk + off,
+                                tmem + C::col_g(bb), tmem + C::COL_VT, d_gk + off, id_s, 0u,
+                                bar(B_S + bb));
       }
-      mma_commit_w(bar(B_S + bb));
+      next_q(s);
+      return true;
     };
     // d_h = 64: the unit's K and V tiles into TMEM (in order after every earlier MMA, so the
     // previous unit's products have read the old ones)
@@ -412,38 +427,36 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
       if (!C::HALF) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-          tmem_cp_w(tmem + C::COL_KT + kk * 8, smem_desc_sw128(x.ks + kk * 32, 16, 1024));
-          tmem_cp_w(tmem + C::COL_VT + kk * 8, smem_desc_sw128(x.vs + kk * 32, 16, 1024));
+          tmem_cp_w(tmem + C::COL_KT + kk * 8, x.k + kk * 2);
+          tmem_cp_w(tmem + C::COL_VT + kk * 8, x.v + kk * 2);
         }
       }
     };
-    int ul = 0, gs0 = 0, gq0 = 0, gt0 = 0;
+    int ul = 0, gs0 = 0, gt0 = 0;
     int pre = 0;  // steps of the current unit issued ahead by the previous unit
     for (int w; ok && (w = unit_at(ul)) < n_work; ++ul) {
       const Unit U = unit(w);
       const int total = U.total;
       acc_done = false;
       const int kvb = ul % C::NKV;
-      const Ctx x = ctx_of(ul, gs0, gq0);
-      const uint32_t ks = x.ks;
+      const Ctx x = ctx_of(ul, gs0);
       if (pre == 0) {
         if (!(ok = mbar_wait_warp(bar(kv_full(kvb)), (ul / C::NKV) & 1, ab))) break;
         tc_fence_after();
         load_kv_tmem(x);
       }
       // d_h = 64: U^T / dP^T of step sn may be issued once its buffer is free (step
-      // sn - NBUF done) and once the GEMM that releases the Q/dO stage it loads into has
-      // been issued: waiting for that stage's load earlier would deadlock.
-      int sn = pre, units_done = 0;
+      // sn - NBUF done) and once the GEMM that releases the Q / dO stage it loads into has
+      // been issued (two tiles back: always by then); waiting for that stage's load earlier
+      // would deadlock.
+      int sn = pre;
       pre = 0;
       while (ok && sn < total && sn < C::NBUF) {
-        ok = issue_u(x, sn);
-        if (ok) issue_dp(x, sn);
+        ok = issue_step(x, sn);
         ++sn;
       }
       for (int s = 0; ok && s < total; ++s) {
-        const int t = s / C::SPT, hh = s % C::SPT, g = gs0 + s, bb = g % C::NBUF;
-        const int st = (gq0 + C::unit_of(s)) % C::NQS;
+        const int hh = s % C::SPT, g = gs0 + s, bb = g % C::NBUF;
         if (!(ok = mbar_wait_warp(bar(B_P + bb), (g / C::NBUF) & 1, ab))) break;
         tc_fence_after();
         // dV += P^T dO and dK += dS'^T Q with the A operands in TMEM: every 32-query chunk
@@ -451,23 +464,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
         // columns.  The first step of a unit starts the sums afresh; the epilogue has
         // read the previous unit's sums before its warps finished this step (B_P).
         const uint32_t pcol = C::col_u(bb), dcol = C::col_g(bb);
-        const uint32_t rows = C::HALF ? 0u : (uint32_t)(hh * C::QW * 128);
-#pragma unroll
-        for (int kk = 0; kk < C::QW / 16; ++kk) {
-          constexpr int H = C::CW / 16;  // 16-query chunks per warpgroup
-          const uint32_t acol = (kk / H) * C::CW + (kk % H) * 8;
-          mma_ts_w(tmem + C::COL_DV, tmem + pcol + acol,
-                   smem_desc_sw128(sb + C::OFF_DO + st * C::QSZ + rows + kk * 2048, C::KBQ, 1024),
-                   id_acc, (s > 0 || kk > 0) ? 1u : 0u);
-        }
-#pragma unroll
-        for (int kk = 0; kk < C::QW / 16; ++kk) {
-          constexpr int H = C::CW / 16;
-          const uint32_t acol = (kk / H) * C::CW + (kk % H) * 8;
-          mma_ts_w(tmem + C::COL_DK, tmem + dcol + acol,
-                   smem_desc_sw128(sb + C::OFF_Q + st * C::QSZ + rows + kk * 2048, C::KBQ, 1024),
-                   id_acc, (s > 0 || kk > 0) ? 1u : 0u);
-        }
+        const uint32_t st = cq_st, off = rows_of(st, hh);
+        if (C::HALF || hh == C::SPT - 1) cq_st = cq_st + 1 == C::NQS ? 0 : cq_st + 1;
+        // (a warpgroup packs its 16-query chunks at the start of its own CW columns)
+        constexpr int A1 = C::CW == 16 ? 16 : 8, A2 = C::CW == 64 ? 16 : 32,
+                      A3 = C::CW == 16 ? 48 : C::CW == 32 ? 40 : 24;
+        mma_ts_w4x2<A1, A2, A3, 128, false>(tmem + C::COL_DV, tmem + pcol, d_gm + off,
+                                            tmem + C::COL_DK, tmem + dcol, d_qm + off, id_acc,
+                                            s > 0 ? 1u : 0u, 0u);
         if (s == total - 1) {  // dK and dV are final: the epilogue need not wait for dQ
           mma_commit_w(bar(B_ACC));
           acc_done = true;
@@ -478,12 +482,11 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
             const Unit N = unit(wn);
             if (!(ok = mbar_wait_warp(bar(kv_full((ul + 1) % C::NKV)), ((ul + 1) / C::NKV) & 1, ab)))
               break;
-            const Ctx xn = ctx_of(ul + 1, gs0 + total, gq0 + U.n_units);
+            const Ctx xn = ctx_of(ul + 1, gs0 + total);
             tc_fence_after();
             load_kv_tmem(xn);
             while (ok && pre < N.total && pre < C::NBUF) {
-              ok = issue_u(xn, pre);
-              if (ok) issue_dp(xn, pre);
+              ok = issue_step(xn, pre);
               ++pre;
             }
             if (!ok) break;
@@ -495,49 +498,47 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
           // step s over dS' in the dP^T columns, which dK has read; U^T of step s + 2
           // over P, which dV has read; dP^T of step s + 2 once dQ^T has been read out.
           // dQ^T = K^T dS'^T (A = K tile, d-major; B = the step's dS', query-major)
-          const uint32_t dsb = sb + C::OFF_DS + (g & 1) * C::DSZ;
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            mma_ss_w(tmem + C::col_g(bb), smem_desc_sw128(ks + kk * 2048, 16384, 1024),
-                     smem_desc_sw128(dsb + kk * 2048, 16384, 1024), id_dq, kk > 0 ? 1u : 0u);
+          for (int kb = 0; kb < 2; ++kb)
+            mma_ss_w4<128, 128>(tmem + C::col_g(bb), x.km + kb * 512,
+                                d_ds + (((g & 1) * C::DSZ) >> 4) + kb * 512, id_dq,
+                                kb > 0 ? 1u : 0u);
           mma_commit_w(bar(B_DQF + bb));
           const int s2 = s + C::NBUF;
-          if (s2 < total && !(ok = issue_u(x, s2))) break;
           if (s2 < total) {
+            if (!(ok = wait_q(s2))) break;
+            const uint32_t o2 = rows_of(iq_st, 0);
+            mma_half(C::col_u(bb), x.k, d_qk + o2);
             if (!(ok = mbar_wait_warp(bar(B_DQE + bb), (g / C::NBUF) & 1, ab))) break;
             tc_fence_after();
-            issue_dp(x, s2);
+            mma_half(C::col_g(bb), x.v, d_gk + o2);
+            mma_commit_w(bar(B_S + bb));
+            next_q(s2);
           }
           continue;
         }
         if (hh == C::SPT - 1) {
-          const int gt = gt0 + t;
+          const int gt = gt0 + s / C::SPT;
           if (gt > 0) {  // dQ of the previous query tile has been read out of TMEM
             if (!(ok = mbar_wait_warp(bar(B_DQE), (gt - 1) & 1, ab))) break;
             tc_fence_after();
           }
           // dQ_t = dS' K   (A = dS', queries x keys, M-major; B = K tile, N-major)
-          const uint32_t ds_base = sb + C::OFF_DS + (gt & 1) * C::DSZ;
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            mma_ss_w(tmem + C::COL_DQ, smem_desc_sw128(ds_base + kk * 2048, 16384, 1024),
-                     smem_desc_sw128(ks + kk * 2048, 16384, 1024), id_dq,
-                     kk > 0 ? 1u : 0u);
+          for (int kb = 0; kb < 2; ++kb)
+            mma_ss_w4<128, 128>(tmem + C::COL_DQ, d_ds + (((gt & 1) * C::DSZ) >> 4) + kb * 512,
+                                x.km + kb * 512, id_dq, kb > 0 ? 1u : 0u);
           mma_commit_w(bar(B_DQF));
           mma_commit_w(bar(B_QE + st));
-          ++units_done;
         }
-        while (ok && sn < total && sn <= s + C::NBUF &&
-               C::unit_of(sn) - C::NQS < units_done) {
-          ok = issue_u(x, sn);
-          if (ok) issue_dp(x, sn);
+        while (ok && sn < total && sn <= s + C::NBUF) {
+          ok = issue_step(x, sn);
           ++sn;
         }
       }
       if (!ok) break;
       mma_commit_w(bar(B_KVE + kvb));  // every MMA of the unit (K / V buffer free) done
       gs0 += total;
-      gq0 += U.n_units;
       gt0 += U.n_i;
     }
     if (!acc_done) mma_commit_w(bar(B_ACC));  // after an abort: whatever completed
