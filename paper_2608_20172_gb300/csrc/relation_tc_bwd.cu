@@ -211,7 +211,9 @@ __device__ __forceinline__ void ew_chunk(const uint32_t (&U)[N], const uint32_t 
   }
 }
 
-template <int D>
+// FULL: d_h = D known at compile time (d_h = 128, whose issue path gains 0.7 % by it; the d_h =
+// 64 kernel measured no slower without).
+template <int D, bool FULL>
 __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
     bwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG,
@@ -352,9 +354,13 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
     // ------------------------------------------------------ MMA issuer
     // Warp-uniform: every lane runs the loop and the waits, one elected lane issues.
     constexpr uint32_t id_s = idesc_bf16_f32(128, C::QW, false, false);  // U^T, dP^T
-    constexpr uint32_t id_acc = idesc_bf16_f32(128, D, false, true);     // dV, dK
-    constexpr uint32_t id_dq = C::HALF ? idesc_bf16_f32(128, C::QW, true, true)  // dQ^T
-                                       : idesc_bf16_f32(128, D, true, true);     // dQ
+    // Head widths below D: the columns of dV, dK (and dQ) up to d_h in 16s only; those past them
+    // are never written, nor read for an output.  (Leaving out U^T's and dP^T's zero k steps
+    // as well costs the full widths more in tests on the issue path than it gives these.)
+    const int dn = FULL ? D : (p.d + 15) & ~15;
+    const uint32_t id_acc = idesc_bf16_f32(128, dn, false, true);              // dV, dK
+    const uint32_t id_dq = C::HALF ? idesc_bf16_f32(128, C::QW, true, true)    // dQ^T
+                                   : idesc_bf16_f32(128, dn, true, true);      // dQ
     bool ok = true;
     bool acc_done = false;  // B_ACC of the current unit committed
     // A unit's running step offset and its K / V tiles' descriptors (K-major; K also as the
@@ -567,6 +573,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
           tmem_ld_wait();
           tc_fence_before();
           mbar_arrive(bar(B_DQE + bb));  // the buffer may take the next dP^T
+          if (!FULL && quad * 32 >= p.d) continue;  // padding rows of dQ^T
           const int row0 = U.bh * t_pad + (U.kt + s / C::SPT) * BT + (s % C::SPT) * C::QW;
           const uint32_t sw = (uint32_t)(lane & 3) << 2;
 #pragma unroll
@@ -604,6 +611,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
             }
 #pragma unroll
             for (int c0 = 0; c0 < 64; c0 += 32, ++chunk) {
+              if (c64 + c0 >= p.d) break;  // padding columns
               const int slot = chunk % C::DQSLOTS;
               if (lane == 0) bulk_wait_read_0();  // the slot's previous reduce has read it
               __syncwarp();
@@ -873,7 +881,8 @@ __global__ void __launch_bounds__(256) pre_kernel(Problem p, BwdWorkspace ws, in
     float* acc = ws.dq_acc + ((long long)bh * ws.t_pad + r) * D + sub * PER;
 #pragma unroll
     for (int c = 0; c < PER; c += 4)
-      *reinterpret_cast<float4*>(acc + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (sub * PER + c < p.d)  // padding columns are never read
+        *reinterpret_cast<float4*>(acc + c) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -978,8 +987,9 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, unsigned stag
     // A runtime call first: it makes the device's primary context current on this thread,
     // which the driver's tensor-map encoder needs (e.g. on a fresh autograd worker thread).
     const int smem = bwd::Cfg<D>::SMEM;
-    e = cudaFuncSetAttribute(bwd::bwd_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem);
+    auto* const tiles =
+        D == 128 && p.d == D ? bwd::bwd_tc_kernel<D, D == 128> : bwd::bwd_tc_kernel<D, false>;
+    e = cudaFuncSetAttribute(tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) { note_failure("backward: shared memory attribute"); return e; }
     CUtensorMap mq, mk, mv, mg, mdq, mdk, mdv;
     constexpr int qrows = bwd::Cfg<D>::QROWS;
@@ -1000,8 +1010,8 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, unsigned stag
     // d_h = 128 (one CTA per unit, dynamic scheduling): heads in groups, one CTA per SM;
     // d_h = 64 (persistent, zigzag over a heaviest-first sequence): one group.
     const int groups = D == 64 ? 1 : head_groups(n_t, p.B * p.H, nsm);
-    bwd::bwd_tc_kernel<D><<<(unsigned)grid, bwd::Cfg<D>::THREADS, smem, s>>>(mq, mk, mv, mg, mdq, mdk,
-                                                                     mdv, p, ws, n_t, t_pad, groups);
+    tiles<<<(unsigned)grid, bwd::Cfg<D>::THREADS, smem, s>>>(mq, mk, mv, mg, mdq, mdk, mdv, p, ws,
+                                                             n_t, t_pad, groups);
     if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("backward: tile kernel launch"); return e; }
   }
   if (stages & 4) {
