@@ -16,8 +16,12 @@
 // dV, I and writes dP1, dP2, dI): one CTA per (sequence, 16 positions) moves 8-element
 // vectors (16 bytes in bf16).  The rotation angles of the CTA's positions are tabulated
 // once in shared memory and reused by every head: m * base^(-2c/d) is formed and reduced
-// modulo 2 pi in fp64 (positions reach 16k, where an fp32 angle would be off by ~1e-3
-// rad), then its cosine and sine are taken in fp32.  dtheta is summed per CTA in a fixed
+// modulo 2 pi as a sum of two floats (positions reach 16k, where an fp32 angle would be off
+// by ~1e-3 rad) from frequencies that come with the launch, then its cosine and sine are
+// taken in fp32.  (In fp64, with an fp64 log and exp per CTA, this chip's fp64 pipe bounded
+// both passes; the rotations and the mixing are CTAs of their own, so that the tables hide.
+// B 4, H 8, T 4096, d 80: prep 48 -> 31 us, grad 63 -> 41; B 2, H 16, T 16384, d 128: 159 ->
+// 126 us (6.4 TB/s), 196 -> 153 (6.1).)  dtheta is summed per CTA in a fixed
 // order and the partials are added up in fp64 by a second kernel, one block per head
 // pair (deterministic).
 #include <math.h>
@@ -37,8 +41,9 @@ template <typename TI>
 struct Vec8;
 template <>
 struct Vec8<__nv_bfloat16> {
-  __device__ static void load(const void* p, float (&x)[8]) {
-    const uint4 w = *reinterpret_cast<const uint4*>(p);
+  using Raw = uint4;
+  __device__ static Raw load(const __nv_bfloat16* p) { return *reinterpret_cast<const uint4*>(p); }
+  __device__ static void unpack(const Raw& w, float (&x)[8]) {
     const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -54,11 +59,15 @@ struct Vec8<__nv_bfloat16> {
 };
 template <>
 struct Vec8<float> {
-  __device__ static void load(const void* p, float (&x)[8]) {
-    const float4 a = reinterpret_cast<const float4*>(p)[0];
-    const float4 b = reinterpret_cast<const float4*>(p)[1];
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  struct Raw {
+    float4 a, b;
+  };
+  __device__ static Raw load(const float* p) {
+    return {reinterpret_cast<const float4*>(p)[0], reinterpret_cast<const float4*>(p)[1]};
+  }
+  __device__ static void unpack(const Raw& w, float (&x)[8]) {
+    x[0] = w.a.x; x[1] = w.a.y; x[2] = w.a.z; x[3] = w.a.w;
+    x[4] = w.b.x; x[5] = w.b.y; x[6] = w.b.z; x[7] = w.b.w;
   }
   __device__ static void store(void* p, const float (&x)[8]) {
     reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
@@ -67,37 +76,49 @@ struct Vec8<float> {
 };
 
 struct Tables {
-  double w[kMaxD / 2];                             // base^(-2c/d), fp64
   float cs[kTok][kMaxD / 2], sn[kTok][kMaxD / 2];  // RoPE of the CTA's positions
-  float tc[kMaxPairs], ts[kMaxPairs];              // cos, sin of the Givens angles
-  float part[kThreads / 32][kMaxPairs];            // dtheta: per-warp partial sums
 };
 
-// cos / sin of m * base^(-2c/d) for the CTA's positions, and of the Givens angles.  The
-// d/2 frequencies first (fp64 exp, the expensive part on this GPU's fp64 pipe), then
-// per entry one fp64 product and a reduction modulo 2 pi.
-__device__ void fill_tables(Tables& tb, const LayerProblem& p, int t0) {
+// The kernels' parameters: the problem and the frequencies base^(-2c/d), each as a sum of two
+// floats (48 bits).
+struct Args {
+  LayerProblem p;
+  float w_hi[kMaxD / 2], w_lo[kMaxD / 2];
+};
+
+// m * w modulo 2 pi (|r| <= pi + rounding) for a position m < 2^22 and w = w_hi + w_lo <= 1:
+// the product and n 2 pi are kept as rounded value and exact remainder (two-product by fma;
+// their leading parts are close, so that their difference is exact), 2 pi as a sum of two
+// floats (48 bits, n < 2^20: 2 pi's tail adds less than 2^-24).
+__device__ __forceinline__ float turn(float m, float w_hi, float w_lo) {
+  constexpr float kTwoPiHi = 6.28318530717958647692f;
+  constexpr float kTwoPiLo = (float)(6.28318530717958647692 - (double)kTwoPiHi);
+  const float a = m * w_hi;
+  const float a_lo = fmaf(m, w_lo, fmaf(m, w_hi, -a));
+  const float n = rintf(a * 0.15915494309189533577f);
+  const float q = n * kTwoPiHi;
+  const float q_lo = fmaf(n, kTwoPiLo, fmaf(n, kTwoPiHi, -q));
+  return (a - q) + (a_lo - q_lo);
+}
+
+// cos / sin of m * base^(-2c/d) for the CTA's positions
+__device__ __forceinline__ void fill_tables(Tables& tb, const Args& ar, int t0) {
+  const LayerProblem& p = ar.p;
   const int half = p.d / 2;
-  const double lnb = log((double)p.rope_base);
-  for (int c = threadIdx.x; c < half; c += kThreads)
-    tb.w[c] = exp(-2.0 * (double)c / (double)p.d * lnb);
-  __syncthreads();
-  const double two_pi = 6.283185307179586476925286766559;
-  const double inv_two_pi = 0.15915494309189533576888376337251;
   for (int e = threadIdx.x; e < kTok * half; e += kThreads) {
     const int tt = e / half, c = e % half;
-    const double a = (double)(t0 + tt) * tb.w[c];
-    const float r = (float)fma(-rint(a * inv_two_pi), two_pi, a);  // |r| <= pi (+ rounding)
+    float r;
+    if (t0 < (1 << 22) - kTok && p.rope_base >= 1.0f) {
+      r = turn((float)(t0 + tt), ar.w_hi[c], ar.w_lo[c]);
+    } else {  // positions or frequencies past turn's range: fp64
+      const double a = (double)(t0 + tt) * exp(-2.0 * (double)c / (double)p.d * log((double)p.rope_base));
+      r = (float)fma(-rint(a * 0.15915494309189533576888376337251),
+                     6.283185307179586476925286766559, a);
+    }
     float s, co;
     sincosf(r, &s, &co);
     tb.cs[tt][c] = co;
     tb.sn[tt][c] = s;
-  }
-  for (int k = threadIdx.x; k < p.H / 2; k += kThreads) {
-    float s, co;
-    sincosf(p.theta[k], &s, &co);
-    tb.tc[k] = co;
-    tb.ts[k] = s;
   }
 }
 
@@ -119,102 +140,155 @@ __device__ __forceinline__ void rotate8(float (&x)[8], const Tables& tb, int tt,
   }
 }
 
+// A CTA's sequence and positions.  Even CTAs rotate, odd ones mix: a rotating CTA's first
+// loads are in flight while it tabulates the angles, and the mixing CTAs beside it have none
+// to wait for.
+struct Where {
+  int b, t0, nt;
+};
+__device__ __forceinline__ Where where(const LayerProblem& p) {
+  const int n_tt = (p.T + kTok - 1) / kTok, w = (int)(blockIdx.x >> 1);
+  const int t0 = (w % n_tt) * kTok;
+  return {w / n_tt, t0, min(kTok, p.T - t0)};
+}
+
 // RoPE (sgn = +1) or its transpose (sgn = -1) of in1 -> out1 and in2 -> out2 over the
 // CTA's (position, head, chunk) items, two items per thread and iteration so that four
-// 16-byte loads are in flight.
+// 16-byte loads are in flight (the first ones during the tables).
 template <typename TI>
-__device__ __forceinline__ void rope_pass(const LayerProblem& p, const Tables& tb, int t0, int nt,
-                                          float sgn) {
+__device__ __forceinline__ void rope_pass(Tables& tb, const Args& ar, const Where& at, float sgn) {
+  using V = Vec8<TI>;
+  const LayerProblem& p = ar.p;
   const int nu = p.d / 8;
-  const int n = nt * p.H * nu;
-  const long long base = (long long)(blockIdx.x / ((p.T + kTok - 1) / kTok)) * p.sB;
-  auto off_of = [&](int e, int& tt, int& u) {
-    u = e % nu;
-    const int h = (e / nu) % p.H;
-    tt = e / (nu * p.H);
-    return base + (long long)(t0 + tt) * p.sT + (long long)h * p.sH + 8 * u;
+  const int n = at.nt * p.H * nu;
+  const long long base = (long long)at.b * p.sB;
+  const TI* in1 = reinterpret_cast<const TI*>(p.in1);
+  const TI* in2 = reinterpret_cast<const TI*>(p.in2);
+  struct Item {
+    long long off;
+    int tt, u;
   };
+  auto item = [&](int e) {  // (clamped: a thread past the end reloads the last item)
+    e = min(e, n - 1);
+    const int r = e / nu, h = r % p.H, tt = r / p.H;
+    Item i;
+    i.u = e - r * nu;
+    i.tt = tt;
+    i.off = base + (long long)(at.t0 + tt) * p.sT + (long long)h * p.sH + 8 * i.u;
+    return i;
+  };
+  auto put = [&](const Item& i, const typename V::Raw& a, const typename V::Raw& b) {
+    float x[8], y[8];
+    V::unpack(a, x);
+    V::unpack(b, y);
+    rotate8(x, tb, i.tt, i.u, sgn);
+    rotate8(y, tb, i.tt, i.u, sgn);
+    V::store(reinterpret_cast<TI*>(p.out1) + i.off, x);
+    V::store(reinterpret_cast<TI*>(p.out2) + i.off, y);
+  };
+  Item i0 = item(threadIdx.x), i1 = item(threadIdx.x + kThreads);
+  typename V::Raw x0 = V::load(in1 + i0.off), y0 = V::load(in2 + i0.off);
+  typename V::Raw x1 = V::load(in1 + i1.off), y1 = V::load(in2 + i1.off);
+  fill_tables(tb, ar, at.t0);
+  __syncthreads();
   for (int e = threadIdx.x; e < n; e += 2 * kThreads) {
-    const int e2 = e + kThreads;
-    const bool two = e2 < n;
-    int tt0, u0, tt1 = 0, u1 = 0;
-    const long long o0 = off_of(e, tt0, u0);
-    const long long o1 = two ? off_of(e2, tt1, u1) : o0;
-    float x0[8], y0[8], x1[8], y1[8];
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in1) + o0, x0);
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in2) + o0, y0);
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in1) + o1, x1);
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in2) + o1, y1);
-    rotate8(x0, tb, tt0, u0, sgn);
-    rotate8(y0, tb, tt0, u0, sgn);
-    Vec8<TI>::store(reinterpret_cast<TI*>(p.out1) + o0, x0);
-    Vec8<TI>::store(reinterpret_cast<TI*>(p.out2) + o0, y0);
-    if (two) {
-      rotate8(x1, tb, tt1, u1, sgn);
-      rotate8(y1, tb, tt1, u1, sgn);
-      Vec8<TI>::store(reinterpret_cast<TI*>(p.out1) + o1, x1);
-      Vec8<TI>::store(reinterpret_cast<TI*>(p.out2) + o1, y1);
+    if (e != (int)threadIdx.x) {
+      i0 = item(e);
+      i1 = item(e + kThreads);
+      x0 = V::load(in1 + i0.off);
+      y0 = V::load(in2 + i0.off);
+      x1 = V::load(in1 + i1.off);
+      y1 = V::load(in2 + i1.off);
     }
+    put(i0, x0, y0);
+    if (e + kThreads < n) put(i1, x1, y1);
   }
 }
 
 template <typename TI>
-__global__ void __launch_bounds__(kThreads) prep_kernel(LayerProblem p) {
-  __shared__ Tables tb;
-  const int n_tt = (p.T + kTok - 1) / kTok;
-  const int b = blockIdx.x / n_tt, t0 = (blockIdx.x % n_tt) * kTok;
-  const int nt = min(kTok, p.T - t0);
-  fill_tables(tb, p, t0);
-  __syncthreads();
-  const int nu = p.d / 8;  // 8-element chunks per row
-  const long long base = (long long)b * p.sB;
-  rope_pass<TI>(p, tb, t0, nt, 1.f);  // Q = RoPE(P1), K = RoPE(P2)
-  // Givens mixing of the information states: (token, pair, chunk) items
-  const int np = p.H / 2;
-  for (int e = threadIdx.x; e < nt * np * nu; e += kThreads) {
-    const int u = e % nu, k = (e / nu) % np, tt = e / (nu * np);
-    int ha, hb;
-    pair_heads(p, k, ha, hb);
-    const long long row = base + (long long)(t0 + tt) * p.sT + 8 * u;
-    const long long oa = row + (long long)ha * p.sH, ob = row + (long long)hb * p.sH;
-    float ia[8], ib[8], va[8], vb[8];
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in3) + oa, ia);
-    Vec8<TI>::load(reinterpret_cast<const TI*>(p.in3) + ob, ib);
-    const float co = tb.tc[k], s = tb.ts[k];
+__global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ Args ar) {
+  using V = Vec8<TI>;
+  const LayerProblem& p = ar.p;
+  const Where at = where(p);
+  if (!(blockIdx.x & 1)) {  // Q = RoPE(P1), K = RoPE(P2)
+    __shared__ Tables tb;
+    rope_pass<TI>(tb, ar, at, 1.f);
+    return;
+  }
+  // Givens mixing of the information states: (token, pair, chunk) items, two per thread and
+  // iteration
+  const int nu = p.d / 8, np = p.H / 2, n = at.nt * np * nu;
+  const long long base = (long long)at.b * p.sB;
+  const TI* in = reinterpret_cast<const TI*>(p.in3);
+  TI* out = reinterpret_cast<TI*>(p.out3);
+  for (int e0 = threadIdx.x; e0 < n; e0 += 2 * kThreads) {
+    typename V::Raw ra[2], rb[2];
+    long long oa[2], ob[2];
+    float th[2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      va[i] = co * ia[i] - s * ib[i];
-      vb[i] = s * ia[i] + co * ib[i];
+    for (int i = 0; i < 2; ++i) {
+      const int e = min(e0 + i * kThreads, n - 1);
+      const int r = e / nu, k = r % np, tt = r / np;
+      int ha, hb;
+      pair_heads(p, k, ha, hb);
+      const long long row = base + (long long)(at.t0 + tt) * p.sT + 8 * (e - r * nu);
+      oa[i] = row + (long long)ha * p.sH;
+      ob[i] = row + (long long)hb * p.sH;
+      ra[i] = V::load(in + oa[i]);
+      rb[i] = V::load(in + ob[i]);
+      th[i] = p.theta[k];
     }
-    Vec8<TI>::store(reinterpret_cast<TI*>(p.out3) + oa, va);
-    Vec8<TI>::store(reinterpret_cast<TI*>(p.out3) + ob, vb);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (e0 + i * kThreads >= n) break;
+      float ia[8], ib[8], va[8], vb[8], s, co;
+      sincosf(th[i], &s, &co);
+      V::unpack(ra[i], ia);
+      V::unpack(rb[i], ib);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        va[j] = co * ia[j] - s * ib[j];
+        vb[j] = s * ia[j] + co * ib[j];
+      }
+      V::store(out + oa[i], va);
+      V::store(out + ob[i], vb);
+    }
   }
 }
 
 template <typename TI>
-__global__ void __launch_bounds__(kThreads) grad_kernel(LayerProblem p) {
-  __shared__ Tables tb;
-  const int n_tt = (p.T + kTok - 1) / kTok;
-  const int b = blockIdx.x / n_tt, t0 = (blockIdx.x % n_tt) * kTok;
-  const int nt = min(kTok, p.T - t0);
+__global__ void __launch_bounds__(kThreads) grad_kernel(const __grid_constant__ Args ar) {
+  using V = Vec8<TI>;
+  const LayerProblem& p = ar.p;
+  const Where at = where(p);
+  if (!(blockIdx.x & 1)) {  // transposed RoPE: dP1 from dQ, dP2 from dK
+    __shared__ Tables tb;
+    rope_pass<TI>(tb, ar, at, -1.f);
+    return;
+  }
+  __shared__ float part[kThreads / 32][kMaxPairs], tc[kMaxPairs], ts[kMaxPairs];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  fill_tables(tb, p, t0);
-  for (int k = lane; k < p.H / 2; k += 32) tb.part[warp][k] = 0.f;
+  for (int k = threadIdx.x; k < p.H / 2; k += kThreads) {
+    float s, co;
+    sincosf(p.theta[k], &s, &co);
+    tc[k] = co;
+    ts[k] = s;
+  }
+  for (int k = lane; k < p.H / 2; k += 32) part[warp][k] = 0.f;
   __syncthreads();
-  const int nu = p.d / 8;
-  const long long base = (long long)b * p.sB;
-  rope_pass<TI>(p, tb, t0, nt, -1.f);  // transposed RoPE: dP1 from dQ, dP2 from dK
+  const int nu = p.d / 8, t0 = at.t0;
+  const long long base = (long long)at.b * p.sB;
   // transposed Givens: dI from dV = dI~, and dtheta.  The loop runs the same number of
   // times on every lane (items past the end are idle), so the warp can reduce dtheta
   // over runs of lanes with the same pair (items are ordered chunk, pair, position) and
   // add each run's sum to its pair's slot in lane order (deterministic).
   const int np = p.H / 2;
-  const int n_items = nt * np * nu;
+  const int n_items = at.nt * np * nu;
   for (int e0 = 0; e0 < n_items; e0 += kThreads) {
     const int e = e0 + (int)threadIdx.x;
     const bool live = e < n_items;
     const int ec = live ? e : 0;
-    const int u = ec % nu, k = (ec / nu) % np, tt = ec / (nu * np);
+    const int rr = ec / nu, u = ec - rr * nu, k = rr % np, tt = rr / np;
     float dt = 0.f;
     if (live) {
       int ha, hb;
@@ -222,11 +296,15 @@ __global__ void __launch_bounds__(kThreads) grad_kernel(LayerProblem p) {
       const long long row = base + (long long)(t0 + tt) * p.sT + 8 * u;
       const long long oa = row + (long long)ha * p.sH, ob = row + (long long)hb * p.sH;
       float ga[8], gb[8], ia[8], ib[8], da[8], db[8];
-      Vec8<TI>::load(reinterpret_cast<const TI*>(p.in3) + oa, ga);
-      Vec8<TI>::load(reinterpret_cast<const TI*>(p.in3) + ob, gb);
-      Vec8<TI>::load(reinterpret_cast<const TI*>(p.in4) + oa, ia);
-      Vec8<TI>::load(reinterpret_cast<const TI*>(p.in4) + ob, ib);
-      const float co = tb.tc[k], s = tb.ts[k];
+      const typename V::Raw r1 = V::load(reinterpret_cast<const TI*>(p.in3) + oa);
+      const typename V::Raw r2 = V::load(reinterpret_cast<const TI*>(p.in3) + ob);
+      const typename V::Raw r3 = V::load(reinterpret_cast<const TI*>(p.in4) + oa);
+      const typename V::Raw r4 = V::load(reinterpret_cast<const TI*>(p.in4) + ob);
+      V::unpack(r1, ga);
+      V::unpack(r2, gb);
+      V::unpack(r3, ia);
+      V::unpack(r4, ib);
+      const float co = tc[k], s = ts[k];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         da[i] = co * ga[i] + s * gb[i];
@@ -252,7 +330,7 @@ __global__ void __launch_bounds__(kThreads) grad_kernel(LayerProblem p) {
     const int run = __popc(heads & (0xffffffffu >> (31 - lane))) - 1;
     const int n_runs = __popc(heads);
     for (int r = 0; r < n_runs; ++r) {
-      if (tail && live && run == r) tb.part[warp][k] += dt;
+      if (tail && live && run == r) part[warp][k] += dt;
       __syncwarp();
     }
   }
@@ -260,24 +338,38 @@ __global__ void __launch_bounds__(kThreads) grad_kernel(LayerProblem p) {
   for (int k = threadIdx.x; k < np; k += kThreads) {
     float s = 0.f;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += tb.part[w][k];
-    p.dtheta_part[(long long)blockIdx.x * np + k] = s;
+    for (int w = 0; w < kThreads / 32; ++w) s += part[w][k];
+    p.dtheta_part[(long long)(blockIdx.x >> 1) * np + k] = s;
   }
 }
 
 // dtheta_k = sum over CTAs of the partials, in fp64 and a fixed order; one block per pair
 __global__ void __launch_bounds__(256) dtheta_kernel(LayerProblem p, int n_cta) {
-  __shared__ double red[256];
+  __shared__ double red[8];
   const int np = p.H / 2, k = blockIdx.x;
   double s = 0.0;
   for (int c = threadIdx.x; c < n_cta; c += 256) s += (double)p.dtheta_part[(long long)c * np + k];
-  red[threadIdx.x] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += red[w];
+    p.dtheta[k] = (float)s;
   }
-  if (threadIdx.x == 0) p.dtheta[k] = (float)red[0];
+}
+
+Args args_of(const LayerProblem& p) {
+  Args ar;
+  ar.p = p;
+  const double lnb = log((double)p.rope_base);
+  for (int c = 0; c < p.d / 2; ++c) {
+    const double w = exp(-2.0 * (double)c / (double)p.d * lnb);
+    ar.w_hi[c] = (float)w;
+    ar.w_lo[c] = (float)(w - (double)ar.w_hi[c]);
+  }
+  return ar;
 }
 
 int ctas(const LayerProblem& p) { return p.B * ((p.T + kTok - 1) / kTok); }
@@ -295,10 +387,11 @@ size_t layer_grad_workspace_bytes(int B, int T, int H) {
 
 cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
   const int grid = layer::ctas(p);
+  const layer::Args ar = layer::args_of(p);
   if (p.dtype == RELATION_F32)
-    layer::prep_kernel<float><<<grid, layer::kThreads, 0, s>>>(p);
+    layer::prep_kernel<float><<<2 * grid, layer::kThreads, 0, s>>>(ar);
   else
-    layer::prep_kernel<__nv_bfloat16><<<grid, layer::kThreads, 0, s>>>(p);
+    layer::prep_kernel<__nv_bfloat16><<<2 * grid, layer::kThreads, 0, s>>>(ar);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) note_failure("layer prep: launch");
   return e;
@@ -306,10 +399,11 @@ cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
 
 cudaError_t launch_layer_grad(const LayerProblem& p, cudaStream_t s) {
   const int grid = layer::ctas(p);
+  const layer::Args ar = layer::args_of(p);
   if (p.dtype == RELATION_F32)
-    layer::grad_kernel<float><<<grid, layer::kThreads, 0, s>>>(p);
+    layer::grad_kernel<float><<<2 * grid, layer::kThreads, 0, s>>>(ar);
   else
-    layer::grad_kernel<__nv_bfloat16><<<grid, layer::kThreads, 0, s>>>(p);
+    layer::grad_kernel<__nv_bfloat16><<<2 * grid, layer::kThreads, 0, s>>>(ar);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { note_failure("layer grad: launch"); return e; }
   layer::dtheta_kernel<<<p.H / 2, 256, 0, s>>>(p, grid);
