@@ -108,7 +108,10 @@ __global__ void __launch_bounds__(kWarps * 32) pre_kernel(Problem p, BwdWorkspac
     }
     const float u = qk * p.inv_sqrt_d;
     const float S = 1.0f / (1.0f + expf(-u / p.tau_s));
-    const float F = expf(S - p.logz_in[gr]);
+    Sum2 t;  // S - logZ with its rounding, as a factor of F
+    t.add(-p.logz_in[gr]);
+    t.add(S);
+    const float F = expf(t.s) * (fabsf(t.s) < INFINITY ? 1.f + t.c : 1.f);
     const float dR = F * (gv - gy);
     const float dS = dR * S * (1.0f - S) / p.tau_s;
     if (lane == 0) {

@@ -21,6 +21,33 @@ namespace rel {
 // ---------------------------------------------------------------------------
 constexpr unsigned long long kWaitTimeoutNs = 1000ull * 1000ull * 1000ull;  // 1 s
 
+// Compensated sum of a few floats: s the rounded sum, c the sum of the additions' errors.
+struct Sum2 {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = s + x, z = t - s;
+    c += (s - (t - z)) + (x - z);
+    s = t;
+  }
+  // + f * log(x) for x > 0: x = 2^e y with y near 1, so that e ln 2 (ln 2 as a sum of two floats)
+  // and log y, each with its rounding small against 1, take the place of one rounded logarithm
+  __device__ __forceinline__ void add_log(float x, float f) {
+    constexpr float kLn2 = 0.693147180559945309417f;
+    constexpr float kLn2Lo = (float)(0.693147180559945309417 - (double)kLn2);
+    int e;
+    float y = frexpf(x, &e);
+    if (y < 0.7071f) {
+      y *= 2.f;
+      --e;
+    }
+    const float a = (float)e * kLn2, b = logf(y), fa = f * a, fb = f * b;
+    add(fa);
+    add(fb);
+    c += fmaf(f, a, -fa) + fmaf(f, b, -fb) +
+         f * fmaf((float)e, kLn2Lo, fmaf((float)e, kLn2, -a));
+  }
+};
+
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -1,8 +1,8 @@
 // relation_simt.cu -- CUDA-core (SIMT) FlashRelation kernels, fp32 and bf16 I/O.
 //
 // These kernels run the exact causal Relation operator with fp32 arithmetic on the
-// CUDA cores.  They serve the fp32 workloads (accurate expf / logf / division, no
-// approximate transcendental instructions) and every (dtype, d_h) the tensor-core
+// CUDA cores.  They serve the fp32 workloads (expf and logf, not the fast forms; the row
+// statistics and the sums that cancel in two floats) and every (dtype, d_h) the tensor-core
 // kernels do not cover.
 //
 // Work split.  A CTA of W warps owns 8 W rows of one head (queries in the forward and dQ,
@@ -15,7 +15,7 @@
 // [8][64] buffer.  Bound: shared-memory bandwidth and the FP32 pipe (backward: 78 % of the
 // wavefronts, 58 % of the pipe), 2 + 7 products of d_h over the causal pairs (forward +
 // backward); the forward's longest CTAs also end alone.  Measured, B 2, H 8, T 1000, d 64,
-// forward + backward: 1478 -> 331 us (forward 567 -> 107, backward tiles 920 -> 209) against a
+// forward + backward: 1478 -> 335 us (forward 567 -> 108, backward tiles 920 -> 212) against a
 // thread per quarter row (one 16-byte shared read per four multiply-adds, two shuffles per
 // entry); B 1, H 2, T 128, d 32: 49 -> 11 and 77 -> 12 us.
 //
@@ -25,6 +25,9 @@
 // Self-Exchange split:
 //   A_i = m + log l - lambda log i, g_i = sigmoid(A_i - S_i),
 //   Y_i = (1 - g_i) v_i + g_i z / l,  logZ_i = logaddexp(S_i, A_i)   (App. A.3.5).
+// logZ's error is a relative error of all weights of its row in the backward, so A_i is a sum
+// of two floats: logZ to 2.5e-8 of 64 bits instead of 1.1e-7 (T 1000, d 64; rms over the rows),
+// dL/dlambda to 1.1e-6 instead of 4.9e-6 (rms over inputs), for 1 % of the time.
 //
 // Backward (App. A.1.7): the Self part and D_i come from the shared row kernel
 // (aux_kernels.cu); one launch holds key-stationary CTAs that accumulate dK, dV over query
@@ -342,11 +345,18 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
     float g = 0.f, lz = S;
     float inv_l = 0.f, fself = 1.0f;  // F_ii = 1 - g: the Self flow
     if (row > 0 && lr > 0.f) {
-      const float A = m[r] + logf(lr) - p.lambda * logf((float)(row + 1));
-      g = 1.0f / (1.0f + expf(S - A));
-      fself = 1.0f / (1.0f + expf(A - S));
-      const float hi = fmaxf(S, A), lo = fminf(S, A);
-      lz = hi + log1pf(expf(lo - hi));
+      // A = m + log l - lambda log i as a sum of two floats (where it is finite): logZ's error is
+      // a relative error of the whole row's weights in the backward
+      Sum2 a;
+      a.add(m[r]);
+      a.add_log(lr, 1.f);
+      a.add_log((float)(row + 1), -p.lambda);
+      const float A = a.s, Alo = fabsf(A) < INFINITY ? a.c : 0.f;
+      const float t = (A - S) + Alo;  // A - S
+      g = 1.0f / (1.0f + expf(-t));
+      fself = 1.0f / (1.0f + expf(t));
+      const float x = log1pf(expf(-fabsf(t)));
+      lz = t > 0.f ? A + (Alo + x) : S + x;
       inv_l = 1.0f / lr;
     }
     float y[D / 16];
@@ -412,7 +422,7 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < D / 16; ++c) dk[r][c] = dv[r][c] = 0.f;
-  float dlam = 0.f;  // -sum_i log i F_ii dR_ij over the lane's Exchange pairs
+  Sum2 dlam;  // -sum_i log i F_ii dR_ij over the lane's Exchange pairs (they cancel within a row)
   stage<TI, D, NT>(Ks, K, p.sT, k0, ROWS, p.T);
   stage<TI, D, NT>(Vs, V, p.sT, k0, ROWS, p.T);
   for (int q0 = k0 / kTile * kTile; q0 < p.T; q0 += kTile) {
@@ -422,16 +432,25 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
     stage_commit();
     for (int ii = threadIdx.x; ii < kTile; ii += NT) {
       const int i = q0 + ii;
-      const float li = logf((float)(i + 1));
-      cs[ii] = i < p.T ? -p.lambda * li - logz[i] : -INFINITY;
-      Ds[ii] = i < p.T ? Drow[i] : 0.f;
-      wl[ii] = i < p.T ? li * Fs[i] : 0.f;
+      if (i < p.T) {
+        // cs rounds; its error times P is in every P of the row, and taken out of dlambda's weight
+        Sum2 c;
+        c.add_log((float)(i + 1), -p.lambda);
+        c.add(-logz[i]);
+        cs[ii] = c.s;
+        wl[ii] = logf((float)(i + 1)) * Fs[i] * (fabsf(c.s) < INFINITY ? 1.f + c.c : 1.f);
+        Ds[ii] = Drow[i];
+      } else {
+        cs[ii] = -INFINITY;
+        wl[ii] = Ds[ii] = 0.f;
+      }
     }
     stage_wait<0>();
     __syncthreads();
     float P[4][4], dS[4][4];
     dots<D>(Ks + warp * kWarpRows * LD, Qs, ty, tx, P);
     dots<D>(Vs + warp * kWarpRows * LD, Gs, ty, tx, dS);
+    float dl = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int ii = 16 * i + tx, q = q0 + ii;
@@ -443,10 +462,11 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
         const bool in = q > j0 + r && q < p.T;
         P[r][i] = in ? pv : 0.f;
         dS[r][i] = in ? ds : 0.f;
-        dlam = in ? fmaf(-wi, dR, dlam) : dlam;
+        dl = in ? fmaf(-wi, dR, dl) : dl;
         Pw[(4 * ty + r) * PW + ii] = P[r][i];
       }
     }
+    dlam.add(dl);
     __syncwarp();
     // queries after every key of the warp, and before them the (at most 8) mixed ones
     const int first = k0 + warp * kWarpRows + 1 - q0;  // the first query any key takes
@@ -465,9 +485,10 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
     axpys<D, false>(Pw, Qs, ty, tx, full, kTile, dk, use);
   }
   // the CTA's dlambda partial
+  double lsum = (double)dlam.s + (double)dlam.c;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) dlam += __shfl_xor_sync(0xffffffffu, dlam, o);
-  if (lane == 0) red[warp] = dlam;
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+  if (lane == 0) red[warp] = (float)lsum;
   __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
