@@ -65,6 +65,8 @@ _lib = None
 def load(path: str | None = None):
     """Load librelation.so (default: the in-tree build) and declare its signatures."""
     global _lib
+    if path is None and _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -146,37 +148,40 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 def shape_of(t: torch.Tensor) -> Shape:
     """relation_shape of a [B, T, H, d_h] tensor with d_h contiguous."""
-    if t.dim() != 4:
+    st = t.stride()
+    if len(st) != 4:
         raise ValueError("expected a [B, T, H, d_h] tensor")
-    if t.stride(3) != 1:
+    if st[3] != 1:
         raise ValueError("d_h must be contiguous")
-    B, T, H, d = t.shape
-    return Shape(B, T, H, d, t.stride(0), t.stride(1), t.stride(2))
+    return Shape(*t.shape, *st[:3])
 
 
 def _same_layout(ref: torch.Tensor, *others: torch.Tensor):
+    shape, stride, dtype, device = ref.shape, ref.stride(), ref.dtype, ref.device
     for o in others:
-        if o.shape != ref.shape or o.stride() != ref.stride() or o.dtype != ref.dtype:
+        if o.shape != shape or o.stride() != stride or o.dtype != dtype:
             raise ValueError("all tensors of a call need the same shape, strides and dtype")
-        if not o.is_cuda or o.device != ref.device:
+        if not o.is_cuda or o.device != device:
             raise ValueError("all tensors must live on the same CUDA device")
 
 
 def _like(t: torch.Tensor) -> torch.Tensor:
     """An output with t's shape, dtype, device and strides.  The C ABI writes an output
     with its input's element strides, which torch.empty_like does not keep for a view that
-    is not dense (e.g. a slice of a padded tensor)."""
+    is not dense (e.g. a slice of a padded tensor); for a contiguous one it does."""
+    if type(t) is torch.Tensor and t.is_contiguous():
+        return torch.empty_like(t)
     return torch.empty_strided(t.size(), t.stride(), dtype=t.dtype, device=t.device)
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+    if stream is None:  # (torch.cuda.current_stream().cuda_stream without the Stream object)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def workspace_size(q: torch.Tensor) -> int:
@@ -190,12 +195,13 @@ def fwd(q, k, v, lam: float, tau_s: float = 2.0, *, kernel: str = "auto", out=No
     B, T, H, _ = q.shape
     if out is None:
         out = _like(q)
-    _same_layout(q, out)
+    else:
+        _same_layout(q, out)
     if logz is None:
         logz = torch.empty((B, H, T), device=q.device, dtype=torch.float32)
     rc = load().relation_fwd_ex(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(logz), float(lam),
                                 float(tau_s), shape_of(q), _dtype_code(q), KERNELS[kernel],
-                                _ptr(dev_status), ctypes.c_void_p(_stream(stream)))
+                                _ptr(dev_status), _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_fwd")
     return out, logz
@@ -209,7 +215,8 @@ def fwd_flow(q, k, v, lam: float, tau_s: float = 2.0, *, kernel: str = "auto", o
     B, T, H, _ = q.shape
     if out is None:
         out = _like(q)
-    _same_layout(q, out)
+    else:
+        _same_layout(q, out)
     if logz is None:
         logz = torch.empty((B, H, T), device=q.device, dtype=torch.float32)
     if self_flow is None:
@@ -217,7 +224,7 @@ def fwd_flow(q, k, v, lam: float, tau_s: float = 2.0, *, kernel: str = "auto", o
     rc = load().relation_fwd_flow(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(logz),
                                   _ptr(self_flow), float(lam), float(tau_s), shape_of(q),
                                   _dtype_code(q), KERNELS[kernel], _ptr(dev_status),
-                                  ctypes.c_void_p(_stream(stream)))
+                                  _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_fwd_flow")
     return out, logz, self_flow
@@ -232,12 +239,14 @@ def linear_fwd(p1, p2, v, alpha, tau_s: float = 2.0, *, kernel: str = "auto", ou
     if alpha.dtype != torch.float32 or tuple(alpha.shape) != tuple(p1.shape) or \
             tuple(alpha.stride()) != tuple(p1.stride()):
         raise ValueError("alpha must be fp32 with p1's shape and strides")
-    out = _like(p1) if out is None else out
-    _same_layout(p1, out)
+    if out is None:
+        out = _like(p1)
+    else:
+        _same_layout(p1, out)
     rc = load().relation_linear_fwd_ex(_ptr(p1), _ptr(p2), _ptr(v), _ptr(alpha), _ptr(out),
                                        float(tau_s), shape_of(p1), _dtype_code(p1),
                                        KERNELS[kernel], _ptr(dev_status),
-                                       ctypes.c_void_p(_stream(stream)))
+                                       _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_linear_fwd_ex")
     return out
@@ -269,7 +278,7 @@ def fwd_state(q, k, v, causal: bool, *, out=None, dev_status=None, stream=None):
     _check_summary(out, B, H, Tq, d, q.device)
     rc = load().relation_fwd_state(_ptr(q), _ptr(k), _ptr(v), _ptr(m), _ptr(l), _ptr(z),
                                    shape_of(q), shape_of(k), int(bool(causal)), _dtype_code(q),
-                                   _ptr(dev_status), ctypes.c_void_p(_stream(stream)))
+                                   _ptr(dev_status), _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_fwd_state")
     return m, l, z
@@ -285,7 +294,7 @@ def state_merge(state, other, *, stream=None):
     _check_summary(other, B, H, T, d, z.device)
     rc = load().relation_state_merge(_ptr(m), _ptr(l), _ptr(z), _ptr(m2), _ptr(l2), _ptr(z2),
                                      Shape(B, T, H, d, T * H * d, H * d, d),
-                                     ctypes.c_void_p(_stream(stream)))
+                                     _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_state_merge")
     return state
@@ -298,8 +307,10 @@ def state_finish(q, k, v, state, lam: float, tau_s: float = 2.0, pos0: int = 0, 
     _same_layout(q, k, v)
     m, l, z = state
     B, T, H, d = q.shape
-    out = _like(q) if out is None else out
-    _same_layout(q, out)
+    if out is None:
+        out = _like(q)
+    else:
+        _same_layout(q, out)
     logz = torch.empty((B, H, T), dtype=torch.float32, device=q.device) if logz is None else logz
     _check_summary(state, B, H, T, d, q.device)
     if tuple(logz.shape) != (B, H, T) or logz.dtype != torch.float32 or not logz.is_contiguous():
@@ -307,7 +318,7 @@ def state_finish(q, k, v, state, lam: float, tau_s: float = 2.0, pos0: int = 0, 
     rc = load().relation_state_finish(_ptr(q), _ptr(k), _ptr(v), _ptr(m), _ptr(l), _ptr(z),
                                       _ptr(out), _ptr(logz), _ptr(self_flow), float(lam),
                                       float(tau_s), int(pos0), shape_of(q), _dtype_code(q),
-                                      ctypes.c_void_p(_stream(stream)))
+                                      _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_state_finish")
     return out, logz
@@ -326,15 +337,16 @@ def linear_fwd_ws(p1, p2, v, alpha, tau_s: float = 2.0, *, workspace=None, out=N
     if alpha.dtype != torch.float32 or tuple(alpha.shape) != tuple(p1.shape) or \
             tuple(alpha.stride()) != tuple(p1.stride()):
         raise ValueError("alpha must be fp32 with p1's shape and strides")
-    out = _like(p1) if out is None else out
-    _same_layout(p1, out)
-    need = linear_fwd_workspace_size(p1)
+    if out is None:
+        out = _like(p1)
+    else:
+        _same_layout(p1, out)
     if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=p1.device)
+        workspace = torch.empty(max(linear_fwd_workspace_size(p1), 16), dtype=torch.uint8, device=p1.device)
     rc = load().relation_linear_fwd_ws(_ptr(p1), _ptr(p2), _ptr(v), _ptr(alpha), _ptr(out),
                                        float(tau_s), shape_of(p1), _dtype_code(p1),
                                        _ptr(workspace), workspace.numel(), _ptr(dev_status),
-                                       ctypes.c_void_p(_stream(stream)))
+                                       _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_linear_fwd_ws")
     return out
@@ -358,15 +370,15 @@ def linear_bwd(p1, p2, v, alpha, dy, tau_s: float = 2.0, *, kernel: str = "auto"
         raise ValueError("alpha must be fp32 with p1's shape and strides")
     dp1, dp2, dv = _like(p1), _like(p1), _like(p1)
     dalpha = _like(alpha)
-    need = linear_bwd_workspace_size(p1, kernel)
     if workspace is None:
-        workspace = torch.empty(max(need, 16), device=p1.device, dtype=torch.uint8)
+        workspace = torch.empty(max(linear_bwd_workspace_size(p1, kernel), 16), device=p1.device,
+                                dtype=torch.uint8)
     rc = load().relation_linear_bwd_ex(_ptr(p1), _ptr(p2), _ptr(v), _ptr(alpha), _ptr(dy),
                                        _ptr(dp1), _ptr(dp2), _ptr(dv), _ptr(dalpha),
                                        float(tau_s), shape_of(p1), _dtype_code(p1),
                                        KERNELS[kernel], _ptr(workspace),
                                        workspace.numel() * workspace.element_size(),
-                                       _ptr(dev_status), ctypes.c_void_p(_stream(stream)))
+                                       _ptr(dev_status), _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_linear_bwd_ex")
     return dp1, dp2, dv, dalpha
@@ -386,12 +398,14 @@ def layer_prep(p1, p2, info, theta, pairing: int = 0, rope_base: float = 1.0e4, 
     RoPE(p2), Givens(info)) for [B, T, H, d] inputs of one layout, theta fp32 [H/2]."""
     _same_layout(p1, p2, info)
     theta, pairing, rope_base = _layer_args(theta, pairing, rope_base, p1)
-    q, k, v = out if out is not None else (_like(p1), _like(p1),
-                                           _like(p1))
-    _same_layout(p1, q, k, v)
+    if out is None:
+        q, k, v = _like(p1), _like(p1), _like(p1)
+    else:
+        q, k, v = out
+        _same_layout(p1, q, k, v)
     rc = load().relation_layer_prep(_ptr(p1), _ptr(p2), _ptr(info), _ptr(theta), pairing,
                                     rope_base, _ptr(q), _ptr(k), _ptr(v), shape_of(p1),
-                                    _dtype_code(p1), ctypes.c_void_p(_stream(stream)))
+                                    _dtype_code(p1), _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_layer_prep")
     return q, k, v
@@ -409,14 +423,14 @@ def layer_grad(dq, dk, dv, info, theta, pairing: int = 0, rope_base: float = 1.0
     theta, pairing, rope_base = _layer_args(theta, pairing, rope_base, dq)
     dp1, dp2, dinfo = _like(dq), _like(dq), _like(dq)
     dtheta = _like(theta)
-    need = layer_grad_workspace_size(dq)
     if workspace is None:
-        workspace = torch.empty(max(need, 16), device=dq.device, dtype=torch.uint8)
+        workspace = torch.empty(max(layer_grad_workspace_size(dq), 16), device=dq.device,
+                                dtype=torch.uint8)
     rc = load().relation_layer_grad(_ptr(dq), _ptr(dk), _ptr(dv), _ptr(info), _ptr(theta),
                                     pairing, rope_base, _ptr(dp1), _ptr(dp2), _ptr(dinfo),
                                     _ptr(dtheta), shape_of(dq), _dtype_code(dq), _ptr(workspace),
                                     workspace.numel() * workspace.element_size(),
-                                    ctypes.c_void_p(_stream(stream)))
+                                    _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_layer_grad")
     return dp1, dp2, dinfo, dtheta
@@ -439,18 +453,17 @@ def decode(q, k_cache, v_cache, lengths, lam: float, tau_s: float = 2.0, *, out=
     if lengths.dtype != torch.int32 or lengths.numel() != B or not lengths.is_contiguous():
         raise ValueError("lengths must be a contiguous int32 tensor of B entries")
     out = _like(q) if out is None else out
-    if tuple(out.stride()) != tuple(q.stride()):
+    if out.stride() != q.stride():
         raise ValueError("out must have q's layout")
     if logz is None:
         logz = torch.empty((B, H), device=q.device, dtype=torch.float32)
-    need = decode_workspace_size(k_cache)
     if workspace is None:
-        workspace = torch.empty(need, device=q.device, dtype=torch.uint8)
+        workspace = torch.empty(decode_workspace_size(k_cache), device=q.device, dtype=torch.uint8)
     rc = load().relation_decode(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(lengths), _ptr(out),
                                 _ptr(logz), float(lam), float(tau_s), shape_of(k_cache),
                                 q.stride(0), q.stride(1), _dtype_code(q), _ptr(workspace),
                                 workspace.numel() * workspace.element_size(), _ptr(dev_status),
-                                ctypes.c_void_p(_stream(stream)))
+                                _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_decode")
     return out, logz
@@ -465,21 +478,22 @@ def bwd(q, k, v, o, dout, logz, lam: float, tau_s: float = 2.0, *, kernel: str =
     """Backward.  Returns (dQ, dK, dV, dlambda) with dlambda a 1-element fp32 device tensor.
     ``stages`` selects a subset of the three backward stages (see relation_bwd_stages)."""
     _same_layout(q, k, v, o, dout)
+    given = [t for t in (dq, dk, dv) if t is not None]
+    if given:
+        _same_layout(q, *given)
     dq = _like(q) if dq is None else dq
     dk = _like(q) if dk is None else dk
     dv = _like(q) if dv is None else dv
-    _same_layout(q, dq, dk, dv)
     if dlambda is None:
         dlambda = torch.empty(1, device=q.device, dtype=torch.float32)
-    need = workspace_size(q)
     if workspace is None:
-        workspace = torch.empty(need, device=q.device, dtype=torch.uint8)
+        workspace = torch.empty(workspace_size(q), device=q.device, dtype=torch.uint8)
     rc = load().relation_bwd_stages(_ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(dout), _ptr(logz),
                                     _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dlambda), float(lam),
                                     float(tau_s), shape_of(q), _dtype_code(q),
                                     _ptr(workspace), workspace.numel() * workspace.element_size(),
                                     KERNELS[kernel], int(stages), _ptr(dev_status),
-                                    ctypes.c_void_p(_stream(stream)))
+                                    _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_bwd")
     return dq, dk, dv, dlambda
@@ -503,7 +517,7 @@ def bwd_no_alloc(q, k, v, o, dout, logz, lam: float, tau_s: float = 2.0, *,
     rc = load().relation_bwd_static(_ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(dout), _ptr(logz),
                                     _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dlambda), float(lam),
                                     float(tau_s), shape_of(q), _dtype_code(q), KERNELS[kernel],
-                                    _ptr(dev_status), ctypes.c_void_p(_stream(stream)))
+                                    _ptr(dev_status), _stream(stream))
     if rc != OK:
         raise RelationError(rc, "relation_bwd_static")
     return dq, dk, dv, dlambda
@@ -512,7 +526,7 @@ def bwd_no_alloc(q, k, v, o, dout, logz, lam: float, tau_s: float = 2.0, *,
 def selftest_wait_timeout(dev_status: torch.Tensor, timeout_us: int = 1000, stream=None) -> int:
     """Launch the bounded-wait self-test; returns the launch status."""
     return int(load().relation_selftest_wait_timeout(_ptr(dev_status), int(timeout_us),
-                                                     ctypes.c_void_p(_stream(stream))))
+                                                     _stream(stream)))
 
 
 class RelationFunction(torch.autograd.Function):
