@@ -26,10 +26,14 @@
 // bounds it but the latency of those phases, so their work is spread over as many warps as
 // the SM holds: four groups on the sequential walk (one CTA per SM, its next block's loads
 // in flight), two on the one-block modes at d_h = 64, which leave room for a second CTA per SM
-// whose phases fill this one's waits.  With one group (one CTA per SM) the sequential walk took
-// 126 us at B 8, H 12, T 2048, d 64; four groups 93; with the logarithms on every warp, the next
-// block's sums taken while the output product runs and the stores on the TMA warp 82.  At B 1,
-// H 12, T 32768 DELTA, the scan and OUT took 140, 27 and 177 us, now 78, 16 and 95.
+// whose phases fill this one's waits.  The one-block modes' CTAs are as many as fit and take
+// blocks in steps of the grid; every part of the next block's inputs is loaded as soon as its
+// place is free (a CTA per block, with its launch and its loads exposed, took 1.1 to 1.2 times as
+// long).  With one group (one CTA per SM) the sequential walk took 126 us at B 8, H 12, T 2048,
+// d 64; four groups 93; with the logarithms on every warp, the next block's sums taken while the
+// output product runs and the stores on the TMA warp 82; with one instruction per logarithm and
+// no test per element for the clamp and the mask 76.  At B 1, H 12, T 32768 DELTA, the scan and
+// OUT took 140, 27 and 177 us, now 64, 16 and 72 (half of the issue slots in OUT).
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps
 // meeting the warpgroups' barriers and skips the work between them.
 #include <cudaTypedefs.h>
@@ -75,8 +79,10 @@ struct Cfg {
   static constexpr int SCB = 5 * LT * 4;
   static constexpr int OFF_BAR = IN_C0 ? OFF_C0 + C0T : OFF_SC + (AHEAD ? 2 : 1) * SCB;
   static constexpr int SMEM = OFF_BAR + 128 + 1024;
-  static constexpr uint32_t LOAD_BYTES =
-      2 * PT + VT + AT + (MODE == MODE_OUT ? C0T : 0) + (MODE == MODE_BOTH ? VT : 0);
+  // p1, p2, alpha; and I~ (dY, the state), which the one-block modes await on their own
+  static constexpr uint32_t LOAD_PA = 2 * PT + AT;
+  static constexpr uint32_t LOAD_V =
+      VT + (MODE == MODE_OUT ? C0T : 0) + (MODE == MODE_BOTH ? VT : 0);
   // TMEM columns: S 128 | E 64 | P 64 (S masked, bf16) | C 64; DELTA: C 64 (BOTH: 128) alone
   static constexpr int COL_S = 0, COL_E = 128, COL_P = 192, COL_C = DELTA ? 0 : 256;
   static constexpr int TMEM = SEQ ? 512 : (DELTA ? 128 : 256);
@@ -116,13 +122,24 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NSPLIT = D / NC;
   const int nb = (p.T + LT - 1) / LT;
-  // SEQ: one CTA per (head, split) over blocks [0, nb); DELTA / BOTH / OUT: one block per CTA
-  const int cta_blk = SEQ ? 0 : (int)(blockIdx.x % nb);
-  const int bhs = SEQ ? (int)blockIdx.x : (int)(blockIdx.x / nb);
-  const int split = bhs % NSPLIT;
-  const int bh = bhs / NSPLIT;
-  const int b = bh / p.H, h = bh % p.H;
-  const int blk_first = cta_blk, blk_end = SEQ ? nb : cta_blk + 1;
+  // SEQ: one CTA per (head, split) over its blocks; DELTA / BOTH / OUT: any block, in steps of
+  // the grid
+  const int n_it =
+      SEQ ? nb : (p.B * p.H * NSPLIT * nb - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+  struct Where {
+    int blk, bhs, split, h, b;
+  };
+  auto where = [&](int it) -> Where {
+    const int item = (int)(blockIdx.x + it * gridDim.x);
+    Where w;
+    w.bhs = SEQ ? (int)blockIdx.x : item / nb;
+    w.blk = SEQ ? it : item - w.bhs * nb;
+    const int bh = w.bhs / NSPLIT;
+    w.split = w.bhs - bh * NSPLIT;
+    w.b = bh / p.H;
+    w.h = bh - w.b * p.H;
+    return w;
+  };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NBAR; ++i)  // arrivals of the elementwise threads, or one
@@ -142,49 +159,103 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   if (warp == C::W_TMA) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      // Y of block it (staged in its p1 tile) by TMA, once every elementwise thread has
-      // written its part and read the stage's I~
-      auto store_y = [&](int it) -> bool {
+      // Y of block it (staged in its p1 tile; OUT: in Qs) by TMA, once every elementwise
+      // thread has written its part and read the stage's I~
+      auto put_y = [&](int it) {
         const int st = it % C::STAGES;
-        if (!mbar_wait(bar(B_EPI + st), (it / C::STAGES) & 1, ab)) return false;
-        for (int q = 0; q < LT && (blk_first + it) * LT + q < p.T; q += 32)
-          tma_store_4d(&tmY, sb + st * C::STAGE + C::OFF_P1 + q * 128, split * NC,
-                       (blk_first + it) * LT + q, h, b);
+        const Where w = where(it);
+        for (int q = 0; q < LT && w.blk * LT + q < p.T; q += 32)
+          tma_store_4d(&tmY, sb + (SEQ ? st * C::STAGE + C::OFF_P1 : C::OFF_QS) + q * 128,
+                       w.split * NC, w.blk * LT + q, w.h, w.b);
         tma_store_commit();
+      };
+      auto store_y = [&](int it) -> bool {
+        if (!mbar_wait(bar(B_EPI + it % C::STAGES), (it / C::STAGES) & 1, ab)) return false;
+        put_y(it);
         tma_store_wait_read_all();  // before the stage is loaded again (or the CTA exits)
         return true;
       };
-      const int n_it = blk_end - blk_first;
+      // the parts of block it's inputs, to stage base sg on barrier lb
+      auto load_p = [&](const Where& w, uint32_t sg, uint32_t lb) {
+        for (int kb = 0; kb < C::KB; ++kb) {
+          tma_load_4d(sg + C::OFF_P1 + kb * LT * 128, &tmP1, lb, kb * 64, w.blk * LT, w.h, w.b);
+          tma_load_4d(sg + C::OFF_P2 + kb * LT * 128, &tmP2, lb, kb * 64, w.blk * LT, w.h, w.b);
+        }
+      };
+      auto load_a = [&](const Where& w, uint32_t sg, uint32_t lb) {
+        for (int k = 0; k < D / 32; ++k)
+          tma_load_4d(sg + C::OFF_A + k * LT * 128, &tmA, lb, k * 32, w.blk * LT, w.h, w.b);
+      };
+      auto load_v = [&](const Where& w, uint32_t sg, uint32_t lb) {
+        tma_load_4d(sg + C::OFF_V, &tmV, lb, w.split * NC, w.blk * LT, w.h, w.b);
+        if (BOTH) tma_load_4d(sg + C::OFF_G, &tmG, lb, w.split * NC, w.blk * LT, w.h, w.b);
+        if (MODE == MODE_OUT)  // the state the block starts from, in the MN-major B layout
+          tma_load_2d(sb + C::OFF_C0, &tmC0, lb, 0, (w.bhs * nb + w.blk) * D);
+      };
       int issued = 0;
       bool ok = true;
-      for (int blk = blk_first; blk < blk_end; ++blk) {
-        const int it = blk - blk_first;
-        const int st = it % C::STAGES, use = it / C::STAGES;
-        // the stage's previous block: its MMAs are done and its output is stored
-        if (use > 0 && (!(ok = store_y(it - C::STAGES)) ||
-                        !(ok = mbar_wait(bar(B_FREE + st), (use - 1) & 1, ab))))
-          break;
-        const int t0 = blk * LT;
-        const uint32_t sg = sb + st * C::STAGE;
-        const uint32_t lb = bar(B_LOAD + st);
-        mbar_arrive_expect_tx(lb, C::LOAD_BYTES);
-        for (int kb = 0; kb < C::KB; ++kb) {
-          tma_load_4d(sg + C::OFF_P1 + kb * LT * 128, &tmP1, lb, kb * 64, t0, h, b);
-          tma_load_4d(sg + C::OFF_P2 + kb * LT * 128, &tmP2, lb, kb * 64, t0, h, b);
+      if constexpr (SEQ) {
+        for (int it = 0; it < n_it; ++it) {
+          const int st = it % C::STAGES, use = it / C::STAGES;
+          // the stage's previous block: its MMAs are done and its output is stored
+          if (use > 0 && (!(ok = store_y(it - C::STAGES)) ||
+                          !(ok = mbar_wait(bar(B_FREE + st), (use - 1) & 1, ab))))
+            break;
+          const Where w = where(it);
+          const uint32_t sg = sb + st * C::STAGE, lb = bar(B_LOAD + st);
+          mbar_arrive_expect_tx(lb, C::LOAD_PA + C::LOAD_V);
+          load_p(w, sg, lb);
+          load_a(w, sg, lb);
+          load_v(w, sg, lb);
+          issued = it + 1;
         }
-        for (int k = 0; k < D / 32; ++k)
-          tma_load_4d(sg + C::OFF_A + k * LT * 128, &tmA, lb, k * 32, t0, h, b);
-        tma_load_4d(sg + C::OFF_V, &tmV, lb, split * NC, t0, h, b);
-        if (BOTH) tma_load_4d(sg + C::OFF_G, &tmG, lb, split * NC, t0, h, b);
-        if (MODE == MODE_OUT)  // the state the block starts from, in the MN-major B layout
-          tma_load_2d(sb + C::OFF_C0, &tmC0, lb, 0, (bhs * nb + blk) * D);
-        issued = it + 1;
-      }
-      if (!DELTA)
         for (int it = max(0, n_it - C::STAGES); ok && it < n_it; ++it) ok = store_y(it);
-      if (ab.raised())  // copies in flight land before the CTA releases its shared memory
-        for (int it = issued - C::STAGES > 0 ? issued - C::STAGES : 0; it < issued; ++it)
-          drain_wait(bar(B_LOAD + it % C::STAGES), (it / C::STAGES) & 1);
+        if (ab.raised())  // copies in flight land before the CTA releases its shared memory
+          for (int it = issued - C::STAGES > 0 ? issued - C::STAGES : 0; it < issued; ++it)
+            drain_wait(bar(B_LOAD + it % C::STAGES), (it / C::STAGES) & 1);
+      } else {
+        // One stage, whose parts are loaded for the next block as this one lets go of them:
+        // alpha when the operands are made, p1 and p2 when their product is done (DELTA, BOTH:
+        // with I~ and dY, when the state product is), I~ and the state after the epilogue
+        const uint32_t lb = bar(B_LOAD), lv = bar(B_LOADV);
+        mbar_arrive_expect_tx(lb, C::LOAD_PA);
+        load_p(where(0), sb, lb);
+        load_a(where(0), sb, lb);
+        mbar_arrive_expect_tx(lv, C::LOAD_V);
+        load_v(where(0), sb, lv);
+        issued = 1;
+        for (int it = 0; ok && it < n_it; ++it) {
+          const bool more = it + 1 < n_it;
+          const Where nx = where(more ? it + 1 : it);
+          const uint32_t ph = it & 1;
+          if (more) {
+            if (!(ok = mbar_wait(bar(B_OPS), ph, ab))) break;
+            mbar_arrive_expect_tx(lb, C::LOAD_PA);
+            load_a(nx, sb, lb);
+            issued = it + 2;
+            if (!(ok = mbar_wait(bar(DELTA ? B_STATE : B_S), ph, ab))) break;
+            load_p(nx, sb, lb);
+            if (DELTA) {
+              mbar_arrive_expect_tx(lv, C::LOAD_V);
+              load_v(nx, sb, lv);
+            }
+          }
+          if (!DELTA) {
+            if (!(ok = mbar_wait(bar(B_EPI), ph, ab))) break;
+            put_y(it);
+            if (more) {
+              mbar_arrive_expect_tx(lv, C::LOAD_V);
+              load_v(nx, sb, lv);
+            }
+            tma_store_wait_read_all();
+            mbar_arrive(bar(B_QFREE));  // Qs may be written again
+          }
+        }
+        if (ab.raised()) {  // copies in flight land before the CTA exits
+          drain_wait(bar(B_LOAD), (issued - 1) & 1);
+          drain_wait(bar(B_LOADV), (issued - 1) & 1);
+        }
+      }
     }
   } else if (warp == C::W_MMA) {
     // ------------------------------------------------------------------ MMA issuer
@@ -192,8 +263,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     constexpr uint32_t id_e = idesc_bf16_f32(128, NC, false, true);
     constexpr uint32_t id_c = idesc_bf16_f32(128, BOTH ? 2 * NC : NC, true, true);
     bool ok = true;
-    for (int blk = blk_first; ok && blk < blk_end; ++blk) {
-      const int it = blk - blk_first;
+    for (int it = 0; ok && it < n_it; ++it) {
       const uint32_t ph = it & 1;
       const int st = it % C::STAGES;
       const uint32_t sg = sb + st * C::STAGE;
@@ -207,10 +277,8 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
                    smem_desc_sw128(sg + C::OFF_P2 + koff, 16, 1024), id_s, kk > 0 ? 1u : 0u);
         }
         mma_commit_w(bar(B_S));
-        if (SEQ) {  // (OUT: C0 came with the block's inputs)
-          if (!(ok = mbar_wait_warp(bar(B_C0), ph, ab))) break;
-          tc_fence_after();
-        }
+        if (!(ok = mbar_wait_warp(bar(SEQ ? B_C0 : B_LOADV), ph, ab))) break;
+        tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {  // E = Qs C_0
           const uint32_t koff = (kk >> 2) * (LT * 128) + (kk & 3) * 32;
@@ -226,6 +294,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
                    smem_desc_sw128(sg + C::OFF_V + kk * 16 * 128, LT * 128, 1024), id_e, 1u);
         mma_commit_w(bar(B_E));
       }
+      if (DELTA && !(ok = mbar_wait_warp(bar(B_LOADV), ph, ab))) break;
       if (MODE != MODE_OUT) {
         // SEQ: C += KL^T I~ (C decayed by the threads); DELTA: the block's own sum; BOTH:
         // [KL | Qs]^T [I~ | dY], whose diagonal quarters are the two contributions
@@ -234,14 +303,14 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
           mma_ss_w(tmem + C::COL_C,
                    smem_desc_sw128(sb + C::OFF_KL + kk * 16 * 128, LT * 128, 1024),
                    smem_desc_sw128(sg + C::OFF_V + kk * 16 * 128, LT * 128, 1024), id_c,
-                   ((SEQ && blk > 0) || kk > 0) ? 1u : 0u);
+                   ((SEQ && it > 0) || kk > 0) ? 1u : 0u);
         mma_commit_w(bar(B_STATE));
       }
       if (SEQ) mma_commit_w(bar(B_FREE + st));
     }
     // SEQ: the last commits land before the CTA exits (EW warps have waited for the others)
     if (SEQ && ok)
-      for (int it = max(0, nb - C::STAGES); it < nb; ++it)
+      for (int it = max(0, n_it - C::STAGES); it < n_it; ++it)
         mbar_wait_warp(bar(B_FREE + it % C::STAGES), (it / C::STAGES) & 1, ab);
     __syncwarp();
   } else {
@@ -267,25 +336,31 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     // on the same four warps they took 3900 cycles of a block's 10600.  Visible after the
     // warpgroups' next barrier.
     auto sums = [&](int it) {
-      const int t0 = (blk_first + it) * LT, st = it % C::STAGES;
+      const int t0 = where(it).blk * LT, st = it % C::STAGES;
       uint8_t* const sg = smem + st * C::STAGE;
       float* const al = reinterpret_cast<float*>(sg + C::OFF_A);
       float* const s_dot = scalars(it);
       float* const l_a = s_dot + 3 * LT;
       float* const l_b = l_a + LT;
       ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_LOAD + st), (it / C::STAGES) & 1, ab));
-      if (ok) {
+      auto logs = [&](bool full) {
 #pragma unroll
         for (int i0 = 0; i0 < LT * D / 4; i0 += C::EW) {
           const int i = i0 + threadIdx.x;  // 16-byte group of the tile, of token (i / 8) % 128
-          const bool live = t0 + ((i >> 3) & 127) < p.T;
+          const bool live = full || t0 + ((i >> 3) & 127) < p.T;
           float4 v = reinterpret_cast<float4*>(al)[i];
-          v.x = live ? __log2f(v.x) : 0.f;
-          v.y = live ? __log2f(v.y) : 0.f;
-          v.z = live ? __log2f(v.z) : 0.f;
-          v.w = live ? __log2f(v.w) : 0.f;
+          v.x = live ? log2_alpha(v.x) : 0.f;
+          v.y = live ? log2_alpha(v.y) : 0.f;
+          v.z = live ? log2_alpha(v.z) : 0.f;
+          v.w = live ? log2_alpha(v.w) : 0.f;
           reinterpret_cast<float4*>(al)[i] = v;
         }
+      };
+      if (ok) {
+        if (t0 + LT <= p.T)
+          logs(true);
+        else
+          logs(false);
       }
       ew_sync<NG>();
       if (!ok) return;
@@ -312,10 +387,10 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
       }
     };
     if (C::AHEAD) sums(0);
-    for (int blk = blk_first; blk < blk_end; ++blk) {
-      const int it = blk - blk_first;
+    for (int it = 0; it < n_it; ++it) {
       const uint32_t ph = it & 1;
-      const int t0 = blk * LT;
+      const Where w = where(it);
+      const int t0 = w.blk * LT;
       const int st = it % C::STAGES;
       uint8_t* const sg = smem + st * C::STAGE;
       uint8_t* const p1s = sg + C::OFF_P1;
@@ -336,14 +411,17 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         if (t < D) l_end = D == 64 ? l_a[c] + l_b[c] : l_b[c];
         // Qs, KL and the state are single buffers: the last block's state product (the last
         // reader of KL; Qs's reader precedes B_E) must be done before they are written
-        if (SEQ && blk > 0) {
-          ok = __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), (blk - 1) & 1, ab));
+        if (SEQ && it > 0) {
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), (it - 1) & 1, ab));
           tc_fence_after();
         }
+        if (MODE == MODE_OUT && it > 0)  // Qs: the last block's Y has left it
+          ok = __all_sync(0xffffffffu, mbar_wait(bar(B_QFREE), (it - 1) & 1, ab));
       }
       if (ok) {
         // ---- the operands of token t over the group's channels, 8 per 16-byte access: Qm
         // and Km in place of p1 and p2, Qs, KL (DELTA: KL in place of p2; BOTH: and Qs of p1)
+        const float later = D == 64 && t >= 64 ? 1.f : 0.f;
         float s1 = 0.f, s2 = 0.f;  // rows past T give zero operands
         if (t0 + t < p.T) {
           const float S = 1.0f / (1.0f + __expf(-s_dot[t] * inv_tau_sqrt_d));
@@ -369,6 +447,15 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
           const float Ev[8] = {E0.x, E0.y, E0.z, E0.w, E1.x, E1.y, E1.z, E1.w};
           const uint32_t aw[4] = {a4.x, a4.y, a4.z, a4.w}, bw[4] = {b4.x, b4.y, b4.z, b4.w};
           uint32_t qm[4], km[4], qs[4], kl[4];
+          // L_t (the second half's sums (d_h = 64) are relative to the half's start) and log2 of
+          // a_t / a_m
+          float Lt[8], dm[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            Lt[i] = D == 64 ? fmaf(Mv[i], later, Lv[i]) : Lv[i];
+            dm[i] = Lt[i] - Mv[i];
+          }
+          if (!DELTA) clamp_exponents(dm, my_clamp);
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[e]));
@@ -377,17 +464,11 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
               const int ch = 2 * e + u;
-              // the second half's sums (d_h = 64) are relative to the half's start
-              const float L = Lv[ch] + ((D == 64 && t >= 64) ? Mv[ch] : 0.f);
+              const float L = Lt[ch];
               const float xv = u ? x.y : x.x, yv = u ? y.y : y.x;
               if (!DELTA) {
-                float dm = L - Mv[ch];  // log2 of a_t / a_m
-                if (fabsf(dm) > kClampLog2) {
-                  dm = copysignf(kClampLog2, dm);
-                  my_clamp = true;
-                }
-                r[u][0] = xv * s1 * ex2_approx(dm);      // Qm
-                r[u][1] = yv * s2 * ex2_approx(-dm);     // Km
+                r[u][0] = xv * s1 * ex2_approx(dm[ch]);   // Qm
+                r[u][1] = yv * s2 * ex2_approx(-dm[ch]);  // Km
               }
               if (!DELTA || BOTH) r[u][2] = xv * s1 * ex2_approx(L);  // Qs (factor <= 1)
               if (MODE != MODE_OUT) {  // KL (factor <= 1)
@@ -419,7 +500,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
       if (C::IN_C0) ew_sync<NG>();  // the scalars have been read: C0 takes their place
       if (DELTA) {
         // the block's state (and adjoint) contribution and decay, to the workspace
-        ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), 0, ab));
+        ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_STATE), ph, ab));
         tc_fence_after();
         constexpr int CG = NC / NG;  // columns per group
         const bool upper = BOTH && t >= 64;  // rows of Qs^T dY, in columns 64 .. 127
@@ -431,12 +512,13 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
           else
             tmem_ld16(col, *reinterpret_cast<uint32_t(*)[16]>(z));
           tmem_ld_wait();
-          const long long row = (long long)(bhs * nb + blk) * D + (upper ? t - 64 : t);
+          const long long row = (long long)(w.bhs * nb + w.blk) * D + (upper ? t - 64 : t);
           float* dst = (upper ? cp.dQ : cp.dC) + row * 64 + grp * CG;
 #pragma unroll
           for (int k = 0; k < CG / 8; ++k) st_global_32(dst + 8 * k, z + 8 * k);
           if (grp == 0 && !upper) cp.g[row] = ex2_approx(l_end);
         }
+        tc_fence_before();  // the sums have been read: the next block's product may start
         continue;
       }
       if (SEQ && ok) {
@@ -444,7 +526,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         // decayed by a_L
         if (t < D) {  // (whole warps)
           uint32_t z[16];
-          if (blk > 0) {
+          if (it > 0) {
             tmem_ld16(trow + C::COL_C + grp * 16, z);
             tmem_ld_wait();
           } else {
@@ -462,7 +544,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
             *reinterpret_cast<uint4*>(crow + (((2 * grp + k) ^ (t & 7)) << 4)) =
                 make_uint4(w[0], w[1], w[2], w[3]);
           }
-          if (blk > 0) {
+          if (it > 0) {
             const float decay = ex2_approx(l_end);
 #pragma unroll
             for (int n = 0; n < 16; ++n) z[n] = __float_as_uint(__uint_as_float(z[n]) * decay);
@@ -486,12 +568,13 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
             uint32_t s[32];
             tmem_ld32(trow + C::COL_S + col, s);
             tmem_ld_wait();
+            if (col == (warp & 3) * 32) {  // the warp's diagonal square
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              const float lo = (col + j < t) ? __uint_as_float(s[j]) : 0.f;
-              const float hi = (col + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
-              pk[j >> 1] = pack_bf16x2(lo, hi);
+              for (int j = 0; j < 32; ++j) s[j] = col + j < t ? s[j] : 0u;
             }
+#pragma unroll
+            for (int j = 0; j < 32; j += 2)
+              pk[j >> 1] = pack_bf16x2(__uint_as_float(s[j]), __uint_as_float(s[j + 1]));
           } else {
 #pragma unroll
             for (int j = 0; j < 16; ++j) pk[j] = 0u;
@@ -502,9 +585,10 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
         tc_fence_before();
         mbar_arrive(bar(B_A));
       }
-      if (C::AHEAD && blk + 1 < blk_end) sums(it + 1);
-      // ---- Y = I~ + E, staged in p1's tile (stored by the TMA warp)
+      if (C::AHEAD && it + 1 < n_it) sums(it + 1);
+      // ---- Y = I~ + E, staged in p1's tile (OUT: in Qs; stored by the TMA warp)
       ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_E), ph, ab));
+      if (!SEQ) ok = ok && __all_sync(0xffffffffu, mbar_wait(bar(B_LOADV), ph, ab));
       if (ok) {
         tc_fence_after();
         constexpr int CG = NC / NG;
@@ -515,7 +599,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
           tmem_ld16(trow + C::COL_E + grp * CG, z);
         tmem_ld_wait();
         const uint8_t* vrow = sg + C::OFF_V + t * 128;
-        uint8_t* yrow = sg + C::OFF_P1 + t * 128;
+        uint8_t* yrow = (SEQ ? sg + C::OFF_P1 : smem + C::OFF_QS) + t * 128;
 #pragma unroll
         for (int k0 = 0; k0 < CG / 8; ++k0) {
           const int k = grp * (CG / 8) + k0;
@@ -630,6 +714,19 @@ static size_t cp_bytes(long long heads, long long nb, int d, LinCp* out, void* b
   return b_dc + b_g + b_c0;
 }
 
+// CTAs of the one-block modes: as many as are resident at once, which share the blocks evenly
+static cudaError_t block_grid(long long blocks, int per_sm, unsigned* grid) {
+  int dev = 0, nsm = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) {
+    note_failure("linear chunked: device attributes");
+    return e;
+  }
+  *grid = (unsigned)(blocks < (long long)per_sm * nsm ? blocks : (long long)per_sm * nsm);
+  return cudaSuccess;
+}
+
 template <int D, int MODE>
 static cudaError_t set_smem() {
   return cudaFuncSetAttribute(lin_tc_fwd_kernel<D, MODE>,
@@ -673,17 +770,20 @@ static cudaError_t fwd_t(const LinearProblem& lp, void* workspace, cudaStream_t 
     lin_tc_fwd_kernel<D, MODE_SEQ>
         <<<(unsigned)heads, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
   } else {
-    const long long grid = heads * nb, ctas = heads * (D / 8);
-    if (grid > 0x7fffffffLL || ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     using CD = Cfg<D, MODE_DELTA>;
     using CO = Cfg<D, MODE_OUT>;
+    const long long ctas = heads * (D / 8);
+    if (heads * nb > 0x7fffffffLL || ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    unsigned grid = 0;
+    if ((e = block_grid(heads * nb, CD::CTAS, &grid)) != cudaSuccess) return e;
+    static_assert(CD::CTAS == CO::CTAS, "one grid for both");
     lin_tc_fwd_kernel<D, MODE_DELTA>
-        <<<(unsigned)grid, CD::THREADS, CD::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
+        <<<grid, CD::THREADS, CD::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
     if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
     scan_kernel<D, false><<<(unsigned)ctas, 256, 0, s>>>(cp, (int)ctas);
     if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
     lin_tc_fwd_kernel<D, MODE_OUT>
-        <<<(unsigned)grid, CO::THREADS, CO::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
+        <<<grid, CO::THREADS, CO::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked forward: launch");
   return e;
@@ -726,12 +826,14 @@ cudaError_t launch_states(const LinearProblem& lp, const void* dy, void* workspa
     note_failure("linear chunked backward: TMA descriptors");
     return cudaErrorInvalidValue;
   }
-  const long long grid = heads * nb, ctas = heads * (D / 8);
-  if (grid > 0x7fffffffLL || 2 * ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   // (the Y and state maps are unused in this mode; m1 stands in)
   using C = Cfg<D, MODE_BOTH>;
+  const long long ctas = heads * (D / 8);
+  if (heads * nb > 0x7fffffffLL || 2 * ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  unsigned grid = 0;
+  if ((e = block_grid(heads * nb, C::CTAS, &grid)) != cudaSuccess) return e;
   lin_tc_fwd_kernel<D, MODE_BOTH>
-      <<<(unsigned)grid, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mg, ma, m1, m1, lp, cp);
+      <<<grid, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mg, ma, m1, m1, lp, cp);
   if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked backward: launch"); return e; }
   scan_kernel<D, true><<<(unsigned)(2 * ctas), 256, 0, s>>>(cp, (int)ctas);
   if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked backward: launch");

@@ -40,6 +40,8 @@ struct LinCp {
 
 // B_LOAD, B_FREE, B_EPI: one per input stage (stage s at + s)
 enum : int { B_LOAD = 0, B_FREE = 2, B_EPI = 4, B_OPS = 6, B_C0, B_S, B_A, B_E, B_STATE, NBAR };
+// the one-block modes have one stage: I~'s (and the state's) loads, and Y has left Qs
+enum : int { B_LOADV = B_LOAD + 1, B_QFREE = B_FREE };
 
 __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
   const unsigned long long t0 = globaltimer_ns();
@@ -65,6 +67,37 @@ __device__ __forceinline__ void ew_sync() {  // the elementwise warpgroups
 __device__ __forceinline__ uint32_t swz(int r, int c, int rows) {
   return (uint32_t)((c >> 6) * rows * 128 + r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4) +
                     (c & 7) * 2);
+}
+// log2 of a retention.  The flushing form takes one instruction where the other scales denormal
+// arguments; those (and 0) give -150 instead: any factor that holds one is 0 in fp32 or beyond
+// kClampLog2 with the true logarithm (below -126) as well.  NaN stays NaN.
+__device__ __forceinline__ float log2_alpha(float a) {
+  float x, y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(a));
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(x), "f"(-150.0f));
+  return y;
+}
+// The same for one exponent already reported (NaN stays NaN)
+__device__ __forceinline__ float clamp_exponent(float dm) {
+  float y;
+  asm("{\n\t.reg .f32 t;\n\tmax.NaN.f32 t, %1, %2;\n\tmin.NaN.f32 %0, t, %3;\n\t}"
+      : "=f"(y)
+      : "f"(dm), "f"(-kClampLog2), "f"(kClampLog2));
+  return y;
+}
+// Exponents of intra-block factors clamped to +-kClampLog2 (the test for all first: none is, but
+// for channels whose result is reported as not exact)
+template <int N>
+__device__ __forceinline__ void clamp_exponents(float (&dm)[N], bool& clamped) {
+  float mx = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) mx = fmaxf(mx, fabsf(dm[i]));
+  if (mx > kClampLog2) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (fabsf(dm[i]) > kClampLog2) dm[i] = copysignf(kClampLog2, dm[i]);
+    clamped = true;
+  }
 }
 // Ask Self's sums of token t over its D channels (p1, p2: 128-byte-swizzled bf16 tiles),
 // those of `which`: 1 p1 . p2, 2 |p1|^2, 4 |p2|^2.  Each is one chain of multiply-adds in

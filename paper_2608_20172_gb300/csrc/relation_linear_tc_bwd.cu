@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) a[e] = live ? __log2f(a[e]) : 0.f;
+        for (int e = 0; e < 4; ++e) a[e] = live ? log2_alpha(a[e]) : 0.f;
         reinterpret_cast<float4*>(al)[i] = make_float4(a[0], a[1], a[2], a[3]);
       }
     }
@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int n_early = n_small <= kFix ? n_small : 0;
     float* const coef = reinterpret_cast<float*>(smem + OFF_COEF);
     float S = 0.f, i1 = 0.f, i2 = 0.f, s1 = 0.f, s2 = 0.f;  // token t (zero past T)
+    const float later = t >= 64 ? 1.f : 0.f;
     uint4 ra[2], rb[2];  // p1, p2 of token t, the group's 16 channels: Qm, Km take their place
     if (ok) {
       if (t0 + t < p.T) {
@@ -405,6 +406,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float4 E4 = *reinterpret_cast<const float4*>(sum_l + 64 + 8 * k + 4 * q);
           const float Lv[4] = {L4.x, L4.y, L4.z, L4.w}, Mv[4] = {M4.x, M4.y, M4.z, M4.w};
           const float Ev[4] = {E4.x, E4.y, E4.z, E4.w};
+          float Lt[4], dm[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            Lt[j] = fmaf(Mv[j], later, Lv[j]);
+            dm[j] = Lt[j] - Mv[j];
+          }
+          clamp_exponents(dm, my_clamp);
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const float2 x = bf2(aw[2 * q + e]), y = bf2(bw[2 * q + e]);
@@ -412,12 +420,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
               const int j = 2 * e + u;
-              const float L = Lv[j] + (t >= 64 ? Mv[j] : 0.f);
-              const float dm = dm_of(Lv[j], Mv[j], t >= 64, my_clamp);
               const float xs = (u ? x.y : x.x) * s1, ys = (u ? y.y : y.x) * s2;
-              r[u][0] = xs * ex2_approx(dm);
-              r[u][1] = ys * ex2_approx(-dm);
-              r[u][2] = ys * ex2_approx((Mv[j] + Ev[j]) - L);  // KL (factor <= 1)
+              r[u][0] = xs * ex2_approx(dm[j]);
+              r[u][1] = ys * ex2_approx(-dm[j]);
+              r[u][2] = ys * ex2_approx((Mv[j] + Ev[j]) - Lt[j]);  // KL (factor <= 1)
             }
             qm[2 * q + e] = pack_bf16x2(r[0][0], r[1][0]);
             km[2 * q + e] = pack_bf16x2(r[0][1], r[1][1]);
@@ -445,12 +451,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t s[32];
         tmem_ld32(trow + COL_SC + c0, s);
         tmem_ld_wait();
+        if (grp == (warp & 3)) {  // the warp's diagonal square
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          const float lo = (c0 + j < t) ? __uint_as_float(s[j]) : 0.f;
-          const float hi = (c0 + j + 1 < t) ? __uint_as_float(s[j + 1]) : 0.f;
-          pk[j >> 1] = pack_bf16x2(lo, hi);
+          for (int j = 0; j < 32; ++j) s[j] = c0 + j < t ? s[j] : 0u;
         }
+#pragma unroll
+        for (int j = 0; j < 32; j += 2)
+          pk[j >> 1] = pack_bf16x2(__uint_as_float(s[j]), __uint_as_float(s[j + 1]));
       } else {
 #pragma unroll
         for (int j = 0; j < 16; ++j) pk[j] = 0u;
@@ -484,7 +491,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     float dq[16], dk[16];
     if (ok) {
       tc_fence_after();
-      bool unused_clamp = false;
       // dq' = 2^{L_t - L_m} X, dk' = 2^{L_m - L_t} Y (Y = dA^T Qm + Ys), the group's shares of
       // p1 . dq' and p2 . dk', dL = Qm X - Km Y and Km Ys (Qm, Km as the products read them),
       // dv = dI~ + dY (in dY's place)
@@ -523,10 +529,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int u = 0; u < 2; ++u) {
             const int i = 2 * e + u, j = 8 * k + i;
             const float pv = u ? xa.y : xa.x, kv = u ? yb.y : yb.x;
-            const float dm = dm_of(Lv[2 * e + u], Mv[2 * e + u], t >= 64, unused_clamp);
             const float qm = u ? qm2.y : qm2.x, km = u ? km2.y : km2.x;
             const float X = __uint_as_float(x[i]), Ysv = __uint_as_float(ys[i]);
             const float Y = __uint_as_float(y[i]) + Ysv;
+            const float dm = clamp_exponent(fmaf(Mv[i], later, Lv[i]) - Mv[i]);
             dq[j] = ex2_approx(dm) * X;
             dk[j] = ex2_approx(-dm) * Y;
             A1 = fmaf(pv, dq[j], A1);

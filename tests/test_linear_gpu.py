@@ -333,3 +333,40 @@ def test_linear_chunked_backward_small_retentions(n_small, T):
     ref = binding.linear_bwd(*args, kernel="simt")[3].float().cpu().numpy()
     for h in range(w.H):
         pu.check(f"dalpha head {h}", got[0, :, h], ref[0, :, h], "bf16", "grad")
+
+
+@pytest.mark.parametrize("B,T,H,d", [(3, 3000, 5, 64), (1, 2100, 5, 128)])
+def test_linear_chunk_parallel_more_blocks_than_ctas(B, T, H, d):
+    """The one-block kernels share out more blocks than CTAs fit (two per SM at d_h = 64, one at
+    128, rest not even) and the last block of a head is ragged: the workspace forward against the
+    sequential one, whose states are the same up to bf16 (the bound of two bf16 results)."""
+    g = torch.Generator().manual_seed(B + d)
+    dev = torch.device("cuda:0")
+    p1, p2, v = (torch.randn((B, T, H, d), generator=g).to(torch.bfloat16).to(dev) for _ in range(3))
+    alpha = (1.0 - 0.1 * torch.rand((B, T, H, d), generator=g)).to(dev)
+    ref = binding.linear_fwd(p1, p2, v, alpha, kernel="tcgen05")
+    got = binding.linear_fwd_ws(p1, p2, v, alpha)
+    again = binding.linear_fwd_ws(p1, p2, v, alpha)
+    torch.cuda.synchronize()
+    assert torch.equal(got, again)
+    pu.check("Y", got.double().cpu().numpy(), ref.double().cpu().numpy(), "bf16", "out")
+
+
+def test_linear_retention_below_the_normal_range():
+    """Retentions of 0 and of a denormal at a block's first token: a state that starts anew there,
+    no exponent out of range, nothing reported; the recurrence is the reference."""
+    g = torch.Generator().manual_seed(4)
+    dev = torch.device("cuda:0")
+    p1, p2, v = (torch.randn((1, 300, 2, 64), generator=g).to(torch.bfloat16).to(dev)
+                 for _ in range(3))
+    alpha = (1.0 - 0.1 * torch.rand((1, 300, 2, 64), generator=g)).to(dev)
+    alpha[0, 128, 0, :5] = 0.0
+    alpha[0, 256, 1, 7:] = 1e-40
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    ref = binding.linear_fwd(p1, p2, v, alpha, kernel="simt")
+    outs = [binding.linear_fwd(p1, p2, v, alpha, kernel="tcgen05", dev_status=status),
+            binding.linear_fwd_ws(p1, p2, v, alpha, dev_status=status)]
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    for y in outs:
+        pu.check("Y", y.double().cpu().numpy(), ref.double().cpu().numpy(), "bf16", "out")
