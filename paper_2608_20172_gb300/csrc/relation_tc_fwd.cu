@@ -38,6 +38,7 @@ namespace tc {
 
 constexpr int BM = 128;        // query rows per CTA
 constexpr int BN = 128;        // keys per K/V tile (TMA granularity)
+constexpr int kMaxSplit = 8;   // CTAs of a cluster that share a query tile
 constexpr int HN = 64;         // half a K/V tile: the register scan's step, the d_h = 64 load
 constexpr int kSCol = 0;       // U/P buffer b at kSCol + SK b
 constexpr float kRescaleLog2 = 8.0f;  // rescale z only when the max grows by > 2^8
@@ -76,7 +77,8 @@ struct FwdCfg {
   static constexpr int OFF_K = OFF_Q + TILE;
   static constexpr int OFF_V = OFF_K + STAGES * KVT;
   static constexpr int OFF_BAR = OFF_V + STAGES * KVT;
-  static constexpr int SMEM = OFF_BAR + 256 + 1024;  // barriers + 1024-byte alignment slack
+  static constexpr int OFF_ST = OFF_BAR + 256;       // SPLIT: m, l, U_ii of the rows
+  static constexpr int SMEM = OFF_ST + 3 * BM * 4 + 1024;  // + 1024-byte alignment slack
   static_assert(CTAS * (SMEM + 1024) <= 233472, "CTAs per SM");
   static_assert(OCOL + D <= TMEM_COLS, "TMEM");
 };
@@ -237,10 +239,49 @@ __device__ __forceinline__ float2 scan_p32(const uint32_t (&U)[32], int t, float
   return sum;
 }
 
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+// All threads of the cluster, their shared memory writes visible to each other
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+// 16 bytes / 4 bytes at this CTA's shared address `a` in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ uint4 ld_peer16(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_peer(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
+// SPLIT: a cluster of CTAs per query tile, each with a contiguous share of the key tiles (the
+// last with the diagonal one; a share may be empty).  Every CTA leaves its rows' (m, l, z) in
+// its own shared memory (z over the Q and K tiles, fp32) and finishes an equal share of the
+// rows from all of them through distributed shared memory.
 // MODE 0: the forward (epilogue: Y, logZ, F_ii).  MODE 1: the Exchange summary only
 // (st.m, st.l, st.z), over the queries' own earlier tokens (st.causal) or over every key
 // of k, v (st.Tk of them, all preceding the queries; the ragged last tile masked).
-template <int D, int MODE>
+template <int D, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
     fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -258,12 +299,15 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int BH = p.B * p.H;
   int tq, bh;  // heaviest query tiles first, heads in groups (common.cuh)
-  grouped_unit((int)blockIdx.x, n_qt, BH, n_groups, tq, bh);
+  const int n_cl = SPLIT ? (int)cluster_size() : 1, rank = SPLIT ? (int)cluster_rank() : 0;
+  grouped_unit((int)blockIdx.x / n_cl, n_qt, BH, n_groups, tq, bh);
   const int qt = n_qt - 1 - tq;
   const int b = bh / p.H, h = bh % p.H;
   const int q0 = qt * BM;
   const bool causal = MODE == 0 || sa.causal;
-  const int n_kv = causal ? qt + 1 : (sa.Tk + BN - 1) / BN;
+  const int n_all = causal ? qt + 1 : (sa.Tk + BN - 1) / BN;  // key tiles, and this CTA's
+  const int kv0 = SPLIT ? n_all * rank / n_cl : 0;
+  const int n_kv = SPLIT ? n_all * (rank + 1) / n_cl - kv0 : n_all;
 
   if (threadIdx.x == 0) {
     mbar_init(bar(B_Q), 1);
@@ -308,7 +352,7 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
         mbar_arrive_expect_tx(bar(B_KF + s), C::KVT);
         for (int kb = 0; kb < C::KB; ++kb)
           tma_load_4d(sb + C::OFF_K + s * C::KVT + kb * C::KVR * 128, &tmK, bar(B_KF + s),
-                      kb * 64, j * C::KVR, h, b);
+                      kb * 64, kv0 * BN + j * C::KVR, h, b);
         if (u > 0 && !mbar_wait(bar(B_VE + s), (u - 1) & 1, ab)) {
           issued = j + 1;  // K of unit j is in flight, V is not
           break;
@@ -316,7 +360,7 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
         mbar_arrive_expect_tx(bar(B_VF + s), C::KVT);
         for (int kb = 0; kb < C::KB; ++kb)
           tma_load_4d(sb + C::OFF_V + s * C::KVT + kb * C::KVR * 128, &tmV, bar(B_VF + s),
-                      kb * 64, j * C::KVR, h, b);
+                      kb * 64, kv0 * BN + j * C::KVR, h, b);
         issued = j + 1;
       }
       if (ab.raised()) {
@@ -442,8 +486,8 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
       const uint32_t ucol = trow + kSCol + bf * C::SK;
       // causal: the diagonal tile masks the keys at and after the row (tl, relative to the
       // step's first key); otherwise keys at and past Tk (a ragged last tile) are masked
-      const int tl = causal ? t - hh * C::SK : sa.Tk - j * BN - hh * C::SK;
-      const bool diag = causal ? (j == qt) : (tl < C::SK);
+      const int tl = causal ? t - hh * C::SK : sa.Tk - (kv0 + j) * BN - hh * C::SK;
+      const bool diag = causal ? (kv0 + j == qt) : (tl < C::SK);
       float umax;
       float2 rs;
       if constexpr (C::NBUF == 1 || C::SK != HN) {
@@ -526,7 +570,27 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
     // (a scale still pending at the end needs nothing: m, l and z agree)
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_O), 0, ab));
     tc_fence_after();
-    if (MODE == 1 && ok) {
+    if (SPLIT) {
+      // this CTA's (m, l, U_ii, z) of row t, 16-byte groups of z rotated within 128 bytes by the
+      // row; an empty share has m = -inf and no z
+      float* const st = reinterpret_cast<float*>(smem + C::OFF_ST);
+      st[t] = ok ? m : -INFINITY;
+      st[BM + t] = l;
+      st[2 * BM + t] = u_self;
+      if (ok && n_kv > 0) {
+#pragma unroll
+        for (int c0 = 0; c0 < D; c0 += 32) {
+          uint32_t z[32];
+          tmem_ld32(trow + C::OCOL + c0, z);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 32; c += 4)
+            *reinterpret_cast<uint4*>(smem + C::OFF_Q + t * (D * 4) +
+                                      ((((c0 + c) >> 2) ^ (t & 7)) << 4)) =
+                make_uint4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+        }
+      }
+    } else if (MODE == 1 && ok) {
       // the Exchange summary of row r: m in natural-log units, l, and z (real columns).
       // The TMEM loads are warp-collective: every lane loads, rows past T store nothing.
       const bool live = r < p.T;
@@ -612,6 +676,111 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
   }
 
   tc_fence_before();
+  if constexpr (SPLIT) {
+    __syncwarp();
+    cluster_sync_all();
+    if (threadIdx.x < BM) {
+      // row rank BM / n + (thread / n), columns 8 (thread % n), + 8 n, ...
+      const int t = rank * (BM / n_cl) + (int)threadIdx.x / n_cl, r = q0 + t;
+      const int part = (int)threadIdx.x % n_cl;
+      const uint32_t a_st = sb + C::OFF_ST + 4 * t, a_z = sb + C::OFF_Q + t * (D * 4);
+      // (every loop's loads before their first use: a trip to a peer takes long)
+      float w[kMaxSplit], lk[kMaxSplit], m = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int k = 0; k < kMaxSplit; ++k) {
+        w[k] = k < n_cl ? ld_peer(peer_addr(a_st, k)) : -INFINITY;
+        lk[k] = k < n_cl ? ld_peer(peer_addr(a_st + 4 * BM, k)) : 0.f;
+      }
+      const float u_self = ld_peer(peer_addr(a_st + 8 * BM, n_cl - 1));
+#pragma unroll
+      for (int k = 0; k < kMaxSplit; ++k) m = fmaxf(m, w[k]);
+#pragma unroll
+      for (int k = 0; k < kMaxSplit; ++k) {
+        w[k] = w[k] == -INFINITY ? 0.f : ex2_approx(w[k] - m);  // (0: no z there either)
+        l = w[k] == 0.f ? l : fmaf(w[k], lk[k], l);
+      }
+      float g = 0.f, inv_l = 0.f, fself = 1.0f, lz = 0.f;
+      if (MODE == 0) {
+        const float S = 1.0f / (1.0f + __expf(-(u_self * p.inv_sqrt_d) / p.tau_s));
+        lz = S;  // empty history (row 1)
+        if (l > 0.f) {
+          const float A = m * kLn2 + __logf(l) - p.lambda * __logf((float)(r + 1));
+          g = 1.0f / (1.0f + __expf(S - A));
+          fself = 1.0f / (1.0f + __expf(A - S));
+          const float hi = fmaxf(S, A), lo = fminf(S, A);
+          lz = hi + log1pf(__expf(lo - hi));
+          inv_l = 1.0f / l;
+        }
+      }
+      const long long row = (long long)bh * p.T + r;
+      if (r < p.T) {
+        for (int c = 8 * part; c < p.d; c += 8 * n_cl) {
+          float z[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) z[e] = 0.f;
+          // v_i from the diagonal tile's V rows, in the last CTA's stages (as above)
+          uint4 vv = make_uint4(0, 0, 0, 0);
+          if (MODE == 0)
+            vv = ld_peer16(peer_addr(
+                sb + C::OFF_V + (c >> 6) * C::KVR * 128 +
+                    (C::QUAD ? (t >> 6) * C::KVT + (t & 63) * 128 : t * 128) +
+                    ((((c & 63) >> 3) ^ (t & 7)) << 4),
+                n_cl - 1));
+#pragma unroll
+          for (int k0 = 0; k0 < kMaxSplit; k0 += 4) {
+            if (k0 >= n_cl) break;
+            uint4 x[4][2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                x[k][q] = make_uint4(0, 0, 0, 0);
+                if (w[k0 + k] != 0.f)
+                  x[k][q] = ld_peer16(peer_addr(a_z + ((((c >> 2) + q) ^ (t & 7)) << 4), k0 + k));
+              }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                z[4 * q] = fmaf(w[k0 + k], __uint_as_float(x[k][q].x), z[4 * q]);
+                z[4 * q + 1] = fmaf(w[k0 + k], __uint_as_float(x[k][q].y), z[4 * q + 1]);
+                z[4 * q + 2] = fmaf(w[k0 + k], __uint_as_float(x[k][q].z), z[4 * q + 2]);
+                z[4 * q + 3] = fmaf(w[k0 + k], __uint_as_float(x[k][q].w), z[4 * q + 3]);
+              }
+          }
+          if (MODE == 1) {
+            float4* o = reinterpret_cast<float4*>(sa.z + row * p.d + c);
+            o[0] = make_float4(z[0], z[1], z[2], z[3]);
+            o[1] = make_float4(z[4], z[5], z[6], z[7]);
+          } else {
+            const uint32_t vw[4] = {vv.x, vv.y, vv.z, vv.w};
+            uint32_t yw[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 vf =
+                  __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&vw[e]));
+              yw[e] = pack_bf16x2(fmaf(g, z[2 * e] * inv_l - vf.x, vf.x),
+                                  fmaf(g, z[2 * e + 1] * inv_l - vf.y, vf.y));
+            }
+            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + (long long)b * p.sB +
+                                      (long long)h * p.sH + (long long)r * p.sT + c) =
+                make_uint4(yw[0], yw[1], yw[2], yw[3]);
+          }
+        }
+        if (part == 0) {
+          if (MODE == 1) {
+            sa.m[row] = m == -INFINITY ? -INFINITY : m * kLn2;
+            sa.l[row] = l;
+          } else {
+            p.logz[row] = lz;
+            if (p.fself) p.fself[row] = fself;
+          }
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();  // this CTA's shared memory has been read
+  }
   __syncthreads();
   if (warp == C::W_MMA) {
     tc_fence_after();
@@ -658,12 +827,13 @@ bool supports(relation_dtype dt, int d) {
   return dt == RELATION_BF16 && d >= 8 && d <= 128 && d % 8 == 0;
 }
 
-template <int D, int MODE>
-static cudaError_t fwd_t(const Problem& p, const StateArgs& sa, cudaStream_t s) {
+template <int D, int MODE, bool SPLIT>
+static cudaError_t launch_t(const Problem& p, const StateArgs& sa, int n_qt, unsigned tiles,
+                            int split, int groups, cudaStream_t s) {
   // A runtime call first: it makes the primary context current on this thread, which the
   // driver's tensor-map encoder needs.
-  const int smem = FwdCfg<D>::SMEM;
-  cudaError_t e = cudaFuncSetAttribute(fwd_tc_kernel<D, MODE>,
+  constexpr int smem = FwdCfg<D>::SMEM;
+  cudaError_t e = cudaFuncSetAttribute(fwd_tc_kernel<D, MODE, SPLIT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) { note_failure("forward: shared memory attribute"); return e; }
   Problem pk = p;  // the keys' view: their own strides, and count (the state over other keys)
@@ -678,18 +848,46 @@ static cudaError_t fwd_t(const Problem& p, const StateArgs& sa, cudaStream_t s) 
     note_failure("forward: TMA descriptor of Q/K/V/Y");
     return cudaErrorInvalidValue;
   }
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)split;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(tiles * (unsigned)split);
+  cfg.blockDim = dim3(FwdCfg<D>::THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = SPLIT ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, fwd_tc_kernel<D, MODE, SPLIT>, mq, mk, mv, mo, p, n_qt, groups, sa);
+  if (e != cudaSuccess) note_failure("forward: kernel launch");
+  return e;
+}
+
+template <int D, int MODE>
+static cudaError_t fwd_t(const Problem& p, const StateArgs& sa, cudaStream_t s) {
   const int n_qt = (p.T + BM - 1) / BM;
-  const long long grid = (long long)n_qt * p.B * p.H;
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  const long long tiles = (long long)n_qt * p.B * p.H;
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   int dev = 0, nsm = 148;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     nsm = 148;
-  const int groups = head_groups(n_qt, p.B * p.H, FwdCfg<D>::CTAS * nsm);
-  fwd_tc_kernel<D, MODE><<<(unsigned)grid, FwdCfg<D>::THREADS, smem, s>>>(mq, mk, mv, mo, p,
-                                                                         n_qt, groups, sa);
-  if ((e = cudaGetLastError()) != cudaSuccess) note_failure("forward: kernel launch");
-  return e;
+  const int slots = FwdCfg<D>::CTAS * nsm;
+  const int groups = head_groups(n_qt, p.B * p.H, slots);
+  // Few query tiles leave SMs idle and the time is the longest row's chain of key tiles (one
+  // step after the other, 2.2 us per tile at d_h = 64): clusters of 2, 4 or 8 CTAs share them
+  // while all are resident at once.  The merge costs 2 to 3 us, so a share keeps two key tiles of
+  // the longest row (d_h = 128, twice the state: five).  Forward, split 1 -> as chosen, warm:
+  // H 12, T 777, d 64 21.6 -> 17.3 us; H 1, T 2048 42 -> 14; H 1, T 8192 154 -> 39; H 12, T 2048
+  // 43 -> 32; H 4, T 4096, d 128 58 -> 41; H 8, T 2048, d 80 33 -> 25.  Past the lines: H 12, T 384
+  // 12.2 -> 12.6; H 16, T 512, d 128 12.9 -> 13.7; H 16, T 2048, d 128 34 -> 44.
+  const int most = MODE == 0 || sa.causal ? n_qt : (sa.Tk + BN - 1) / BN;  // key tiles of a row
+  constexpr int kShare = FwdCfg<D>::QUAD ? 2 : 5;
+  int split = 1;
+  while (split < kMaxSplit && kShare * 2 * split <= most && 2 * split * tiles <= slots) split *= 2;
+  return split > 1 ? launch_t<D, MODE, true>(p, sa, n_qt, (unsigned)tiles, split, groups, s)
+                   : launch_t<D, MODE, false>(p, sa, n_qt, (unsigned)tiles, 1, groups, s);
 }
 
 cudaError_t launch_fwd(const Problem& p, cudaStream_t s) {
