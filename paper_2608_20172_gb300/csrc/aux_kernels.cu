@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kWarps * 32) pre_kernel(Problem p, BwdWorkspac
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long gr = (long long)blockIdx.x * kWarps + warp;
   const long long nrows = (long long)p.B * p.H * p.T;
+  pdl_wait_and_launch();
   float contrib = 0.f;
   if (gr < nrows) {
     const int bh = (int)(gr / p.T), r = (int)(gr % p.T);
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(kWarps * 32) pre_kernel(Problem p, BwdWorkspac
 __global__ void __launch_bounds__(1024) dlambda_kernel(const float* pre, int n_pre,
                                                        const float* main, int n_main, float* out) {
   __shared__ double red[32];
+  pdl_wait_and_launch();
   double s = 0.0;
   for (int i = threadIdx.x; i < n_pre; i += 1024) s += (double)pre[i];
   for (int i = threadIdx.x; i < n_main; i += 1024) s += (double)main[i];
@@ -155,16 +157,14 @@ __global__ void __launch_bounds__(1024) dlambda_kernel(const float* pre, int n_p
 cudaError_t launch_pre(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
   dim3 grid(ws.n_pre_blocks);
   if (p.dtype == RELATION_F32)
-    pre_kernel<float><<<grid, kWarps * 32, 0, s>>>(p, ws);
-  else
-    pre_kernel<__nv_bfloat16><<<grid, kWarps * 32, 0, s>>>(p, ws);
-  return cudaGetLastError();
+    return launch_pdl(pre_kernel<float>, grid, kWarps * 32, 0, s, 1, p, ws);
+  return launch_pdl(pre_kernel<__nv_bfloat16>, grid, kWarps * 32, 0, s, 1, p, ws);
 }
 
 cudaError_t launch_dlambda(const Problem& p, const BwdWorkspace& ws, const float* main, int n_main,
                            cudaStream_t s) {
-  dlambda_kernel<<<1, 1024, 0, s>>>(ws.dlam_part, ws.n_pre_blocks, main, n_main, p.dlambda);
-  return cudaGetLastError();
+  return launch_pdl(dlambda_kernel, dim3(1), 1024, 0, s, 1, (const float*)ws.dlam_part,
+                    ws.n_pre_blocks, main, n_main, p.dlambda);
 }
 
 }  // namespace bwd_common

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(256) merge_kernel(float* m, float* l, float* z
                                                     long long rows, int d) {
   const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait_and_launch();
   if (row >= rows) return;
   const float ma = m[row], mb = m2[row], la = l[row], lb = l2[row];
   const float M = fmaxf(ma, mb);
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(256) finish_kernel(Problem p, const float* m, 
   const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const long long rows = (long long)p.B * p.H * p.T;
+  pdl_wait_and_launch();
   if (row >= rows) return;
   const int bh = (int)(row / p.T), r = (int)(row % p.T);
   const int b = bh / p.H, h = bh % p.H;
@@ -122,8 +124,8 @@ cudaError_t launch_state_merge(float* m, float* l, float* z, const float* m2, co
   if (rows < 1 || d < 4 || d > 128 || d % 4) return cudaErrorInvalidValue;
   const long long blocks = (rows + 7) / 8;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  cp::merge_kernel<<<(unsigned)blocks, 256, 0, s>>>(m, l, z, m2, l2, z2, rows, d);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(cp::merge_kernel, dim3((unsigned)blocks), 256, 0, s, 1, m, l, z, m2,
+                                   l2, z2, rows, d);
   if (e != cudaSuccess) note_failure("state merge: launch");
   return e;
 }
@@ -134,11 +136,9 @@ cudaError_t launch_state_finish(const Problem& p, const float* m, const float* l
   if (rows < 1 || p.d < 4 || p.d > 128 || p.d % 4) return cudaErrorInvalidValue;
   const long long blocks = (rows + 7) / 8;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  if (p.dtype == RELATION_BF16)
-    cp::finish_kernel<__nv_bfloat16><<<(unsigned)blocks, 256, 0, s>>>(p, m, l, z, pos0);
-  else
-    cp::finish_kernel<float><<<(unsigned)blocks, 256, 0, s>>>(p, m, l, z, pos0);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(
+      p.dtype == RELATION_BF16 ? cp::finish_kernel<__nv_bfloat16> : cp::finish_kernel<float>,
+      dim3((unsigned)blocks), 256, 0, s, 1, p, m, l, z, pos0);
   if (e != cudaSuccess) note_failure("state finish: launch");
   return e;
 }

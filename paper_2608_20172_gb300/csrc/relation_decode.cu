@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(32 * kClWarps) cluster_kernel(DecodeProblem p)
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)blockIdx.x % kCluster;
   const int bh = (int)blockIdx.x / kCluster, b = bh / p.H, h = bh % p.H;
+  pdl_wait_and_launch();
   const int len = length_of(p, b, threadIdx.x == 0 && rank == 0);
   const TI* qv = reinterpret_cast<const TI*>(p.q) + (long long)b * p.qsB + (long long)h * p.qsH;
   const long long head = (long long)b * p.sB + (long long)h * p.sH;
@@ -446,7 +447,7 @@ template <typename TI, int NQ>
 __global__ void __launch_bounds__(32 * kClWarps) scan_kernel(DecodeProblem p, float* part) {
   __shared__ Smem sm;
   extern __shared__ uint4 ring[];
-  cudaTriggerProgrammaticLaunchCompletion();  // the combine pass may come in beside the last CTAs
+  pdl_wait_and_launch();  // the combine pass may come in beside the last CTAs
   const int bh = blockIdx.x, chunk = blockIdx.y, b = bh / p.H, h = bh % p.H;
   const int len = length_of(p, b, threadIdx.x == 0 && chunk == 0);
   const int c0 = chunk * kChunk, n = min(kChunk, len - 1 - c0);
@@ -470,9 +471,9 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.x, chunk = blockIdx.y;
   const int b = bh / p.H, h = bh % p.H;
+  pdl_wait_and_launch();  // the combine pass may come in beside the last CTAs
   const int len = length_of(p, b, threadIdx.x == 0 && chunk == 0);
   if (len == 0) return;  // invalid: no cache row is touched
-  cudaTriggerProgrammaticLaunchCompletion();  // the combine pass may come in beside the last CTAs
   const int hist = len - 1;  // history rows
   const int c0 = chunk * kChunk;
   const int n = max(0, min(kChunk, hist - c0));
@@ -572,6 +573,7 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
   __shared__ float self;
   const int bh = blockIdx.x, c = threadIdx.x, b = bh / p.H, h = bh % p.H;
   const int lane = c & 31, warp = c >> 5;
+  // (the partial pass's CTAs let this one in after their own wait: what came before is complete)
   const int len = length_of(p, b, false);  // (reported by the partial pass)
   const TI* qv = reinterpret_cast<const TI*>(p.q) + (long long)b * p.qsB + (long long)h * p.qsH;
   const long long row = (long long)b * p.sB + (long long)h * p.sH + (long long)(len - 1) * p.sT;
@@ -579,7 +581,7 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
     const float s = self_dot<TI>(p, qv, reinterpret_cast<const TI*>(p.k) + row, lane);
     if (lane == 0) self = s;
   }
-  cudaGridDependencySynchronize();  // the partial pass is complete
+  pdl_wait_and_launch();  // the partial pass is complete
   if (len == 0) return;
   const int used = (len - 1 + kChunk - 1) / kChunk;  // <= n_chunks
   const float* pb = part + (long long)bh * n_chunks * (2 + kMaxD);
@@ -625,11 +627,6 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
   const bool qal = (reinterpret_cast<uintptr_t>(p.q) & 15u) == 0 &&
                    (p.qsB * (long long)sizeof(TI)) % 16 == 0 &&
                    (p.qsH * (long long)sizeof(TI)) % 16 == 0;
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr{};
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
   constexpr int smem = Scan<TI, NQ>::kRing;
   auto allow = [&](const void* f) {
     const cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -643,32 +640,23 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
   // d 128: 21 against 17; 128 heads: 30 against 16) the CTAs are too few or come in waves.
   if (kCluster * heads <= 2 * nsm && n_chunks <= kCluster) {
     if ((e = allow((const void*)cluster_kernel<TI, NQ>)) != cudaSuccess) return e;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = kCluster;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)heads * kCluster);
-    cfg.blockDim = dim3(32 * kClWarps);
-    cfg.dynamicSmemBytes = smem;
-    e = cudaLaunchKernelEx(&cfg, cluster_kernel<TI, NQ>, p);
+    e = launch_pdl(cluster_kernel<TI, NQ>, dim3((unsigned)heads * kCluster), 32 * kClWarps, smem, s,
+                   kCluster, p);
     if (e != cudaSuccess) note_failure("decode: cluster launch");
     return e;
   }
   const dim3 grid((unsigned)heads, (unsigned)n_chunks);
   if (NQ > 0 && p.d == 128 && qal) {
-    partial_kernel<TI, 128><<<grid, 32 * kWarps, 0, s>>>(p, part);
+    e = launch_pdl(partial_kernel<TI, 128>, grid, 32 * kWarps, 0, s, 1, p, part);
   } else if (NQ > 0 && p.d == 64 && qal) {
-    partial_kernel<TI, 64><<<grid, 32 * kWarps, 0, s>>>(p, part);
+    e = launch_pdl(partial_kernel<TI, 64>, grid, 32 * kWarps, 0, s, 1, p, part);
   } else {
     if ((e = allow((const void*)scan_kernel<TI, NQ>)) != cudaSuccess) return e;
-    scan_kernel<TI, NQ><<<grid, 32 * kClWarps, smem, s>>>(p, part);
+    e = launch_pdl(scan_kernel<TI, NQ>, grid, 32 * kClWarps, smem, s, 1, p, part);
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) { note_failure("decode: partial pass launch"); return e; }
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)heads);
-  cfg.blockDim = dim3(kMaxD);
-  e = cudaLaunchKernelEx(&cfg, combine_kernel<TI>, p, (const float*)part, n_chunks);
+  e = launch_pdl(combine_kernel<TI>, dim3((unsigned)heads), kMaxD, 0, s, 1, p, (const float*)part,
+                 n_chunks);
   if (e != cudaSuccess) note_failure("decode: combine launch");
   return e;
 }

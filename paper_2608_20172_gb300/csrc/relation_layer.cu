@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
   using V = Vec8<TI>;
   const LayerProblem& p = ar.p;
   const Where at = where(p);
+  pdl_wait_and_launch();
   if (!(blockIdx.x & 1)) {  // Q = RoPE(P1), K = RoPE(P2)
     __shared__ Tables tb;
     rope_pass<TI>(tb, ar, at, 1.f);
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(kThreads) grad_kernel(const __grid_constant__ 
   using V = Vec8<TI>;
   const LayerProblem& p = ar.p;
   const Where at = where(p);
+  pdl_wait_and_launch();
   if (!(blockIdx.x & 1)) {  // transposed RoPE: dP1 from dQ, dP2 from dK
     __shared__ Tables tb;
     rope_pass<TI>(tb, ar, at, -1.f);
@@ -347,6 +349,7 @@ __global__ void __launch_bounds__(kThreads) grad_kernel(const __grid_constant__ 
 __global__ void __launch_bounds__(256) dtheta_kernel(LayerProblem p, int n_cta) {
   __shared__ double red[8];
   const int np = p.H / 2, k = blockIdx.x;
+  pdl_wait_and_launch();
   double s = 0.0;
   for (int c = threadIdx.x; c < n_cta; c += 256) s += (double)p.dtheta_part[(long long)c * np + k];
 #pragma unroll
@@ -388,11 +391,11 @@ size_t layer_grad_workspace_bytes(int B, int T, int H) {
 cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
   const int grid = layer::ctas(p);
   const layer::Args ar = layer::args_of(p);
+  cudaError_t e;
   if (p.dtype == RELATION_F32)
-    layer::prep_kernel<float><<<2 * grid, layer::kThreads, 0, s>>>(ar);
+    e = launch_pdl(layer::prep_kernel<float>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
   else
-    layer::prep_kernel<__nv_bfloat16><<<2 * grid, layer::kThreads, 0, s>>>(ar);
-  cudaError_t e = cudaGetLastError();
+    e = launch_pdl(layer::prep_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
   if (e != cudaSuccess) note_failure("layer prep: launch");
   return e;
 }
@@ -400,14 +403,14 @@ cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
 cudaError_t launch_layer_grad(const LayerProblem& p, cudaStream_t s) {
   const int grid = layer::ctas(p);
   const layer::Args ar = layer::args_of(p);
+  cudaError_t e;
   if (p.dtype == RELATION_F32)
-    layer::grad_kernel<float><<<2 * grid, layer::kThreads, 0, s>>>(ar);
+    e = launch_pdl(layer::grad_kernel<float>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
   else
-    layer::grad_kernel<__nv_bfloat16><<<2 * grid, layer::kThreads, 0, s>>>(ar);
-  cudaError_t e = cudaGetLastError();
+    e = launch_pdl(layer::grad_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
   if (e != cudaSuccess) { note_failure("layer grad: launch"); return e; }
-  layer::dtheta_kernel<<<p.H / 2, 256, 0, s>>>(p, grid);
-  if ((e = cudaGetLastError()) != cudaSuccess) note_failure("layer grad: dtheta launch");
+  e = launch_pdl(layer::dtheta_kernel, dim3(p.H / 2), 256, 0, s, 1, p, grid);
+  if (e != cudaSuccess) note_failure("layer grad: dtheta launch");
   return e;
 }
 

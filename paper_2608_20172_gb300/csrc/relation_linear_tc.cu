@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
+  pdl_wait();
 
   if (warp == C::W_TMA) {
     // ------------------------------------------------------------------ TMA producer
@@ -689,6 +690,7 @@ __device__ __forceinline__ void scan_blocks(float* rows, const float* g, int nb,
 // CTAs of 8 channels; with BOTH the second half of the grid scans the adjoints.
 template <int D, bool BOTH>
 __global__ void __launch_bounds__(256) scan_kernel(LinCp cp, int ctas) {
+  pdl_wait_and_launch();
   const bool rev = BOTH && (int)blockIdx.x >= ctas;
   const int w = (int)blockIdx.x - (rev ? ctas : 0);
   const int c = (w % (D / 8)) * 8 + (int)(threadIdx.x >> 5), n = (int)(threadIdx.x & 31) * 2;
@@ -767,8 +769,8 @@ static cudaError_t fwd_t(const LinearProblem& lp, void* workspace, cudaStream_t 
   if (!cp_path) {
     if (heads > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     using C = Cfg<D, MODE_SEQ>;
-    lin_tc_fwd_kernel<D, MODE_SEQ>
-        <<<(unsigned)heads, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
+    e = launch_pdl(lin_tc_fwd_kernel<D, MODE_SEQ>, dim3((unsigned)heads), C::THREADS, C::SMEM, s, 1,
+                   m1, m2, mv, mv, ma, my, mc, lp, cp);
   } else {
     using CD = Cfg<D, MODE_DELTA>;
     using CO = Cfg<D, MODE_OUT>;
@@ -777,15 +779,14 @@ static cudaError_t fwd_t(const LinearProblem& lp, void* workspace, cudaStream_t 
     unsigned grid = 0;
     if ((e = block_grid(heads * nb, CD::CTAS, &grid)) != cudaSuccess) return e;
     static_assert(CD::CTAS == CO::CTAS, "one grid for both");
-    lin_tc_fwd_kernel<D, MODE_DELTA>
-        <<<grid, CD::THREADS, CD::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
-    if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
-    scan_kernel<D, false><<<(unsigned)ctas, 256, 0, s>>>(cp, (int)ctas);
-    if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked forward: launch"); return e; }
-    lin_tc_fwd_kernel<D, MODE_OUT>
-        <<<grid, CO::THREADS, CO::SMEM, s>>>(m1, m2, mv, mv, ma, my, mc, lp, cp);
+    if ((e = launch_pdl(lin_tc_fwd_kernel<D, MODE_DELTA>, dim3(grid), CD::THREADS, CD::SMEM, s, 1, m1,
+                        m2, mv, mv, ma, my, mc, lp, cp)) == cudaSuccess &&
+        (e = launch_pdl(scan_kernel<D, false>, dim3((unsigned)ctas), 256, 0, s, 1, cp, (int)ctas)) ==
+            cudaSuccess)
+      e = launch_pdl(lin_tc_fwd_kernel<D, MODE_OUT>, dim3(grid), CO::THREADS, CO::SMEM, s, 1, m1, m2,
+                     mv, mv, ma, my, mc, lp, cp);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked forward: launch");
+  if (e != cudaSuccess) note_failure("linear chunked forward: launch");
   return e;
 }
 
@@ -832,11 +833,10 @@ cudaError_t launch_states(const LinearProblem& lp, const void* dy, void* workspa
   if (heads * nb > 0x7fffffffLL || 2 * ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   unsigned grid = 0;
   if ((e = block_grid(heads * nb, C::CTAS, &grid)) != cudaSuccess) return e;
-  lin_tc_fwd_kernel<D, MODE_BOTH>
-      <<<grid, C::THREADS, C::SMEM, s>>>(m1, m2, mv, mg, ma, m1, m1, lp, cp);
-  if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("linear chunked backward: launch"); return e; }
-  scan_kernel<D, true><<<(unsigned)(2 * ctas), 256, 0, s>>>(cp, (int)ctas);
-  if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked backward: launch");
+  if ((e = launch_pdl(lin_tc_fwd_kernel<D, MODE_BOTH>, dim3(grid), C::THREADS, C::SMEM, s, 1, m1, m2,
+                      mv, mg, ma, m1, m1, lp, cp)) == cudaSuccess)
+    e = launch_pdl(scan_kernel<D, true>, dim3((unsigned)(2 * ctas)), 256, 0, s, 1, cp, (int)ctas);
+  if (e != cudaSuccess) note_failure("linear chunked backward: launch");
   return e;
 }
 

@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
+  pdl_wait();
 
   if (warp == W_TMA) {
     // ------------------------------------------------------------------ TMA producer
@@ -781,9 +782,9 @@ cudaError_t launch_linear_tc_bwd(const LinearProblem& p, cudaStream_t s) {
     note_failure("linear chunked backward: TMA descriptors");
     return cudaErrorInvalidValue;
   }
-  bwd::lin_tc_bwd_kernel<<<(unsigned)grid, bwd::kThreads, bwd::SMEM, s>>>(m1, m2, mv, mg, ma, mc0, mdc,
-                                                                    o1, o2, ov, p, nb);
-  if ((e = cudaGetLastError()) != cudaSuccess) note_failure("linear chunked backward: launch");
+  e = launch_pdl(bwd::lin_tc_bwd_kernel, dim3((unsigned)grid), bwd::kThreads, bwd::SMEM, s, 1, m1, m2,
+                 mv, mg, ma, mc0, mdc, o1, o2, ov, p, nb);
+  if (e != cudaSuccess) note_failure("linear chunked backward: launch");
   return e;
 }
 

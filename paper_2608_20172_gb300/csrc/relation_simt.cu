@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
   float* Pw = Vs + kTile * LD + warp * kWarpRows * PW;
   const float* Qw = Qs + warp * kWarpRows * LD;
+  pdl_wait();
   const int BH = p.B * p.H;
   const int qt = n_t - 1 - (int)(blockIdx.x / BH);  // most key tiles first
   const int bh = (int)(blockIdx.x % BH), b = bh / p.H, h = bh % p.H;
@@ -600,6 +601,7 @@ __global__ void __launch_bounds__(32 * W) bwd_kernel(Problem p, BwdWorkspace ws,
   float* smem = reinterpret_cast<float*>(smem_f4);
   const int BH = p.B * p.H;
   const int t = (int)((blockIdx.x >> 1) / BH), bh = (int)((blockIdx.x >> 1) % BH);
+  pdl_wait();
   if (blockIdx.x & 1)
     bwd_dq<TI, D, W>(p, ws, smem, n_t - 1 - t, bh);
   else
@@ -635,8 +637,7 @@ static cudaError_t fwd_t(const Problem& p, cudaStream_t s) {
   const int n_t = tiles(p);
   const long long grid = (long long)n_t * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  fwd_kernel<TI, D, W><<<(unsigned)grid, 32 * W, smem, s>>>(p, n_t);
-  return cudaGetLastError();
+  return launch_pdl(fwd_kernel<TI, D, W>, dim3((unsigned)grid), 32 * W, smem, s, 1, p, n_t);
 }
 
 template <typename TI, int D>
@@ -650,8 +651,8 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t 
   const int n_t = tiles(p);
   const long long grid = 2LL * n_t * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  bwd_kernel<TI, D, W><<<(unsigned)grid, 32 * W, smem, s>>>(p, ws, main_partials(ws), n_t);
-  return cudaGetLastError();
+  return launch_pdl(bwd_kernel<TI, D, W>, dim3((unsigned)grid), 32 * W, smem, s, 1, p, ws,
+                    main_partials(ws), n_t);
 }
 
 // The tile kernel's dlambda partials, one per dK / dV CTA (at most one per 16 rows): in the

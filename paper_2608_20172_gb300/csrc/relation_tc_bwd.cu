@@ -287,6 +287,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
+  pdl_wait();
 
   if (warp == C::W_TMA) {
     // ------------------------------------------------------ TMA + per-query scalars
@@ -820,6 +821,7 @@ __global__ void __launch_bounds__(256) pre_kernel(Problem p, BwdWorkspace ws, in
   const bool real = live && r < p.T;
   const int b = bh / p.H, h = bh % p.H;
   const long long off = (long long)b * p.sB + (long long)h * p.sH + (long long)r * p.sT + sub * PER;
+  pdl_wait();
   float gy = 0.f, gv = 0.f, qk = 0.f;
   if (real) {
     auto bf = [](const void* base, long long o) {
@@ -900,6 +902,7 @@ __global__ void __launch_bounds__(256) pre_kernel(Problem p, BwdWorkspace ws, in
 template <int D>
 __global__ void __launch_bounds__(256) finalize_kernel(Problem p, BwdWorkspace ws, int n_pre,
                                                        int n_cta) {
+  pdl_wait();
   if (blockIdx.x == 0) {
     __shared__ double part[256];
     double s = 0.0;
@@ -980,8 +983,9 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, unsigned stag
   cudaError_t e = cudaSuccess;
   if (stages & 1) {
     const long long rows_pad = (long long)p.B * p.H * t_pad;
-    bwd::pre_kernel<D><<<(unsigned)((rows_pad * 8 + 255) / 256), 256, 0, s>>>(p, ws, n_t);
-    if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("backward: row pass launch"); return e; }
+    e = launch_pdl(bwd::pre_kernel<D>, dim3((unsigned)((rows_pad * 8 + 255) / 256)), 256, 0, s, 1, p,
+                   ws, n_t);
+    if (e != cudaSuccess) { note_failure("backward: row pass launch"); return e; }
   }
   if (stages & 2) {
     // A runtime call first: it makes the device's primary context current on this thread,
@@ -1010,17 +1014,17 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, unsigned stag
     // d_h = 128 (one CTA per unit, dynamic scheduling): heads in groups, one CTA per SM;
     // d_h = 64 (persistent, zigzag over a heaviest-first sequence): one group.
     const int groups = D == 64 ? 1 : head_groups(n_t, p.B * p.H, nsm);
-    tiles<<<(unsigned)grid, bwd::Cfg<D>::THREADS, smem, s>>>(mq, mk, mv, mg, mdq, mdk, mdv, p, ws,
-                                                             n_t, t_pad, groups);
-    if ((e = cudaGetLastError()) != cudaSuccess) { note_failure("backward: tile kernel launch"); return e; }
+    e = launch_pdl(tiles, dim3((unsigned)grid), bwd::Cfg<D>::THREADS, smem, s, 1, mq, mk, mv, mg, mdq,
+                   mdk, mdv, p, ws, n_t, t_pad, groups);
+    if (e != cudaSuccess) { note_failure("backward: tile kernel launch"); return e; }
   }
   if (stages & 4) {
     const long long chunks = rows * (p.d / 8);
     const long long fblocks = (chunks + 255) / 256;
     const int n_pre = (int)((long long)p.B * p.H * t_pad / 32);  // row-pass blocks
-    bwd::finalize_kernel<D><<<(unsigned)(fblocks > 0 ? fblocks : 1), 256, 0, s>>>(p, ws, n_pre,
-                                                                                (int)grid);
-    if ((e = cudaGetLastError()) != cudaSuccess) note_failure("backward: finalisation launch");
+    e = launch_pdl(bwd::finalize_kernel<D>, dim3((unsigned)(fblocks > 0 ? fblocks : 1)), 256, 0, s, 1,
+                   p, ws, n_pre, (int)grid);
+    if (e != cudaSuccess) note_failure("backward: finalisation launch");
   }
   return e;
 }

@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, p.dev_status};
+  pdl_wait();
 
   if (warp == C::W_TMA) {
     // ------------------------------------------------------------------ TMA producer
@@ -848,18 +849,8 @@ static cudaError_t launch_t(const Problem& p, const StateArgs& sa, int n_qt, uns
     note_failure("forward: TMA descriptor of Q/K/V/Y");
     return cudaErrorInvalidValue;
   }
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)split;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.gridDim = dim3(tiles * (unsigned)split);
-  cfg.blockDim = dim3(FwdCfg<D>::THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = SPLIT ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, fwd_tc_kernel<D, MODE, SPLIT>, mq, mk, mv, mo, p, n_qt, groups, sa);
+  e = launch_pdl(fwd_tc_kernel<D, MODE, SPLIT>, dim3(tiles * (unsigned)split), FwdCfg<D>::THREADS,
+                 smem, s, (unsigned)split, mq, mk, mv, mo, p, n_qt, groups, sa);
   if (e != cudaSuccess) note_failure("forward: kernel launch");
   return e;
 }
