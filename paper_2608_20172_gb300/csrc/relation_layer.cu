@@ -13,15 +13,15 @@
 //       dtheta_k = sum dI~_a (-sin I_a - cos I_b) + dI~_b (cos I_a - sin I_b).
 //
 // Both passes are HBM-bound (prep reads P1, P2, I and writes Q, K, V; grad reads dQ, dK,
-// dV, I and writes dP1, dP2, dI): one CTA per (sequence, 16 positions) moves 8-element
+// dV, I and writes dP1, dP2, dI): CTAs of 8 or 16 positions of a sequence move 8-element
 // vectors (16 bytes in bf16).  The rotation angles of the CTA's positions are tabulated
 // once in shared memory and reused by every head: m * base^(-2c/d) is formed and reduced
 // modulo 2 pi as a sum of two floats (positions reach 16k, where an fp32 angle would be off
 // by ~1e-3 rad) from frequencies that come with the launch, then its cosine and sine are
 // taken in fp32.  (In fp64, with an fp64 log and exp per CTA, this chip's fp64 pipe bounded
 // both passes; the rotations and the mixing are CTAs of their own, so that the tables hide.
-// B 4, H 8, T 4096, d 80: prep 48 -> 31 us, grad 63 -> 41; B 2, H 16, T 16384, d 128: 159 ->
-// 126 us (6.4 TB/s), 196 -> 153 (6.1).)  dtheta is summed per CTA in a fixed
+// B 4, H 8, T 4096, d 80: prep 48 -> 26 us, grad 63 -> 36; B 2, H 16, T 16384, d 128: 159 ->
+// 122 us (6.6 TB/s), 196 -> 149 (6.3).)  dtheta is summed per CTA in a fixed
 // order and the partials are added up in fp64 by a second kernel, one block per head
 // pair (deterministic).
 #include <math.h>
@@ -32,8 +32,11 @@
 namespace rel {
 namespace layer {
 
-constexpr int kTok = 16;       // positions per CTA
-constexpr int kThreads = 256;
+// Positions and threads of a CTA.  prep: small CTAs, whose last wave is short (16 and 256 take
+// 28.4 instead of 25.5 us at B 4, H 8, T 4096, d 80, 29.9 instead of 27.4 at B 32, T 1024, d 48).
+// grad keeps 16, whose dtheta partials its workspace holds.
+constexpr int kPrepTok = 8, kPrepThreads = 128;
+constexpr int kTok = 16, kThreads = 256;
 constexpr int kMaxD = 256;     // head size limit of these passes
 constexpr int kMaxPairs = 128; // H / 2 limit
 
@@ -75,8 +78,9 @@ struct Vec8<float> {
   }
 };
 
+template <int TOK>
 struct Tables {
-  float cs[kTok][kMaxD / 2], sn[kTok][kMaxD / 2];  // RoPE of the CTA's positions
+  float cs[TOK][kMaxD / 2], sn[TOK][kMaxD / 2];  // RoPE of the CTA's positions
 };
 
 // The kernels' parameters: the problem and the frequencies base^(-2c/d), each as a sum of two
@@ -102,13 +106,14 @@ __device__ __forceinline__ float turn(float m, float w_hi, float w_lo) {
 }
 
 // cos / sin of m * base^(-2c/d) for the CTA's positions
-__device__ __forceinline__ void fill_tables(Tables& tb, const Args& ar, int t0) {
+template <int TOK, int NT>
+__device__ __forceinline__ void fill_tables(Tables<TOK>& tb, const Args& ar, int t0) {
   const LayerProblem& p = ar.p;
   const int half = p.d / 2;
-  for (int e = threadIdx.x; e < kTok * half; e += kThreads) {
+  for (int e = threadIdx.x; e < TOK * half; e += NT) {
     const int tt = e / half, c = e % half;
     float r;
-    if (t0 < (1 << 22) - kTok && p.rope_base >= 1.0f) {
+    if (t0 < (1 << 22) - TOK && p.rope_base >= 1.0f) {
       r = turn((float)(t0 + tt), ar.w_hi[c], ar.w_lo[c]);
     } else {  // positions or frequencies past turn's range: fp64
       const double a = (double)(t0 + tt) * exp(-2.0 * (double)c / (double)p.d * log((double)p.rope_base));
@@ -129,7 +134,8 @@ __device__ __forceinline__ void pair_heads(const LayerProblem& p, int k, int& a,
 }
 
 // rotate the 4 pairs of an 8-element chunk starting at channel 8 u by +-angle
-__device__ __forceinline__ void rotate8(float (&x)[8], const Tables& tb, int tt, int u,
+template <int TOK>
+__device__ __forceinline__ void rotate8(float (&x)[8], const Tables<TOK>& tb, int tt, int u,
                                         float sgn) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -146,17 +152,18 @@ __device__ __forceinline__ void rotate8(float (&x)[8], const Tables& tb, int tt,
 struct Where {
   int b, t0, nt;
 };
+template <int TOK>
 __device__ __forceinline__ Where where(const LayerProblem& p) {
-  const int n_tt = (p.T + kTok - 1) / kTok, w = (int)(blockIdx.x >> 1);
-  const int t0 = (w % n_tt) * kTok;
-  return {w / n_tt, t0, min(kTok, p.T - t0)};
+  const int n_tt = (p.T + TOK - 1) / TOK, w = (int)(blockIdx.x >> 1);
+  const int t0 = (w % n_tt) * TOK;
+  return {w / n_tt, t0, min(TOK, p.T - t0)};
 }
 
 // RoPE (sgn = +1) or its transpose (sgn = -1) of in1 -> out1 and in2 -> out2 over the
 // CTA's (position, head, chunk) items, two items per thread and iteration so that four
 // 16-byte loads are in flight (the first ones during the tables).
-template <typename TI>
-__device__ __forceinline__ void rope_pass(Tables& tb, const Args& ar, const Where& at, float sgn) {
+template <typename TI, int TOK, int NT>
+__device__ __forceinline__ void rope_pass(Tables<TOK>& tb, const Args& ar, const Where& at, float sgn) {
   using V = Vec8<TI>;
   const LayerProblem& p = ar.p;
   const int nu = p.d / 8;
@@ -186,34 +193,34 @@ __device__ __forceinline__ void rope_pass(Tables& tb, const Args& ar, const Wher
     V::store(reinterpret_cast<TI*>(p.out1) + i.off, x);
     V::store(reinterpret_cast<TI*>(p.out2) + i.off, y);
   };
-  Item i0 = item(threadIdx.x), i1 = item(threadIdx.x + kThreads);
+  Item i0 = item(threadIdx.x), i1 = item(threadIdx.x + NT);
   typename V::Raw x0 = V::load(in1 + i0.off), y0 = V::load(in2 + i0.off);
   typename V::Raw x1 = V::load(in1 + i1.off), y1 = V::load(in2 + i1.off);
-  fill_tables(tb, ar, at.t0);
+  fill_tables<TOK, NT>(tb, ar, at.t0);
   __syncthreads();
-  for (int e = threadIdx.x; e < n; e += 2 * kThreads) {
+  for (int e = threadIdx.x; e < n; e += 2 * NT) {
     if (e != (int)threadIdx.x) {
       i0 = item(e);
-      i1 = item(e + kThreads);
+      i1 = item(e + NT);
       x0 = V::load(in1 + i0.off);
       y0 = V::load(in2 + i0.off);
       x1 = V::load(in1 + i1.off);
       y1 = V::load(in2 + i1.off);
     }
     put(i0, x0, y0);
-    if (e + kThreads < n) put(i1, x1, y1);
+    if (e + NT < n) put(i1, x1, y1);
   }
 }
 
 template <typename TI>
-__global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ Args ar) {
+__global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constant__ Args ar) {
   using V = Vec8<TI>;
   const LayerProblem& p = ar.p;
-  const Where at = where(p);
+  const Where at = where<kPrepTok>(p);
   pdl_wait_and_launch();
   if (!(blockIdx.x & 1)) {  // Q = RoPE(P1), K = RoPE(P2)
-    __shared__ Tables tb;
-    rope_pass<TI>(tb, ar, at, 1.f);
+    __shared__ Tables<kPrepTok> tb;
+    rope_pass<TI, kPrepTok, kPrepThreads>(tb, ar, at, 1.f);
     return;
   }
   // Givens mixing of the information states: (token, pair, chunk) items, two per thread and
@@ -222,13 +229,13 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
   const long long base = (long long)at.b * p.sB;
   const TI* in = reinterpret_cast<const TI*>(p.in3);
   TI* out = reinterpret_cast<TI*>(p.out3);
-  for (int e0 = threadIdx.x; e0 < n; e0 += 2 * kThreads) {
+  for (int e0 = threadIdx.x; e0 < n; e0 += 2 * kPrepThreads) {
     typename V::Raw ra[2], rb[2];
     long long oa[2], ob[2];
     float th[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int e = min(e0 + i * kThreads, n - 1);
+      const int e = min(e0 + i * kPrepThreads, n - 1);
       const int r = e / nu, k = r % np, tt = r / np;
       int ha, hb;
       pair_heads(p, k, ha, hb);
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const __grid_constant__ 
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      if (e0 + i * kThreads >= n) break;
+      if (e0 + i * kPrepThreads >= n) break;
       float ia[8], ib[8], va[8], vb[8], s, co;
       sincosf(th[i], &s, &co);
       V::unpack(ra[i], ia);
@@ -261,11 +268,11 @@ template <typename TI>
 __global__ void __launch_bounds__(kThreads) grad_kernel(const __grid_constant__ Args ar) {
   using V = Vec8<TI>;
   const LayerProblem& p = ar.p;
-  const Where at = where(p);
+  const Where at = where<kTok>(p);
   pdl_wait_and_launch();
   if (!(blockIdx.x & 1)) {  // transposed RoPE: dP1 from dQ, dP2 from dK
-    __shared__ Tables tb;
-    rope_pass<TI>(tb, ar, at, -1.f);
+    __shared__ Tables<kTok> tb;
+    rope_pass<TI, kTok, kThreads>(tb, ar, at, -1.f);
     return;
   }
   __shared__ float part[kThreads / 32][kMaxPairs], tc[kMaxPairs], ts[kMaxPairs];
@@ -375,7 +382,7 @@ Args args_of(const LayerProblem& p) {
   return ar;
 }
 
-int ctas(const LayerProblem& p) { return p.B * ((p.T + kTok - 1) / kTok); }
+int ctas(const LayerProblem& p, int tok) { return p.B * ((p.T + tok - 1) / tok); }
 
 }  // namespace layer
 
@@ -389,19 +396,19 @@ size_t layer_grad_workspace_bytes(int B, int T, int H) {
 }
 
 cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
-  const int grid = layer::ctas(p);
+  const int grid = layer::ctas(p, layer::kPrepTok);
   const layer::Args ar = layer::args_of(p);
   cudaError_t e;
   if (p.dtype == RELATION_F32)
-    e = launch_pdl(layer::prep_kernel<float>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
+    e = launch_pdl(layer::prep_kernel<float>, dim3(2 * grid), layer::kPrepThreads, 0, s, 1, ar);
   else
-    e = launch_pdl(layer::prep_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
+    e = launch_pdl(layer::prep_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kPrepThreads, 0, s, 1, ar);
   if (e != cudaSuccess) note_failure("layer prep: launch");
   return e;
 }
 
 cudaError_t launch_layer_grad(const LayerProblem& p, cudaStream_t s) {
-  const int grid = layer::ctas(p);
+  const int grid = layer::ctas(p, layer::kTok);
   const layer::Args ar = layer::args_of(p);
   cudaError_t e;
   if (p.dtype == RELATION_F32)
