@@ -14,10 +14,11 @@
 // warp's: the weights pass between the two kinds of product through a warp-private
 // [8][64] buffer.  Bound: shared-memory bandwidth and the FP32 pipe (backward: 78 % of the
 // wavefronts, 58 % of the pipe), 2 + 7 products of d_h over the causal pairs (forward +
-// backward); the forward's longest CTAs also end alone.  Measured, B 2, H 8, T 1000, d 64,
-// forward + backward: 1478 -> 335 us (forward 567 -> 108, backward tiles 920 -> 212) against a
-// thread per quarter row (one 16-byte shared read per four multiply-adds, two shuffles per
-// entry); B 1, H 2, T 128, d 32: 49 -> 11 and 77 -> 12 us.
+// backward); in small grids, the chain of tiles of the longest rows, which two groups of warps
+// then share (two_groups).  Measured, B 2, H 8, T 1000, d 64, forward + backward: 1478 -> 293 us
+// (forward 567 -> 80, backward tiles 920 -> 210) against a thread per quarter row (one 16-byte
+// shared read per four multiply-adds, two shuffles per entry); B 1, H 2, T 128, d 32: 49 -> 9 and
+// 77 -> 11 us.
 //
 // Forward (Sec. 5.1, App. A.3): per tile the row's Exchange entries E_ij = SiLU(U_ij) (j < i)
 // update the running (m, l, z) state; the diagonal entry gives S_i = sigmoid(U_ii / tau_S)
@@ -134,14 +135,26 @@ __device__ __forceinline__ void store_cols(TI* row, int tx, const float (&x)[D /
   }
 }
 
+// NG groups of W warps share the tiles of a CTA's rows (group g the tiles g, g + NG, ...) and add
+// up their sums at the end: the NT threads of group g meet.
+template <int NT, int NG>
+__device__ __forceinline__ void group_sync(int g) {
+  if (NG == 1)
+    __syncthreads();
+  else if (g == 0)
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+  else
+    asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
+}
+
 // Stage `rows` rows from r0 of one head into shared memory as fp32 (rows >= T are zero).
 // fp32 rows go by cp.async (16 bytes, zero-filled past T) and are complete after
 // stage_wait and a barrier; bf16 rows are converted on the way.
 template <typename TI, int D, int NT>
 __device__ __forceinline__ void stage(float* dst, const TI* src, long long sT, int r0, int rows,
-                                      int T) {
+                                      int T, int tid) {  // tid: of the NT threads that stage it
   constexpr int LD = Ld<D>::V;
-  for (int idx = threadIdx.x; idx < rows * (D / 4); idx += NT) {
+  for (int idx = tid; idx < rows * (D / 4); idx += NT) {
     const int rr = idx / (D / 4), c4 = idx % (D / 4);
     const int r = r0 + rr;
     float* to = dst + rr * LD + 4 * c4;
@@ -240,20 +253,22 @@ __device__ __forceinline__ float row_max(float x) {
 // ---------------------------------------------------------------------------
 // Forward
 // ---------------------------------------------------------------------------
-template <int D, int W>
+template <int D, int W, int NG>
 constexpr size_t fwd_smem() {
-  return (size_t)(kWarpRows * W + 2 * kTile) * Ld<D>::V * 4 + (size_t)W * kWarpRows * PW * 4;
+  return (size_t)(kWarpRows * W + NG * 2 * kTile) * Ld<D>::V * 4 +
+         (size_t)NG * W * kWarpRows * PW * 4;
 }
 
-template <typename TI, int D, int W>
-__global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
+template <typename TI, int D, int W, int NG>
+__global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) fwd_kernel(Problem p, int n_t) {
   constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
   extern __shared__ float4 smem_f4[];
   float* Qs = reinterpret_cast<float*>(smem_f4);
-  float* Ks = Qs + ROWS * LD;
+  const int grp = NG == 1 ? 0 : threadIdx.x / NT, tid = NG == 1 ? threadIdx.x : threadIdx.x % NT;
+  float* Ks = Qs + ROWS * LD + grp * 2 * kTile * LD;
   float* Vs = Ks + kTile * LD;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
-  float* Pw = Vs + kTile * LD + warp * kWarpRows * PW;
+  const int warp = tid >> 5, lane = tid & 31, ty = lane >> 4, tx = lane & 15;
+  float* Pw = Qs + (ROWS + NG * 2 * kTile) * LD + (threadIdx.x >> 5) * kWarpRows * PW;
   const float* Qw = Qs + warp * kWarpRows * LD;
   pdl_wait();
   const int BH = p.B * p.H;
@@ -275,14 +290,18 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
     for (int c = 0; c < D / 16; ++c) z[r][c] = 0.f;
   }
   const int kend = min(p.T, q0 + ROWS);
-  stage<TI, D, NT>(Qs, Q, p.sT, q0, ROWS, p.T);
-  stage<TI, D, NT>(Ks, K, p.sT, 0, kTile, p.T);
+  constexpr int STEP = NG * kTile;
+  stage<TI, D, NT * NG>(Qs, Q, p.sT, q0, ROWS, p.T, threadIdx.x);
   stage_commit();
-  stage<TI, D, NT>(Vs, V, p.sT, 0, kTile, p.T);
+  if (grp * kTile < kend) stage<TI, D, NT>(Ks, K, p.sT, grp * kTile, kTile, p.T, tid);
   stage_commit();
-  for (int k0 = 0; k0 < kend; k0 += kTile) {
+  if (grp * kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, grp * kTile, kTile, p.T, tid);
+  stage_commit();
+  stage_wait<2>();
+  __syncthreads();  // Q is in
+  for (int k0 = grp * kTile; k0 < kend; k0 += STEP) {
     stage_wait<1>();
-    __syncthreads();  // Q and K are in
+    group_sync<NT, NG>(grp);  // K is in
     const int hist = q0 + warp * kWarpRows + kWarpRows - 1 - k0;  // the warp's last history key + 1
     float sc[4];
     {
@@ -314,11 +333,11 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
         m[r] = mn;
       }
     }
-    __syncthreads();  // K has been read
-    if (k0 + kTile < kend) stage<TI, D, NT>(Ks, K, p.sT, k0 + kTile, kTile, p.T);
+    group_sync<NT, NG>(grp);  // K has been read
+    if (k0 + STEP < kend) stage<TI, D, NT>(Ks, K, p.sT, k0 + STEP, kTile, p.T, tid);
     stage_commit();
     stage_wait<1>();
-    __syncthreads();  // V is in
+    group_sync<NT, NG>(grp);  // V is in
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -328,8 +347,8 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
     const int some = max(0, min(kTile, (hist + 3) & ~3));
     axpys<D, false>(Pw, Vs, ty, tx, 0, full, z, [](int, int) { return true; });
     axpys<D, true>(Pw, Vs, ty, tx, full, some, z, [&](int r, int k) { return k0 + k < r0 + r; });
-    __syncthreads();  // V has been read
-    if (k0 + kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + kTile, kTile, p.T);
+    group_sync<NT, NG>(grp);  // V has been read
+    if (k0 + STEP < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + STEP, kTile, p.T, tid);
     stage_commit();
   }
 
@@ -337,6 +356,33 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
   for (int r = 0; r < 4; ++r) {
     l[r] = row_sum(l[r]);
     u_self[r] = row_sum(u_self[r]);  // held by the lane whose key it was, 0 elsewhere
+  }
+  if constexpr (NG == 2) {
+    // the second group's (m, l, U_ii, z) through its own tiles to the first, which finishes the rows
+    float* const zs = Qs + (ROWS + 2 * kTile) * LD + (warp * kWarpRows + 4 * ty) * LD;
+    float* const st = Qs + (ROWS + 3 * kTile) * LD + (warp * kWarpRows + 4 * ty) * 4;
+    if (grp == 1) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        store_cols<float, D>(zs + r * LD, tx, z[r]);
+        if (tx == 0) *reinterpret_cast<float4*>(st + 4 * r) = make_float4(m[r], l[r], u_self[r], 0.f);
+      }
+    }
+    __syncthreads();
+    if (grp == 1) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float4 o = *reinterpret_cast<const float4*>(st + 4 * r);
+      u_self[r] += o.z;
+      if (o.x == -INFINITY) continue;  // no history there
+      const float mn = fmaxf(m[r], o.x), a = m[r] == -INFINITY ? 0.f : expf(m[r] - mn), b2 = expf(o.x - mn);
+      float zo[D / 16];
+      load_cols<float, D>(zs + r * LD, tx, zo);
+      m[r] = mn;
+      l[r] = fmaf(l[r], a, o.y * b2);
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) z[r][c] = fmaf(z[r][c], a, zo[c] * b2);
+    }
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -375,10 +421,10 @@ __global__ void __launch_bounds__(32 * W) fwd_kernel(Problem p, int n_t) {
 // ---------------------------------------------------------------------------
 // Backward
 // ---------------------------------------------------------------------------
-template <int D, int W>
+template <int D, int W, int NG>
 constexpr size_t bwd_smem() {
-  return (size_t)(2 * kWarpRows * W + 2 * kTile) * Ld<D>::V * 4 +
-         (size_t)W * kWarpRows * PW * 4 + 3 * kTile * 4 + W * 4;
+  return (size_t)(2 * kWarpRows * W + NG * 2 * kTile) * Ld<D>::V * 4 +
+         (size_t)NG * (W * kWarpRows * PW * 4 + 3 * kTile * 4 + W * 4);
 }
 
 // P_ij and dS_ij of one Exchange pair: ci = -lambda log i - logZ_i
@@ -392,20 +438,22 @@ __device__ __forceinline__ void pair_grad(float u, float dP, float ci, float Di,
 }
 
 // dK, dV (key-stationary): the CTA's ROWS keys over the query tiles from its first key on
-template <typename TI, int D, int W>
+template <typename TI, int D, int W, int NG>
 __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& ws, float* dlam_part,
                                          float* smem, int kt, int bh) {
   constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
   float* Ks = smem;
   float* Vs = Ks + ROWS * LD;
-  float* Qs = Vs + ROWS * LD;
+  const int grp = NG == 1 ? 0 : threadIdx.x / NT, tid = NG == 1 ? threadIdx.x : threadIdx.x % NT;
+  float* Qs = Vs + ROWS * LD + grp * 2 * kTile * LD;
   float* Gs = Qs + kTile * LD;  // dO tile
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
-  float* Pw = Gs + kTile * LD + warp * kWarpRows * PW;
-  float* cs = Gs + kTile * LD + W * kWarpRows * PW;  // -lambda log i - logZ_i
+  const int warp = tid >> 5, lane = tid & 31, ty = lane >> 4, tx = lane & 15;
+  float* const after = Vs + (ROWS + NG * 2 * kTile) * LD;
+  float* Pw = after + (threadIdx.x >> 5) * kWarpRows * PW;
+  float* cs = after + NG * W * kWarpRows * PW + grp * 3 * kTile;  // -lambda log i - logZ_i
   float* Ds = cs + kTile;                            // D_i
   float* wl = Ds + kTile;                            // log i * F_ii (Exchange weight of dlambda)
-  float* red = wl + kTile;
+  float* red = after + NG * (W * kWarpRows * PW + 3 * kTile);
   const int b = bh / p.H, h = bh % p.H;
   const int k0 = kt * ROWS;
   const int j0 = k0 + warp * kWarpRows + 4 * ty;  // the lane's keys j0 .. j0 + 3
@@ -424,14 +472,19 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
 #pragma unroll
     for (int c = 0; c < D / 16; ++c) dk[r][c] = dv[r][c] = 0.f;
   Sum2 dlam;  // -sum_i log i F_ii dR_ij over the lane's Exchange pairs (they cancel within a row)
-  stage<TI, D, NT>(Ks, K, p.sT, k0, ROWS, p.T);
-  stage<TI, D, NT>(Vs, V, p.sT, k0, ROWS, p.T);
-  for (int q0 = k0 / kTile * kTile; q0 < p.T; q0 += kTile) {
-    __syncthreads();  // the previous tile has been read
-    stage<TI, D, NT>(Qs, Q, p.sT, q0, kTile, p.T);
-    stage<TI, D, NT>(Gs, G, p.sT, q0, kTile, p.T);
+  stage<TI, D, NT * NG>(Ks, K, p.sT, k0, ROWS, p.T, threadIdx.x);
+  stage<TI, D, NT * NG>(Vs, V, p.sT, k0, ROWS, p.T, threadIdx.x);
+  if (NG > 1) {  // both groups read all of them
     stage_commit();
-    for (int ii = threadIdx.x; ii < kTile; ii += NT) {
+    stage_wait<0>();
+    __syncthreads();
+  }
+  for (int q0 = k0 / kTile * kTile + grp * kTile; q0 < p.T; q0 += NG * kTile) {
+    group_sync<NT, NG>(grp);  // the previous tile has been read
+    stage<TI, D, NT>(Qs, Q, p.sT, q0, kTile, p.T, tid);
+    stage<TI, D, NT>(Gs, G, p.sT, q0, kTile, p.T, tid);
+    stage_commit();
+    for (int ii = tid; ii < kTile; ii += NT) {
       const int i = q0 + ii;
       if (i < p.T) {
         // cs rounds; its error times P is in every P of the row, and taken out of dlambda's weight
@@ -447,7 +500,7 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
       }
     }
     stage_wait<0>();
-    __syncthreads();
+    group_sync<NT, NG>(grp);
     float P[4][4], dS[4][4];
     dots<D>(Ks + warp * kWarpRows * LD, Qs, ty, tx, P);
     dots<D>(Vs + warp * kWarpRows * LD, Gs, ty, tx, dS);
@@ -489,12 +542,37 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
   double lsum = (double)dlam.s + (double)dlam.c;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-  if (lane == 0) red[warp] = (float)lsum;
-  __syncthreads();
+  if (lane == 0) red[threadIdx.x >> 5] = (float)lsum;
+  if (NG > 1) {  // the second group's dK, dV through its own tiles
+    float* const xs = Vs + (ROWS + 2 * kTile) * LD + (warp * kWarpRows + 4 * ty) * LD;
+    if (grp == 1) {
+      group_sync<NT, NG>(grp);  // the last tile has been read
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        store_cols<float, D>(xs + r * LD, tx, dk[r]);
+        store_cols<float, D>(xs + (kTile + r) * LD, tx, dv[r]);
+      }
+    }
+    __syncthreads();
+    if (grp == 1) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float a[D / 16], b2[D / 16];
+      load_cols<float, D>(xs + r * LD, tx, a);
+      load_cols<float, D>(xs + (kTile + r) * LD, tx, b2);
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) {
+        dk[r][c] += a[c];
+        dv[r][c] += b2[c];
+      }
+    }
+  } else {
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < W; ++w) t += red[w];
+    for (int w = 0; w < W * NG; ++w) t += red[w];
     dlam_part[kt * (p.B * p.H) + bh] = t;
   }
   // Self terms of key j: dv_j += F_jj dO_j, dk_j += dS_jj q_j; then the 1/sqrt(d) of U.
@@ -517,16 +595,17 @@ __device__ __forceinline__ void bwd_dkdv(const Problem& p, const BwdWorkspace& w
 }
 
 // dQ (query-stationary): the CTA's ROWS queries over the key tiles up to its last query
-template <typename TI, int D, int W>
+template <typename TI, int D, int W, int NG>
 __device__ __forceinline__ void bwd_dq(const Problem& p, const BwdWorkspace& ws, float* smem,
                                        int qt, int bh) {
   constexpr int LD = Ld<D>::V, ROWS = kWarpRows * W, NT = 32 * W;
   float* Qs = smem;
   float* Gs = Qs + ROWS * LD;
-  float* Ks = Gs + ROWS * LD;
+  const int grp = NG == 1 ? 0 : threadIdx.x / NT, tid = NG == 1 ? threadIdx.x : threadIdx.x % NT;
+  float* Ks = Gs + ROWS * LD + grp * 2 * kTile * LD;
   float* Vs = Ks + kTile * LD;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 4, tx = lane & 15;
-  float* Pw = Vs + kTile * LD + warp * kWarpRows * PW;
+  const int warp = tid >> 5, lane = tid & 31, ty = lane >> 4, tx = lane & 15;
+  float* Pw = Gs + (ROWS + NG * 2 * kTile) * LD + (threadIdx.x >> 5) * kWarpRows * PW;
   const int b = bh / p.H, h = bh % p.H;
   const int q0 = qt * ROWS;
   const int r0 = q0 + warp * kWarpRows + 4 * ty;  // the lane's queries r0 .. r0 + 3
@@ -547,20 +626,25 @@ __device__ __forceinline__ void bwd_dq(const Problem& p, const BwdWorkspace& ws,
     for (int c = 0; c < D / 16; ++c) dq[r][c] = 0.f;
   }
   const int kend = min(p.T, q0 + ROWS);
-  stage<TI, D, NT>(Qs, Q, p.sT, q0, ROWS, p.T);
-  stage<TI, D, NT>(Gs, G, p.sT, q0, ROWS, p.T);
-  stage<TI, D, NT>(Vs, V, p.sT, 0, kTile, p.T);
+  constexpr int STEP = NG * kTile;
+  stage<TI, D, NT * NG>(Qs, Q, p.sT, q0, ROWS, p.T, threadIdx.x);
+  stage<TI, D, NT * NG>(Gs, G, p.sT, q0, ROWS, p.T, threadIdx.x);
+  if (grp * kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, grp * kTile, kTile, p.T, tid);
   stage_commit();
-  for (int k0 = 0; k0 < kend; k0 += kTile) {
-    stage<TI, D, NT>(Ks, K, p.sT, k0, kTile, p.T);
+  if (NG > 1) {  // both groups read all of Q and dO
+    stage_wait<0>();
+    __syncthreads();
+  }
+  for (int k0 = grp * kTile; k0 < kend; k0 += STEP) {
+    stage<TI, D, NT>(Ks, K, p.sT, k0, kTile, p.T, tid);
     stage_commit();
     stage_wait<1>();
-    __syncthreads();  // V (and Q, dO) are in
+    group_sync<NT, NG>(grp);  // V (and Q, dO) are in
     float dS[4][4], u[4][4];
     dots<D>(Gs + warp * kWarpRows * LD, Vs, ty, tx, dS);
     stage_wait<0>();
-    __syncthreads();  // V has been read, K is in
-    if (k0 + kTile < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + kTile, kTile, p.T);
+    group_sync<NT, NG>(grp);  // V has been read, K is in
+    if (k0 + STEP < kend) stage<TI, D, NT>(Vs, V, p.sT, k0 + STEP, kTile, p.T, tid);
     stage_commit();
     dots<D>(Qs + warp * kWarpRows * LD, Ks, ty, tx, u);
 #pragma unroll
@@ -578,7 +662,23 @@ __device__ __forceinline__ void bwd_dq(const Problem& p, const BwdWorkspace& ws,
     const int some = max(0, min(kTile, (hist + 3) & ~3));
     axpys<D, false>(Pw, Ks, ty, tx, 0, full, dq, [](int, int) { return true; });
     axpys<D, true>(Pw, Ks, ty, tx, full, some, dq, [&](int r, int k) { return k0 + k < r0 + r; });
-    __syncthreads();  // K has been read
+    group_sync<NT, NG>(grp);  // K has been read
+  }
+  if (NG > 1) {  // the second group's dQ through its own tiles
+    float* const xs = Gs + (ROWS + 2 * kTile) * LD + (warp * kWarpRows + 4 * ty) * LD;
+    if (grp == 1) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) store_cols<float, D>(xs + r * LD, tx, dq[r]);
+    }
+    __syncthreads();
+    if (grp == 1) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float a[D / 16];
+      load_cols<float, D>(xs + r * LD, tx, a);
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) dq[r][c] += a[c];
+    }
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -594,8 +694,8 @@ __device__ __forceinline__ void bwd_dq(const Problem& p, const BwdWorkspace& ws,
 }
 
 // Even CTAs dK / dV, odd ones dQ, the longest first in both.
-template <typename TI, int D, int W>
-__global__ void __launch_bounds__(32 * W) bwd_kernel(Problem p, BwdWorkspace ws, float* dlam_part,
+template <typename TI, int D, int W, int NG>
+__global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) bwd_kernel(Problem p, BwdWorkspace ws, float* dlam_part,
                                                      int n_t) {
   extern __shared__ float4 smem_f4[];
   float* smem = reinterpret_cast<float*>(smem_f4);
@@ -603,9 +703,9 @@ __global__ void __launch_bounds__(32 * W) bwd_kernel(Problem p, BwdWorkspace ws,
   const int t = (int)((blockIdx.x >> 1) / BH), bh = (int)((blockIdx.x >> 1) % BH);
   pdl_wait();
   if (blockIdx.x & 1)
-    bwd_dq<TI, D, W>(p, ws, smem, n_t - 1 - t, bh);
+    bwd_dq<TI, D, W, NG>(p, ws, smem, n_t - 1 - t, bh);
   else
-    bwd_dkdv<TI, D, W>(p, ws, dlam_part, smem, t, bh);
+    bwd_dkdv<TI, D, W, NG>(p, ws, dlam_part, smem, t, bh);
 }
 
 // ---------------------------------------------------------------------------
@@ -627,32 +727,57 @@ static int tiles(const Problem& p) {
   return (p.T + kWarpRows * kWarps - 1) / (kWarpRows * kWarps);
 }
 
+// Two groups per CTA where the longest row's chain of tiles decides: more than one tile, and no
+// more CTAs than are resident at once (`per_sm` of them on each SM).  Elsewhere they only cost
+// registers and the joining.  us with one and with two groups.  Forward: B 1, H 4, T 1000, d 64
+// 74 / 52; B 2, H 8, T 1000 (512 CTAs) 106 / 80; B 4, H 8 (1024) 139 / 149; B 2, H 4, T 777, d 128
+// (200) 94 / 72; B 4 (400) 108 / 111.  Backward: B 1, H 4, T 1000 (256) 184 / 133; B 2, H 8 (1024)
+// 210 / 218; B 2, H 4, T 777, d 128 (400) 198 / 148; B 4 (800) 261 / 282.
+static bool two_groups(const Problem& p, long long ctas, int per_sm) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    nsm = 0;
+  return p.T > kTile && ctas <= (long long)per_sm * nsm;
+}
+
+template <typename TI, int D, int NG>
+static cudaError_t fwd_g(const Problem& p, unsigned grid, cudaStream_t s) {
+  constexpr int W = kWarps;
+  constexpr size_t smem = fwd_smem<D, W, NG>();
+  static_assert(smem <= 232448, "shared memory");
+  const cudaError_t e = cudaFuncSetAttribute(
+      fwd_kernel<TI, D, W, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(fwd_kernel<TI, D, W, NG>, dim3(grid), 32 * W * NG, smem, s, 1, p, tiles(p));
+}
+
+template <typename TI, int D, int NG>
+static cudaError_t bwd_g(const Problem& p, const BwdWorkspace& ws, unsigned grid, cudaStream_t s) {
+  constexpr int W = kWarps;
+  constexpr size_t smem = bwd_smem<D, W, NG>();
+  static_assert(smem <= 232448, "shared memory");
+  const cudaError_t e = cudaFuncSetAttribute(
+      bwd_kernel<TI, D, W, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(bwd_kernel<TI, D, W, NG>, dim3(grid), 32 * W * NG, smem, s, 1, p, ws,
+                    main_partials(ws), tiles(p));
+}
+
 template <typename TI, int D>
 static cudaError_t fwd_t(const Problem& p, cudaStream_t s) {
-  constexpr int W = kWarps;
-  constexpr size_t smem = fwd_smem<D, W>();
-  cudaError_t e = cudaFuncSetAttribute(fwd_kernel<TI, D, W>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int n_t = tiles(p);
-  const long long grid = (long long)n_t * p.B * p.H;
+  const long long grid = (long long)tiles(p) * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return launch_pdl(fwd_kernel<TI, D, W>, dim3((unsigned)grid), 32 * W, smem, s, 1, p, n_t);
+  return two_groups(p, grid, D < 128 ? 4 : 2) ? fwd_g<TI, D, 2>(p, (unsigned)grid, s)
+                             : fwd_g<TI, D, 1>(p, (unsigned)grid, s);
 }
 
 template <typename TI, int D>
 static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
-  constexpr int W = kWarps;
-  constexpr size_t smem = bwd_smem<D, W>();
-  static_assert(smem <= 232448, "shared memory");
-  cudaError_t e = cudaFuncSetAttribute(bwd_kernel<TI, D, W>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int n_t = tiles(p);
-  const long long grid = 2LL * n_t * p.B * p.H;
+  const long long grid = 2LL * tiles(p) * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return launch_pdl(bwd_kernel<TI, D, W>, dim3((unsigned)grid), 32 * W, smem, s, 1, p, ws,
-                    main_partials(ws), n_t);
+  return two_groups(p, grid, D < 128 ? 4 : 3) ? bwd_g<TI, D, 2>(p, ws, (unsigned)grid, s)
+                             : bwd_g<TI, D, 1>(p, ws, (unsigned)grid, s);
 }
 
 // The tile kernel's dlambda partials, one per dK / dV CTA (at most one per 16 rows): in the

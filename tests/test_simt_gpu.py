@@ -41,3 +41,28 @@ def test_rows_outside_the_history_never_enter(cut):
     _, dkn, dvn, _ = binding.bwd(q, k, v, y, dn, logz, LAM, kernel="simt")
     assert torch.equal(dkn[:, cut:], dk[:, cut:]) and torch.equal(dvn[:, cut:], dv[:, cut:])
     assert np.isfinite(dk.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("T,d", [(65, 64), (96, 32), (129, 64), (160, 128), (193, 32), (300, 64),
+                                 (321, 128)])
+def test_one_and_two_groups_of_warps(T, d, dtype):
+    """A few heads take CTAs whose two groups of warps share a row's tiles, the same heads in a
+    large batch CTAs of one group: the large batch against the oracle, and both against each other
+    (fp32 sums in another order, a few 1e-7 of the largest value; bf16 outputs then rounded)."""
+    H, n = 2, -(-1300 // (2 * (T // 32)))
+    w = workloads.custom(1, H, T, d, dtype, qk_std=1.0)
+    x = workloads.make_inputs(w, seed=T + d)
+    many = [t.expand(n, T, H, d).contiguous() for t in x]
+    out = []
+    for q, k, v, do in (x, many):
+        q, k, v, do = (t.cuda() for t in (q, k, v, do))
+        y, lz = binding.fwd(q, k, v, LAM, kernel="simt")
+        dq, dk, dv, dl = binding.bwd(q, k, v, y, do, lz, LAM, kernel="simt")
+        out.append([t[:1].float() for t in (y, lz, dq, dk, dv)])
+    for a, b in zip(*out):
+        tol = 2e-6 if a.dtype == torch.float32 and dtype == "fp32" else 2.0 ** -7
+        assert float((a - b).abs().max()) <= tol * float(b.abs().max())
+    res = {k: t.cpu() for k, t in zip(("Y", "logZ", "dQ", "dK", "dV"), out[1])}
+    ref = pu.oracle_heads(*x, LAM, [(0, h) for h in range(H)])
+    pu.compare_heads(res, ref, dtype)
