@@ -33,7 +33,8 @@
 // d 64; four groups 93; with the logarithms on every warp, the next block's sums taken while the
 // output product runs and the stores on the TMA warp 82; with one instruction per logarithm and
 // no test per element for the clamp and the mask 76.  At B 1, H 12, T 32768 DELTA, the scan and
-// OUT took 140, 27 and 177 us, now 64, 16 and 72 (half of the issue slots in OUT).
+// OUT took 140, 27 and 177 us, now 64, 16 and 66 (4.5 TB/s in DELTA, half of the issue slots in
+// OUT, which takes the blocks in the opposite order: 72 us in the same one).
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps
 // meeting the warpgroups' barriers and skips the work between them.
 #include <cudaTypedefs.h>
@@ -130,7 +131,9 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     int blk, bhs, split, h, b;
   };
   auto where = [&](int it) -> Where {
-    const int item = (int)(blockIdx.x + it * gridDim.x);
+    // (OUT from the last block down: what DELTA read last is still in L2)
+    const int n = (int)(blockIdx.x + it * gridDim.x);
+    const int item = MODE == MODE_OUT ? p.B * p.H * NSPLIT * nb - 1 - n : n;
     Where w;
     w.bhs = SEQ ? (int)blockIdx.x : item / nb;
     w.blk = SEQ ? it : item - w.bhs * nb;
