@@ -33,8 +33,8 @@
 // d 64; four groups 93; with the logarithms on every warp, the next block's sums taken while the
 // output product runs and the stores on the TMA warp 82; with one instruction per logarithm and
 // no test per element for the clamp and the mask 76.  At B 1, H 12, T 32768 DELTA, the scan and
-// OUT took 140, 27 and 177 us, now 64, 16 and 66 (4.5 TB/s in DELTA, half of the issue slots in
-// OUT, which takes the blocks in the opposite order: 72 us in the same one).
+// OUT took 140, 27 and 177 us, now 57, 15 and 67 (5.1 TB/s in DELTA, half of the issue slots in
+// OUT; in head order, and both from the first block on, 64 and 72).
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps
 // meeting the warpgroups' barriers and skips the work between them.
 #include <cudaTypedefs.h>
@@ -131,16 +131,28 @@ __global__ void __launch_bounds__(Cfg<D, MODE>::THREADS, Cfg<D, MODE>::CTAS)
     int blk, bhs, split, h, b;
   };
   auto where = [&](int it) -> Where {
-    // (OUT from the last block down: what DELTA read last is still in L2)
+    // The heads of a block of tokens side by side, as they lie in memory; OUT and BOTH from the
+    // last tokens back, which DELTA, and the forward before a backward, have read last and left
+    // in L2
     const int n = (int)(blockIdx.x + it * gridDim.x);
-    const int item = MODE == MODE_OUT ? p.B * p.H * NSPLIT * nb - 1 - n : n;
+    const int item =
+        MODE == MODE_OUT || BOTH ? p.B * p.H * NSPLIT * nb - 1 - n : n;
     Where w;
-    w.bhs = SEQ ? (int)blockIdx.x : item / nb;
-    w.blk = SEQ ? it : item - w.bhs * nb;
-    const int bh = w.bhs / NSPLIT;
-    w.split = w.bhs - bh * NSPLIT;
-    w.b = bh / p.H;
-    w.h = bh - w.b * p.H;
+    if (SEQ) {
+      w.bhs = (int)blockIdx.x;
+      w.blk = it;
+      const int bh = w.bhs / NSPLIT;
+      w.split = w.bhs - bh * NSPLIT;
+      w.b = bh / p.H;
+      w.h = bh - w.b * p.H;
+    } else {
+      const int hs = p.H * NSPLIT, tb = item / hs, e = item - tb * hs;
+      w.b = tb / nb;
+      w.blk = tb - w.b * nb;
+      w.h = e / NSPLIT;
+      w.split = e - w.h * NSPLIT;
+      w.bhs = (w.b * p.H + w.h) * NSPLIT + w.split;
+    }
     return w;
   };
 

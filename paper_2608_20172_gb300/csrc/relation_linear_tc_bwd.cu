@@ -188,9 +188,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint16_t* fix_early = reinterpret_cast<uint16_t*>(e0_s + 64);  // [kFix] (token, channel)s
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int blk = (int)(blockIdx.x % nb);
-  const int bh = (int)(blockIdx.x / nb);  // one 64-column split per head at d_h = 64
-  const int b = bh / p.H, h = bh % p.H;
+  // one 64-column split per head at d_h = 64; the heads of a block of tokens side by side
+  const int tb = (int)blockIdx.x / p.H, h = (int)blockIdx.x - tb * p.H;
+  const int b = tb / nb, blk = tb - b * nb, bh = b * p.H + h;
   const int t0 = blk * LT;
 
   if (threadIdx.x == 0) {
