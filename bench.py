@@ -613,7 +613,7 @@ def linear_measure(binding, dev, peaks, steps=20, warmup=3):
                                      "unit": "TFLOP/s", "frac": tcb_ach / peaks["bf16_tflops"],
                                      "flops_per_call": tcb_fl},
             "long_context_sweep": {"kernel": "chunked forward with a workspace (chunk-parallel "
-                                             "below one (head, column) pair per SM)",
+                                             "where that takes less time)",
                                    "H": 12, "d_h": 64,
                                    "tokens_per_point": LINEAR_SWEEP_TOKENS, "points": sweep},
             "gpu_launches_per_step": {"fwd_chunked": 1, "bwd_chunked": 5, "fwd": 1, "bwd": 2}}

@@ -169,8 +169,9 @@ relation_status relation_linear_fwd_ex(const void* p1, const void* p2, const voi
  *               B H (d_h / 64) (ceil(T / 128) + 1) d_h rows of 64 bf16),
  *               16-byte aligned, or RELATION_ERR_WORKSPACE / RELATION_ERR_ALIGNMENT with
  *               nothing launched.
- * The chunk-parallel form runs when B H (d_h / 64) is below half the device's SM count, the
- * sequential chunked kernel otherwise (same results up to rounding).  Requests the chunked
+ * The chunk-parallel form runs where it takes less time (few such pairs, or a last round of
+ * the SMs that is nearly empty), the sequential chunked kernel otherwise (same results up to
+ * rounding).  Requests the chunked
  * kernel does not serve (workspace size 0: fp32, d_h other than 64 and 128, strides not
  * multiples of 8) go to relation_linear_fwd_ex(..., RELATION_KERNEL_AUTO, ...) and ignore the
  * workspace.  Other arguments, results and the decay-range report are those of

@@ -240,9 +240,15 @@ relation_status relation_linear_fwd_ws(const void* p1, const void* p2, const voi
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return RELATION_ERR_CUDA;
   const long long ctas = (long long)shp.B * shp.H * (shp.d_h / 64);
-  // enough (head, column) pairs for the sequential walk (measured on GB300: 96 pairs on 152
-  // SMs still favour it, 0.14 against 0.19 ms; 12 pairs at T = 32768 take 1.9 ms against 0.38)
-  if (2 * ctas >= nsm)
+  const long long nb = (shp.T + 127) / 128, waves = nsm > 0 ? (ctas + nsm - 1) / nsm : 0;
+  // The sequential walk takes `waves` rounds of the SMs, one (head, column) pair each, however
+  // full the last one is; the chunk-parallel passes share out the blocks evenly, at 1.52 times a
+  // round's time per block of all SMs (d_h = 128: 1.61) and 1.75 (2.0) blocks' time for the
+  // launches and the scan.  us, chunk-parallel and sequential, d_h = 64: 12 pairs, T 8192 44 / 262;
+  // 84 pairs, T 2048 66 / 74; 96 76 / 74; 144 108 / 78; 156 112 / 139; 216 152 / 142; 60 pairs,
+  // T 640 22 / 26; 72 28 / 26.  d_h = 128, T 2048: 80 132 / 144; 96 157 / 147; 160 249 / 277.
+  const long long per_block = shp.d_h == 64 ? 152 : 161, fixed = shp.d_h == 64 ? 175 : 200;
+  if (100 * waves * nb * nsm <= fixed * nsm + per_block * ctas * nb)
     return relation_linear_fwd_ex(p1, p2, v, alpha, y, tau_s, shp, dt, RELATION_KERNEL_TCGEN05,
                                   dev_status, stream);
   relation_status st;

@@ -335,10 +335,10 @@ def test_linear_chunked_backward_small_retentions(n_small, T):
         pu.check(f"dalpha head {h}", got[0, :, h], ref[0, :, h], "bf16", "grad")
 
 
-@pytest.mark.parametrize("B,T,H,d", [(3, 3000, 5, 64), (1, 2100, 5, 128)])
+@pytest.mark.parametrize("B,T,H,d", [(3, 3000, 5, 64), (1, 2100, 5, 128), (13, 1300, 12, 64)])
 def test_linear_chunk_parallel_more_blocks_than_ctas(B, T, H, d):
     """The one-block kernels share out more blocks than CTAs fit (two per SM at d_h = 64, one at
-    128, rest not even) and the last block of a head is ragged: the workspace forward against the
+    128, rest not even; the last shape has more pairs than SMs) and the last block of a head is ragged: the workspace forward against the
     sequential one, whose states are the same up to bf16 (the bound of two bf16 results)."""
     g = torch.Generator().manual_seed(B + d)
     dev = torch.device("cuda:0")
