@@ -869,14 +869,15 @@ static cudaError_t fwd_t(const Problem& p, const StateArgs& sa, cudaStream_t s) 
   // Few query tiles leave SMs idle and the time is the longest row's chain of key tiles (one
   // step after the other, 2.2 us per tile at d_h = 64): clusters of 2, 4 or 8 CTAs share them
   // while all are resident at once.  The merge costs 2 to 3 us, so a share keeps two key tiles of
-  // the longest row (d_h = 128, twice the state: five).  Forward, split 1 -> as chosen, warm:
-  // H 12, T 777, d 64 21.6 -> 17.3 us; H 1, T 2048 42 -> 14; H 1, T 8192 154 -> 39; H 12, T 2048
-  // 43 -> 32; H 4, T 4096, d 128 58 -> 41; H 8, T 2048, d 80 33 -> 25.  Past the lines: H 12, T 384
-  // 12.2 -> 12.6; H 16, T 512, d 128 12.9 -> 13.7; H 16, T 2048, d 128 34 -> 44.
+  // the longest row (d_h = 128, twice the state: two and a half).  Forward, split 1 -> as chosen,
+  // on cold caches: H 12, T 777, d 64 21.2 -> 17.8 us; H 4, T 1500 33 -> 17; H 1, T 2048 42 -> 14;
+  // H 8, T 640, d 128 17.3 -> 16.0; H 16, T 1024 22.8 -> 20.1; H 4, T 1536 28.9 -> 19.3; H 6, T 2048,
+  // d 80 36 -> 25.  Past the lines: H 12, T 384, d 64 12.0 -> 12.7; H 16, T 512, d 128 (warm) 12.9 ->
+  // 13.7; H 2, T 2048, d 128 in eight 20.4 instead of 18.0; H 16, T 1024 in four 35.7.
   const int most = MODE == 0 || sa.causal ? n_qt : (sa.Tk + BN - 1) / BN;  // key tiles of a row
-  constexpr int kShare = FwdCfg<D>::QUAD ? 2 : 5;
+  constexpr int kShare2 = FwdCfg<D>::QUAD ? 4 : 5;  // half key tiles
   int split = 1;
-  while (split < kMaxSplit && kShare * 2 * split <= most && 2 * split * tiles <= slots) split *= 2;
+  while (split < kMaxSplit && kShare2 * 2 * split <= 2 * most && 2 * split * tiles <= slots) split *= 2;
   return split > 1 ? launch_t<D, MODE, true>(p, sa, n_qt, (unsigned)tiles, split, groups, s)
                    : launch_t<D, MODE, false>(p, sa, n_qt, (unsigned)tiles, 1, groups, s);
 }

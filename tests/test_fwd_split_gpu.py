@@ -14,10 +14,10 @@ DEV = torch.device("cuda:0")
 LAM = workloads.LAMBDA_INIT
 
 
-# clusters of 2, 4 and 8 at d_h <= 64 (T 512 is their first length) and of 2 above (1280), ragged
+# clusters of 2, 4 and 8 at d_h <= 64 (T 512 is their first length), of 2 and 4 above (640, 1280), ragged
 # last tiles, padded widths; the first query tiles of a head leave shares empty
 @pytest.mark.parametrize("T,d,reps", [(512, 64, 320), (777, 40, 320), (1024, 64, 320),
-                                      (2048, 64, 320), (2047, 8, 320), (1280, 128, 64),
+                                      (2048, 64, 320), (2047, 8, 320), (640, 128, 64), (1280, 128, 64),
                                       (1409, 80, 64)])
 def test_split_rows(T, d, reps):
     H = 2 if T < 2047 else 1
