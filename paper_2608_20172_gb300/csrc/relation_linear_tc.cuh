@@ -21,7 +21,7 @@ constexpr int NC = 64;           // information columns per CTA
 constexpr float kClampLog2 = 120.0f;
 
 // Modes of the kernel: SEQ walks all blocks of a (head, split) in order with the state in
-// TMEM; the chunk-parallel pair takes one block per CTA: DELTA writes the block's state
+// TMEM; the chunk-parallel pair takes any block by itself: DELTA writes the block's state
 // contribution sum_j KL_j I~_j^T and decay a_L (fp32) to the workspace, OUT reads the
 // state the block starts from (bf16, produced by scan_kernel) and writes the block's Y.
 // BOTH (the backward, d_h = 64) is DELTA together with the block's contribution to the

@@ -31,7 +31,9 @@
 // barriers around small products, nothing else resident.  B 8, H 12, T 2048, the whole backward:
 // 535 us with one elementwise warpgroup and four state launches, 270 with four groups and two,
 // 254 with p1 and p2 kept in registers past Qm and Km (they were loaded again) and the small
-// retentions' fix-up beside the products.
+// retentions' fix-up beside the products, 228 with fewer instructions per element, the state
+// pass's blocks shared out among resident CTAs and launches that overlap.  (Persistent CTAs here,
+// the next block's tiles loaded early: the same; the registers spill.)
 // Every mbarrier wait is bounded (common.cuh); a warp whose wait gave up keeps meeting the
 // warpgroups' barriers and skips the work between them.
 #include "relation_linear_tc.cuh"
