@@ -91,7 +91,7 @@ struct Cfg {
   static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory");
 };
 
-// 32 bytes to global memory (one sector)
+// 32 bytes to global memory (one sector); p 32-byte aligned (ws_base)
 __device__ __forceinline__ void st_global_32(float* p, const uint32_t* r) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]),
                "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
@@ -715,6 +715,15 @@ __global__ void __launch_bounds__(256) scan_kernel(LinCp cp, int ctas) {
     scan_blocks<D, false>(cp.dC, cp.g, cp.nb, w / (D / 8), c, n);
 }
 
+// Where the arrays start in a workspace, which is 16-byte aligned only: the stores of whole sectors
+// (st_global_32) take 32 bytes, and rows of 256 bytes should not straddle more cache lines than
+// they fill.  The up to 240 bytes this skips are in the size already: of the bf16 rows that it
+// counts for nb + 1 states per (head, split), the forward uses none and the backward leaves at
+// least d rows of 128 bytes.
+static uint8_t* ws_base(void* base) {
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(base) + 255) & ~(uintptr_t)255);
+}
+
 // Workspace of the chunk-parallel forward: dC and g per (head, split, block) (see LinCp).  The
 // size also holds bf16 rows for nb + 1 states per (head, split), which the scan now keeps in
 // dC's rows: the backward's second array of fp32 rows takes that place.
@@ -723,7 +732,7 @@ static size_t cp_bytes(long long heads, long long nb, int d, LinCp* out, void* b
   const size_t b_dc = align256((size_t)rows * 64 * 4), b_g = align256((size_t)rows * 4);
   const size_t b_c0 = align256((size_t)rows_c0 * 64 * 2);
   if (out) {
-    uint8_t* q = static_cast<uint8_t*>(base);
+    uint8_t* q = ws_base(base);
     out->dC = reinterpret_cast<float*>(q);
     out->g = reinterpret_cast<float*>(q + b_dc);
     out->dQ = nullptr;
@@ -813,8 +822,7 @@ size_t bwd_bytes(long long heads, long long nb, int d, LinCp* cp, void* base) {
   const size_t f = cp_bytes(heads, nb, d, cp, base);
   // dQ's fp32 rows fill what the forward's nb + 1 and the adjoints' nb bf16 rows would take
   if (cp)
-    cp->dQ = reinterpret_cast<float*>(static_cast<uint8_t*>(base) +
-                                      align256((size_t)(heads * nb * d) * 64 * 4) +
+    cp->dQ = reinterpret_cast<float*>(ws_base(base) + align256((size_t)(heads * nb * d) * 64 * 4) +
                                       align256((size_t)(heads * nb * d) * 4));
   return f + align256((size_t)(heads * nb * d) * 64 * 2);
 }
