@@ -18,9 +18,9 @@
 // Self-Exchange epilogue.  There the time is latency: launches, and dependent trips to memory.
 // Otherwise two launches: the partial pass splits each history into chunks of kChunk rows, one
 // CTA per (head, chunk), with (m, l, z) to the workspace; the combine pass (one CTA per head)
-// merges them by the associative (m, l, z) rule of the tiled scan (App. A.3).  It comes in
-// while the last partial CTAs run and takes the Self evidence meanwhile, and reads the chunks'
-// weights a thread each (a serial loop over dependent loads before).
+// merges them by the associative (m, l, z) rule of the tiled scan (App. A.3).  Its CTAs come in
+// while the last partial CTAs run, and it reads the chunks' weights a thread each (a serial loop
+// over dependent loads before).
 // Measured in one graph over caches that together exceed L2, bf16, before -> now:
 // B 1, H 12, T 2048, d 64 18.6 -> 9.3 us; B 1, H 32, T 2048, d 80 78 -> 12.8;
 // B 32, H 8, T 2048, d 80 148 -> 58.6; B 1, H 16, T 32768, d 128 92.7 -> 64.8;
@@ -573,16 +573,17 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
   __shared__ float self;
   const int bh = blockIdx.x, c = threadIdx.x, b = bh / p.H, h = bh % p.H;
   const int lane = c & 31, warp = c >> 5;
-  // (the partial pass's CTAs let this one in after their own wait: what came before is complete)
+  // Before anything is read: that the partial CTAs have waited orders this kernel behind what came
+  // before them, but only its own wait makes those writes visible here.
+  pdl_wait_and_launch();
   const int len = length_of(p, b, false);  // (reported by the partial pass)
+  if (len == 0) return;
   const TI* qv = reinterpret_cast<const TI*>(p.q) + (long long)b * p.qsB + (long long)h * p.qsH;
   const long long row = (long long)b * p.sB + (long long)h * p.sH + (long long)(len - 1) * p.sT;
-  if (len > 0 && warp == 0) {
+  if (warp == kMaxD / 32 - 1) {  // (beside the first warps' loads of the chunks' weights)
     const float s = self_dot<TI>(p, qv, reinterpret_cast<const TI*>(p.k) + row, lane);
     if (lane == 0) self = s;
   }
-  pdl_wait_and_launch();  // the partial pass is complete
-  if (len == 0) return;
   const int used = (len - 1 + kChunk - 1) / kChunk;  // <= n_chunks
   const float* pb = part + (long long)bh * n_chunks * (2 + kMaxD);
   float M = -INFINITY;
