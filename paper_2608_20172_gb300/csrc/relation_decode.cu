@@ -18,9 +18,9 @@
 // Self-Exchange epilogue.  There the time is latency: launches, and dependent trips to memory.
 // Otherwise two launches: the partial pass splits each history into chunks of kChunk rows, one
 // CTA per (head, chunk), with (m, l, z) to the workspace; the combine pass (one CTA per head)
-// merges them by the associative (m, l, z) rule of the tiled scan (App. A.3).  Its CTAs come in
-// while the last partial CTAs run, and it reads the chunks' weights a thread each (a serial loop
-// over dependent loads before).
+// merges them by the associative (m, l, z) rule of the tiled scan (App. A.3), the chunks' weights
+// a thread each (a serial loop over dependent loads before).  Its CTAs come in
+// while the last partial CTAs run.
 // Measured in one graph over caches that together exceed L2, bf16, before -> now:
 // B 1, H 12, T 2048, d 64 18.6 -> 9.3 us; B 1, H 32, T 2048, d 80 78 -> 12.8;
 // B 32, H 8, T 2048, d 80 148 -> 58.6; B 1, H 16, T 32768, d 128 92.7 -> 64.8;
@@ -442,7 +442,7 @@ __device__ __forceinline__ void ld_vec(const TI* p, float* out) {
 }
 
 // Partial (m, l, z) of history rows [c0, min(c0 + kChunk, len - 1)) of head (b, h), into part.
-// Any d and alignment:
+// Aligned rows of any whole number of 16-byte groups:
 template <typename TI, int NQ>
 __global__ void __launch_bounds__(32 * kClWarps) scan_kernel(DecodeProblem p, float* part) {
   __shared__ Smem sm;
@@ -460,9 +460,13 @@ __global__ void __launch_bounds__(32 * kClWarps) scan_kernel(DecodeProblem p, fl
   sc.merge(out, out + 1, out + 2);
 }
 
-// The same, D = 64 or 128 and aligned rows: the chunk's scores first, four lanes per key and a
-// quarter of the row each, then P V with D / 32 consecutive columns per lane.  Fewer instructions
-// per row than scan_kernel and twice the warps: where every SM is full, these bound the pass.
+// The same in two steps, the chunk's scores first, then P V.  D = 64 or 128 and aligned rows: four
+// lanes per key and a quarter of the row each, then D / 32 consecutive columns per lane.  Fewer
+// instructions per row than scan_kernel and twice the warps: where every SM is full, these bound
+// the pass.  D = 0: any d and alignment, one element per lane and load, a warp per row; the warps
+// keep many rows' loads in flight, where scan_kernel's plain loads wait tile by tile (bf16, d 64,
+// rows of 65 elements, us with these and with those: 40 heads, T 300 18 / 31; 40 heads, T 4096
+// 40 / 52; 512 heads, T 4096 269 / 315).
 template <typename TI, int D>
 __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, float* part) {
   __shared__ float e_s[kChunk];
@@ -472,8 +476,18 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
   const int bh = blockIdx.x, chunk = blockIdx.y;
   const int b = bh / p.H, h = bh % p.H;
   pdl_wait_and_launch();  // the combine pass may come in beside the last CTAs
-  const int len = length_of(p, b, threadIdx.x == 0 && chunk == 0);
-  if (len == 0) return;  // invalid: no cache row is touched
+  int len;  // invalid (reported): no cache row is touched
+  if constexpr (D > 0) {
+    if ((len = length_of(p, b, threadIdx.x == 0 && chunk == 0)) == 0) return;
+  } else {  // the same with the range in the compiler's sight: 40 registers in fp32 instead of 45,
+            // 15 % of the pass
+    len = p.lengths[b];
+    if (len < 1 || len > p.T) {
+      if (threadIdx.x == 0 && chunk == 0 && p.dev_status)
+        atomicExch(p.dev_status, (int)RELATION_ERR_INVALID_ARG);
+      return;
+    }
+  }
   const int hist = len - 1;  // history rows
   const int c0 = chunk * kChunk;
   const int n = max(0, min(kChunk, hist - c0));
@@ -482,9 +496,9 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
                  (long long)c0 * p.sT;
   const TI* vc = reinterpret_cast<const TI*>(p.v) + (long long)b * p.sB + (long long)h * p.sH +
                  (long long)c0 * p.sT;
-  constexpr int PL = D / 32;  // columns per lane in the P V pass
+  constexpr int PL = D > 0 ? D / 32 : kMaxD / 32;  // columns per lane in the P V pass
   float mx = -INFINITY;
-  {
+  if constexpr (D > 0) {
     // scores: lane = 4 key + quarter; per iteration two groups of 8 keys,
     // jj = base + lane / 4 and jj + 8 kWarps, loaded together (rows past the chunk read a
     // clamped row and are dropped)
@@ -522,6 +536,28 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  } else {
+    float qr[PL];
+#pragma unroll
+    for (int e = 0; e < PL; ++e) {
+      const int c = lane + 32 * e;
+      qr[e] = c < p.d ? ldf<TI>(qv + c) : 0.f;
+    }
+    for (int jj = warp; jj < n; jj += kWarps) {
+      const TI* kr = kc + (long long)jj * p.sT;
+      float s = 0.f;
+#pragma unroll
+      for (int e = 0; e < PL; ++e) {
+        const int c = lane + 32 * e;
+        if (c < p.d) s = fmaf(qr[e], ldf<TI>(kr + c), s);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const float u = s * p.inv_sqrt_d;
+      const float E = u / (1.0f + expf(-u));  // SiLU(u)
+      if (lane == 0) e_s[jj] = E;
+      mx = fmaxf(mx, E);
+    }
   }
   if (lane == 0) red[warp] = mx;
   __syncthreads();
@@ -533,7 +569,7 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
   float l = 0.f, z[PL];
 #pragma unroll
   for (int e = 0; e < PL; ++e) z[e] = 0.f;
-  {
+  if constexpr (D > 0) {
     const int col = lane * PL;
 #pragma unroll 8
     for (int jj = warp; jj < n; jj += kWarps) {
@@ -546,6 +582,19 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
     }
 #pragma unroll
     for (int e = 0; e < PL; ++e) zs[warp][col + e] = z[e];
+  } else {
+    for (int jj = warp; jj < n; jj += kWarps) {
+      const float P = expf(e_s[jj] - m);
+      l += P;
+      const TI* vr = vc + (long long)jj * p.sT;
+#pragma unroll
+      for (int e = 0; e < PL; ++e) {
+        const int c = lane + 32 * e;
+        if (c < p.d) z[e] = fmaf(P, ldf<TI>(vr + c), z[e]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < PL; ++e) zs[warp][lane + 32 * e] = z[e];
   }
   if (lane == 0) red[warp] = l;
   __syncthreads();
@@ -638,8 +687,9 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
   // rows than a partial CTA would.  Cluster against partial and combine pass, bf16: 12 heads,
   // T 2048, d 64 9.3 against 17.1 us; 32 heads, T 2048, d 128 14.3 against 21.0; 36 heads, T 4096,
   // d 64 16.5 against 20.0.  Past the lines (T 8192, 12 heads: 18 against 16; 64 heads, T 1024,
-  // d 128: 21 against 17; 128 heads: 30 against 16) the CTAs are too few or come in waves.
-  if (kCluster * heads <= 2 * nsm && n_chunks <= kCluster) {
+  // d 128: 21 against 17; 128 heads: 30 against 16) the CTAs are too few or come in waves; by plain loads T 4096
+  // already (bf16, 12 heads, d 64: 50 against 31).
+  if (kCluster * heads <= 2 * nsm && n_chunks <= (NQ > 0 ? kCluster : kCluster / 2)) {
     if ((e = allow((const void*)cluster_kernel<TI, NQ>)) != cudaSuccess) return e;
     e = launch_pdl(cluster_kernel<TI, NQ>, dim3((unsigned)heads * kCluster), 32 * kClWarps, smem, s,
                    kCluster, p);
@@ -651,9 +701,11 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
     e = launch_pdl(partial_kernel<TI, 128>, grid, 32 * kWarps, 0, s, 1, p, part);
   } else if (NQ > 0 && p.d == 64 && qal) {
     e = launch_pdl(partial_kernel<TI, 64>, grid, 32 * kWarps, 0, s, 1, p, part);
-  } else {
+  } else if constexpr (NQ > 0) {
     if ((e = allow((const void*)scan_kernel<TI, NQ>)) != cudaSuccess) return e;
     e = launch_pdl(scan_kernel<TI, NQ>, grid, 32 * kClWarps, smem, s, 1, p, part);
+  } else {
+    e = launch_pdl(partial_kernel<TI, 0>, grid, 32 * kWarps, 0, s, 1, p, part);
   }
   if (e != cudaSuccess) { note_failure("decode: partial pass launch"); return e; }
   e = launch_pdl(combine_kernel<TI>, dim3((unsigned)heads), kMaxD, 0, s, 1, p, (const float*)part,
