@@ -19,8 +19,9 @@
 // Otherwise two launches: the partial pass splits each history into chunks of kChunk rows, one
 // CTA per (head, chunk), with (m, l, z) to the workspace; the combine pass (one CTA per head)
 // merges them by the associative (m, l, z) rule of the tiled scan (App. A.3), the chunks' weights
-// a thread each (a serial loop over dependent loads before).  Its CTAs come in
-// while the last partial CTAs run.
+// a thread each (a serial loop over dependent loads before).  It starts when the partial pass has
+// ended: CTAs that come in early (pdl_launch) cost a grid of 512 heads 0.7 to 1.7 us and gain
+// nothing elsewhere.
 // Measured in one graph over caches that together exceed L2, bf16, before -> now:
 // B 1, H 12, T 2048, d 64 18.6 -> 9.3 us; B 1, H 32, T 2048, d 80 78 -> 12.8;
 // B 32, H 8, T 2048, d 80 148 -> 58.6; B 1, H 16, T 32768, d 128 92.7 -> 64.8;
@@ -447,7 +448,7 @@ template <typename TI, int NQ>
 __global__ void __launch_bounds__(32 * kClWarps) scan_kernel(DecodeProblem p, float* part) {
   __shared__ Smem sm;
   extern __shared__ uint4 ring[];
-  pdl_wait_and_launch();  // the combine pass may come in beside the last CTAs
+  pdl_wait();
   const int bh = blockIdx.x, chunk = blockIdx.y, b = bh / p.H, h = bh % p.H;
   const int len = length_of(p, b, threadIdx.x == 0 && chunk == 0);
   const int c0 = chunk * kChunk, n = min(kChunk, len - 1 - c0);
@@ -475,7 +476,7 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.x, chunk = blockIdx.y;
   const int b = bh / p.H, h = bh % p.H;
-  pdl_wait_and_launch();  // the combine pass may come in beside the last CTAs
+  pdl_wait();
   int len;  // invalid (reported): no cache row is touched
   if constexpr (D > 0) {
     if ((len = length_of(p, b, threadIdx.x == 0 && chunk == 0)) == 0) return;
@@ -683,13 +684,17 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
     if (r != cudaSuccess) note_failure("decode: shared memory");
     return r;
   };
-  // One launch while its CTAs are all resident at once (two per SM fit) and a CTA has no more
-  // rows than a partial CTA would.  Cluster against partial and combine pass, bf16: 12 heads,
-  // T 2048, d 64 9.3 against 17.1 us; 32 heads, T 2048, d 128 14.3 against 21.0; 36 heads, T 4096,
-  // d 64 16.5 against 20.0.  Past the lines (T 8192, 12 heads: 18 against 16; 64 heads, T 1024,
-  // d 128: 21 against 17; 128 heads: 30 against 16) the CTAs are too few or come in waves; by plain loads T 4096
-  // already (bf16, 12 heads, d 64: 50 against 31).
-  if (kCluster * heads <= 2 * nsm && n_chunks <= (NQ > 0 ? kCluster : kCluster / 2)) {
+  // One launch while its CTAs are all resident at once (two per SM fit) and a CTA has no more than
+  // half of a partial CTA's rows, or as many where the heads are few.  us, cluster against partial
+  // and combine pass, caches that exceed L2 / a cache that stays in it, bf16: 12 heads, T 2048, d 64
+  // 8.9 against 17.8 / 8.5 against 10.8; 32 heads, T 2048, d 128 15.8 against 20.8 / 14.8 against
+  // 13.1; 12 heads, T 4096, d 64 12.6 against 16.4 / 12.3 against 10.8.  Past the lines (32 heads,
+  // T 4096, d 128: 24.7 against 22.7 / 23.6 against 16.6; fp32, 16 heads: 26.5 against 24.9; T 8192,
+  // 12 heads: 18 against 16; 64 heads, T 1024, d 128: 21 against 17) the CTAs are too few or come in
+  // waves.
+  if (kCluster * heads <= 2 * nsm &&
+      (n_chunks <= kCluster / 2 ||
+       (NQ > 0 && n_chunks <= kCluster && heads * p.d * (long long)sizeof(TI) <= 2048))) {
     if ((e = allow((const void*)cluster_kernel<TI, NQ>)) != cudaSuccess) return e;
     e = launch_pdl(cluster_kernel<TI, NQ>, dim3((unsigned)heads * kCluster), 32 * kClWarps, smem, s,
                    kCluster, p);
