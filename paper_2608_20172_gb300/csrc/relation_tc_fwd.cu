@@ -874,10 +874,19 @@ static cudaError_t fwd_t(const Problem& p, const StateArgs& sa, cudaStream_t s) 
   // H 8, T 640, d 128 17.3 -> 16.0; H 16, T 1024 22.8 -> 20.1; H 4, T 1536 28.9 -> 19.3; H 6, T 2048,
   // d 80 36 -> 25.  Past the lines: H 12, T 384, d 64 12.0 -> 12.7; H 16, T 512, d 128 (warm) 12.9 ->
   // 13.7; H 2, T 2048, d 128 in eight 20.4 instead of 18.0; H 16, T 1024 in four 35.7.
-  const int most = MODE == 0 || sa.causal ? n_qt : (sa.Tk + BN - 1) / BN;  // key tiles of a row
+  // Short rows split unevenly (five tiles: two and three) and gain less than a second CTA on
+  // every SM costs: below six key tiles the split stops at half of the places, and with rows all of
+  // one length (no causal mask: the unsplit tiles take one round anyway) below twelve, d_h = 128 ten.
+  // One CTA -> two, us: H 32, T 640, d 64 17.8 -> 18.5; H 64, T 512 16.4 -> 20.6; H 24, T 640, d 128
+  // 16.1 -> 18.4; summaries of H 40, T 777, d 64 27.1 -> 32.4; H 16, T 777, d 128 18.4 -> 21.7; beyond:
+  // H 32, T 777, d 64 22.9 -> 21.4; H 16, T 1024, d 128 21.1 -> 20.3; H 12, T 1536 26.7 -> 25.2.
+  const bool causal = MODE == 0 || sa.causal;
+  const int most = causal ? n_qt : (sa.Tk + BN - 1) / BN;  // key tiles of a row
   constexpr int kShare2 = FwdCfg<D>::QUAD ? 4 : 5;  // half key tiles
+  const int few = causal ? 6 : FwdCfg<D>::QUAD ? 12 : 10;
+  const int places = most < few ? slots / 2 : slots;
   int split = 1;
-  while (split < kMaxSplit && kShare2 * 2 * split <= 2 * most && 2 * split * tiles <= slots) split *= 2;
+  while (split < kMaxSplit && kShare2 * 2 * split <= 2 * most && 2 * split * tiles <= places) split *= 2;
   return split > 1 ? launch_t<D, MODE, true>(p, sa, n_qt, (unsigned)tiles, split, groups, s)
                    : launch_t<D, MODE, false>(p, sa, n_qt, (unsigned)tiles, 1, groups, s);
 }
