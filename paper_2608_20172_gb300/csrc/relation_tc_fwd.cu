@@ -697,7 +697,9 @@ __global__ void __launch_bounds__(FwdCfg<D>::THREADS, FwdCfg<D>::CTAS)
       for (int k = 0; k < kMaxSplit; ++k) m = fmaxf(m, w[k]);
 #pragma unroll
       for (int k = 0; k < kMaxSplit; ++k) {
-        w[k] = w[k] == -INFINITY ? 0.f : ex2_approx(w[k] - m);  // (0: no z there either)
+        // no key seen (l = 0): 0, and no z there; m is -inf too where every score so far is NaN
+        // (l NaN): NaN, so that it reaches the row
+        w[k] = w[k] == -INFINITY ? 0.f * lk[k] : ex2_approx(w[k] - m);
         l = w[k] == 0.f ? l : fmaf(w[k], lk[k], l);
       }
       float g = 0.f, inv_l = 0.f, fself = 1.0f, lz = 0.f;
