@@ -320,12 +320,13 @@ __global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) fwd_k
           mt = fmaxf(mt, e[r][i]);
         }
         const float mn = fmaxf(m[r], row_max(mt));
-        // no history seen yet (mn = -inf): every weight is 0
-        sc[r] = mn == -INFINITY ? 1.f : expf(m[r] - mn);
+        // no history seen yet (mn = -inf): every weight is 0, but for a NaN score's
+        const float ms = mn == -INFINITY ? 0.f : mn;
+        sc[r] = expf(m[r] - ms);
         float ls = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float w = mn == -INFINITY ? 0.f : expf(e[r][i] - mn);
+          const float w = expf(e[r][i] - ms);
           ls += w;
           Pw[(4 * ty + r) * PW + 16 * i + tx] = w;
         }
@@ -374,8 +375,9 @@ __global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) fwd_k
     for (int r = 0; r < 4; ++r) {
       const float4 o = *reinterpret_cast<const float4*>(st + 4 * r);
       u_self[r] += o.z;
-      if (o.x == -INFINITY) continue;  // no history there
-      const float mn = fmaxf(m[r], o.x), a = m[r] == -INFINITY ? 0.f : expf(m[r] - mn), b2 = expf(o.x - mn);
+      // (no history there: a factor of 0; l and z are 0 then, or NaN where every score was)
+      const float mn = fmaxf(m[r], o.x), a = m[r] == -INFINITY ? 0.f : expf(m[r] - mn);
+      const float b2 = o.x == -INFINITY ? 0.f : expf(o.x - mn);
       float zo[D / 16];
       load_cols<float, D>(zs + r * LD, tx, zo);
       m[r] = mn;

@@ -50,3 +50,18 @@ def test_nan_key_split(T, d, j):
     bad = _rows(y)
     assert bool(bad[j + 1:].all()) and not bool(bad[:j].any())
     assert torch.equal(y[0, :j], y0[0, :j])
+
+
+# T 65 and 70: the second group of warps has one to six keys of the last rows; T 300: several tiles;
+# many heads: one group
+@pytest.mark.parametrize("T,d,H,j", [(70, 64, 1, 64), (70, 32, 1, 0), (300, 64, 1, 64), (300, 128, 1, 192),
+                                     (300, 64, 256, 64), (40, 64, 1, 0)])
+def test_nan_key_simt(T, d, H, j):
+    q, k, v = _inputs(T, H, d, torch.float32, T + j)
+    y0, _ = binding.fwd(q, k, v, LAM)
+    k[0, j] = float("nan")
+    y, _ = binding.fwd(q, k, v, LAM)
+    torch.cuda.synchronize()
+    bad = _rows(y)
+    assert bool(bad[j + 1:].all()) and not bool(bad[:j].any())
+    assert torch.equal(y[0, :j], y0[0, :j])
