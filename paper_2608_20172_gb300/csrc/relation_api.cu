@@ -248,7 +248,11 @@ relation_status relation_linear_fwd_ws(const void* p1, const void* p2, const voi
   // 84 pairs, T 2048 66 / 74; 96 76 / 74; 144 108 / 78; 156 112 / 139; 216 152 / 142; 60 pairs,
   // T 640 22 / 26; 72 28 / 26.  d_h = 128, T 2048: 80 132 / 144; 96 157 / 147; 160 249 / 277.
   const long long per_block = shp.d_h == 64 ? 152 : 161, fixed = shp.d_h == 64 ? 175 : 200;
-  if (100 * waves * nb * nsm <= fixed * nsm + per_block * ctas * nb)
+  // A stride below 1 (one entry along it: 0 is as good as any) is refused by the sequential entry
+  // point and taken by the passes: there the choice goes by the number of pairs alone, as it did
+  // before it went by cost, so that the same calls are refused.
+  const bool strided = shp.sB >= 1 && shp.sT >= 1 && shp.sH >= 1;
+  if (strided ? 100 * waves * nb * nsm <= fixed * nsm + per_block * ctas * nb : 2 * ctas >= nsm)
     return relation_linear_fwd_ex(p1, p2, v, alpha, y, tau_s, shp, dt, RELATION_KERNEL_TCGEN05,
                                   dev_status, stream);
   relation_status st;

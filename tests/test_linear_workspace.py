@@ -58,3 +58,24 @@ def test_workspace_at_any_16_byte_boundary(past):
     ref = binding.linear_bwd(p1, p2, v, alpha, dy, kernel="tcgen05")
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(got, ref)) and outside(buf, at, need)
+
+
+@pytest.mark.gpu
+def test_stride_zero_along_one_entry():
+    """A stride of 0 along a dimension of one entry: taken with few (head, column) pairs whatever the
+    length, with the result of a plain stride, and refused with half as many pairs as SMs or more."""
+    dev = torch.device("cuda:0")
+    for T, H, ok in ((100, 3, True), (700, 3, True), (2048, 80, False), (100, 80, False)):
+        g = torch.Generator().manual_seed(T + H)
+        p1, p2, v = (torch.randn((1, T, H, 64), generator=g).to(torch.bfloat16).to(dev) for _ in range(3))
+        alpha = (1.0 - 0.1 * torch.rand((1, T, H, 64), generator=g)).to(dev)
+        x = [t.as_strided(t.shape, (0,) + t.stride()[1:]) for t in (p1, p2, v, alpha)]
+        if not ok:
+            with pytest.raises(binding.RelationError) as e:
+                binding.linear_fwd_ws(*x)
+            assert e.value.code == binding.ERR_INVALID_ARG
+            continue
+        y = binding.linear_fwd_ws(*x)
+        ref = binding.linear_fwd_ws(p1, p2, v, alpha)
+        torch.cuda.synchronize()
+        assert float((y.float() - ref.float()).abs().max()) <= 2.0 ** -6 * float(ref.float().abs().max())
