@@ -382,7 +382,29 @@ Args args_of(const LayerProblem& p) {
   return ar;
 }
 
-int ctas(const LayerProblem& p, int tok) { return p.B * ((p.T + tok - 1) / tok); }
+int per_sequence(const LayerProblem& p, int tok) { return p.T / tok + (p.T % tok != 0); }
+
+// A grid holds 2^31 - 1 CTAs, two for every `tok` positions of a sequence: more sequences than that
+// come in several launches.
+template <typename K>
+cudaError_t launch_sequences(K kernel, const LayerProblem& p, int tok, unsigned threads, cudaStream_t s) {
+  Args ar = args_of(p);
+  const int per = per_sequence(p, tok), most = 0x7fffffff / (2 * per);
+  const long long esz = p.dtype == RELATION_F32 ? 4 : 2;
+  for (long long b = 0; b < p.B; b += most) {
+    const int n = (int)(p.B - b < most ? p.B - b : most);
+    const long long off = b * p.sB * esz;
+    auto in = [&](const void* x) -> const void* { return x ? static_cast<const char*>(x) + off : x; };
+    auto out = [&](void* x) -> void* { return x ? static_cast<char*>(x) + off : x; };
+    ar.p.B = n;
+    ar.p.in1 = in(p.in1); ar.p.in2 = in(p.in2); ar.p.in3 = in(p.in3); ar.p.in4 = in(p.in4);
+    ar.p.out1 = out(p.out1); ar.p.out2 = out(p.out2); ar.p.out3 = out(p.out3);
+    if (p.dtheta_part) ar.p.dtheta_part = p.dtheta_part + b * per * (p.H / 2);
+    const cudaError_t e = launch_pdl(kernel, dim3(2u * n * per), threads, 0, s, 1, ar);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 }  // namespace layer
 
@@ -396,27 +418,20 @@ size_t layer_grad_workspace_bytes(int B, int T, int H) {
 }
 
 cudaError_t launch_layer_prep(const LayerProblem& p, cudaStream_t s) {
-  const int grid = layer::ctas(p, layer::kPrepTok);
-  const layer::Args ar = layer::args_of(p);
-  cudaError_t e;
-  if (p.dtype == RELATION_F32)
-    e = launch_pdl(layer::prep_kernel<float>, dim3(2 * grid), layer::kPrepThreads, 0, s, 1, ar);
-  else
-    e = launch_pdl(layer::prep_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kPrepThreads, 0, s, 1, ar);
+  const cudaError_t e = layer::launch_sequences(
+      p.dtype == RELATION_F32 ? layer::prep_kernel<float> : layer::prep_kernel<__nv_bfloat16>, p,
+      layer::kPrepTok, layer::kPrepThreads, s);
   if (e != cudaSuccess) note_failure("layer prep: launch");
   return e;
 }
 
 cudaError_t launch_layer_grad(const LayerProblem& p, cudaStream_t s) {
-  const int grid = layer::ctas(p, layer::kTok);
-  const layer::Args ar = layer::args_of(p);
-  cudaError_t e;
-  if (p.dtype == RELATION_F32)
-    e = launch_pdl(layer::grad_kernel<float>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
-  else
-    e = launch_pdl(layer::grad_kernel<__nv_bfloat16>, dim3(2 * grid), layer::kThreads, 0, s, 1, ar);
+  cudaError_t e = layer::launch_sequences(
+      p.dtype == RELATION_F32 ? layer::grad_kernel<float> : layer::grad_kernel<__nv_bfloat16>, p,
+      layer::kTok, layer::kThreads, s);
   if (e != cudaSuccess) { note_failure("layer grad: launch"); return e; }
-  e = launch_pdl(layer::dtheta_kernel, dim3(p.H / 2), 256, 0, s, 1, p, grid);
+  e = launch_pdl(layer::dtheta_kernel, dim3(p.H / 2), 256, 0, s, 1, p,
+                 p.B * layer::per_sequence(p, layer::kTok));
   if (e != cudaSuccess) note_failure("layer grad: dtheta launch");
   return e;
 }
