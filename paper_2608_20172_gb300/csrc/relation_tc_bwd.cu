@@ -453,9 +453,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, 1)
         load_kv_tmem(x);
       }
       // d_h = 64: U^T / dP^T of step sn may be issued once its buffer is free (step
-      // sn - NBUF done) and once the GEMM that releases the Q / dO stage it loads into has
-      // been issued (two tiles back: always by then); waiting for that stage's load earlier
-      // would deadlock.
+      // sn - NBUF done) and once the GEMM that releases the Q / dO stage it loads into, NQS
+      // tiles back, has been issued; waiting for that stage's load earlier would deadlock.
+      // Behind step s the steps up to s + NBUF are issued, with (s + 1) / SPT tiles released;
+      // ahead of a unit's last dQ the next unit's first NBUF, with all tiles but one:
+      static_assert(C::HALF || C::NBUF <= (C::NQS - 1) * C::SPT + 1, "step s + NBUF's stage");
+      static_assert(C::HALF || (C::NBUF - 1) / C::SPT <= C::NQS - 2, "the next unit's stages");
       int sn = pre;
       pre = 0;
       while (ok && sn < total && sn < C::NBUF) {
