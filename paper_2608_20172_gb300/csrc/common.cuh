@@ -36,12 +36,14 @@ __device__ __forceinline__ void pdl_wait_and_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Compensated sum of a few floats: s the rounded sum, c the sum of the additions' errors.
+// Compensated sum of a few floats: s the rounded sum, c the sum of the additions' errors.  Every
+// product and sum whose rounding error is taken is rounded on its own (the _rn forms are never
+// contracted to a multiply-add, which would round otherwise).
 struct Sum2 {
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float t = s + x, z = t - s;
-    c += (s - (t - z)) + (x - z);
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
     s = t;
   }
   // + f * log(x) for x > 0: x = 2^e y with y near 1, so that e ln 2 (ln 2 as a sum of two floats)
@@ -55,7 +57,7 @@ struct Sum2 {
       y *= 2.f;
       --e;
     }
-    const float a = (float)e * kLn2, b = logf(y), fa = f * a, fb = f * b;
+    const float a = __fmul_rn((float)e, kLn2), b = logf(y), fa = __fmul_rn(f, a), fb = __fmul_rn(f, b);
     add(fa);
     add(fb);
     c += fmaf(f, a, -fa) + fmaf(f, b, -fb) +

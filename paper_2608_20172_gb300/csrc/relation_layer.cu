@@ -93,16 +93,17 @@ struct Args {
 // m * w modulo 2 pi (|r| <= pi + rounding) for a position m < 2^22 and w = w_hi + w_lo <= 1:
 // the product and n 2 pi are kept as rounded value and exact remainder (two-product by fma;
 // their leading parts are close, so that their difference is exact), 2 pi as a sum of two
-// floats (48 bits, n < 2^20: 2 pi's tail adds less than 2^-24).
+// floats (48 bits, n < 2^20: 2 pi's tail adds less than 2^-24).  The _rn forms: a product that was
+// contracted into the difference would have its remainder counted twice.
 __device__ __forceinline__ float turn(float m, float w_hi, float w_lo) {
   constexpr float kTwoPiHi = 6.28318530717958647692f;
   constexpr float kTwoPiLo = (float)(6.28318530717958647692 - (double)kTwoPiHi);
-  const float a = m * w_hi;
+  const float a = __fmul_rn(m, w_hi);
   const float a_lo = fmaf(m, w_lo, fmaf(m, w_hi, -a));
-  const float n = rintf(a * 0.15915494309189533577f);
-  const float q = n * kTwoPiHi;
+  const float n = rintf(__fmul_rn(a, 0.15915494309189533577f));
+  const float q = __fmul_rn(n, kTwoPiHi);
   const float q_lo = fmaf(n, kTwoPiLo, fmaf(n, kTwoPiHi, -q));
-  return (a - q) + (a_lo - q_lo);
+  return __fadd_rn(__fsub_rn(a, q), __fsub_rn(a_lo, q_lo));
 }
 
 // cos / sin of m * base^(-2c/d) for the CTA's positions
