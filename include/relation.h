@@ -314,7 +314,8 @@ relation_status relation_state_finish(const void* q, const void* k, const void* 
  *       may alias its input (q = p1, k = p2, v = info).
  *   theta : device float[H/2], fp32.
  * H even, d_h a multiple of 8 up to 256, H/2 <= 128; fp32 or bf16 (rotations in fp32; the
- * RoPE angles are reduced modulo 2 pi in fp64).  Other shapes: RELATION_ERR_UNSUPPORTED.
+ * RoPE angles are formed and reduced modulo 2 pi in 48 bits, as sums of two floats, up to
+ * position 32767 and in fp64 from there on and for bases below 1).  Other shapes: RELATION_ERR_UNSUPPORTED.
  * Asynchronous on `stream`; nothing is allocated.
  */
 relation_status relation_layer_prep(const void* p1, const void* p2, const void* info,

@@ -17,8 +17,8 @@
 // vectors (16 bytes in bf16).  The rotation angles of the CTA's positions are tabulated
 // once in shared memory and reused by every head: m * base^(-2c/d) is formed and reduced
 // modulo 2 pi as a sum of two floats (positions reach 16k, where an fp32 angle would be off
-// by ~1e-3 rad) from frequencies that come with the launch, then its cosine and sine are
-// taken in fp32.  (In fp64, with an fp64 log and exp per CTA, this chip's fp64 pipe bounded
+// by ~1e-3 rad; past 32k in fp64) from frequencies that come with the launch, then its cosine and
+// sine are taken in fp32.  (In fp64, with an fp64 log and exp per CTA, this chip's fp64 pipe bounded
 // both passes; the rotations and the mixing are CTAs of their own, so that the tables hide.
 // B 4, H 8, T 4096, d 80: prep 48 -> 26 us, grad 63 -> 36; B 2, H 16, T 16384, d 128: 159 ->
 // 122 us (6.6 TB/s), 196 -> 149 (6.3).)  dtheta is summed per CTA in a fixed
@@ -90,11 +90,16 @@ struct Args {
   float w_hi[kMaxD / 2], w_lo[kMaxD / 2];
 };
 
-// m * w modulo 2 pi (|r| <= pi + rounding) for a position m < 2^22 and w = w_hi + w_lo <= 1:
-// the product and n 2 pi are kept as rounded value and exact remainder (two-product by fma;
-// their leading parts are close, so that their difference is exact), 2 pi as a sum of two
-// floats (48 bits, n < 2^20: 2 pi's tail adds less than 2^-24).  The _rn forms: a product that was
-// contracted into the difference would have its remainder counted twice.
+// Positions whose angles come from turn: up to there they are as exact as fp64's, both being
+// rounded to fp32 in the end (against 64 bits over d 48 to 256, bases 1 to 5e5: rms 4.66e-8 rad with
+// either, at most 1.193e-7 against 1.192e-7 below 2^15 positions; 1.20e-7 at 2^17, 1.49e-7 at 2^22).
+constexpr int kTurnPositions = 1 << 15;
+
+// m * w modulo 2 pi (|r| <= pi + rounding) for a position m and w = w_hi + w_lo <= 1: the product
+// and n 2 pi are kept as rounded value and exact remainder (two-product by fma; their leading
+// parts are close, so that their difference is exact), 2 pi as a sum of two floats (48 bits).
+// The _rn forms: a product that was contracted into the difference would have its remainder
+// counted twice.
 __device__ __forceinline__ float turn(float m, float w_hi, float w_lo) {
   constexpr float kTwoPiHi = 6.28318530717958647692f;
   constexpr float kTwoPiLo = (float)(6.28318530717958647692 - (double)kTwoPiHi);
@@ -114,7 +119,7 @@ __device__ __forceinline__ void fill_tables(Tables<TOK>& tb, const Args& ar, int
   for (int e = threadIdx.x; e < TOK * half; e += NT) {
     const int tt = e / half, c = e % half;
     float r;
-    if (t0 < (1 << 22) - TOK && p.rope_base >= 1.0f) {
+    if (t0 < kTurnPositions && p.rope_base >= 1.0f) {
       r = turn((float)(t0 + tt), ar.w_hi[c], ar.w_lo[c]);
     } else {  // positions or frequencies past turn's range: fp64
       const double a = (double)(t0 + tt) * exp(-2.0 * (double)c / (double)p.d * log((double)p.rope_base));
