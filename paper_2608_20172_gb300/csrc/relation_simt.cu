@@ -238,6 +238,13 @@ __device__ __forceinline__ void axpys(const float* w, const float* b, int ty, in
   }
 }
 
+// Maximum that keeps a NaN (fmaxf drops it): a NaN score makes its row's scale NaN, and so all of
+// the row's weights, also where no other score has been seen
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
 // Sum / maximum over the 16 lanes that share a row
 __device__ __forceinline__ float row_sum(float x) {
 #pragma unroll
@@ -246,7 +253,7 @@ __device__ __forceinline__ float row_sum(float x) {
 }
 __device__ __forceinline__ float row_max(float x) {
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  for (int o = 8; o > 0; o >>= 1) x = max_nan(x, __shfl_xor_sync(0xffffffffu, x, o));
   return x;
 }
 
@@ -317,16 +324,15 @@ __global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) fwd_k
           const float ev = u * sigmoidf_acc(u);        // E_ij = SiLU(U_ij)
           e[r][i] = j < r0 + r ? ev : -INFINITY;
           u_self[r] = j == r0 + r ? u : u_self[r];
-          mt = fmaxf(mt, e[r][i]);
+          mt = max_nan(mt, e[r][i]);
         }
-        const float mn = fmaxf(m[r], row_max(mt));
-        // no history seen yet (mn = -inf): every weight is 0, but for a NaN score's
-        const float ms = mn == -INFINITY ? 0.f : mn;
-        sc[r] = expf(m[r] - ms);
+        const float mn = max_nan(m[r], row_max(mt));
+        // no history seen yet (mn = -inf): every weight is 0
+        sc[r] = mn == -INFINITY ? 1.f : expf(m[r] - mn);
         float ls = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float w = expf(e[r][i] - ms);
+          const float w = mn == -INFINITY ? 0.f : expf(e[r][i] - mn);
           ls += w;
           Pw[(4 * ty + r) * PW + 16 * i + tx] = w;
         }
@@ -375,9 +381,8 @@ __global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) fwd_k
     for (int r = 0; r < 4; ++r) {
       const float4 o = *reinterpret_cast<const float4*>(st + 4 * r);
       u_self[r] += o.z;
-      // (no history there: a factor of 0; l and z are 0 then, or NaN where every score was)
-      const float mn = fmaxf(m[r], o.x), a = m[r] == -INFINITY ? 0.f : expf(m[r] - mn);
-      const float b2 = o.x == -INFINITY ? 0.f : expf(o.x - mn);
+      if (o.x == -INFINITY) continue;  // no history there
+      const float mn = max_nan(m[r], o.x), a = m[r] == -INFINITY ? 0.f : expf(m[r] - mn), b2 = expf(o.x - mn);
       float zo[D / 16];
       load_cols<float, D>(zs + r * LD, tx, zo);
       m[r] = mn;
