@@ -15,7 +15,7 @@
 // [8][64] buffer.  Bound: shared-memory bandwidth and the FP32 pipe (backward: 78 % of the
 // wavefronts, 58 % of the pipe), 2 + 7 products of d_h over the causal pairs (forward +
 // backward); in small grids, the chain of tiles of the longest rows, which two groups of warps
-// then share (two_groups).  Measured, B 2, H 8, T 1000, d 64, forward + backward: 1478 -> 293 us
+// then share (two_groups, by measured lines).  Measured, B 2, H 8, T 1000, d 64, forward + backward: 1478 -> 293 us
 // (forward 567 -> 80, backward tiles 920 -> 210) against a thread per quarter row (one 16-byte
 // shared read per four multiply-adds, two shuffles per entry); B 1, H 2, T 128, d 32: 49 -> 9 and
 // 77 -> 11 us.
@@ -734,18 +734,25 @@ static int tiles(const Problem& p) {
   return (p.T + kWarpRows * kWarps - 1) / (kWarpRows * kWarps);
 }
 
-// Two groups per CTA where the longest row's chain of tiles decides: more than one tile, and no
-// more CTAs than are resident at once (`per_sm` of them on each SM).  Elsewhere they only cost
-// registers and the joining.  us with one and with two groups.  Forward: B 1, H 4, T 1000, d 64
-// 74 / 52; B 2, H 8, T 1000 (512 CTAs) 106 / 80; B 4, H 8 (1024) 139 / 149; B 2, H 4, T 777, d 128
-// (200) 94 / 72; B 4 (400) 108 / 111.  Backward: B 1, H 4, T 1000 (256) 184 / 133; B 2, H 8 (1024)
-// 210 / 218; B 2, H 4, T 777, d 128 (400) 198 / 148; B 4 (800) 261 / 282.
-static bool two_groups(const Problem& p, long long ctas, int per_sm) {
+// Two groups per CTA where the longest row's chain of tiles decides, which it does up to some number
+// of CTAs per SM.  Beyond it two groups only cost residency (at d 64 two of their CTAs fit an SM, for
+// four (forward) and three (backward) of one group; at d 128 one for two), registers and the
+// joining.  The lines are where both forms take the same time, measured with each forced, and lie
+// lower up to 128 tokens: two tiles, little to share.  us with one and with two groups, below the
+// line and above it (B H, T):
+//   forward, d <= 64:  T <= 128, 2 per SM: 64, 128 14.0 / 12.9, 96, 128 17.0 / 21.5;
+//                      longer, 4: 16, 1000 98 / 81, 48, 500 59 / 68
+//   forward, d 128:    1: 32, 128 17.0 / 15.4, 48, 128 19.3 / 23.9; 2: 16, 500 61 / 53, 24, 500 67 / 76
+//   backward, d <= 64: 3: 48, 128 33.1 / 28.4, 64, 128 34.5 / 34.4; 5: 12, 777 161 / 117,
+//                      16, 1000 210 / 218
+//   backward, d 128:   2: 32, 128 40.0 / 35.7, 48, 128 40.5 / 47.1; 3: 8, 777 197 / 148,
+//                      16, 640 168 / 185
+static bool two_groups(const Problem& p, long long ctas, int short_per_sm, int per_sm) {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     nsm = 0;
-  return p.T > kTile && ctas <= (long long)per_sm * nsm;
+  return p.T > kTile && ctas <= (long long)(p.T > 2 * kTile ? per_sm : short_per_sm) * nsm;
 }
 
 template <typename TI, int D, int NG>
@@ -775,7 +782,7 @@ template <typename TI, int D>
 static cudaError_t fwd_t(const Problem& p, cudaStream_t s) {
   const long long grid = (long long)tiles(p) * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return two_groups(p, grid, D < 128 ? 4 : 2) ? fwd_g<TI, D, 2>(p, (unsigned)grid, s)
+  return two_groups(p, grid, D < 128 ? 2 : 1, D < 128 ? 4 : 2) ? fwd_g<TI, D, 2>(p, (unsigned)grid, s)
                              : fwd_g<TI, D, 1>(p, (unsigned)grid, s);
 }
 
@@ -783,7 +790,7 @@ template <typename TI, int D>
 static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
   const long long grid = 2LL * tiles(p) * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return two_groups(p, grid, D < 128 ? 4 : 3) ? bwd_g<TI, D, 2>(p, ws, (unsigned)grid, s)
+  return two_groups(p, grid, D < 128 ? 3 : 2, D < 128 ? 5 : 3) ? bwd_g<TI, D, 2>(p, ws, (unsigned)grid, s)
                              : bwd_g<TI, D, 1>(p, ws, (unsigned)grid, s);
 }
 
