@@ -98,7 +98,11 @@ struct IO<__nv_bfloat16> {
 };
 
 // The denominator is at least 1: __fdividef (2 ulp, 0 for a denominator above 2^126) takes no
-// branch, so that a lane's 16 entries overlap; the IEEE division's range check kept them apart.
+// branch, so that a lane's 16 entries overlap; the IEEE division's range check kept them apart and
+// costs 12 % of the forward and 5 % of the backward.  Against 64 bits over 42 inputs (d 32 to 128,
+// T 33 to 2048) the outputs' errors are those with the IEEE division: Y 2.379e-7 and 2.377e-7 (rms of
+// the relative errors), logZ 4.42e-8 and 4.44e-8, dQ 3.400e-7 and 3.399e-7, dK 5.087e-7 and 5.082e-7,
+// dV 3.163e-7 and 3.162e-7; the rounding of the products over d and of expf decides them.
 __device__ __forceinline__ float sigmoidf_acc(float x) { return __fdividef(1.0f, 1.0f + expf(-x)); }
 
 // A lane's columns of a row of D: D = 32: 2 tx .., D = 64: 4 tx .., D = 128: 4 tx .. and
