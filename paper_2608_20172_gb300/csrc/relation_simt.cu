@@ -798,8 +798,9 @@ static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t 
                              : bwd_g<TI, D, 1>(p, ws, (unsigned)grid, s);
 }
 
-// The tile kernel's dlambda partials, one per dK / dV CTA (at most one per 16 rows): in the
-// tensor-core path's per-query scalars (four floats per row), which this path does not use.
+// The tile kernel's dlambda partials, one per dK / dV CTA and its 32 rows: in the tensor-core path's
+// per-query scalars (four floats per row, rows padded to 128), which this path does not use.
+static_assert(128 % (kWarpRows * kWarps) == 0, "a head's partials end within its padded rows");
 float* main_partials(const BwdWorkspace& ws) { return ws.stats; }
 int main_ctas(const Problem& p) { return tiles(p) * p.B * p.H; }
 
