@@ -616,7 +616,7 @@ def linear_measure(binding, dev, peaks, steps=20, warmup=3):
                                              "where that takes less time)",
                                    "H": 12, "d_h": 64,
                                    "tokens_per_point": LINEAR_SWEEP_TOKENS, "points": sweep},
-            "gpu_launches_per_step": {"fwd_chunked": 1, "bwd_chunked": 5, "fwd": 1, "bwd": 2}}
+            "gpu_launches_per_step": {"fwd_chunked": 1, "bwd_chunked": 3, "fwd": 1, "bwd": 2}}
 
 
 def measure_workload(binding, w, dev, steps, warmup, family, peaks, dist=None, ws=1,
