@@ -719,6 +719,19 @@ __global__ void __launch_bounds__(32 * W * NG, NG == 2 && D < 128 ? 2 : 0) bwd_k
     bwd_dkdv<TI, D, W, NG>(p, ws, dlam_part, smem, t, bh);
 }
 
+// dQ in the place of Q or dO, which the dK / dV CTAs of every earlier key read: a launch of its own
+// behind theirs.  (A kernel for each: a switch in bwd_kernel costs it registers, 20 % at d 32.)
+template <typename TI, int D, int W, bool DQ>
+__global__ void __launch_bounds__(32 * W) bwd_part_kernel(Problem p, BwdWorkspace ws, float* dlam_part, int n_t) {
+  extern __shared__ float4 smem_f4[];
+  const int BH = p.B * p.H, t = (int)(blockIdx.x / BH), bh = (int)(blockIdx.x % BH);
+  pdl_wait();
+  if (DQ)
+    bwd_dq<TI, D, W, 1>(p, ws, reinterpret_cast<float*>(smem_f4), n_t - 1 - t, bh);
+  else
+    bwd_dkdv<TI, D, W, 1>(p, ws, dlam_part, reinterpret_cast<float*>(smem_f4), t, bh);
+}
+
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
@@ -782,6 +795,17 @@ static cudaError_t bwd_g(const Problem& p, const BwdWorkspace& ws, unsigned grid
                     main_partials(ws), tiles(p));
 }
 
+template <typename TI, int D, bool DQ>
+static cudaError_t bwd_part(const Problem& p, const BwdWorkspace& ws, unsigned grid, cudaStream_t s) {
+  constexpr int W = kWarps;
+  constexpr size_t smem = bwd_smem<D, W, 1>();
+  const cudaError_t e = cudaFuncSetAttribute(
+      bwd_part_kernel<TI, D, W, DQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(bwd_part_kernel<TI, D, W, DQ>, dim3(grid), 32 * W, smem, s, 1, p, ws,
+                    main_partials(ws), tiles(p));
+}
+
 template <typename TI, int D>
 static cudaError_t fwd_t(const Problem& p, cudaStream_t s) {
   const long long grid = (long long)tiles(p) * p.B * p.H;
@@ -794,6 +818,10 @@ template <typename TI, int D>
 static cudaError_t bwd_t(const Problem& p, const BwdWorkspace& ws, cudaStream_t s) {
   const long long grid = 2LL * tiles(p) * p.B * p.H;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  if (p.dq == p.q || p.dq == p.dout) {
+    const cudaError_t e = bwd_part<TI, D, false>(p, ws, (unsigned)(grid / 2), s);
+    return e != cudaSuccess ? e : bwd_part<TI, D, true>(p, ws, (unsigned)(grid / 2), s);
+  }
   return two_groups(p, grid, D < 128 ? 3 : 2, D < 128 ? 5 : 3) ? bwd_g<TI, D, 2>(p, ws, (unsigned)grid, s)
                              : bwd_g<TI, D, 1>(p, ws, (unsigned)grid, s);
 }
