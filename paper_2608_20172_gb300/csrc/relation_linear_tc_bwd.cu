@@ -484,7 +484,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float a = __ldg(p.alpha + at);
         const float pq = fix_up(coef + warp * LT, smem + OFF_V, smem + OFF_G, smem + OFF_C0,
                                 smem + OFF_DCP, u, ch, lane);
-        if (lane == 0) p.dalpha[at] = pq / a;
+        // (where dalpha takes alpha's place: kept, in place of the warp's coefficients, until every
+        // alpha of the block has been read)
+        __syncwarp();
+        if (lane == 0) *(p.dalpha == p.alpha ? coef + warp * LT : p.dalpha + at) = pq / a;
       }
       ew_sync<NG>();  // dY has been read: dv takes its place
     }
@@ -724,6 +727,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) p.dalpha[at] = pq / __ldg(p.alpha + at);
         __syncwarp();
       }
+    }
+    if (p.dalpha == p.alpha && ok && warp < n_early && lane == 0) {
+      const int u = fix_early[warp] >> 6, ch = fix_early[warp] & 63;
+      p.dalpha[(long long)b * p.sB + (long long)h * p.sH + (long long)(t0 + u) * p.sT + ch] =
+          coef[warp * LT];
     }
     if (lane == 0) tma_store_wait_read_all();
     if (my_clamp) atomicExch(clamped, 1);
