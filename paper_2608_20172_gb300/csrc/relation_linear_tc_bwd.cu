@@ -156,6 +156,8 @@ __device__ __forceinline__ float fix_up(const float* coef, const uint8_t* v, con
   return pq;
 }
 
+// IN_PLACE: dalpha stands in alpha's place (a kernel of its own: the tests alone cost 1 %).
+template <bool IN_PLACE>
 __global__ void __launch_bounds__(kThreads, 1)
     lin_tc_bwd_kernel(const __grid_constant__ CUtensorMap tmP1,
                       const __grid_constant__ CUtensorMap tmP2,
@@ -484,10 +486,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float a = __ldg(p.alpha + at);
         const float pq = fix_up(coef + warp * LT, smem + OFF_V, smem + OFF_G, smem + OFF_C0,
                                 smem + OFF_DCP, u, ch, lane);
-        // (where dalpha takes alpha's place: kept, in place of the warp's coefficients, until every
-        // alpha of the block has been read)
-        __syncwarp();
-        if (lane == 0) *(p.dalpha == p.alpha ? coef + warp * LT : p.dalpha + at) = pq / a;
+        if (IN_PLACE) __syncwarp();  // kept, in place of the warp's coefficients, until every alpha
+                                     // of the block has been read
+        if (lane == 0) *(IN_PLACE ? coef + warp * LT : p.dalpha + at) = pq / a;
       }
       ew_sync<NG>();  // dY has been read: dv takes its place
     }
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
       }
     }
-    if (p.dalpha == p.alpha && ok && warp < n_early && lane == 0) {
+    if (IN_PLACE && ok && warp < n_early && lane == 0) {
       const int u = fix_early[warp] >> 6, ch = fix_early[warp] & 63;
       p.dalpha[(long long)b * p.sB + (long long)h * p.sH + (long long)(t0 + u) * p.sT + ch] =
           coef[warp * LT];
@@ -772,7 +773,8 @@ cudaError_t launch_linear_tc_bwd(const LinearProblem& p, cudaStream_t s) {
   const long long grid = heads * nb;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(bwd::lin_tc_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  auto* const kernel = p.dalpha == p.alpha ? bwd::lin_tc_bwd_kernel<true> : bwd::lin_tc_bwd_kernel<false>;
+  if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 bwd::SMEM)) != cudaSuccess) {
     note_failure("linear chunked backward: shared memory attribute");
     return e;
@@ -792,7 +794,7 @@ cudaError_t launch_linear_tc_bwd(const LinearProblem& p, cudaStream_t s) {
     note_failure("linear chunked backward: TMA descriptors");
     return cudaErrorInvalidValue;
   }
-  e = launch_pdl(bwd::lin_tc_bwd_kernel, dim3((unsigned)grid), bwd::kThreads, bwd::SMEM, s, 1, m1, m2,
+  e = launch_pdl(kernel, dim3((unsigned)grid), bwd::kThreads, bwd::SMEM, s, 1, m1, m2,
                  mv, mg, ma, mc0, mdc, o1, o2, ov, p, nb);
   if (e != cudaSuccess) note_failure("linear chunked backward: launch");
   return e;
