@@ -23,9 +23,9 @@
 // ended: CTAs that come in early (pdl_launch) cost a grid of 512 heads 0.7 to 1.7 us and gain
 // nothing elsewhere.
 // Measured in one graph over caches that together exceed L2, bf16, before -> now:
-// B 1, H 12, T 2048, d 64 18.6 -> 9.3 us; B 1, H 32, T 2048, d 80 78 -> 12.8;
-// B 32, H 8, T 2048, d 80 148 -> 58.6; B 1, H 16, T 32768, d 128 92.7 -> 64.8;
-// B 32, H 16, T 8192, d 128 (2.1 GB) 334 -> 322 (6.66 TB/s).
+// B 1, H 12, T 2048, d 64 18.6 -> 8.7 us; B 1, H 32, T 2048, d 80 78 -> 13.6;
+// B 32, H 8, T 2048, d 80 148 -> 54.8; B 1, H 16, T 32768, d 128 92.7 -> 56.6 (68.2 with the merge's
+// loads one behind the other); B 32, H 16, T 8192, d 128 (2.1 GB) 331 -> 319 (6.74 TB/s).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -318,7 +318,7 @@ __device__ __forceinline__ float self_dot(const DecodeProblem& p, const TI* qv, 
 // Column c of the new row from the merged (M, L, Z): the Self-Exchange epilogue
 template <typename TI>
 __device__ __forceinline__ void epilogue(const DecodeProblem& p, int bh, int len, float qk, float M,
-                                         float L, float Z, int c, const TI* vs, TI* o) {
+                                         float L, float Z, int c, float vi, TI* o) {
   const float S = 1.0f / (1.0f + expf(-(qk * p.inv_sqrt_d) / p.tau_s));
   float g = 0.f, lz = S, fz = 0.f;
   if (len > 1 && L > 0.f) {
@@ -328,7 +328,6 @@ __device__ __forceinline__ void epilogue(const DecodeProblem& p, int bh, int len
     lz = hi + log1pf(expf(lo - hi));
     fz = Z / L;
   }
-  const float vi = ldf<TI>(vs + c);
   const float y = fmaf(g, fz - vi, vi);
   if (sizeof(TI) == 4)
     reinterpret_cast<float*>(o)[c] = y;
@@ -390,7 +389,7 @@ __global__ void __launch_bounds__(32 * kClWarps) cluster_kernel(DecodeProblem p)
       L = fmaf(w, o->l, L);
       Z = fmaf(w, o->z[c], Z);
     }
-    epilogue<TI>(p, bh, len, sm.self, M, L, Z, c, vh + (long long)(len - 1) * p.sT,
+    epilogue<TI>(p, bh, len, sm.self, M, L, Z, c, ldf<TI>(vh + (long long)(len - 1) * p.sT + c),
                  reinterpret_cast<TI*>(p.out) + (long long)b * p.qsB + (long long)h * p.qsH);
   }
   cl.sync();  // the other CTAs' shared memory has been read
@@ -619,6 +618,7 @@ __global__ void __launch_bounds__(32 * kWarps) partial_kernel(DecodeProblem p, f
 template <typename TI>
 __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const float* part,
                                                         int n_chunks) {
+  constexpr int kAhead = 16;  // chunks' z in flight
   __shared__ float red[kMaxD / 32], w[kMaxD], lw[kMaxD];
   __shared__ float self;
   const int bh = blockIdx.x, c = threadIdx.x, b = bh / p.H, h = bh % p.H;
@@ -630,10 +630,16 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
   if (len == 0) return;
   const TI* qv = reinterpret_cast<const TI*>(p.q) + (long long)b * p.qsB + (long long)h * p.qsH;
   const long long row = (long long)b * p.sB + (long long)h * p.sH + (long long)(len - 1) * p.sT;
-  if (warp == kMaxD / 32 - 1) {  // (beside the first warps' loads of the chunks' weights)
-    const float s = self_dot<TI>(p, qv, reinterpret_cast<const TI*>(p.k) + row, lane);
-    if (lane == 0) self = s;
+  // the new row, in flight during the merge (K's by the last warp, which has no chunk weights to load)
+  const bool own = warp == kMaxD / 32 - 1;
+  float qr[kMaxD / 32], kr[kMaxD / 32];
+#pragma unroll
+  for (int e = 0; e < kMaxD / 32; ++e) {
+    const bool in = own && lane + 32 * e < p.d;
+    qr[e] = in ? ldf<TI>(qv + lane + 32 * e) : 0.f;
+    kr[e] = in ? ldf<TI>(reinterpret_cast<const TI*>(p.k) + row + lane + 32 * e) : 0.f;
   }
+  const float vi = c < p.d ? ldf<TI>(reinterpret_cast<const TI*>(p.v) + row + c) : 0.f;
   const int used = (len - 1 + kChunk - 1) / kChunk;  // <= n_chunks
   const float* pb = part + (long long)bh * n_chunks * (2 + kMaxD);
   float M = -INFINITY;
@@ -643,6 +649,13 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kMaxD / 32; ++i) M = fmaxf(M, red[i]);
+  if (own) {  // Self evidence q . k_i
+    float s = 0.f;
+#pragma unroll
+    for (int e = 0; e < kMaxD / 32; ++e) s = fmaf(qr[e], kr[e], s);
+    s = warp_sum(s);
+    if (lane == 0) self = s;
+  }
   float L = 0.f, Z = 0.f;
   for (int k0 = 0; k0 < used; k0 += kMaxD) {  // kMaxD chunks' weights at a time
     if (k0 > 0) __syncthreads();
@@ -653,15 +666,22 @@ __global__ void __launch_bounds__(kMaxD) combine_kernel(DecodeProblem p, const f
     }
     __syncthreads();
     const int n = min(kMaxD, used - k0);
-#pragma unroll 8
-    for (int k = 0; k < n; ++k) {
-      L = fmaf(w[k], lw[k], L);
-      if (c < p.d) Z = fmaf(w[k], pb[(long long)(k0 + k) * (2 + kMaxD) + 2 + c], Z);
+    for (int k = 0; k < n; k += kAhead) {  // (left to the unroller, the loads came one by one)
+      float zk[kAhead];
+#pragma unroll
+      for (int e = 0; e < kAhead; ++e)
+        zk[e] = k + e < n && c < p.d ? pb[(long long)(k0 + k + e) * (2 + kMaxD) + 2 + c] : 0.f;
+#pragma unroll
+      for (int e = 0; e < kAhead; ++e) {
+        if (k + e >= n) break;
+        L = fmaf(w[k + e], lw[k + e], L);
+        Z = fmaf(w[k + e], zk[e], Z);
+      }
     }
   }
   if (used == 0) __syncthreads();  // self is in (above: the weights' barrier)
   if (c < p.d)
-    epilogue<TI>(p, bh, len, self, M, L, Z, c, reinterpret_cast<const TI*>(p.v) + row,
+    epilogue<TI>(p, bh, len, self, M, L, Z, c, vi,
                  reinterpret_cast<TI*>(p.out) + (long long)b * p.qsB + (long long)h * p.qsH);
 }
 
