@@ -705,16 +705,19 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
     return r;
   };
   // One launch while its CTAs are all resident at once (two per SM fit) and a CTA has no more than
-  // half of a partial CTA's rows, or as many where the heads are few.  us, cluster against partial
-  // and combine pass, caches that exceed L2 / a cache that stays in it, bf16: 12 heads, T 2048, d 64
-  // 8.9 against 17.8 / 8.5 against 10.8; 32 heads, T 2048, d 128 15.8 against 20.8 / 14.8 against
-  // 13.1; 12 heads, T 4096, d 64 12.6 against 16.4 / 12.3 against 10.8.  Past the lines (32 heads,
-  // T 4096, d 128: 24.7 against 22.7 / 23.6 against 16.6; fp32, 16 heads: 26.5 against 24.9; T 8192,
-  // 12 heads: 18 against 16; 64 heads, T 1024, d 128: 21 against 17) the CTAs are too few or come in
-  // waves.
+  // half of a partial CTA's rows; or as many, where the two passes would scan them by the same tiles
+  // (below), or the cache is small (12K elements of K for every row of a chunk).  us, cluster against
+  // partial and combine pass, caches that together exceed L2 / one cache that stays in it, bf16:
+  // 12 heads, T 2048, d 64 8.6 against 16.5 / 8.2 against 9.7; 32 heads, T 2048, d 128 15.3 against
+  // 19.3 / 14.3 against 11.9; 24 heads, T 4096, d 64 14.2 against 17.9 / 13.5 against 11.7; 38 heads,
+  // T 4096, d 80 21.7 against 23.0 / 20.5 against 21.9.  Past the lines (32 heads, T 4096, d 128:
+  // 24.3 against 22.6 / 23.2 against 15.2; T 8192, 12 heads: 18 against 16; 64 heads, T 1024, d 128:
+  // 21 against 17) the CTAs are too few or come in waves.
+  const bool steps = (p.d == 128 || p.d == 64) && qal;  // the partial pass in two steps
   if (kCluster * heads <= 2 * nsm &&
       (n_chunks <= kCluster / 2 ||
-       (NQ > 0 && n_chunks <= kCluster && heads * p.d * (long long)sizeof(TI) <= 2048))) {
+       (NQ > 0 && n_chunks <= kCluster &&
+        (!steps || n_chunks * heads * p.d <= 12 * 1024)))) {
     if ((e = allow((const void*)cluster_kernel<TI, NQ>)) != cudaSuccess) return e;
     e = launch_pdl(cluster_kernel<TI, NQ>, dim3((unsigned)heads * kCluster), 32 * kClWarps, smem, s,
                    kCluster, p);
@@ -722,9 +725,9 @@ cudaError_t launch_t(const DecodeProblem& p, float* part, int n_chunks, cudaStre
     return e;
   }
   const dim3 grid((unsigned)heads, (unsigned)n_chunks);
-  if (NQ > 0 && p.d == 128 && qal) {
+  if (NQ > 0 && steps && p.d == 128) {
     e = launch_pdl(partial_kernel<TI, 128>, grid, 32 * kWarps, 0, s, 1, p, part);
-  } else if (NQ > 0 && p.d == 64 && qal) {
+  } else if (NQ > 0 && steps) {
     e = launch_pdl(partial_kernel<TI, 64>, grid, 32 * kWarps, 0, s, 1, p, part);
   } else if constexpr (NQ > 0) {
     if ((e = allow((const void*)scan_kernel<TI, NQ>)) != cudaSuccess) return e;
