@@ -166,8 +166,8 @@ relation_status relation_linear_fwd_ex(const void* p1, const void* p2, const voi
  * the state it starts from (stored in bf16 between the passes; three launches).
  *   workspace : device scratch of relation_linear_fwd_workspace_size(shp, dt) bytes
  *               (B H (d_h / 64) ceil(T / 128) d_h rows of 64 + 1 fp32, and
- *               B H (d_h / 64) (ceil(T / 128) + 1) d_h rows of 64 bf16),
- *               16-byte aligned, or RELATION_ERR_WORKSPACE / RELATION_ERR_ALIGNMENT with
+ *               B H (d_h / 64) (ceil(T / 128) + 1) d_h rows of 64 bf16, which hold no more
+ *               than what a base between two 256-byte boundaries skips), 16-byte aligned, or RELATION_ERR_WORKSPACE / RELATION_ERR_ALIGNMENT with
  *               nothing launched.
  * The chunk-parallel form runs where it takes less time (few such pairs, or a last round of
  * the SMs that is nearly empty), the sequential chunked kernel otherwise (same results up to
@@ -216,11 +216,12 @@ relation_status relation_linear_bwd(const void* p1, const void* p2, const void* 
  *                           then per block the gradients as tcgen05 products with bf16
  *                           operands and fp32 accumulation (three launches).  bf16 with d_h = 64,
  *                           element strides multiples of 8 (else RELATION_ERR_UNSUPPORTED or
- *                           RELATION_ERR_ALIGNMENT, nothing launched).  Workspace, in
- *                           256-byte-aligned parts, with n = ceil(T / 128): B H n 64 rows of 64
- *                           fp32 (the states' contributions, then the states), B H n 64 fp32,
- *                           and B H (n + 1) 64 and B H n 64 rows of 64 bf16 (together the
- *                           adjoints' contributions, then the adjoints).
+ *                           RELATION_ERR_ALIGNMENT, nothing launched).  Workspace, in parts
+ *                           that start at 256-byte boundaries, with n = ceil(T / 128): B H n 64
+ *                           rows of 64 fp32 (the states' contributions, then the states),
+ *                           B H n 64 fp32, and B H (n + 1) 64 and B H n 64 rows of 64 bf16
+ *                           (together the adjoints' contributions, then the adjoints, and what
+ *                           a base between two such boundaries skips).
  *                           The decay-range clamp and its report are the chunked forward's.
  *   RELATION_KERNEL_AUTO    the chunked kernel where it applies, else the recurrence.
  * workspace is 16-byte aligned and holds relation_linear_bwd_ex_workspace_size(shp, dt,
@@ -370,8 +371,9 @@ relation_status relation_bwd_ex(const void* q, const void* k, const void* v, con
                                 relation_kernel kernel, int* dev_status, relation_stream_t stream);
 
 /* Number of kernel launches one relation_fwd_ex (backward = 0) or relation_bwd_ex
- * (backward != 0) call makes for this dtype, head width and kernel request; 0 when the
- * request is not supported.  Host-only query. */
+ * (backward != 0) call makes for this dtype, head width and kernel request (one more in a
+ * CUDA-core backward whose dq stands in the place of q or dout); 0 when the request is not
+ * supported.  Host-only query. */
 int relation_launch_count(relation_dtype dt, int d_h, relation_kernel kernel, int backward);
 
 /* The backward as three stages, each launched only when its bit is set in `stages`:
