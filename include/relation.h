@@ -167,8 +167,8 @@ relation_status relation_linear_fwd_ex(const void* p1, const void* p2, const voi
  *   workspace : device scratch of relation_linear_fwd_workspace_size(shp, dt) bytes
  *               (B H (d_h / 64) ceil(T / 128) d_h rows of 64 + 1 fp32, and
  *               B H (d_h / 64) (ceil(T / 128) + 1) d_h rows of 64 bf16, which hold no more
- *               than what a base between two 256-byte boundaries skips), 16-byte aligned, or RELATION_ERR_WORKSPACE / RELATION_ERR_ALIGNMENT with
- *               nothing launched.
+ *               than what a base between two 256-byte boundaries skips), 16-byte aligned,
+ *               or RELATION_ERR_WORKSPACE / RELATION_ERR_ALIGNMENT with nothing launched.
  * The chunk-parallel form runs where it takes less time (few such pairs, or a last round of
  * the SMs that is nearly empty), the sequential chunked kernel otherwise (same results up to
  * rounding).  Requests the chunked
